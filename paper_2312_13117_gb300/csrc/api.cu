@@ -624,17 +624,25 @@ int run_level(Call& c, const std::vector<HostRegion>& regs, bool gate_top, bool 
   }
 
   // ---- waves of whole disks whose solutions fit the wave buffer ----
+  struct ResidentClass {
+    size_t off, count;
+    int max_n, max_l;
+  };
+  // work counters of a wave: FP64, mixed, small, then one per class of resident nodes
+  // (by CTAs per SM)
+  constexpr size_t kResidentClasses = 8, kCounters = 3 + kResidentClasses;
   struct Wave {
     int g0, g1;
     size_t items64_off, n64, items32_off, n32, itemsS_off, nS;
     size_t copies_off, n_copies;  // reused solutions copied into this wave's X
     int max_copy;
+    std::vector<ResidentClass> resident;  // FP64 nodes whose matrices stay in shared memory
   };
   std::vector<Wave> waves;
   std::vector<NodeItem> items;  // all waves: FP64 items then mixed items per wave
   std::vector<VecItem> copies;  // all waves
   size_t x_need = 0, reused_nodes = 0;
-  bool any64 = false, any32 = false, anyS = false;
+  bool any64 = false, any32 = false, anyS = false, anyF = false;
   int t64_n = 0;  // largest n of a precision-form problem with two or more dense terms
   int ysl_n = 0, ysl_nd = 0;  // largest n and dense-term count of the tensor-core residuals
   {
@@ -653,13 +661,17 @@ int run_level(Call& c, const std::vector<HostRegion>& regs, bool gate_top, bool 
       x_need = std::max(x_need, xb);
       // largest n first: the atomic work counter then hands out the long jobs early
       // small problems (n <= 32, l <= 16) go to the warp-per-node kernel whatever the form
-      std::vector<NodeItem> it64, it32, itS;
+      // FP64 nodes that fit shared memory go to the resident kernel, one launch per number of
+      // CTAs an SM holds, so that a small problem of a batch does not pay for a large one
+      std::vector<NodeItem> it64, it32, itS, itF[kResidentClasses];
       const size_t copies_off = copies.size();
       int max_copy = 0;
       for (int g = g0; g < g1; ++g) {
         const ProblemDev& P = c.pd[regs[g].prob];
+        const bool f64 = form_of(regs[g].prob) == PMCIM_PREC_FP64;
+        const int fit = f64 ? resident_ctas(P.n, P.l) : 0;
         std::vector<NodeItem>& dst = small_kernel_fits(P.n, P.l) ? itS
-                                     : (form_of(regs[g].prob) == PMCIM_PREC_FP64 ? it64 : it32);
+                                     : fit > 0 ? itF[fit - 1] : f64 ? it64 : it32;
         if (&dst == &it32 && ((P.n_dense >= 2 && !tc_residual(c.opt)) || P.bie)) t64_n = std::max(t64_n, P.n);
         if (&dst == &it32 && tc_residual(c.opt)) {
           ysl_n = std::max(ysl_n, P.n);
@@ -687,7 +699,7 @@ int run_level(Call& c, const std::vector<HostRegion>& regs, bool gate_top, bool 
       std::stable_sort(it64.begin(), it64.end(), by_n);
       std::stable_sort(it32.begin(), it32.end(), by_n);
       Wave wv{g0, g1, items.size(), it64.size(), 0, it32.size(), 0, itS.size(), copies_off,
-              copies.size() - copies_off, max_copy};
+              copies.size() - copies_off, max_copy, {}};
       items.insert(items.end(), it64.begin(), it64.end());
       wv.items32_off = items.size();
       items.insert(items.end(), it32.begin(), it32.end());
@@ -696,6 +708,18 @@ int run_level(Call& c, const std::vector<HostRegion>& regs, bool gate_top, bool 
       any64 |= !it64.empty();
       any32 |= !it32.empty();
       anyS |= !itS.empty();
+      for (std::vector<NodeItem>& f : itF) {
+        if (f.empty()) continue;
+        std::stable_sort(f.begin(), f.end(), by_n);
+        ResidentClass rc{items.size(), f.size(), 0, 0};
+        for (const NodeItem& it : f) {
+          rc.max_n = std::max(rc.max_n, c.pd[regs[it.region].prob].n);
+          rc.max_l = std::max(rc.max_l, c.pd[regs[it.region].prob].l);
+        }
+        items.insert(items.end(), f.begin(), f.end());
+        wv.resident.push_back(rc);
+        anyF = true;
+      }
       waves.push_back(wv);
       g0 = g1;
     }
@@ -708,8 +732,8 @@ int run_level(Call& c, const std::vector<HostRegion>& regs, bool gate_top, bool 
   }
   CU(ws.items.ensure(std::max<size_t>(1, items.size()) * sizeof(NodeItem)));
   CU(ws.regions.ensure(R * sizeof(RegionDev)));
-  // 3 work counters per wave, then the mixed kernel's error flag
-  CU(ws.counters.ensure((3 * waves.size() + 1) * sizeof(int)));
+  // the waves' work counters, then the mixed kernel's error flag
+  CU(ws.counters.ensure((kCounters * waves.size() + 1) * sizeof(int)));
   CU(cudaMemcpyAsync(ws.items.p, items.data(), items.size() * sizeof(NodeItem), cudaMemcpyHostToDevice, s));
   CU(cudaMemcpyAsync(ws.regions.p, rd.data(), R * sizeof(RegionDev), cudaMemcpyHostToDevice, s));
 
@@ -789,12 +813,13 @@ int run_level(Call& c, const std::vector<HostRegion>& regs, bool gate_top, bool 
   if (any64) CU(prepare_factor_fp64());
   if (any32) CU(prepare_factor_mixed());
   if (anyS) CU(prepare_factor_small());
+  if (anyF) CU(prepare_factor_resident());
 
   // ---- the level as one CUDA graph (profiler events become graph nodes) ----
   cudaGraph_t graph = nullptr;
   CU(cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal));
   auto capture = [&]() -> int {
-    CU(cudaMemsetAsync(ws.counters.p, 0, (3 * waves.size() + 1) * sizeof(int), s));
+    CU(cudaMemsetAsync(ws.counters.p, 0, (kCounters * waves.size() + 1) * sizeof(int), s));
     for (size_t wi = 0; wi < waves.size(); ++wi) {
       const Wave& wv = waves[wi];
       NodeArgs na;
@@ -815,14 +840,14 @@ int run_level(Call& c, const std::vector<HostRegion>& regs, bool gate_top, bool 
       na.max_n = max_n;
       na.max_sweeps = c.opt->max_ir_sweeps;
       na.tol_ir = c.opt->tol_ir > 0.0 ? c.opt->tol_ir : kIrTol;
-      na.err = ws.counters.as<int32_t>() + 3 * waves.size();
+      na.err = ws.counters.as<int32_t>() + kCounters * waves.size();
       na.tc_wait_cycles = wait_limit_tc();
       na.handoff_wait_cycles = wait_limit_handoff();
       if (wv.n64) {
         na.items = ws.items.as<NodeItem>() + wv.items64_off;
         na.n_items = (int)wv.n64;
         na.fp64_tile = fp64_tile;
-        na.counter = ws.counters.as<int>() + 3 * wi;
+        na.counter = ws.counters.as<int>() + kCounters * wi;
         na.work = ws.work64.as<char>();
         na.slot_bytes = slot64;
         na.piv = ws.piv64.as<int32_t>();
@@ -835,7 +860,7 @@ int run_level(Call& c, const std::vector<HostRegion>& regs, bool gate_top, bool 
       if (wv.n32) {
         na.items = ws.items.as<NodeItem>() + wv.items32_off;
         na.n_items = (int)wv.n32;
-        na.counter = ws.counters.as<int>() + 3 * wi + 1;
+        na.counter = ws.counters.as<int>() + kCounters * wi + 1;
         na.work = ws.work32.as<char>();
         na.slot_bytes = slot32;
         na.piv = ws.piv32.as<int32_t>();
@@ -853,10 +878,21 @@ int run_level(Call& c, const std::vector<HostRegion>& regs, bool gate_top, bool 
       if (wv.nS) {
         na.items = ws.items.as<NodeItem>() + wv.itemsS_off;
         na.n_items = (int)wv.nS;
-        na.counter = ws.counters.as<int>() + 3 * wi + 2;
+        na.counter = ws.counters.as<int>() + kCounters * wi + 2;
         na.phase = nullptr;
         prof_begin(PMCIM_K_FACTOR, s);
         CU(launch_factor_solve_small(na, s));
+        prof_end(PMCIM_K_FACTOR, s);
+      }
+      for (size_t k = 0; k < wv.resident.size(); ++k) {
+        const ResidentClass& rc = wv.resident[k];
+        na.items = ws.items.as<NodeItem>() + rc.off;
+        na.n_items = (int)rc.count;
+        na.max_n = rc.max_n;
+        na.counter = ws.counters.as<int>() + kCounters * wi + 3 + k;
+        na.phase = nullptr;
+        prof_begin(PMCIM_K_FACTOR, s);
+        CU(launch_factor_solve_resident(na, rc.max_l, s));
         prof_end(PMCIM_K_FACTOR, s);
       }
       LevelArgs lw = la;
@@ -913,7 +949,7 @@ int run_level(Call& c, const std::vector<HostRegion>& regs, bool gate_top, bool 
   }
   CU(cudaMemcpyAsync(out->node_info.data(), ws.node_info.p, total_nodes * sizeof(int32_t), cudaMemcpyDeviceToHost, s));
   int32_t handoff_err = 0;
-  CU(cudaMemcpyAsync(&handoff_err, ws.counters.as<int32_t>() + 3 * waves.size(), sizeof(int32_t),
+  CU(cudaMemcpyAsync(&handoff_err, ws.counters.as<int32_t>() + kCounters * waves.size(), sizeof(int32_t),
                      cudaMemcpyDeviceToHost, s));
   if (do_beyn) {
     out->p.resize(R);

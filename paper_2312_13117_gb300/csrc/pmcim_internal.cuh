@@ -271,6 +271,10 @@ bool small_kernel_fits(int n, int l);
 cudaError_t prepare_factor_small();
 cudaError_t launch_factor_solve_small(const NodeArgs& a, cudaStream_t s);
 int factor_slots_fp64(int n, int l);
+// FP64 nodes whose matrix and probe columns fit shared memory (lu_resident.cu)
+int resident_ctas(int n, int l);  // CTAs per SM, 0 when a node does not fit
+cudaError_t prepare_factor_resident();
+cudaError_t launch_factor_solve_resident(const NodeArgs& a, int max_l, cudaStream_t s);
 // Phases of the precision-form node kernel timed with clock64 when profiling.
 // assemble, LU panels, first solve, residual, correction solves, fallback, set-up,
 // LU triangular solves, LU trailing updates, 3 unused
