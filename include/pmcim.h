@@ -186,9 +186,9 @@ typedef struct {
   int32_t tc_timeouts;     /* nodes whose tensor-core wait ran out (their LU was
                               finished on the FMA pipes or the node re-solved in
                               FP64; results stay refined)                        */
-  int32_t node_ctas;       /* largest number of CTAs (one per SM) the precision
-                              form's node kernel ran with in the call: fewer than
-                              the SMs when device memory was short               */
+  int32_t node_ctas;       /* the SMs the precision form's factorisation ran on:
+                              fewer than the device has when a call has fewer
+                              nodes or device memory is short                    */
 } pmcim_stats;
 
 typedef struct pmcim_problem_s* pmcim_problem;
@@ -417,13 +417,11 @@ int pmcim_solve_points_noalloc(int32_t n, int32_t K, const pmcim_fterm* f, const
 typedef struct {
   int64_t launches[PMCIM_K_COUNT];
   double ms[PMCIM_K_COUNT]; /* summed event time; 0 unless timing was on */
-  /* precision-form node kernel, with timing on: SM clock cycles summed over
-     CTAs per phase: assembly, LU panels, first solve, FP64 residual,
-     correction solves, FP64 fallback, node set-up, LU triangular solves
-     (U12), LU trailing updates, factor group waiting for a free slot, refine
-     group waiting for a factored node, then the CTAs' lifetimes in ns
-     (globaltimer, summed), then the LU panels' row interchanges on the columns
-     outside the panel (counted apart from the panels); 3 unused */
+  /* precision form, with timing on: SM clock cycles summed over the CTAs of its
+     kernels per step: assembly, LU panels, first solve, residual, correction
+     solves, FP64 fallback, node set-up, LU triangular solves (U12), LU trailing
+     updates, 2 unused, the CTAs' lifetimes in ns (globaltimer, summed), the LU
+     panels' row interchanges on the columns outside the panel; 3 unused */
   double mixed_phase_cycles[PMCIM_PHASE_COUNT];
 } pmcim_profile;
 
@@ -432,18 +430,19 @@ void pmcim_profile_reset(void);
 void pmcim_profile_read(pmcim_profile* out);
 
 /* Limits, in SM clock cycles, of the two kinds of bounded device waits in the
-   precision-form node kernel (no counterpart in the paper; for testing the
-   paths taken when a wait runs out). tc_wait_cycles bounds each wait for a
-   tensor-core commit inside the LU's trailing update: when one runs out the
-   node's LU is finished on the FMA pipes, the node is counted in
-   stats.tc_timeouts, and its refinement (or its FP64 re-solve) still delivers
-   an FP64-accurate solution. handoff_wait_cycles bounds each wait between the
-   kernel's two thread groups: when one runs out both groups end and the call
-   returns PMCIM_ETIMEOUT; the handle stays usable. 0 restores a default
-   (2^30 and 2^35 cycles, about 0.5 s and 16 s at 2 GHz). Process-wide; takes
-   effect for launches prepared after the call. The final wait for a commit in
-   flight before the kernel frees its tensor memory always uses the default.
-   EINVAL for a negative limit. */
+   precision form's kernels (no counterpart in the paper; for testing the paths
+   taken when a wait runs out). tc_wait_cycles bounds each wait for a tensor-core
+   commit inside the LU's trailing update (when one runs out the node's LU is
+   finished on the FMA pipes) and each wait for operands of the refinement
+   residual (its nodes are solved again in FP64); the node is counted in
+   stats.tc_timeouts and still gets an FP64-accurate solution.
+   handoff_wait_cycles bounds each wait between the residual kernel's warp
+   groups: when one runs out the kernel ends and the call returns
+   PMCIM_ETIMEOUT; the handle stays usable. 0 restores a default (2^30 and 2^35
+   cycles, about 0.5 s and 16 s at 2 GHz). Process-wide; takes effect for
+   launches prepared after the call. The final wait for a commit in flight before
+   a kernel frees its tensor memory always uses the default. EINVAL for a
+   negative limit. */
 int pmcim_debug_wait_limits(int64_t tc_wait_cycles, int64_t handoff_wait_cycles);
 
 #ifdef __cplusplus

@@ -97,9 +97,14 @@ struct DevBuf {
 
 // Upper bound on the node solutions kept before one reduction (one HBM wave).
 constexpr size_t kWaveBytes = size_t(16) << 30;
-// Upper bound on the per-CTA factorisation workspaces of one form: at n = 2048 the
-// precision form's 152 CTAs need 41 GB (two complex64 slots and two FP64 T(z_j) each).
+// Upper bound on the factorisation workspaces of one form.
 constexpr size_t kSlotBytes = size_t(48) << 30;
+// The precision forms keep every node of a chunk in device memory. A chunk takes up to
+// this much, but at least kChunkNodesPerSm nodes per SM where kSlotBytes allows: the last
+// wave of two nodes per SM is then at most a quarter of a chunk (n = 1024, l = 16: 1500
+// nodes of 10.6 MB; n = 2048, l = 48: 608 of 47 MB).
+constexpr size_t kChunkBytes = size_t(16) << 30;
+constexpr int kChunkNodesPerSm = 4;
 // indicator-pass solutions kept for reuse by the two-pass schedule, per chunk of disks
 constexpr size_t kKeepBytes = size_t(8) << 30;
 // largest pmCIMa level (disks); beyond it the indicator is marking noise
@@ -196,6 +201,12 @@ void prof_begin(int kind, cudaStream_t s) {
   P.cur_begin[kind] = e;
 }
 
+void prof_count(int kind, int launches) {
+  Prof& P = prof();
+  std::lock_guard<std::mutex> g(P.mu);
+  P.launches[kind] += launches;
+}
+
 void prof_end(int kind, cudaStream_t s) {
   Prof& P = prof();
   std::lock_guard<std::mutex> g(P.mu);
@@ -231,7 +242,8 @@ long long wait_limit_handoff() {
 // Device workspaces, reused across calls on one handle.
 struct Workspace {
   DevBuf probs, regions, items, counters, node_info, X;
-  DevBuf work64, piv64, work32, piv32, t64, phase;
+  DevBuf work64, piv64, work32, t64, phase;
+  DevBuf mstate, mctl, mlists, mubase;  // precision forms: node states, counters, node lists, list bases
   DevBuf C0, C1, pf_half, pf_abs, ind, pf_norm, pf_scale, cand;
   DevBuf bwork, bsigma, bp, blam, bvecs, bkept, bstatus;
   DevBuf vlam, vprob, voff, vsig, vacc, vwork, vvec, vpiv;
@@ -242,7 +254,7 @@ struct Workspace {
   DevBuf ind3, feats, sprob, sparams, sscratch;
   // verification's inverse-iteration step: per-value problem table, pseudo-disks, items, solutions
   DevBuf iprobs, iregions, iitems, iX, iinfo, icounters, ibord, ioffs;
-  DevBuf ysl;                        // per slot: digits of f_k X for the tensor-core residual
+  DevBuf ysl, gexp;                  // per slot: digits of f_k X for the tensor-core residual, exponents
   DevBuf rz, rX, rR, rstat, rysl;    // pmcim_residual: points, solutions, residuals, status, scratch
   DevBuf cW, cidx, cgram, gpart;     // certificates from coefficient products: W, index arrays, Gram data
   // the library's own stream: graphs cannot be captured on the legacy default stream
@@ -253,11 +265,11 @@ struct Workspace {
     if (ordered) cudaEventDestroy(ordered);
     stream = nullptr;
     ordered = nullptr;
-    DevBuf* b[] = {&probs, &regions, &items, &counters, &node_info, &X, &work64, &piv64, &work32, &piv32, &t64,
-                   &phase, &C0, &C1, &pf_half, &pf_abs, &ind, &pf_norm, &pf_scale, &cand, &bwork, &bsigma,
+    DevBuf* b[] = {&probs, &regions, &items, &counters, &node_info, &X, &work64, &piv64, &work32, &t64,
+                   &phase, &mstate, &mctl, &mlists, &mubase, &C0, &C1, &pf_half, &pf_abs, &ind, &pf_norm, &pf_scale, &cand, &bwork, &bsigma,
                    &bp, &blam, &bvecs, &bkept, &bstatus, &vlam, &vprob, &voff, &vsig, &vacc, &vwork,
                    &vvec, &vpiv, &gitems, &gdst, &gperm, &ind3, &feats, &sprob, &sparams, &sscratch, &Xkeep,
-                   &citems, &vout, &Cm, &iprobs, &iregions, &iitems, &iX, &iinfo, &icounters, &ibord, &ioffs, &ysl, &rz,
+                   &citems, &vout, &Cm, &iprobs, &iregions, &iitems, &iX, &iinfo, &icounters, &ibord, &ioffs, &ysl, &gexp, &rz,
                    &rX, &rR, &rstat, &rysl, &cW, &cidx, &cgram, &gpart};
     for (DevBuf* x : b) x->release();
   }
@@ -448,6 +460,135 @@ int n_bucket(int n) {
   int b = 0;
   while ((32 << b) < n) ++b;  // buckets (..32], (32,64], (64,128], ...
   return b;
+}
+
+// ===========================================================================
+// Precision forms: nodes in chunks, each chunk in slots of device memory
+// ===========================================================================
+struct MixedChunk {
+  size_t off, count;  // in the item list
+  int max_n, max_l;
+  int tc;
+};
+
+// The chunks of a call's precision-form nodes, their workspaces and the arguments they share.
+struct MixedPlan {
+  std::vector<std::vector<MixedChunk>> chunks;  // per wave
+  std::vector<int> ubase;                       // per chunk and problem: first unit of its list
+  size_t n_probs = 0, max_count = 0;
+  size_t work = 0, t64 = 0, ysl = 0;
+  size_t t64_stride = 0, ysl_stride = 0;
+  int gexp_stride = 0;
+  int unit_cap = 0;
+};
+
+// Plans a wave's nodes items[off .. off + count) (largest n first).
+void plan_mixed(Workspace& ws, const std::vector<ProblemDev>& pd, const std::vector<RegionDev>& rd,
+                const std::vector<NodeItem>& items, size_t off, size_t count, bool oz, int sms, MixedPlan* mp) {
+  mp->n_probs = pd.size();
+  mp->chunks.emplace_back();
+  if (count == 0) return;
+  int max_l = 1, t64_n = 0, nd = 0;
+  size_t ysl = 0;
+  for (size_t i = 0; i < count; ++i) {
+    const RegionDev& r = rd[items[off + i].region];
+    const ProblemDev& P = pd[r.prob];
+    max_l = std::max(max_l, P.l);
+    if (r.herm || P.bie || (P.n_dense >= 2 && !oz)) t64_n = std::max(t64_n, P.n);
+    if (oz && !r.herm && !P.bie) {
+      ysl = std::max(ysl, oz_slot_bytes(P.n, P.l, P.n_dense));
+      nd = std::max(nd, P.n_dense);
+    }
+  }
+  mp->t64_stride = std::max(mp->t64_stride, (size_t)t64_n * t64_n);
+  mp->ysl_stride = std::max(mp->ysl_stride, ysl);
+  mp->gexp_stride = std::max(mp->gexp_stride, nd * PMCIM_MAX_L);
+  const size_t budget = slot_budget(ws.work32.cap + ws.t64.cap + ws.ysl.cap);
+  for (size_t i = 0; i < count;) {
+    MixedChunk ch{off + i, 0, pd[rd[items[off + i].region].prob].n, max_l, 0};
+    const size_t slot = mixed_slot_bytes(ch.max_n, ch.max_l);
+    const size_t per = slot + mp->t64_stride * sizeof(double2) + mp->ysl_stride;
+    const size_t cap = std::max<size_t>(
+        1, std::min(budget / per, std::max<size_t>(kChunkBytes / per, (size_t)kChunkNodesPerSm * sms)));
+    ch.count = std::min(cap, count - i);
+    std::vector<int> units(pd.size(), 0);
+    for (size_t k = 0; k < ch.count; ++k) {
+      const RegionDev& r = rd[items[off + i + k].region];
+      units[r.prob] += (pd[r.prob].l + 7) / 8;
+      ch.tc |= r.lu_tc != 0;
+    }
+    int base = 0;
+    for (int u : units) {
+      mp->ubase.push_back(base);
+      base += u;
+    }
+    mp->unit_cap = std::max(mp->unit_cap, base);
+    mp->max_count = std::max(mp->max_count, ch.count);
+    mp->work = std::max(mp->work, std::max(ch.count * slot, mixed_fallback_bytes(ch.max_n, ch.max_l)));
+    mp->chunks.back().push_back(ch);
+    i += ch.count;
+  }
+}
+
+// Allocates what the plan needs and fills the arguments that all chunks share.
+int ensure_mixed(Call& c, const MixedPlan& mp, int max_sweeps, MixedArgs* ma) {
+  Workspace& ws = *c.ws;
+  std::memset(ma, 0, sizeof(*ma));
+  const size_t cnt = mp.max_count;
+  CU(ws.work32.ensure(mp.work));
+  if (mp.t64_stride) CU(ws.t64.ensure(cnt * mp.t64_stride * sizeof(double2)));
+  if (mp.ysl_stride) CU(ws.ysl.ensure(cnt * mp.ysl_stride));
+  if (mp.gexp_stride) CU(ws.gexp.ensure(cnt * mp.gexp_stride * sizeof(int32_t)));
+  CU(ws.mstate.ensure(cnt * sizeof(MixedState)));
+  CU(ws.mctl.ensure(mixed_ctl_ints((int)mp.n_probs, max_sweeps) * sizeof(int)));
+  CU(ws.mlists.ensure((3 * cnt + 2 * (size_t)mp.unit_cap) * sizeof(int)));
+  CU(ws.mubase.ensure(std::max<size_t>(1, mp.ubase.size()) * sizeof(int)));
+  CU(cudaMemcpyAsync(ws.mubase.p, mp.ubase.data(), mp.ubase.size() * sizeof(int), cudaMemcpyHostToDevice, c.s));
+  CU(prepare_factor_mixed());
+  ma->n_probs = (int)mp.n_probs;
+  ma->work = ws.work32.as<char>();
+  ma->work_bytes = mp.work;
+  ma->t64 = mp.t64_stride ? ws.t64.as<double2>() : nullptr;
+  ma->t64_stride = mp.t64_stride;
+  ma->ysl = mp.ysl_stride ? ws.ysl.as<unsigned char>() : nullptr;
+  ma->ysl_stride = mp.ysl_stride;
+  ma->oz = mp.ysl_stride ? 1 : 0;
+  ma->gexp = ws.gexp.as<int32_t>();
+  ma->gexp_stride = mp.gexp_stride;
+  ma->state = ws.mstate.as<MixedState>();
+  ma->ctl = ws.mctl.as<int>();
+  ma->act = ws.mlists.as<int>();
+  ma->fallback = ma->act + 2 * cnt;
+  ma->units = ma->fallback + cnt;
+  ma->unit_cap = mp.unit_cap;
+  ma->slots = (int)cnt;
+  ma->max_sweeps = max_sweeps;
+  ma->bie = any_bie(c.groups) ? 1 : 0;
+  ma->tc_wait_cycles = wait_limit_tc();
+  ma->handoff_wait_cycles = wait_limit_handoff();
+  return PMCIM_OK;
+}
+
+// One wave's chunks. items: the device item list; chunk0: index of the wave's first chunk.
+int launch_mixed(const MixedPlan& mp, size_t wave, size_t chunk0, const MixedArgs& shared, const NodeItem* items,
+                 int sms, int prof_kind, cudaStream_t s, const int* d_ubase) {
+  for (size_t k = 0; k < mp.chunks[wave].size(); ++k) {
+    const MixedChunk& ch = mp.chunks[wave][k];
+    MixedArgs a = shared;
+    a.items = items + ch.off;
+    a.count = (int)ch.count;
+    a.max_n = ch.max_n;
+    a.max_l = ch.max_l;
+    a.slot_bytes = mixed_slot_bytes(ch.max_n, ch.max_l);
+    a.tc = ch.tc;
+    a.ubase = d_ubase + (chunk0 + k) * mp.n_probs;
+    int launched = 0;
+    prof_begin(prof_kind, s);
+    CU(launch_factor_solve_mixed(a, sms, s, &launched));
+    prof_end(prof_kind, s);
+    prof_count(prof_kind, launched - 1);
+  }
+  return PMCIM_OK;
 }
 
 struct LevelOut {
@@ -643,8 +784,6 @@ int run_level(Call& c, const std::vector<HostRegion>& regs, bool gate_top, bool 
   std::vector<VecItem> copies;  // all waves
   size_t x_need = 0, reused_nodes = 0;
   bool any64 = false, any32 = false, anyS = false, anyF = false;
-  int t64_n = 0;  // largest n of a precision-form problem with two or more dense terms
-  int ysl_n = 0, ysl_nd = 0;  // largest n and dense-term count of the tensor-core residuals
   {
     int g0 = 0;
     while (g0 < R) {
@@ -672,11 +811,6 @@ int run_level(Call& c, const std::vector<HostRegion>& regs, bool gate_top, bool 
         const int fit = f64 ? resident_ctas(P.n, P.l) : 0;
         std::vector<NodeItem>& dst = small_kernel_fits(P.n, P.l) ? itS
                                      : fit > 0 ? itF[fit - 1] : f64 ? it64 : it32;
-        if (&dst == &it32 && ((P.n_dense >= 2 && !tc_residual(c.opt)) || P.bie)) t64_n = std::max(t64_n, P.n);
-        if (&dst == &it32 && tc_residual(c.opt)) {
-          ysl_n = std::max(ysl_n, P.n);
-          ysl_nd = std::max(ysl_nd, P.n_dense);
-        }
         const bool re = reuse && reuse->src[g] >= 0;
         const int nl = P.n * P.l;
         for (int j = 0; j < regs[g].N; ++j) {
@@ -751,8 +885,8 @@ int run_level(Call& c, const std::vector<HostRegion>& regs, bool gate_top, bool 
   }
   // ---- factorisation workspaces, one slot per resident CTA ----
   const int sms = num_sms();
-  int slots64 = 0, slots32 = 0;
-  size_t slot64 = 0, slot32 = 0, t64_stride = 0, ysl_stride = 0;
+  int slots64 = 0;
+  size_t slot64 = 0;
   if (any64) {
     slot64 = (size_t)max_n * (max_n + max_l) * sizeof(double2);
     const size_t budget = slot_budget(ws.work64.cap);
@@ -760,27 +894,19 @@ int run_level(Call& c, const std::vector<HostRegion>& regs, bool gate_top, bool 
     CU(ws.work64.ensure((size_t)slots64 * slot64));
     CU(ws.piv64.ensure((size_t)slots64 * max_n * sizeof(int32_t)));
   }
+  MixedPlan mp;
+  MixedArgs ma;
   if (any32) {
-    // one CTA per SM, each cycling through mixed_slots_per_cta() slots
-    slot32 = mixed_slot_bytes(max_n, max_l);
-    const size_t per = (size_t)mixed_slots_per_cta();
-    t64_stride = (size_t)t64_n * t64_n;  // FP64 T(z_j) of each slot
-    ysl_stride = y_digit_scratch_bytes(ysl_n, ysl_nd);
-    const size_t cta_bytes = per * (slot32 + t64_stride * sizeof(double2) + ysl_stride);
-    const size_t budget = slot_budget(ws.work32.cap + ws.t64.cap + ws.ysl.cap);
-    const size_t ctas = std::max<size_t>(1, std::min<size_t>(std::min<size_t>(sms, budget / cta_bytes),
-                                                             total_nodes));
-    slots32 = (int)(ctas * per);
-    c.st.node_ctas = std::max(c.st.node_ctas, (int32_t)ctas);
-    CU(ws.work32.ensure((size_t)slots32 * slot32));
-    CU(ws.piv32.ensure((size_t)slots32 * max_n * sizeof(int32_t)));
-    if (t64_stride) CU(ws.t64.ensure((size_t)slots32 * t64_stride * sizeof(double2)));
-    if (ysl_stride) CU(ws.ysl.ensure((size_t)slots32 * ysl_stride));
+    for (const Wave& wv : waves)
+      plan_mixed(ws, c.pd, rd, items, wv.items32_off, wv.n32, tc_residual(c.opt), sms, &mp);
+    CHK(ensure_mixed(c, mp, c.opt->max_ir_sweeps, &ma));
+    c.st.node_ctas = std::max(c.st.node_ctas, (int32_t)std::min<size_t>(sms, mp.max_count));
   }
   const bool timed = prof_on();
+  const int phase_ctas = 3 * sms;  // the largest grid of the precision form's kernels
   if (timed && any32) {
-    CU(ws.phase.ensure((size_t)slots32 * PMCIM_PHASES * sizeof(unsigned long long)));
-    CU(cudaMemsetAsync(ws.phase.p, 0, (size_t)slots32 * PMCIM_PHASES * sizeof(unsigned long long), s));
+    CU(ws.phase.ensure((size_t)phase_ctas * PMCIM_PHASES * sizeof(unsigned long long)));
+    CU(cudaMemsetAsync(ws.phase.p, 0, (size_t)phase_ctas * PMCIM_PHASES * sizeof(unsigned long long), s));
   }
 
   LevelArgs la;
@@ -811,15 +937,30 @@ int run_level(Call& c, const std::vector<HostRegion>& regs, bool gate_top, bool 
   la.status = ws.bstatus.as<int32_t>();
 
   if (any64) CU(prepare_factor_fp64());
-  if (any32) CU(prepare_factor_mixed());
   if (anyS) CU(prepare_factor_small());
   if (anyF) CU(prepare_factor_resident());
 
+  if (any32) {
+    ma.probs = la.probs;
+    ma.regions = la.regions;
+    ma.X = xbuf.as<double2>();
+    ma.node_info = ws.node_info.as<int32_t>();
+    ma.tol_ir = c.opt->tol_ir > 0.0 ? c.opt->tol_ir : kIrTol;
+    ma.err = ws.counters.as<int32_t>() + kCounters * waves.size();
+    ma.phase = timed ? ws.phase.as<unsigned long long>() : nullptr;
+    // nodes whose residuals have no coefficient digits
+    for (const NodeItem& it : items) {
+      const ProblemDev& P = c.pd[rd[it.region].prob];
+      if (P.bie || P.n_dense == 0) ma.res64 = 1;
+    }
+    if (!tc_residual(c.opt)) ma.res64 = 1;
+  }
   // ---- the level as one CUDA graph (profiler events become graph nodes) ----
   cudaGraph_t graph = nullptr;
   CU(cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal));
   auto capture = [&]() -> int {
     CU(cudaMemsetAsync(ws.counters.p, 0, (kCounters * waves.size() + 1) * sizeof(int), s));
+    size_t chunk0 = 0;
     for (size_t wi = 0; wi < waves.size(); ++wi) {
       const Wave& wv = waves[wi];
       NodeArgs na;
@@ -838,11 +979,6 @@ int run_level(Call& c, const std::vector<HostRegion>& regs, bool gate_top, bool 
       }
       na.node_info = ws.node_info.as<int32_t>();
       na.max_n = max_n;
-      na.max_sweeps = c.opt->max_ir_sweeps;
-      na.tol_ir = c.opt->tol_ir > 0.0 ? c.opt->tol_ir : kIrTol;
-      na.err = ws.counters.as<int32_t>() + kCounters * waves.size();
-      na.tc_wait_cycles = wait_limit_tc();
-      na.handoff_wait_cycles = wait_limit_handoff();
       if (wv.n64) {
         na.items = ws.items.as<NodeItem>() + wv.items64_off;
         na.n_items = (int)wv.n64;
@@ -852,34 +988,19 @@ int run_level(Call& c, const std::vector<HostRegion>& regs, bool gate_top, bool 
         na.slot_bytes = slot64;
         na.piv = ws.piv64.as<int32_t>();
         na.slots = slots64;
-        na.phase = nullptr;
         prof_begin(PMCIM_K_FACTOR, s);
         CU(launch_factor_solve_fp64(na, s));
         prof_end(PMCIM_K_FACTOR, s);
       }
       if (wv.n32) {
-        na.items = ws.items.as<NodeItem>() + wv.items32_off;
-        na.n_items = (int)wv.n32;
-        na.counter = ws.counters.as<int>() + kCounters * wi + 1;
-        na.work = ws.work32.as<char>();
-        na.slot_bytes = slot32;
-        na.piv = ws.piv32.as<int32_t>();
-        na.slots = slots32;
-        na.t64 = t64_stride ? ws.t64.as<double2>() : nullptr;
-        na.t64_stride = t64_stride;
-        na.oz = tc_residual(c.opt) ? 1 : 0;
-        na.ysl = ysl_stride ? ws.ysl.as<unsigned char>() : nullptr;
-        na.ysl_stride = ysl_stride;
-        na.phase = timed ? ws.phase.as<unsigned long long>() : nullptr;
-        prof_begin(PMCIM_K_FACTOR32, s);
-        CU(launch_factor_solve_mixed(na, s));
-        prof_end(PMCIM_K_FACTOR32, s);
+        CHK(launch_mixed(mp, wi, chunk0, ma, ws.items.as<NodeItem>(), sms, PMCIM_K_FACTOR32, s,
+                         ws.mubase.as<int>()));
+        chunk0 += mp.chunks[wi].size();
       }
       if (wv.nS) {
         na.items = ws.items.as<NodeItem>() + wv.itemsS_off;
         na.n_items = (int)wv.nS;
         na.counter = ws.counters.as<int>() + kCounters * wi + 2;
-        na.phase = nullptr;
         prof_begin(PMCIM_K_FACTOR, s);
         CU(launch_factor_solve_small(na, s));
         prof_end(PMCIM_K_FACTOR, s);
@@ -890,7 +1011,6 @@ int run_level(Call& c, const std::vector<HostRegion>& regs, bool gate_top, bool 
         na.n_items = (int)rc.count;
         na.max_n = rc.max_n;
         na.counter = ws.counters.as<int>() + kCounters * wi + 3 + k;
-        na.phase = nullptr;
         prof_begin(PMCIM_K_FACTOR, s);
         CU(launch_factor_solve_resident(na, rc.max_l, s));
         prof_end(PMCIM_K_FACTOR, s);
@@ -962,14 +1082,14 @@ int run_level(Call& c, const std::vector<HostRegion>& regs, bool gate_top, bool 
     CU(cudaMemcpyAsync(out->kept.data(), ws.bkept.p, (size_t)R * PMCIM_MAX_L, cudaMemcpyDeviceToHost, s));
   }
   if (timed && any32) {
-    std::vector<unsigned long long> cyc((size_t)slots32 * PMCIM_PHASES);
+    std::vector<unsigned long long> cyc((size_t)phase_ctas * PMCIM_PHASES);
     CU(cudaMemcpyAsync(cyc.data(), ws.phase.p, cyc.size() * sizeof(unsigned long long), cudaMemcpyDeviceToHost, s));
     CU(cudaStreamSynchronize(s));
-    prof_add_phases(cyc.data(), slots32);
+    prof_add_phases(cyc.data(), phase_ctas);
   }
   CU(cudaStreamSynchronize(s));
   if (handoff_err)
-    return fail(PMCIM_ETIMEOUT, "precision-form node kernel: a wait between its thread groups ran out");
+    return fail(PMCIM_ETIMEOUT, "precision form: a wait between a kernel's warp groups ran out");
   if (reuse)  // reused nodes were not solved here: their info words are stale
     for (int g = 0; g < R; ++g)
       if (reuse->src[g] >= 0)
@@ -1344,7 +1464,7 @@ int run_bordered_step(Call& c, const std::vector<double2>& lam_in, const std::ve
   std::vector<int32_t> prob_of(m);
   std::vector<int64_t> x_off(m), b_off(m, -1);
   size_t x_tot = 0, b_tot = 0;
-  int max_n = 1, t64_n = 0;
+  int max_n = 1;
   // the bordered right-hand sides and replacement columns: 2 n per value
   for (int i = 0; i < m; ++i) {
     const int n = c.pd[prob_in[i]].n;
@@ -1382,7 +1502,6 @@ int run_bordered_step(Call& c, const std::vector<double2>& lam_in, const std::ve
       pdv[i].V = bord + b_off[i];       // b; the column alpha c follows it
       d.v_off = b_off[i] + n;           // d.border is set on the device
       it32.push_back(NodeItem{i, 0});
-      t64_n = std::max(t64_n, n);  // T^H in FP64 for the residuals
     }
   }
   std::stable_sort(it32.begin(), it32.end(), [&](const NodeItem& a, const NodeItem& b) {
@@ -1430,55 +1549,33 @@ int run_bordered_step(Call& c, const std::vector<double2>& lam_in, const std::ve
     CU(launch_border_rhs(va, d_b_off, ws.ibord.as<double2>(), ws.iregions.as<RegionDev>(), s));
     prof_end(PMCIM_K_VERIFY, s);
   }
-  NodeArgs na;
-  std::memset(&na, 0, sizeof(na));
-  na.bie = any_bie(c.groups) ? 1 : 0;
-  na.probs = ws.iprobs.as<ProblemDev>();
-  na.regions = ws.iregions.as<RegionDev>();
-  na.X = ws.iX.as<double2>();
-  na.node_info = ws.iinfo.as<int32_t>();
-  na.max_n = max_n;
-  na.max_sweeps = std::max(1, c.opt->max_ir_sweeps);
-  na.tol_ir = kIrTol;
-  na.err = ws.icounters.as<int32_t>() + 3;
-  na.tc_wait_cycles = wait_limit_tc();
-  na.handoff_wait_cycles = wait_limit_handoff();
-  na.border = bord;
   const int sms = num_sms();
   if (!it32.empty()) {
-    const size_t slot32 = mixed_slot_bytes(max_n, 1);
-    const size_t per = (size_t)mixed_slots_per_cta();
-    const size_t t64_stride = (size_t)t64_n * t64_n;
-    const size_t cta_bytes = per * (slot32 + t64_stride * sizeof(double2));
-    const size_t budget = slot_budget(ws.work32.cap + ws.t64.cap);
-    // one value per CTA (its other slot idle): the values are few, and a CTA works
-    // through its slots one node after another
-    const size_t ctas = std::max<size_t>(1, std::min<size_t>(std::min<size_t>(sms, budget / cta_bytes),
-                                                             it32.size()));
-    const int slots32 = (int)(ctas * per);
-    CU(ws.work32.ensure((size_t)slots32 * slot32));
-    CU(ws.piv32.ensure((size_t)slots32 * max_n * sizeof(int32_t)));
-    CU(ws.t64.ensure((size_t)slots32 * t64_stride * sizeof(double2)));
-    CU(prepare_factor_mixed());
-    na.oz = 0;
-    na.ysl = nullptr;
-    na.ysl_stride = 0;
-    na.items = ws.iitems.as<NodeItem>();
-    na.n_items = (int)it32.size();
-    na.counter = ws.icounters.as<int>() + 1;
-    na.work = ws.work32.as<char>();
-    na.slot_bytes = slot32;
-    na.piv = ws.piv32.as<int32_t>();
-    na.slots = slots32;
-    na.t64 = ws.t64.as<double2>();
-    na.t64_stride = t64_stride;
-    na.phase = nullptr;
-    prof_begin(PMCIM_K_VERIFY, s);  // verification work, timed apart from the disks' nodes
-    CU(launch_factor_solve_mixed(na, s));
-    prof_end(PMCIM_K_VERIFY, s);
+    MixedPlan mp;
+    MixedArgs ma;
+    plan_mixed(ws, pdv, rdv, items, 0, it32.size(), false, sms, &mp);
+    CHK(ensure_mixed(c, mp, std::max(1, c.opt->max_ir_sweeps), &ma));
+    ma.probs = ws.iprobs.as<ProblemDev>();
+    ma.regions = ws.iregions.as<RegionDev>();
+    ma.X = ws.iX.as<double2>();
+    ma.node_info = ws.iinfo.as<int32_t>();
+    ma.tol_ir = kIrTol;
+    ma.err = ws.icounters.as<int32_t>() + 3;
+    ma.res64 = 1;
+    ma.border = bord;
+    // verification work, timed apart from the disks' nodes
+    CHK(launch_mixed(mp, 0, 0, ma, ws.iitems.as<NodeItem>(), sms, PMCIM_K_VERIFY, s, ws.mubase.as<int>()));
   }
   if (!itS.empty()) {
     CU(prepare_factor_small());
+    NodeArgs na;
+    std::memset(&na, 0, sizeof(na));
+    na.bie = any_bie(c.groups) ? 1 : 0;
+    na.probs = ws.iprobs.as<ProblemDev>();
+    na.regions = ws.iregions.as<RegionDev>();
+    na.X = ws.iX.as<double2>();
+    na.node_info = ws.iinfo.as<int32_t>();
+    na.max_n = max_n;
     na.items = ws.iitems.as<NodeItem>() + it32.size();
     na.n_items = (int)itS.size();
     na.counter = ws.icounters.as<int>() + 2;
@@ -1499,7 +1596,7 @@ int run_bordered_step(Call& c, const std::vector<double2>& lam_in, const std::ve
   CU(cudaMemcpyAsync(&handoff_err, ws.icounters.as<int32_t>() + 3, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
   CU(cudaStreamSynchronize(s));
   if (handoff_err)
-    return fail(PMCIM_ETIMEOUT, "precision-form node kernel: a wait between its thread groups ran out");
+    return fail(PMCIM_ETIMEOUT, "precision form: a wait between a kernel's warp groups ran out");
   // a value whose certificate is not finite (e.g. an exactly singular T(lambda)) is left
   // to the full sigma_min computation
   for (int i = 0; i < m; ++i)

@@ -7,7 +7,7 @@
 // the FP64 coefficients A_k, and the accumulated solution X.
 //
 // Per node:
-//   1. assemble T(z_j) in FP64 and round to complex64, append V;
+//   1. assemble T(z_j), rounded to complex64, append V;
 //   2. FP32 blocked LU with partial pivoting (also eliminates V), back
 //      substitution -> X_0 (promoted to FP64);
 //   3. sweeps s = 1..max: R = V - T(z_j) X in FP64; delta = LU^-1 (R / |R|max)
@@ -15,16 +15,22 @@
 //      error |delta_s|^2 / |delta_{s-1}| (|delta_0| = |X_0|) is below
 //      tol_ir |X| (max norms);
 //   4. no convergence within max sweeps (or growth) -> the node is solved
-//      again by the FP64 LU in the same workspace and flagged.
-// Steps 1-2 are FP32 (or tensor-core) work, step 3 is FP64 work. One
-// persistent CTA per SM runs them in two warp-specialised groups of 256
-// threads: the factor group (warps 0-7) does steps 1-2 for node k+1 while the
-// refine group (warps 8-15) does steps 3-4 for node k, so the FP64 pipe and
-// the FP32 / tensor pipes of the SM work at the same time. Nodes pass between
-// the groups through three workspace slots per CTA (the factor group can run up
-// to two nodes ahead), each guarded by a pair of mbarriers (full: factor ->
-// refine, empty: refine -> factor); every wait on them is bounded and a wait
-// that runs out ends both groups with an error. The trailing updates of step 2
+//      again by the FP64 LU and flagged.
+//
+// A launch's nodes go through these steps together, one kernel per step, each
+// node's factors staying in a slot of its own in device memory:
+//   k_mixed_factor    steps 1-2 up to the triangular factors, two CTAs per SM;
+//   k_mixed_solve     the back substitution, and each sweep's correction;
+//   k_oz_digits,      (oz_refine.cu) the residuals of all active nodes as one
+//   k_oz_residual     product with the coefficients, which all nodes of a problem
+//                     share: the coefficient digits are read once for 32 solution
+//                     columns of any nodes;
+//   k_mixed_fallback  step 4.
+// The kernels of a sweep read the list of nodes that still refine, which the sweep
+// before appended to; with none left they return at once. Every step is bound by
+// latency when one node has an SM to itself (block barriers, global round trips),
+// so what counts is how many nodes an SM works on at a time; in one kernel per node
+// the residual's tensor memory and operand stages allowed one. The trailing updates
 // run on the FMA pipes, or, for regions marked lu_tc, as complex products on the
 // tensor cores: 3xTF32 (tc_update.cuh) or BF16 3M (tc_update_bf16.cuh).
 // node_info: bits 0-23 = 0 or 1 + first zero-pivot column, bits 24-28 = sweeps
@@ -76,72 +82,58 @@ __device__ __forceinline__ void res_tile_async(double2* dst, const double2* __re
   }
 }
 
-constexpr int GROUPS = 2;                        // factor group, refine group
-constexpr int CTA_THREADS = GROUPS * THREADS;
-constexpr int SLOTS = 3;                         // node slots per CTA
-
-// A group's node context.
+// A CTA's node context.
 struct NodeCtx {
   ProblemDev P;
   double2 fz[PMCIM_MAX_TERMS];
   float2 fz32[PMCIM_MAX_TERMS];  // f_k(z) rounded to complex64
-  float2 fid32;                  // sum over identity terms of f_k(z) id_k, complex64
+  double2 fid;                   // sum over identity terms of f_k(z) id_k
+  float2 fid32;
   double red[THREADS / 32];
   int item;
 };
 
 struct FactorSmem {
-  union {
-    LuSmemT<float2> lu32;
-    // lu32 followed by the tensor-core operand stage, which starts at lu32.Ls
-    unsigned char tc[offsetof(LuSmemT<float2>, Ls) + tcu::STAGE_BYTES];
-  } u;
   NodeCtx c;
-};
-
-struct RefineSmem {
-  union {
-    LuSmemT<float2> lu32;   // correction solves
-    LuSmemT<double2> lu64;  // FP64 fallback
-    ResSmem res;            // residual tiles (FP64 pipe)
-    ozk::Smem oz;           // residual operand stages (tensor cores)
-  } u;
-  NodeCtx c;
-  int ozg[PMCIM_MAX_TERMS * ozk::LC];  // column exponents of the digits of f_k X
-  double ozred[THREADS];
-};
-
-// What the factor group hands over with a slot.
-struct Slot {
-  int item;        // node item, or -1: no more nodes
-  int info;        // 0, or 1 + first zero-pivot column of the FP32 LU
-  int tc_timeout;  // a tensor-core wait ran out during the LU
-};
-
-struct MixedSmem {
-  FactorSmem f;
-  RefineSmem r;
-  Slot slot[SLOTS];
-  uint64_t full[SLOTS];   // THREADS arrivals of the factor group
-  uint64_t empty[SLOTS];  // THREADS arrivals of the refine group
   uint64_t mbar_tc[2];    // tensor-core completion, one per accumulator
-  ozk::Bars ozb;          // the refine group's tensor-core residual: stage rings, drains
-  uint32_t tmem_base;     // TMEM_ALL columns: the factor group's from 0, the refine group's from 256
+  uint32_t tmem_base;     // TMEM_FACTOR columns
   int tc_bad;             // a tensor-core wait ran out: FMA pipes from then on
+  // last: the operand stage of the trailing update starts at lu32.Ls and runs over the
+  // end of the struct
+  LuSmemT<float2> lu32;
+};
+constexpr size_t kFactorHead = offsetof(FactorSmem, lu32) + offsetof(LuSmemT<float2>, Ls);
+
+// Bytes of the scratch that starts at lu32.Ls: the operand stage of the tensor-core
+// updates, or else the FMA pipes' tiles and a panel's sub-panel of 8 columns.
+inline size_t factor_scratch_bytes(int max_n, bool tc) {
+  if (tc) return tcu::STAGE_BYTES;
+  const size_t tiles = sizeof(LuSmemT<float2>) - offsetof(LuSmemT<float2>, Ls);
+  const size_t sub = ((size_t)max_n * 8 + NB * 8 + 40) * sizeof(float2) + 1024;
+  const size_t b = sub < (size_t)tcu::STAGE_BYTES ? sub : (size_t)tcu::STAGE_BYTES;
+  return ((b > tiles ? b : tiles) + 127) & ~size_t(127);
+}
+
+template <bool RES64>
+struct SolveSmem {
+  union {
+    LuSmemT<float2> lu32;   // triangular solves
+    ResSmem res;            // residual tiles on the FP64 pipe
+  };
+  NodeCtx c;
+};
+template <>
+struct SolveSmem<false> {
+  LuSmemT<float2> lu32;
+  NodeCtx c;
 };
 
-__device__ __forceinline__ void mbar_init_count(uint64_t* bar, uint32_t count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(tcu::smem_u32(bar)), "r"(count) : "memory");
-}
+struct FallbackSmem {
+  LuSmemT<double2> lu64;
+  NodeCtx c;
+};
 
-// Arrival with release semantics: this thread's earlier writes (shared and
-// global) are visible to a thread whose wait on the phase succeeds.
-__device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
-  asm volatile("{\n\t.reg .b64 st;\n\tmbarrier.arrive.shared::cta.b64 st, [%0];\n\t}" ::"r"(tcu::smem_u32(bar))
-               : "memory");
-}
-
-// Phase clock: the group's thread 0 adds the cycles since the last mark to counter p.
+// Phase clock: thread 0 adds the cycles since the last mark to counter p.
 struct PhaseClock {
   unsigned long long* c;
   long long t;
@@ -153,29 +145,17 @@ struct PhaseClock {
       t = u;
     }
   }
+  // the CTA's lifetime since t0 (global_ns)
+  __device__ void wall(unsigned long long t0) {
+    if (c && gtid() == 0) c[PH_CTA_WALL_NS] += global_ns() - t0;
+  }
 };
-
-// Phase-clock slots. Factor group: assemble, LU panels / TRSM / updates, first
-// solve, set-up, waiting for a free slot; refine group: residual, correction
-// solves, fallback, waiting for a factored node.
-enum { PH_ASSEMBLE = 0, PH_PANEL = 1, PH_FIRST_SOLVE = 2, PH_RESIDUAL = 3, PH_CORRECTION = 4, PH_FALLBACK = 5,
-       PH_SETUP = 6, PH_TRSM = 7, PH_UPDATE = 8, PH_FACTOR_WAIT = 9, PH_REFINE_WAIT = 10,
-       PH_CTA_WALL_NS = 11,  // ns of CTA lifetime, not cycles
-       PH_SWAPS = 12 };      // the panel's row interchanges on the columns outside it
-static_assert(PH_SWAPS < PMCIM_PHASES, "phase slots");
-
-__device__ __forceinline__ unsigned long long global_ns() {
-  unsigned long long t;
-  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-  return t;
-}
 
 // The FP32 blocked LU of lucore::cta_lu, with the trailing updates on the
 // tensor cores (use_tc, while no wait has run out) or on the FMA pipes.
-// Factor group only: its warps 0-7 are the TMEM lane owners.
 // tc: 0 = trailing updates on the FMA pipes, 1 = 3xTF32 on the tensor cores, 2 = BF16 3M on the tensor cores
 __device__ int cta_lu32(float2* __restrict__ M, int n, int ncols, int* __restrict__ piv, int* __restrict__ lists,
-                        LuSmemT<float2>& sm, tcu::Ctx& cx, int tc, PhaseClock& pc) {
+                        LuSmemT<float2>& sm, tcu::Ctx& cx, int tc, int scratch_bytes, PhaseClock& pc) {
   if (gtid() == 0) sm.info_sh = 0;
   gsync();
   for (int k0 = 0; k0 < n; k0 += NB) {
@@ -183,14 +163,14 @@ __device__ int cta_lu32(float2* __restrict__ M, int n, int ncols, int* __restric
     const int kend = k0 + kb;
     // the panel in shared-memory sub-panels, in the tensor-core stage (idle during the
     // panel), while one sub-panel column fits there; else in global memory
-    constexpr int kScratch = tcu::STAGE_BYTES / (int)sizeof(float2);
+    const int kScratch = scratch_bytes / (int)sizeof(float2);
     // row interchanges in LINPACK's order (none on the L columns left of the panel);
     // each panel's permutation goes to lists for the forward solves
     int* list = lists + (size_t)(k0 / NB) * SWAP_LIST_INTS;
     if (n - k0 + NB * 8 + 40 <= kScratch) {
       const int sb = cta_lu_panel_sub(M, n, ncols, k0, kb, piv, sm, reinterpret_cast<float2*>(cx.stage), kScratch);
       pc.mark(PH_PANEL);
-      cta_panel_swaps_lp(M, n, ncols, k0, kb, piv, sb, list, cx.stage, tcu::STAGE_BYTES);
+      cta_panel_swaps_lp(M, n, ncols, k0, kb, piv, sb, list, cx.stage, scratch_bytes);
       pc.mark(PH_SWAPS);
     } else {
       cta_lu_panel(M, n, ncols, k0, kb, piv, sm, k0);
@@ -494,9 +474,10 @@ __device__ void assemble(const NodeCtx& cx, float2* M32, double2* M64) {
   }
 }
 
-// Node item -> problem, node point and weight in the group's context.
-__device__ void load_node(const NodeArgs& a, int idx, NodeCtx& c, RegionDev& rg, NodeItem& it) {
-  it = a.items[idx];
+// Node item -> problem, node point and, with FZ, the scalar functions in the CTA's context.
+template <bool FZ>
+__device__ void load_node(const MixedArgs& a, int q, NodeCtx& c, RegionDev& rg, NodeItem& it) {
+  it = a.items[q];
   rg = a.regions[it.region];
   {
     const int* src = reinterpret_cast<const int*>(a.probs + rg.prob);
@@ -504,6 +485,7 @@ __device__ void load_node(const NodeArgs& a, int idx, NodeCtx& c, RegionDev& rg,
     for (int i = gtid(); i < (int)(sizeof(ProblemDev) / sizeof(int)); i += THREADS) dst[i] = src[i];
   }
   gsync();
+  if (!FZ) return;
   double2 z, w;
   node_weight(rg.cre, rg.cim, rg.r, rg.N, it.j, &z, &w);
   if (gtid() < c.P.K) {
@@ -517,71 +499,70 @@ __device__ void load_node(const NodeArgs& a, int idx, NodeCtx& c, RegionDev& rg,
     for (int k = 0; k < c.P.K; ++k)
       if (!c.P.term[k].dense && c.P.term[k].kind != PMCIM_F_HELMHOLTZ_DLP)
         id = cadd(id, cmul(c.fz[k], c.P.term[k].id));
+    c.fid = id;
     c.fid32 = make_float2((float)id.x, (float)id.y);
   }
   gsync();
 }
 
-// True in every thread of the group when v is true in every thread (a group barrier).
-__device__ __forceinline__ bool group_all(bool v) {
-  int r;
-  asm volatile(
-      "{\n\t.reg .pred p, q;\n\tsetp.ne.s32 p, %1, 0;\n\t"
-      "bar.red.and.pred q, %2, %3, p;\n\tselp.s32 %0, 1, 0, q;\n\t}"
-      : "=r"(r)
-      : "r"((int)v), "r"(1 + (int)(threadIdx.x / THREADS)), "n"(THREADS)
-      : "memory");
-  return r != 0;
+// The next index of a work list of `total` entries, -1 past its end or once the launch has
+// failed; every thread gets it.
+__device__ __forceinline__ int next_index(const MixedArgs& a, int counter, int total, NodeCtx& c) {
+  gsync();  // the previous item is no longer read
+  if (gtid() == 0) {
+    const int k = atomicAdd(a.ctl + counter, 1);
+    c.item = k < total && *reinterpret_cast<volatile int32_t*>(a.err) == 0 ? k : -1;
+  }
+  gsync();
+  return c.item;
 }
 
-// Bounded wait of the whole group on a hand-off barrier; the group agrees on
-// the outcome, so that it never splits at a timeout.
-__device__ bool handoff_wait(uint64_t* bar, uint32_t parity, int32_t* err, long long limit) {
-  const bool ok = group_all(tcu::wait_parity(bar, parity, limit));
-  if (!ok && gtid() == 0) atomicExch(err, 1);
-  return ok;
+// Whether the node's residuals are formed on the tensor cores.
+__device__ __forceinline__ bool node_oz(const MixedArgs& a, const ProblemDev& P, const RegionDev& rg) {
+  return a.oz && P.Adig != nullptr && !rg.herm && P.bie == nullptr;
 }
 
-constexpr uint32_t TMEM_ALL = 512;
-constexpr uint32_t TMEM_REFINE = 256;  // first column of the refine group's accumulators
-static_assert(tcu::TMEM_COLS <= TMEM_REFINE && TMEM_REFINE + ozk::TMEM_COLS <= TMEM_ALL, "TMEM split");
+constexpr uint32_t TMEM_FACTOR = 256;  // columns per CTA, two CTAs per SM
+static_assert(tcu::TMEM_COLS <= TMEM_FACTOR && 2 * tcb::ACC_COLS <= TMEM_FACTOR, "TMEM columns");
 
-// Steps 1-2 for one node after another, into the CTA's slots in turn.
+// Steps 1-2: node after node, each into its own slot.
 // BIE: the instantiation for launches with a boundary-integral term (bie.cuh); the
-// other leaves its code out.
-template <bool BIE>
-__device__ void factor_group(const NodeArgs& a, MixedSmem& sm, tcu::Ctx& cx, PhaseClock& pc) {
+// other leaves its code out. TC: a region of the launch updates on the tensor cores.
+template <bool BIE, bool TC>
+__global__ void __launch_bounds__(THREADS, TC ? 2 : 3) k_mixed_factor(MixedArgs a, int scratch_bytes) {
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  FactorSmem& sm = *reinterpret_cast<FactorSmem*>(smem_raw);
   const int tid = gtid();
-  NodeCtx& c = sm.f.c;
-  for (int k = 0;; ++k) {
-    const int s = k % SLOTS, use = k / SLOTS;
-    // the slot is free again once the refine group has finished its previous node
-    if (use > 0 && !handoff_wait(&sm.empty[s], (uint32_t)((use - 1) & 1), a.err, a.handoff_wait_cycles)) return;
-    pc.mark(PH_FACTOR_WAIT);
-    if (tid == 0) c.item = atomicAdd(a.counter, 1);
-    gsync();
-    const int idx = c.item;
-    Slot& sl = sm.slot[s];
-    if (idx >= a.n_items) {
-      if (tid == 0) sl.item = -1;
-      mbar_arrive(&sm.full[s]);
-      return;
-    }
-    const size_t si = (size_t)blockIdx.x * SLOTS + s;
-    char* slot = a.work + si * a.slot_bytes;
+  NodeCtx& c = sm.c;
+  PhaseClock pc(a.phase ? a.phase + (size_t)blockIdx.x * PMCIM_PHASES : nullptr);
+  const unsigned long long t_start = global_ns();
+  if (TC && tid < 32) tcu::tmem_alloc_cols(&sm.tmem_base, TMEM_FACTOR);
+  if (tid == 0) {
+    tcu::mbar_init(&sm.mbar_tc[0]);
+    tcu::mbar_init(&sm.mbar_tc[1]);
+    sm.tc_bad = 0;
+  }
+  tcu::fence_async_smem();
+  tcu::fence_before();
+  __syncthreads();
+  tcu::fence_after();
+  tcu::Ctx cx{smem_raw + kFactorHead, sm.mbar_tc, TC ? sm.tmem_base : 0u, {0u, 0u}, &sm.tc_bad, a.tc_wait_cycles};
+  for (;;) {
+    const int q = next_index(a, MIXED_CTL_FACTOR, a.count, c);
+    if (q < 0) break;
+    char* slot = a.work + (size_t)q * a.slot_bytes;
     float2* M32 = reinterpret_cast<float2*>(slot);
-    int* piv = a.piv + si * a.max_n;
     NodeItem it;
     RegionDev rg;
-    load_node(a, idx, c, rg, it);
+    load_node<true>(a, q, c, rg, it);
     const ProblemDev& P = c.P;
     const int n = P.n, l = P.l, ncols = n + l;
     const size_t nn = (size_t)n * n, nl = (size_t)n * l;
     pc.mark(PH_SETUP);
-    // T(z_j) in FP64 for the refine group's FP64 residual, and rounded; T(z_j)^H likewise;
+    // T(z_j) in FP64 for the residuals on the FP64 pipe, and rounded; T(z_j)^H likewise;
     // always with a boundary-integral term (no stored coefficients to take residuals from)
     if (rg.herm || (P.n_dense >= 2 && !a.oz) || (BIE && P.bie))
-      assemble_fp64<BIE>(c, a.t64 + si * a.t64_stride, M32, rg.herm != 0,
+      assemble_fp64<BIE>(c, a.t64 + (size_t)q * a.t64_stride, M32, rg.herm != 0,
                          reinterpret_cast<double2*>(slot + mixed_residual_offset(n, l)));
     else
       assemble32(c, M32);
@@ -596,140 +577,122 @@ __device__ void factor_group(const NodeArgs& a, MixedSmem& sm, tcu::Ctx& cx, Pha
     pc.mark(PH_ASSEMBLE);
     const int bad_before = sm.tc_bad;
     int* lists = reinterpret_cast<int*>(slot + mixed_lists_offset(n, l));
-    const int info = cta_lu32(M32, n, ncols, piv, lists, sm.f.u.lu32, cx, rg.lu_tc, pc);
+    int* piv = lists + (size_t)((n + NB - 1) / NB) * SWAP_LIST_INTS;
+    const int info = cta_lu32(M32, n, ncols, piv, lists, sm.lu32, cx, TC ? rg.lu_tc : 0, scratch_bytes, pc);
     if (tid == 0) {
-      sl.item = idx;
-      sl.info = info;
-      sl.tc_timeout = sm.tc_bad != bad_before;
+      MixedState st{};
+      st.info = info;
+      st.lost = sm.tc_bad != bad_before ? MIXED_LOST_LU : 0;
+      st.id = c.fid;
+      a.state[q] = st;
     }
-    mbar_arrive(&sm.full[s]);
   }
+  if (TC) {
+    // a commit whose wait ran out may still be in flight: wait once more, with the
+    // default limit whatever the update's own limit was, before the columns are given back
+    if (sm.tc_bad) {
+      // returns at once for a barrier with no commit outstanding
+      tcu::wait_parity(&sm.mbar_tc[0], cx.phase[0] ^ 1u, tcu::WAIT_CYCLES);
+      tcu::wait_parity(&sm.mbar_tc[1], cx.phase[1] ^ 1u, tcu::WAIT_CYCLES);
+    }
+    tcu::fence_before();
+    __syncthreads();
+    tcu::fence_after();
+    if (tid < 32) tcu::tmem_dealloc_cols(sm.tmem_base, TMEM_FACTOR);
+  }
+  pc.wall(t_start);
 }
 
-// Step 4: the node solved again by the FP64 LU in its slot. Kept out of line:
-// it is rare, and its registers should not weigh on the refinement loop.
-__device__ __noinline__ int fallback_fp64(const NodeCtx& c, double2* M64, int* piv, double2* X,
-                                          LuSmemT<double2>& lu, const double2* __restrict__ T64) {
-  const ProblemDev& P = c.P;
-  const int n = P.n, l = P.l;
-  const size_t nn = (size_t)n * n, nl = (size_t)n * l;
-  gsync();
-  if (T64)  // T(z_j) as the factor group assembled it in FP64 (a boundary-integral term)
-    for (size_t e = gtid(); e < nn; e += THREADS) M64[e] = T64[e];
-  else
-    assemble(c, nullptr, M64);
-  for (size_t e = gtid(); e < nl; e += THREADS) M64[nn + e] = P.V[e];
-  gsync();
-  const int info = cta_lu(M64, n, n + l, piv, lu);
-  cta_back_blocked(M64, n, l, lu);
-  for (size_t e = gtid(); e < nl; e += THREADS) X[e] = M64[nn + e];
-  gsync();
-  return info;
+// Thread 0: a finished node's info word.
+__device__ __forceinline__ void finish_node(const MixedArgs& a, const RegionDev& rg, const NodeItem& it,
+                                            const MixedState& st, bool ok) {
+  a.node_info[rg.node_off + it.j] =
+      st.info | (st.sweeps << 24) | (st.lost ? (1 << 29) : 0) | (ok ? 0 : (1 << 30));
 }
 
-// Steps 3-4 for the nodes the factor group hands over, in the same order.
-template <bool BIE>
-__device__ void refine_group(const NodeArgs& a, MixedSmem& sm, PhaseClock& pc) {
+// The back substitution (sw = 0, every node) or sweep sw's correction (the active nodes).
+// RES64: a node of the launch forms its residuals on the FP64 pipe.
+template <bool RES64>
+__global__ void __launch_bounds__(THREADS, 3) k_mixed_solve(MixedArgs a, int sw) {
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  SolveSmem<RES64>& sm = *reinterpret_cast<SolveSmem<RES64>*>(smem_raw);
   const int tid = gtid();
-  NodeCtx& c = sm.r.c;
-  for (int k = 0;; ++k) {
-    const int s = k % SLOTS, use = k / SLOTS;
-    if (!handoff_wait(&sm.full[s], (uint32_t)(use & 1), a.err, a.handoff_wait_cycles)) return;
-    pc.mark(PH_REFINE_WAIT);
-    const Slot sl = sm.slot[s];
-    if (sl.item < 0) return;
-    const size_t si = (size_t)blockIdx.x * SLOTS + s;
-    char* slot = a.work + si * a.slot_bytes;
+  NodeCtx& c = sm.c;
+  const int total = sw == 0 ? a.count : a.ctl[MIXED_CTL_ACTIVE + sw];
+  if (total == 0) return;
+  PhaseClock pc(a.phase ? a.phase + (size_t)blockIdx.x * PMCIM_PHASES : nullptr);
+  const unsigned long long t_start = global_ns();
+  for (;;) {
+    const int k = next_index(a, sw == 0 ? MIXED_CTL_FIRST : MIXED_CTL_SWEEP + sw, total, c);
+    if (k < 0) break;
+    const int q = sw == 0 ? k : a.act[(size_t)(sw & 1) * a.slots + k];
+    char* slot = a.work + (size_t)q * a.slot_bytes;
     float2* M32 = reinterpret_cast<float2*>(slot);
-    double2* M64 = reinterpret_cast<double2*>(slot);  // fallback only; aliases M32
-    int* piv = a.piv + si * a.max_n;
     NodeItem it;
     RegionDev rg;
-    load_node(a, sl.item, c, rg, it);
+    load_node<RES64>(a, q, c, rg, it);
     const ProblemDev& P = c.P;
     const int n = P.n, l = P.l;
     const size_t nn = (size_t)n * n, nl = (size_t)n * l;
     double2* R = reinterpret_cast<double2*>(slot + mixed_residual_offset(n, l));
     const int* lists = reinterpret_cast<const int*>(slot + mixed_lists_offset(n, l));
     double2* X = a.X + rg.x_off + (size_t)it.j * nl;
-    int info = sl.info;
-    bool ok = (info == 0);
-    // the first solve, X_0 = U^-1 (L^-1 P V) in FP32 (the factor group eliminated V
-    // with the LU), here so that the factor group can start the next node
-    double xm = 0.0;
-    if (ok) {
-      cta_back_blocked(M32, n, l, sm.r.u.lu32);
-      for (size_t e = tid; e < nl; e += THREADS) {
-        const float2 y = M32[nn + e];
-        const double2 x = make_double2((double)y.x, (double)y.y);
-        X[e] = x;
-        xm = fmax(xm, fmax(fabs(x.x), fabs(x.y)));
-      }
-      xm = block_max(xm, c.red);
-    }
-    pc.mark(PH_FIRST_SOLVE);
-    bool tc_lost = sl.tc_timeout != 0;
-    int sweeps = 0;
-    // residuals on the tensor cores (exact digit products), unless a wait of that
-    // path ran out earlier in this CTA; then the node is solved in FP64 below
-    const bool bie = BIE && P.bie;
-    const bool use_oz = a.oz && P.Adig != nullptr && !rg.herm && !bie;
-    if (use_oz && sm.ozb.bad) {
-      ok = false;
-      tc_lost = true;
-    }
-    // max_sweeps == 0: the FP32 solve alone (a direction for a certificate), no refinement
-    // and no FP64 re-solve
-    const bool refine = a.max_sweeps > 0;
-    if (ok && refine) {
-      // the matrix each residual multiplies: T(z_j) assembled once, or the one dense term
-      const double2* M = nullptr;
-      double2 fM = make_double2(0.0, 0.0), id = make_double2(0.0, 0.0);
-      if (use_oz) {
-        // every dense term through the digit products; nothing to set up here
-      } else if (P.n_dense >= 2 || rg.herm || bie) {  // assembled by the factor group with the slot
-        M = a.t64 + si * a.t64_stride;
-        fM = make_double2(1.0, 0.0);
-      } else {
-        for (int k = 0; k < P.K; ++k) {
-          const TermDesc& t = P.term[k];
-          if (t.dense) {
-            M = P.A + (size_t)t.mat_index * nn;
-            fM = c.fz[k];
-          } else {
-            id = cadd(id, cmul(c.fz[k], t.id));
-          }
+    MixedState st = a.state[q];
+    const bool oz = node_oz(a, P, rg);
+    bool ok = st.info == 0, done = false;
+    if (sw == 0) {
+      if (ok) {
+        // X_0 = U^-1 (L^-1 P V) in FP32 (the LU eliminated V)
+        double xm = 0.0;
+        cta_back_blocked(M32, n, l, sm.lu32);
+        for (size_t e = tid; e < nl; e += THREADS) {
+          const float2 y = M32[nn + e];
+          const double2 x = make_double2((double)y.x, (double)y.y);
+          X[e] = x;
+          xm = fmax(xm, fmax(fabs(x.x), fabs(x.y)));
         }
+        st.dprev = block_max(xm, c.red);
       }
-      double dprev = xm;
-      bool conv = false;
-      for (int sw = 1; sw <= a.max_sweeps && ok; ++sw) {
-        if (use_oz) {
-          if (!ozk::residual(P, c.fz, X, R, sm.r.u.oz, sm.ozb, a.ysl + si * a.ysl_stride,
-                             sm.tmem_base + TMEM_REFINE, sm.r.ozg, sm.r.ozred, a.tc_wait_cycles)) {
-            ok = false;
-            tc_lost = true;
-            break;
-          }
+      // max_sweeps == 0: the FP32 solve alone (a direction for a certificate), no refinement
+      // and no FP64 re-solve
+      done = a.max_sweeps == 0;
+      pc.mark(PH_FIRST_SOLVE);
+    } else {
+      if (oz) {
+        ok = (st.lost & MIXED_LOST_RESIDUAL) == 0;  // R is not valid where a wait ran out
+      } else if (RES64) {
+        // the matrix the residual multiplies: T(z_j) assembled once, or the one dense term
+        const double2* M = nullptr;
+        double2 fM = make_double2(1.0, 0.0), id = make_double2(0.0, 0.0);
+        if (P.n_dense >= 2 || rg.herm || P.bie) {
+          M = a.t64 + (size_t)q * a.t64_stride;
         } else {
-          if (l == 1) residual_fp64_col(X, R, c, sm.r.u.res, M, fM, id);
-          else residual_fp64(X, R, c, sm.r.u.res, M, fM, id);
+          id = c.fid;
+          for (int t = 0; t < P.K; ++t)
+            if (P.term[t].dense) {
+              M = P.A + (size_t)P.term[t].mat_index * nn;
+              fM = c.fz[t];
+            }
         }
-        if (rg.border > 0) {
-          // bordered system M u = b, M = T(z_j) + (c - T(z_j) e_s) e_s^T with b = -T(z_j) e_s:
-          // R = b - T X - (c + b) X_s (l = 1)
-          const double2 xs = X[rg.border - 1];
-          const double2* bc = a.border + rg.v_off;
-          for (size_t e = tid; e < nl; e += THREADS) cfms(R[e], cadd(bc[e], P.V[e]), xs);
-        }
-        pc.mark(PH_RESIDUAL);
-        double rm = 0.0;
+        ResSmem& res = *reinterpret_cast<ResSmem*>(smem_raw);
+        if (l == 1) residual_fp64_col(X, R, c, res, M, fM, id);
+        else residual_fp64(X, R, c, res, M, fM, id);
+      }
+      if (ok && rg.border > 0) {
+        // bordered system M u = b, M = T(z_j) + (c - T(z_j) e_s) e_s^T with b = -T(z_j) e_s:
+        // R = b - T X - (c + b) X_s (l = 1)
+        const double2 xs = X[rg.border - 1];
+        const double2* bc = a.border + rg.v_off;
+        for (size_t e = tid; e < nl; e += THREADS) cfms(R[e], cadd(bc[e], P.V[e]), xs);
+      }
+      pc.mark(PH_RESIDUAL);
+      double rm = 0.0;
+      if (ok) {
         for (size_t e = tid; e < nl; e += THREADS) rm = fmax(rm, fmax(fabs(R[e].x), fabs(R[e].y)));
         rm = block_max(rm, c.red);
-        if (rm == 0.0) {
-          conv = true;
-          break;
-        }
+        done = rm == 0.0;
+      }
+      if (ok && !done) {
         const double inv = 1.0 / rm;
         // right-hand side R / |R|max; the forward solve applies the row interchanges
         for (size_t e = tid; e < nl; e += THREADS) {
@@ -737,8 +700,8 @@ __device__ void refine_group(const NodeArgs& a, MixedSmem& sm, PhaseClock& pc) {
           M32[nn + e] = make_float2((float)(rv.x * inv), (float)(rv.y * inv));
         }
         gsync();
-        cta_fwd_blocked_lp(M32, n, l, sm.r.u.lu32, lists);
-        cta_back_blocked(M32, n, l, sm.r.u.lu32);
+        cta_fwd_blocked_lp(M32, n, l, sm.lu32, lists);
+        cta_back_blocked(M32, n, l, sm.lu32);
         double dm = 0.0, xmx = 0.0;
         for (size_t e = tid; e < nl; e += THREADS) {
           const float2 d = M32[nn + e];
@@ -752,109 +715,120 @@ __device__ void refine_group(const NodeArgs& a, MixedSmem& sm, PhaseClock& pc) {
         }
         dm = block_max(dm, c.red);
         xmx = block_max(xmx, c.red);
-        pc.mark(PH_CORRECTION);
-        sweeps = sw;
-        if (!(dm < dprev) && sw > 1) {  // no contraction
-          ok = false;
-          break;
-        }
-        if (dm * dm <= a.tol_ir * xmx * dprev) {
-          conv = true;
-          break;
-        }
-        dprev = dm;
+        st.sweeps = sw;
+        if (!(dm < st.dprev) && sw > 1) ok = false;  // no contraction
+        else if (dm * dm <= a.tol_ir * xmx * st.dprev) done = true;
+        else if (sw >= a.max_sweeps) ok = false;
+        st.dprev = dm;
       }
-      if (!conv) ok = false;
+      pc.mark(PH_CORRECTION);
     }
-    if (!ok && refine && rg.border == 0) {
-      info = fallback_fp64(c, M64, piv, X, sm.r.u.lu64, bie ? a.t64 + si * a.t64_stride : nullptr);
-      pc.mark(PH_FALLBACK);
-    }
-    if (rg.border > 0) {
+    const bool refine = a.max_sweeps > 0;
+    if ((done || !ok) && rg.border > 0) {
       // the certificate's vector y = e_s + (u - u_s e_s): T(z_j) y = -u_s c
       gsync();
       if (tid == 0) X[rg.border - 1] = make_double2(1.0, 0.0);
     }
-    if (tid == 0)
-      a.node_info[rg.node_off + it.j] =
-          info | (sweeps << 24) | (tc_lost ? (1 << 29) : 0) | (ok ? 0 : (1 << 30));
-    gsync();
-    mbar_arrive(&sm.empty[s]);
+    if (tid == 0) {
+      a.state[q] = st;
+      if (!ok && refine && rg.border == 0) {
+        a.fallback[atomicAdd(a.ctl + MIXED_CTL_FALLBACK_COUNT, 1)] = q;
+      } else if (done || !ok) {
+        finish_node(a, rg, it, st, ok);
+      } else {  // active in the next sweep
+        const int nx = sw + 1;
+        a.act[(size_t)(nx & 1) * a.slots + atomicAdd(a.ctl + MIXED_CTL_ACTIVE + nx, 1)] = q;
+        if (oz) {
+          const int ncg = (l + 7) / 8;
+          const int u = a.ubase[rg.prob] + atomicAdd(mixed_ucount(a, nx) + rg.prob, ncg);
+          for (int g = 0; g < ncg; ++g) a.units[(size_t)(nx & 1) * a.unit_cap + u + g] = q * 8 + g;
+        }
+      }
+    }
   }
+  pc.wall(t_start);
 }
 
-template <bool BIE>
-__global__ void __launch_bounds__(CTA_THREADS, 1) k_factor_solve_mixed(NodeArgs a) {
+// Step 4: the nodes that did not converge, by the FP64 LU. The chunk's other nodes are
+// done, so the FP64 matrices take the slots' place.
+__global__ void __launch_bounds__(THREADS, 2) k_mixed_fallback(MixedArgs a, size_t bytes_per_cta) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
-  MixedSmem& sm = *reinterpret_cast<MixedSmem*>(smem_raw);
-  const int tid = threadIdx.x;
+  FallbackSmem& sm = *reinterpret_cast<FallbackSmem*>(smem_raw);
+  NodeCtx& c = sm.c;
+  const int total = a.ctl[MIXED_CTL_FALLBACK_COUNT];
+  if (total == 0) return;
   PhaseClock pc(a.phase ? a.phase + (size_t)blockIdx.x * PMCIM_PHASES : nullptr);
-  unsigned long long t_start = 0;
-  if (a.phase && tid == 0) t_start = global_ns();
-
-  // tensor memory (all of it: one CTA per SM) and the barriers, for the whole persistent CTA
-  if (tid < 32) tcu::tmem_alloc_cols(&sm.tmem_base, TMEM_ALL);
-  if (tid == 0) {
-    ozk::init_bars(sm.ozb);
-    for (int s = 0; s < SLOTS; ++s) {
-      mbar_init_count(&sm.full[s], THREADS);
-      mbar_init_count(&sm.empty[s], THREADS);
+  const unsigned long long t_start = global_ns();
+  for (;;) {
+    const int k = next_index(a, MIXED_CTL_FALLBACK, total, c);
+    if (k < 0) break;
+    const int q = a.fallback[k];
+    NodeItem it;
+    RegionDev rg;
+    load_node<true>(a, q, c, rg, it);
+    const ProblemDev& P = c.P;
+    const int n = P.n, l = P.l;
+    const size_t nn = (size_t)n * n, nl = (size_t)n * l;
+    double2* M64 = reinterpret_cast<double2*>(a.work + (size_t)blockIdx.x * bytes_per_cta);
+    int* piv = reinterpret_cast<int*>(M64 + nn + nl);
+    double2* X = a.X + rg.x_off + (size_t)it.j * nl;
+    if (P.bie) {  // T(z_j) as k_mixed_factor assembled it in FP64
+      const double2* T64 = a.t64 + (size_t)q * a.t64_stride;
+      for (size_t e = gtid(); e < nn; e += THREADS) M64[e] = T64[e];
+    } else {
+      assemble(c, nullptr, M64);
     }
-    tcu::mbar_init(&sm.mbar_tc[0]);
-    tcu::mbar_init(&sm.mbar_tc[1]);
-    sm.tc_bad = 0;
+    for (size_t e = gtid(); e < nl; e += THREADS) M64[nn + e] = P.V[e];
+    gsync();
+    MixedState st = a.state[q];
+    st.info = cta_lu(M64, n, n + l, piv, sm.lu64);
+    cta_back_blocked(M64, n, l, sm.lu64);
+    for (size_t e = gtid(); e < nl; e += THREADS) X[e] = M64[nn + e];
+    if (gtid() == 0) finish_node(a, rg, it, st, false);
+    pc.mark(PH_FALLBACK);
   }
-  tcu::fence_async_smem();
-  tcu::fence_before();
-  __syncthreads();
-  tcu::fence_after();
-
-  if (tid < THREADS) {
-    tcu::Ctx cx{sm.f.u.tc + offsetof(LuSmemT<float2>, Ls), sm.mbar_tc, sm.tmem_base, {0u, 0u}, &sm.tc_bad,
-                a.tc_wait_cycles};
-    factor_group<BIE>(a, sm, cx, pc);
-    // a commit whose wait ran out may still be in flight: wait once more, with the
-    // default limit whatever the update's own limit was, before the columns are given back
-    if (sm.tc_bad) {
-      // returns at once for a barrier with no commit outstanding
-      tcu::wait_parity(&sm.mbar_tc[0], cx.phase[0] ^ 1u, tcu::WAIT_CYCLES);
-      tcu::wait_parity(&sm.mbar_tc[1], cx.phase[1] ^ 1u, tcu::WAIT_CYCLES);
-    }
-  } else {
-    refine_group<BIE>(a, sm, pc);
-  }
-  // both groups are done with tensor memory before it is given back
-  tcu::fence_before();
-  __syncthreads();
-  tcu::fence_after();
-  if (tid < 32) tcu::tmem_dealloc_cols(sm.tmem_base, TMEM_ALL);
-  if (a.phase && tid == 0)  // the CTA's lifetime, for cycles per ns
-    a.phase[(size_t)blockIdx.x * PMCIM_PHASES + PH_CTA_WALL_NS] += global_ns() - t_start;
+  pc.wall(t_start);
 }
 
 }  // namespace
 
 // Slot layout: [FP32 matrix n x (n + l)] [FP64 residual n x l] [the panels' row
-// permutations, SWAP_LIST_INTS ints each], or, after a fallback, the FP64 matrix
-// n x (n + l) over the whole slot.
+// permutations, SWAP_LIST_INTS ints each] [pivots].
 size_t mixed_slot_bytes(int n, int l) {
-  const size_t fp64 = (size_t)n * (n + l) * sizeof(double2);
-  const size_t mixed = mixed_lists_offset(n, l) + (size_t)((n + NB - 1) / NB) * SWAP_LIST_INTS * sizeof(int);
-  const size_t b = fp64 > mixed ? fp64 : mixed;
+  const size_t b = mixed_lists_offset(n, l) +
+                   ((size_t)((n + NB - 1) / NB) * SWAP_LIST_INTS + (size_t)n) * sizeof(int);
   return (b + 255) & ~(size_t)255;
 }
-
-static_assert(sizeof(MixedSmem) + 1024 <= 227 * 1024, "one CTA per SM");
-
-cudaError_t prepare_factor_mixed() {
-  cudaError_t e = cudaFuncSetAttribute(k_factor_solve_mixed<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)sizeof(MixedSmem));
-  if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(k_factor_solve_mixed<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)sizeof(MixedSmem));
+// Bytes a slot area needs at the least: one FP64 fallback.
+size_t mixed_fallback_bytes(int n, int l) {
+  return (((size_t)n * (n + l) * sizeof(double2) + (size_t)n * sizeof(int)) + 255) & ~(size_t)255;
 }
 
-int mixed_slots_per_cta() { return SLOTS; }
+namespace {
+const void* factor_kernel(bool bie, bool tc) {
+  if (bie) return tc ? (const void*)k_mixed_factor<true, true> : (const void*)k_mixed_factor<true, false>;
+  return tc ? (const void*)k_mixed_factor<false, true> : (const void*)k_mixed_factor<false, false>;
+}
+}  // namespace
+
+static_assert(2 * (kFactorHead + tcu::STAGE_BYTES + 1024) <= 228 * 1024, "two CTAs per SM");
+
+cudaError_t prepare_factor_mixed() {
+  for (int i = 0; i < 4; ++i) {
+    cudaError_t e = cudaFuncSetAttribute(factor_kernel(i & 1, i & 2), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)(kFactorHead + tcu::STAGE_BYTES));
+    if (e != cudaSuccess) return e;
+  }
+  cudaError_t e = cudaFuncSetAttribute(k_mixed_solve<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)sizeof(SolveSmem<true>));
+  if (e != cudaSuccess) return e;
+  e = cudaFuncSetAttribute(k_mixed_solve<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           (int)sizeof(SolveSmem<false>));
+  if (e != cudaSuccess) return e;
+  e = cudaFuncSetAttribute(k_mixed_fallback, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(FallbackSmem));
+  if (e != cudaSuccess) return e;
+  return prepare_oz_refine();
+}
 
 namespace {
 __global__ void k_round_c64(const double2* __restrict__ src, float2* __restrict__ dst, size_t count) {
@@ -870,15 +844,41 @@ cudaError_t round_coefficients_c64(const double2* src, float2* dst, size_t count
   return cudaGetLastError();
 }
 
-// Launch only; prepare_factor_mixed() must have set the shared-memory limit.
-// One CTA per a.slots / SLOTS workspace slots.
-cudaError_t launch_factor_solve_mixed(const NodeArgs& a, cudaStream_t s) {
-  if (a.n_items <= 0) return cudaSuccess;
-  const size_t smem = sizeof(MixedSmem);
-  int grid = a.slots / SLOTS;
-  if (grid > a.n_items) grid = a.n_items;
-  if (grid < 1) return cudaErrorInvalidValue;
-  if (a.bie) k_factor_solve_mixed<true><<<grid, CTA_THREADS, smem, s>>>(a);
-  else k_factor_solve_mixed<false><<<grid, CTA_THREADS, smem, s>>>(a);
+// One chunk's kernels in order (no synchronisation, so that they can be captured);
+// prepare_factor_mixed() must have set the shared-memory limits. *launched: kernels.
+cudaError_t launch_factor_solve_mixed(const MixedArgs& a, int sms, cudaStream_t s, int* launched) {
+  *launched = 0;
+  if (a.count <= 0) return cudaSuccess;
+  cudaError_t e = cudaMemsetAsync(a.ctl, 0, mixed_ctl_zero_ints(a.n_probs, a.max_sweeps) * sizeof(int), s);
+  if (e != cudaSuccess) return e;
+  auto grid = [&](int per_sm) { return per_sm * sms < a.count ? per_sm * sms : a.count; };
+  {
+    const int scratch = (int)factor_scratch_bytes(a.max_n, a.tc != 0);
+    const size_t smem = kFactorHead + scratch;
+    const int g = grid(a.tc ? 2 : 3);
+    if (a.bie && a.tc) k_mixed_factor<true, true><<<g, THREADS, smem, s>>>(a, scratch);
+    else if (a.bie) k_mixed_factor<true, false><<<g, THREADS, smem, s>>>(a, scratch);
+    else if (a.tc) k_mixed_factor<false, true><<<g, THREADS, smem, s>>>(a, scratch);
+    else k_mixed_factor<false, false><<<g, THREADS, smem, s>>>(a, scratch);
+    ++*launched;
+  }
+  for (int sw = 0; sw <= a.max_sweeps; ++sw) {
+    if (sw > 0 && a.oz) {
+      e = launch_oz_residual(a, sw, sms, s);
+      if (e != cudaSuccess) return e;
+      *launched += 2;
+    }
+    if (a.res64) k_mixed_solve<true><<<grid(3), THREADS, sizeof(SolveSmem<true>), s>>>(a, sw);
+    else k_mixed_solve<false><<<grid(3), THREADS, sizeof(SolveSmem<false>), s>>>(a, sw);
+    ++*launched;
+  }
+  if (a.max_sweeps > 0) {
+    const size_t per = mixed_fallback_bytes(a.max_n, a.max_l);
+    size_t g = a.work_bytes / per;
+    if (g < 1) return cudaErrorInvalidValue;
+    if (g > (size_t)grid(2)) g = (size_t)grid(2);
+    k_mixed_fallback<<<(unsigned)g, THREADS, sizeof(FallbackSmem), s>>>(a, per);
+    ++*launched;
+  }
   return cudaGetLastError();
 }

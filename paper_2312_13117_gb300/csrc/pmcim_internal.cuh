@@ -8,6 +8,8 @@
 #include "bie.cuh"
 
 #define PMCIM_MAX_TERMS 16
+// phases of the precision form timed with clock64 when profiling
+#define PMCIM_PHASES PMCIM_PHASE_COUNT
 // ||P f|_N|| at or below this fraction of ||sum_j |w_j| |x_j||| counts as zero
 constexpr double kPfFloor = 1e-10;
 #define PMCIM_MAX_L 64
@@ -220,37 +222,108 @@ struct NodeArgs {
   int n_items;
   int* counter;             // work counter, zero before the launch
   double2* X;
-  int32_t* node_info;       // FP64: 0 or 1 + zero-pivot column. Mixed: bits 0-23 the same,
-                            // 24-29 sweeps run, 30 FP64 fallback
+  int32_t* node_info;       // 0 or 1 + zero-pivot column
   char* work;               // slots * slot_bytes
   size_t slot_bytes;
   int32_t* piv;             // slots * max_n
   int max_n;
   int slots;
-  int max_sweeps;             // mixed kernel: refinement sweeps; 0 = the FP32 solve only
-  double tol_ir;
-  unsigned long long* phase;  // NULL, or slots * PMCIM_PHASES clock64 counters (mixed kernel)
-  int32_t* err;               // mixed kernel: set to 1 when a wait between its thread groups ran out
-  double2* t64;               // mixed kernel: per slot, T(z_j) in FP64 for the residuals (problems
-  size_t t64_stride;          // with two or more dense terms); double2 elements per slot
-  int oz;                     // mixed kernel: 1 = refinement residuals on the tensor cores
-  unsigned char* ysl;         // mixed kernel: per slot, the digits of f_k X (ozaki.cuh)
-  size_t ysl_stride;          // bytes per slot
-  long long tc_wait_cycles;       // mixed kernel: limit of a wait for a tensor-core commit
-  long long handoff_wait_cycles;  // mixed kernel: limit of a wait between its thread groups
-  const double2* border;          // mixed kernel: the replacement columns of bordered nodes
   int fp64_tile;                  // FP64 kernel: trailing-update tile, 32 or 64 (0: 64)
   int bie;                        // FP64 and small kernels: a problem has a boundary-integral term
 };
-// Limits of the precision-form kernel's bounded waits (clock64 cycles): the
+
+// Precision forms (lu_mixed.cu, oz_refine.cu): a chunk of nodes goes through the steps
+// together, one kernel per step, node q of the chunk in slot q.
+struct MixedState {
+  double dprev;    // max norm of X_0 or of the last correction
+  double2 id;      // sum over identity terms of f_k(z_j) id_k
+  int32_t info;    // 0, or 1 + first zero-pivot column of the FP32 LU
+  int32_t sweeps;  // refinement sweeps run
+  int32_t lost;    // MIXED_LOST_*: a tensor-core wait ran out
+  int32_t pad;
+};
+constexpr int MIXED_LOST_LU = 1, MIXED_LOST_RESIDUAL = 2;
+// ctl: work counters, active nodes per sweep, then the column groups per sweep and problem
+// (all zero at a chunk's start), then the residual tiles before each problem
+constexpr int MIXED_CTL_FACTOR = 0, MIXED_CTL_FIRST = 1, MIXED_CTL_FALLBACK = 2, MIXED_CTL_FALLBACK_COUNT = 3,
+              MIXED_CTL_ACTIVE = 16, MIXED_CTL_SWEEP = 32, MIXED_CTL_UNITS = 48;
+constexpr int MIXED_MAX_SWEEPS = 10;
+static_assert(MIXED_CTL_ACTIVE + MIXED_MAX_SWEEPS + 1 < MIXED_CTL_SWEEP &&
+                  MIXED_CTL_SWEEP + MIXED_MAX_SWEEPS + 1 < MIXED_CTL_UNITS,
+              "a counter per sweep");
+struct MixedArgs {
+  const ProblemDev* probs;
+  int n_probs;
+  const RegionDev* regions;
+  const NodeItem* items;  // the chunk's, largest n first
+  int count;
+  double2* X;
+  int32_t* node_info;  // bits 0-23: 0 or 1 + zero-pivot column, 24-28 sweeps run, 29 a
+                       // tensor-core wait ran out, 30 FP64 fallback
+  char* work;          // slots * slot_bytes
+  size_t slot_bytes, work_bytes;
+  int slots;
+  int max_n, max_l;    // of the chunk
+  int max_sweeps;      // 0 = the FP32 solve only
+  double tol_ir;
+  int tc;              // a region updates on the tensor cores (RegionDev::lu_tc)
+  int bie;             // a problem has a boundary-integral term
+  int oz;              // refinement residuals on the tensor cores
+  int res64;           // a node forms its residuals on the FP64 pipe
+  double2* t64;        // per slot, T(z_j) in FP64 for those
+  size_t t64_stride;
+  unsigned char* ysl;  // per slot, the digits of f_k X (oz_refine.cu)
+  size_t ysl_stride;
+  int32_t* gexp;       // per slot, their column exponents: [dense term][column]
+  int gexp_stride;     // PMCIM_MAX_L per dense term
+  MixedState* state;   // per slot
+  int* ctl;
+  int* act;            // [sweep & 1][slots]: nodes that still refine
+  int* fallback;       // [slots]
+  int* units;          // [sweep & 1][unit_cap]: their groups of 8 solution columns, 8 slot + group,
+  int unit_cap;        // those of problem p from ubase[p] on
+  const int* ubase;
+  const double2* border;       // the replacement columns of bordered nodes
+  unsigned long long* phase;   // NULL, or PMCIM_PHASES clock64 counters per CTA
+  int32_t* err;                // set to 1 when a wait between a kernel's warp groups ran out
+  long long tc_wait_cycles;       // limit of a wait for a tensor-core commit or its operands
+  long long handoff_wait_cycles;  // limit of a wait between warp groups
+};
+__host__ __device__ inline size_t mixed_ctl_zero_ints(int n_probs, int max_sweeps) {
+  return MIXED_CTL_UNITS + (size_t)(max_sweeps + 1) * n_probs;
+}
+__host__ __device__ inline size_t mixed_ctl_ints(int n_probs, int max_sweeps) {
+  return mixed_ctl_zero_ints(n_probs, max_sweeps) + n_probs + 1;
+}
+__device__ __forceinline__ int* mixed_ucount(const MixedArgs& a, int sw) {
+  return a.ctl + MIXED_CTL_UNITS + (size_t)sw * a.n_probs;
+}
+__device__ __forceinline__ int* mixed_tiles(const MixedArgs& a) {
+  return a.ctl + mixed_ctl_zero_ints(a.n_probs, a.max_sweeps);
+}
+// Phase-clock slots (PMCIM_PHASES): SM cycles summed over CTAs, by step.
+enum { PH_ASSEMBLE = 0, PH_PANEL = 1, PH_FIRST_SOLVE = 2, PH_RESIDUAL = 3, PH_CORRECTION = 4, PH_FALLBACK = 5,
+       PH_SETUP = 6, PH_TRSM = 7, PH_UPDATE = 8,
+       PH_CTA_WALL_NS = 11,  // ns of CTA lifetime, not cycles
+       PH_SWAPS = 12 };      // the panel's row interchanges on the columns outside it
+__device__ __forceinline__ unsigned long long global_ns() {
+  unsigned long long t;
+  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+  return t;
+}
+
+// Limits of the precision-form kernels' bounded waits (clock64 cycles): the
 // defaults, or the values a test set with pmcim_debug_wait_limits.
 long long wait_limit_tc();
 long long wait_limit_handoff();
 cudaError_t prepare_factor_fp64();   // shared-memory limits; call outside graph capture
 cudaError_t prepare_factor_mixed();
 cudaError_t launch_factor_solve_fp64(const NodeArgs& a, cudaStream_t s);
-cudaError_t launch_factor_solve_mixed(const NodeArgs& a, cudaStream_t s);
-int mixed_slots_per_cta();  // workspace slots each CTA of the mixed kernel cycles through
+cudaError_t launch_factor_solve_mixed(const MixedArgs& a, int sms, cudaStream_t s, int* launched);
+// the residuals of sweep sw's active nodes (oz_refine.cu)
+cudaError_t prepare_oz_refine();
+cudaError_t launch_oz_residual(const MixedArgs& a, int sw, int sms, cudaStream_t s);
+size_t oz_slot_bytes(int n, int l, int n_dense);  // digits of f_k X of one slot
 // dst[i] = complex64(src[i]), i < count (the FP32 copy of the coefficients)
 cudaError_t round_coefficients_c64(const double2* src, float2* dst, size_t count, cudaStream_t s);
 // Exact BF16 digits of the n_dense dense coefficients (ozaki.cu): row exponents
@@ -275,10 +348,6 @@ int factor_slots_fp64(int n, int l);
 int resident_ctas(int n, int l);  // CTAs per SM, 0 when a node does not fit
 cudaError_t prepare_factor_resident();
 cudaError_t launch_factor_solve_resident(const NodeArgs& a, int max_l, cudaStream_t s);
-// Phases of the precision-form node kernel timed with clock64 when profiling.
-// assemble, LU panels, first solve, residual, correction solves, fallback, set-up,
-// LU triangular solves, LU trailing updates, 3 unused
-#define PMCIM_PHASES PMCIM_PHASE_COUNT
 __host__ __device__ inline size_t mixed_residual_offset(int n, int l) {
   return (((size_t)n * (n + l) * 8) + 255) & ~(size_t)255;
 }
@@ -287,6 +356,7 @@ __host__ __device__ inline size_t mixed_lists_offset(int n, int l) {
   return (mixed_residual_offset(n, l) + (size_t)n * l * 16 + 255) & ~(size_t)255;
 }
 size_t mixed_slot_bytes(int n, int l);
+size_t mixed_fallback_bytes(int n, int l);
 
 struct LevelArgs {
   const ProblemDev* probs;
@@ -389,5 +459,6 @@ cudaError_t launch_gather_vecs(const double2* src, double2* dst, const VecItem* 
 // caller has synchronised the stream.
 // ---------------------------------------------------------------------------
 void prof_begin(int kind, cudaStream_t s);
+void prof_count(int kind, int launches);  // kernels of a bracket beyond its first
 void prof_end(int kind, cudaStream_t s);
 void prof_flush();

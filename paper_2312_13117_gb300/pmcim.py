@@ -174,7 +174,7 @@ def pmcim_profile_reset():
 
 
 def debug_wait_limits(tc_wait_cycles: int = 0, handoff_wait_cycles: int = 0):
-    """Limits of the precision-form kernel's bounded waits (0 = default); for tests."""
+    """Limits of the precision-form kernels' bounded waits (0 = default); for tests."""
     _check(load().pmcim_debug_wait_limits(int(tc_wait_cycles), int(handoff_wait_cycles)), "pmcim_debug_wait_limits")
 
 
@@ -187,23 +187,17 @@ def pmcim_profile_read() -> dict:
     cyc[11] = 0.0
     tot = sum(cyc)
     if tot > 0:
-        # the node kernel runs two thread groups side by side: each phase is given
-        # as a share of its own group's clock
         names = ["assemble", "lu_panel", "first_solve", "residual_fp64", "correction_solve", "fp64_fallback",
-                 "node_setup", "lu_trsm", "lu_update", "factor_wait", "refine_wait", "cta_wall", "lu_swaps",
+                 "node_setup", "lu_trsm", "lu_update", "unused9", "unused10", "cta_wall", "lu_swaps",
                  "unused13", "unused14", "unused15"]
-        factor = {0, 1, 6, 7, 8, 9, 12}
-        tot_f = sum(c for i, c in enumerate(cyc) if i in factor) or 1.0
-        tot_r = sum(c for i, c in enumerate(cyc) if i not in factor) or 1.0
-        share = {nm: c / (tot_f if i in factor else tot_r) for i, (nm, c) in enumerate(zip(names, cyc)) if c > 0}
+        share = {nm: c / tot for nm, c in zip(names, cyc) if c > 0}
         share["lu_fp32"] = sum(share.get(k, 0.0) for k in ("lu_panel", "lu_swaps", "lu_trsm", "lu_update"))
         out["factor_fp32"]["phase_share"] = share
         out["factor_fp32"]["phase_cycles"] = {nm: c for nm, c in zip(names, cyc) if c > 0}
         if wall_ns > 0:
-            # SM cycles the refine group accounted for per ns of CTA lifetime: the
-            # effective SM clock the node kernel ran at, in GHz
+            # SM cycles in the steps per ns of CTA lifetime: the effective SM clock, in GHz
             out["factor_fp32"]["cta_wall_ns"] = wall_ns
-            out["factor_fp32"]["effective_clock_ghz"] = tot_r / wall_ns
+            out["factor_fp32"]["effective_clock_ghz"] = tot / wall_ns
     return out
 
 
