@@ -74,10 +74,11 @@ extern "C" {
    PMCIM_PREC_FP32_IR for it, and pmcim_residual refuses it (EINVAL: the
    tensor-core residual needs coefficient matrices). The entries are formed on
    the device from J_1 and H_1^(1) of complex argument w = z r (ascending series
-   for |w| <= 13, Hankel's expansion above), for Re(z) > 0: relative error at
-   most about 5e-12 where Im(w) <= 0 (the scattering poles lie in Im z < 0) and
-   4e-11 for 0 < Im(w) <= 2; above that the series loses about e^{2 Im w}
-   rounding units to cancellation in H_1^(1) = J_1 + i Y_1. */
+   for |w| <= 6, backward recurrence up to 13, Hankel's expansion above), for
+   Re(z) > 0: relative error at most about 1e-14 for |w| <= 13 and 3e-12 above
+   where Im(w) <= 0 (the scattering poles lie in Im z < 0), and 1e-13 and 2e-12
+   for 0 < Im(w) <= 2; above that H_1^(1) = J_1 + i Y_1 loses about e^{2 Im w}
+   rounding units to cancellation. */
 #define PMCIM_F_HELMHOLTZ_DLP 2
 
 typedef struct {

@@ -17,7 +17,8 @@ LIBDIR = os.path.join(HERE, "lib")
 OBJDIR = os.path.join(HERE, "_build")
 LIB = os.path.join(LIBDIR, "libpmcim.so")
 SOURCES = ["api.cu", "lu_fp64.cu", "lu_mixed.cu", "reduce.cu", "beyn.cu", "screen.cu", "lu_small.cu", "lu_resident.cu",
-           "ozaki.cu", "oz_refine.cu"]
+           "ozaki.cu", "oz_refine.cu",
+           "bie_nodes.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", "-O2",
          "--expt-relaxed-constexpr", "-Xptxas", "-warn-spills"]

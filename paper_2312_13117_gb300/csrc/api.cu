@@ -243,6 +243,7 @@ long long wait_limit_handoff() {
 struct Workspace {
   DevBuf probs, regions, items, counters, node_info, X;
   DevBuf work64, piv64, work32, t64, phase;
+  DevBuf tdig, texp;                     // boundary-integral nodes: digits of T(z_j), row exponents
   DevBuf mstate, mctl, mlists, mubase;  // precision forms: node states, counters, node lists, list bases
   DevBuf C0, C1, pf_half, pf_abs, ind, pf_norm, pf_scale, cand;
   DevBuf bwork, bsigma, bp, blam, bvecs, bkept, bstatus;
@@ -266,7 +267,7 @@ struct Workspace {
     stream = nullptr;
     ordered = nullptr;
     DevBuf* b[] = {&probs, &regions, &items, &counters, &node_info, &X, &work64, &piv64, &work32, &t64,
-                   &phase, &mstate, &mctl, &mlists, &mubase, &C0, &C1, &pf_half, &pf_abs, &ind, &pf_norm, &pf_scale, &cand, &bwork, &bsigma,
+                   &phase, &tdig, &texp, &mstate, &mctl, &mlists, &mubase, &C0, &C1, &pf_half, &pf_abs, &ind, &pf_norm, &pf_scale, &cand, &bwork, &bsigma,
                    &bp, &blam, &bvecs, &bkept, &bstatus, &vlam, &vprob, &voff, &vsig, &vacc, &vwork,
                    &vvec, &vpiv, &gitems, &gdst, &gperm, &ind3, &feats, &sprob, &sparams, &sscratch, &Xkeep,
                    &citems, &vout, &Cm, &iprobs, &iregions, &iitems, &iX, &iinfo, &icounters, &ibord, &ioffs, &ysl, &gexp, &rz,
@@ -477,8 +478,8 @@ struct MixedPlan {
   std::vector<int> ubase;                       // per chunk and problem: first unit of its list
   size_t n_probs = 0, max_count = 0;
   size_t work = 0, t64 = 0, ysl = 0;
-  size_t t64_stride = 0, ysl_stride = 0;
-  int gexp_stride = 0;
+  size_t t64_stride = 0, ysl_stride = 0, tdig_stride = 0;
+  int gexp_stride = 0, texp_stride = 0;
   int unit_cap = 0;
 };
 
@@ -488,26 +489,32 @@ void plan_mixed(Workspace& ws, const std::vector<ProblemDev>& pd, const std::vec
   mp->n_probs = pd.size();
   mp->chunks.emplace_back();
   if (count == 0) return;
-  int max_l = 1, t64_n = 0, nd = 0;
-  size_t ysl = 0;
+  int max_l = 1, nd = 0;
+  size_t ysl = 0, t64 = 0;
   for (size_t i = 0; i < count; ++i) {
     const RegionDev& r = rd[items[off + i].region];
     const ProblemDev& P = pd[r.prob];
     max_l = std::max(max_l, P.l);
-    if (r.herm || P.bie || (P.n_dense >= 2 && !oz)) t64_n = std::max(t64_n, P.n);
-    if (oz && !r.herm && !P.bie) {
-      ysl = std::max(ysl, oz_slot_bytes(P.n, P.l, P.n_dense));
-      nd = std::max(nd, P.n_dense);
+    const bool column = oz && P.bie && P.bie_circ && P.n_dense == 0;  // mixed_column_only
+    if (r.herm || P.bie || (P.n_dense >= 2 && !oz)) t64 = std::max(t64, (size_t)P.n * (column ? 1 : P.n));
+    if (oz && !r.herm) {
+      const int terms = P.bie ? 1 : P.n_dense;
+      ysl = std::max(ysl, oz_slot_bytes(P.n, P.l, terms));
+      nd = std::max(nd, terms);
+      if (P.bie) {
+        mp->tdig_stride = std::max(mp->tdig_stride, coefficient_digit_bytes(P.n, 1));
+        mp->texp_stride = std::max(mp->texp_stride, (P.n + 127) / 128 * 128);
+      }
     }
   }
-  mp->t64_stride = std::max(mp->t64_stride, (size_t)t64_n * t64_n);
+  mp->t64_stride = std::max(mp->t64_stride, t64);
   mp->ysl_stride = std::max(mp->ysl_stride, ysl);
   mp->gexp_stride = std::max(mp->gexp_stride, nd * PMCIM_MAX_L);
-  const size_t budget = slot_budget(ws.work32.cap + ws.t64.cap + ws.ysl.cap);
+  const size_t budget = slot_budget(ws.work32.cap + ws.t64.cap + ws.ysl.cap + ws.tdig.cap);
   for (size_t i = 0; i < count;) {
     MixedChunk ch{off + i, 0, pd[rd[items[off + i].region].prob].n, max_l, 0};
     const size_t slot = mixed_slot_bytes(ch.max_n, ch.max_l);
-    const size_t per = slot + mp->t64_stride * sizeof(double2) + mp->ysl_stride;
+    const size_t per = slot + mp->t64_stride * sizeof(double2) + mp->ysl_stride + mp->tdig_stride;
     const size_t cap = std::max<size_t>(
         1, std::min(budget / per, std::max<size_t>(kChunkBytes / per, (size_t)kChunkNodesPerSm * sms)));
     ch.count = std::min(cap, count - i);
@@ -539,6 +546,14 @@ int ensure_mixed(Call& c, const MixedPlan& mp, int max_sweeps, MixedArgs* ma) {
   if (mp.t64_stride) CU(ws.t64.ensure(cnt * mp.t64_stride * sizeof(double2)));
   if (mp.ysl_stride) CU(ws.ysl.ensure(cnt * mp.ysl_stride));
   if (mp.gexp_stride) CU(ws.gexp.ensure(cnt * mp.gexp_stride * sizeof(int32_t)));
+  if (mp.tdig_stride) {
+    CU(ws.tdig.ensure(cnt * mp.tdig_stride));
+    CU(ws.texp.ensure(cnt * mp.texp_stride * sizeof(int32_t)));
+    ma->tdig = ws.tdig.as<unsigned char>();
+    ma->tdig_stride = mp.tdig_stride;
+    ma->texp = ws.texp.as<int32_t>();
+    ma->texp_stride = mp.texp_stride;
+  }
   CU(ws.mstate.ensure(cnt * sizeof(MixedState)));
   CU(ws.mctl.ensure(mixed_ctl_ints((int)mp.n_probs, max_sweeps) * sizeof(int)));
   CU(ws.mlists.ensure((3 * cnt + 2 * (size_t)mp.unit_cap) * sizeof(int)));
@@ -951,7 +966,7 @@ int run_level(Call& c, const std::vector<HostRegion>& regs, bool gate_top, bool 
     // nodes whose residuals have no coefficient digits
     for (const NodeItem& it : items) {
       const ProblemDev& P = c.pd[rd[it.region].prob];
-      if (P.bie || P.n_dense == 0) ma.res64 = 1;
+      if (P.bie ? !ma.tdig : P.n_dense == 0) ma.res64 = 1;
     }
     if (!tc_residual(c.opt)) ma.res64 = 1;
   }

@@ -33,29 +33,35 @@ namespace bie {
 
 constexpr double kPi = 3.14159265358979323846;
 constexpr double kEulerGamma = 0.57721566490153286061;
-constexpr double kSeriesMax = 13.0;  // |w| at or below: ascending series; above: Hankel's expansion
-constexpr int kSeriesTerms = 96, kAsymTerms = 64;
+constexpr double kSeriesMax = 6.0;   // |w| at or below: ascending series
+constexpr double kMillerMax = 13.0;  // at or below: backward recurrence; above: Hankel's expansion
+constexpr int kMillerTop = 46;       // J_46(w) is below 1e-20 of the largest J_k for |w| <= 13
+constexpr int kSeriesTerms = 32, kAsymTerms = 64;
 
-// The series' coefficients, made at compile time in the order the loops below would
-// compute them (so the results are those of dividing in the loop), and read from the
-// constant cache on the device instead of two FP64 divisions per term:
-//   inv_kk1[k] = 1 / (k (k+1)),  psi2[k] = psi(k+1) + psi(k+2) = 2 (H_k - gamma) + 1/(k+1),
+// The series' coefficients, made at compile time and read from the constant cache:
+//   cj[k] = 1 / (k! (k+1)!),  cs[k] = (psi(k+1) + psi(k+2)) / (k! (k+1)!) with
+//   psi(k+1) + psi(k+2) = 2 (H_k - gamma) + 1/(k+1),
+//   nm[2k+1] = (-1)^k (2k+1) / (k (k+1))  (Neumann's series),
 //   ak[k] = prod_{j=1..k} (4 - (2j-1)^2) / (8 j)  (Hankel's a_k for order 1).
 struct SeriesTables {
-  double inv_kk1[kSeriesTerms];
-  double psi2[kSeriesTerms];
+  double cj[kSeriesTerms];
+  double cs[kSeriesTerms];
+  double nm[kMillerTop + 1];
   double ak[kAsymTerms];
 };
 constexpr SeriesTables make_series_tables() {
   SeriesTables T{};
-  double Hk = 0.0;
-  T.inv_kk1[0] = 0.0;
-  T.psi2[0] = 1.0 - 2.0 * kEulerGamma;
+  double Hk = 0.0, f = 1.0;
+  T.cj[0] = 1.0;
+  T.cs[0] = 1.0 - 2.0 * kEulerGamma;
   for (int k = 1; k < kSeriesTerms; ++k) {
-    T.inv_kk1[k] = 1.0 / ((double)k * (double)(k + 1));
+    f /= (double)k * (double)(k + 1);
     Hk += 1.0 / (double)k;
-    T.psi2[k] = 2.0 * (Hk - kEulerGamma) + 1.0 / (double)(k + 1);
+    T.cj[k] = f;
+    T.cs[k] = f * (2.0 * (Hk - kEulerGamma) + 1.0 / (double)(k + 1));
   }
+  for (int k = 1; 2 * k + 1 <= kMillerTop; ++k)
+    T.nm[2 * k + 1] = ((k & 1) ? -1.0 : 1.0) * (double)(2 * k + 1) / ((double)k * (double)(k + 1));
   double a = 1.0;
   T.ak[0] = 1.0;
   for (int k = 1; k < kAsymTerms; ++k) {
@@ -87,49 +93,112 @@ BIE_HD double2 crec(double2 b) {                                    // 1 / b (Sm
   return make_double2(t / d, -1.0 / d);
 }
 
-// J_1(w) and H_1^(1)(w) for Re w > 0.
-//  |w| <= 13: the ascending series J_1(w) = sum_k (-1)^k (w/2)^{2k+1} / (k! (k+1)!) and
+// What the entries of one wave number kappa share.
+struct Wave {
+  double2 kappa, inv;   // kappa, 1 / kappa
+  double2 lg;           // log(kappa / 2)
+  double2 pref;         // sqrt(2 / (pi kappa))
+  double mod;           // |kappa|
+};
+BIE_HD Wave wave_of(double2 kappa) {
+  Wave W;
+  W.kappa = kappa;
+  W.inv = crec(kappa);
+  W.mod = hypot(kappa.x, kappa.y);
+  const double arg = atan2(kappa.y, kappa.x);
+  W.lg = make_double2(log(0.5 * W.mod), arg);
+  double s, c;
+  sincos(-0.5 * arg, &s, &c);
+  const double m = sqrt(2.0 / (kPi * W.mod));
+  W.pref = make_double2(m * c, m * s);
+  return W;
+}
+
+// J_1(w) and H_1^(1)(w), w = kappa r, for Re w > 0; ri = 1 / r, lr = log r.
+//  |w| <= 6: the ascending series J_1(w) = sum_k (-1)^k (w/2)^{2k+1} / (k! (k+1)!) and
 //    Y_1(w) = -2 / (pi w) + (2/pi) log(w/2) J_1(w)
 //             - (1/pi) sum_k (psi(k+1) + psi(k+2)) (-1)^k (w/2)^{2k+1} / (k! (k+1)!)
 //    (DLMF 10.2.2 and 10.8.1; psi(k+1) = -gamma + H_k with H_k the harmonic number),
-//    H_1^(1) = J_1 + i Y_1 (DLMF 10.4.3). Summed until a term falls below 1e-17 of the
-//    largest one.
+//    H_1^(1) = J_1 + i Y_1 (DLMF 10.4.3). Both sums are polynomials in -(w/2)^2 with real
+//    coefficients, by Horner's rule, 8 FP64 operations per term (a term with a running
+//    product and a stopping test took about 20, and FP64 bounds the assembly). The number
+//    of terms, ceil(5.9 + 3 |w| - 0.095 |w|^2), leaves out less than 1e-17 of the largest
+//    term; a warp takes its largest, so that its lanes read the same coefficients. Near the
+//    real axis the sums cancel to e^{-|w|} of their largest term, which sets the range.
+//  6 < |w| <= 13: J_k by the backward recurrence J_{k-1} = (2k / w) J_k - J_{k+1} (DLMF
+//    3.6(iii)) from k = 46, scaled by e^{+-iw} = J_0 + 2 sum_k (+-i)^k J_k (DLMF 10.12.1; the
+//    sign that makes the left side large), and Y_1 by Neumann's series (Abramowitz & Stegun
+//    9.1.88): Y_1 = -2 J_0 / (pi w) + (2/pi) ((log(w/2) + gamma - 1) J_1
+//    - sum_k (-1)^k (2k+1) / (k (k+1)) J_{2k+1}).
 //  |w| > 13: Hankel's expansions (DLMF 10.17.5, 10.17.6)
 //    H_1^(1,2)(w) ~ sqrt(2 / (pi w)) e^{+-i (w - 3 pi / 4)} sum_k (+-i)^k a_k / w^k,
 //    a_k = prod_{j=1..k} (4 - (2j - 1)^2) / (k! 8^k), truncated before the smallest term
 //    grows again, and J_1 = (H_1^(1) + H_1^(2)) / 2 (DLMF 10.4.4).
-BIE_HD void j1_h1(double2 w, double2* J, double2* H) {
-  const double aw = hypot(w.x, w.y);
+BIE_HD void j1_h1(const Wave& W, double r, double ri, double lr, double2* J, double2* H) {
+  const SeriesTables& TB = BIE_TABLES;
+  const double2 w = cs(W.kappa, r);
+  const double aw = W.mod * r;
+  const double2 iw = cs(W.inv, ri);
   if (aw <= kSeriesMax) {
     const double2 h = cs(w, 0.5);
-    const double2 hh = cm(h, h);
-    const double2 u = make_double2(-hh.x, -hh.y);  // -(w/2)^2
-    const SeriesTables& TB = BIE_TABLES;
-    double2 t = h;                                 // k = 0 term
-    double2 Js = t;
-    double2 S = cs(t, TB.psi2[0]);                 // psi(1) + psi(2)
-    double tmax = fabs(t.x) + fabs(t.y);
-    const double au = hypot(u.x, u.y);
-    for (int k = 1; k < kSeriesTerms; ++k) {
-      t = cs(cm(t, u), TB.inv_kk1[k]);
-      Js = ca(Js, t);
-      S = ca(S, cs(t, TB.psi2[k]));
-      const double at = fabs(t.x) + fabs(t.y);
-      tmax = fmax(tmax, at);
-      if ((double)k * (double)(k + 1) > au && at <= 1e-17 * tmax) break;
+    const double2 u = make_double2(h.y * h.y - h.x * h.x, -2.0 * h.x * h.y);  // -(w/2)^2
+    const float fw = (float)aw;
+    int k = (int)ceilf(5.9f + fw * (3.0f - 0.095f * fw)) - 1;
+#if defined(__CUDA_ARCH__)
+    k = __reduce_max_sync(__activemask(), k);
+#endif
+    double2 p = make_double2(TB.cj[k], 0.0), q = make_double2(TB.cs[k], 0.0);
+    for (--k; k >= 0; --k) {
+      const double px = fma(p.x, u.x, fma(-p.y, u.y, TB.cj[k])), qx = fma(q.x, u.x, fma(-q.y, u.y, TB.cs[k]));
+      p.y = fma(p.x, u.y, p.y * u.x);
+      q.y = fma(q.x, u.y, q.y * u.x);
+      p.x = px;
+      q.x = qx;
     }
-    // log(w/2) = log|w/2| + i arg(w)
-    const double2 lg = make_double2(log(0.5 * aw), atan2(w.y, w.x));
-    const double2 iw = crec(w);
-    double2 Y = cs(iw, -2.0 / kPi);
-    Y = ca(Y, cs(cm(lg, Js), 2.0 / kPi));
-    Y = ca(Y, cs(S, -1.0 / kPi));
+    const double2 Js = cm(h, p), S = cm(h, q);
+    const double2 lg = make_double2(W.lg.x + lr, W.lg.y);  // log(w/2)
+    const double2 lj = cm(lg, Js);
+    const double2 Y = make_double2((2.0 / kPi) * (lj.x - iw.x) - (1.0 / kPi) * S.x,
+                                   (2.0 / kPi) * (lj.y - iw.y) - (1.0 / kPi) * S.y);
     *J = Js;
     *H = ca(Js, ci(Y));
     return;
   }
-  const SeriesTables& TB = BIE_TABLES;
-  const double2 iw = crec(w);
+  if (aw <= kMillerMax) {
+    const double sg = w.y <= 0.0 ? 1.0 : -1.0;
+    double2 up = make_double2(0.0, 0.0), cur = make_double2(1e-30, 0.0);  // J_{k+1}, J_k up to a factor
+    double2 sum = up, nm = up, j1 = up;  // sum_k (+-i)^k J_k, Neumann's series
+    for (int k = kMillerTop; k >= 1; --k) {
+      switch (k & 3) {  // (sg i)^k
+        case 0: sum.x += cur.x; sum.y += cur.y; break;
+        case 1: sum.x -= sg * cur.y; sum.y += sg * cur.x; break;
+        case 2: sum.x -= cur.x; sum.y -= cur.y; break;
+        default: sum.x += sg * cur.y; sum.y -= sg * cur.x; break;
+      }
+      if ((k & 1) && k > 1) {
+        nm.x = fma(TB.nm[k], cur.x, nm.x);
+        nm.y = fma(TB.nm[k], cur.y, nm.y);
+      }
+      if (k == 1) j1 = cur;
+      const double2 f = cs(iw, 2.0 * (double)k);
+      const double2 dn = make_double2(fma(f.x, cur.x, fma(-f.y, cur.y, -up.x)),
+                                      fma(f.x, cur.y, fma(f.y, cur.x, -up.y)));
+      up = cur;
+      cur = dn;
+    }
+    sum = make_double2(fma(2.0, sum.x, cur.x), fma(2.0, sum.y, cur.y));
+    double so, co;
+    sincos(sg * w.x, &so, &co);
+    const double em = exp(-sg * w.y);
+    const double2 scale = cm(make_double2(em * co, em * so), crec(sum));
+    const double2 J0 = cm(cur, scale), Js = cm(j1, scale), S = cm(nm, scale);
+    const double2 lg = make_double2(W.lg.x + lr + (kEulerGamma - 1.0), W.lg.y);
+    const double2 lj = cm(lg, Js), jw = cm(iw, J0);
+    const double2 Y = cs(make_double2(lj.x - S.x - jw.x, lj.y - S.y - jw.y), 2.0 / kPi);
+    *J = Js;
+    *H = ca(Js, ci(Y));
+    return;
+  }
   double2 p = make_double2(1.0, 0.0);   // 1 / w^k
   double2 s1 = p, s2 = p;               // sums with (+i)^k and (-i)^k
   double prev = 1.0;
@@ -151,12 +220,7 @@ BIE_HD void j1_h1(double2 w, double2* J, double2* H) {
     prev = mag;
     if (mag < 1e-17) break;
   }
-  // sqrt(2 / (pi w)) = sqrt(2 / pi) |w|^{-1/2} e^{-i arg(w) / 2}
-  const double ph = -0.5 * atan2(w.y, w.x);
-  double sp, cp;
-  sincos(ph, &sp, &cp);
-  const double mod = sqrt(2.0 / (kPi * aw));
-  const double2 pref = make_double2(mod * cp, mod * sp);
+  const double2 pref = cs(W.pref, sqrt(ri));
   double so, co;
   sincos(w.x - 0.75 * kPi, &so, &co);
   const double eu = exp(-w.y), ed = exp(w.y);
@@ -167,28 +231,59 @@ BIE_HD void j1_h1(double2 w, double2* J, double2* H) {
   *H = h1;
   *J = cs(ca(h1, h2), 0.5);
 }
+BIE_HD void j1_h1(double2 w, double2* J, double2* H) { j1_h1(wave_of(w), 1.0, 1.0, 0.0, J, H); }
 
-// Entry (i, j) of K_n(kappa). G: the device geometry of the term (n >= 4, even),
+// Entries (i, j) and (j, i), i != j, of K_n(kappa). They share r and with it the Bessel
+// values, and differ in the normal: K_ij = (n(t_j).(x_i - x_j) / r) F, K_ji =
+// (n(t_i).(x_j - x_i) / r) F with F = kappa ((i h / 2) H_1 - (G[5 n + m] / 2 pi) J_1).
+// G: the device geometry of the term (n >= 4, even),
 //   G[5 j + 0..4] = x1, x2, n1 = x2', n2 = -x1', d = n.x'' / (2 pi |x'|^2) at t_j,
 //   G[5 n + m]    = R_m - (2 pi / n) log(4 sin^2(pi m / n))  (m = 1..n-1; m = 0 unused),
 //   G[6 n]        = 1 when the sampled curve is invariant under the shift j -> j + 1 (a
 //                   circle), so that K_n is circulant: K_ij = K_{(i-j) mod n, 0}; else 0.
-BIE_ENTRY double2 dlp_entry(const double* G, int n, int i, int j, double2 kappa) {
+BIE_ENTRY void dlp_pair(const double* G, int n, int i, int j, const Wave& W, double2* Kij, double2* Kji) {
   const double h = 2.0 * kPi / (double)n;
-  const double* pj = G + 5 * (size_t)j;
-  if (i == j) return make_double2(h * pj[4], 0.0);
   const double* pi_ = G + 5 * (size_t)i;
+  const double* pj = G + 5 * (size_t)j;
   const double ex = pi_[0] - pj[0], ey = pi_[1] - pj[1];
-  const double r = hypot(ex, ey);
-  const double qr = (pj[2] * ex + pj[3] * ey) / r;  // n(t_j).(x_i - x_j) / r
+  const double rr = ex * ex + ey * ey;
+#if defined(__CUDA_ARCH__)
+  const double ri = rsqrt(rr);
+#else
+  const double ri = 1.0 / sqrt(rr);
+#endif
+  const double r = rr * ri;
   double2 J1, H1;
-  j1_h1(cs(kappa, r), &J1, &H1);
-  const double2 kq = cs(kappa, qr);
-  const double2 L = ci(cs(cm(kq, H1), 0.5));             // (i kappa / 2) q H_1 / r
-  const double2 L1 = cs(cm(kq, J1), -1.0 / (2.0 * kPi));  // -(kappa / 2 pi) q J_1 / r
-  int m = i - j;
-  if (m < 0) m += n;
-  return ca(cs(L, h), cs(L1, G[5 * (size_t)n + m]));
+  j1_h1(W, r, ri, log(r), &J1, &H1);
+  const int m = i > j ? i - j : i - j + n;
+  const double wj = G[5 * (size_t)n + m] * (1.0 / (2.0 * kPi)), wh = 0.5 * h;
+  const double2 F = cm(W.kappa, make_double2(-wh * H1.y - wj * J1.x, wh * H1.x - wj * J1.y));
+  *Kij = cs(F, (pj[2] * ex + pj[3] * ey) * ri);
+  *Kji = cs(F, -(pi_[2] * ex + pi_[3] * ey) * ri);
+}
+// A diagonal entry.
+BIE_HD double2 dlp_diagonal(const double* G, int n, int j) {
+  return make_double2(2.0 * kPi / (double)n * G[5 * (size_t)j + 4], 0.0);
+}
+// Entry (i, j) alone.
+BIE_HD double2 dlp_entry(const double* G, int n, int i, int j, const Wave& W) {
+  if (i == j) return dlp_diagonal(G, n, j);
+  double2 a, b;
+  dlp_pair(G, n, i, j, W, &a, &b);
+  return a;
+}
+BIE_HD double2 dlp_entry(const double* G, int n, int i, int j, double2 kappa) {
+  return dlp_entry(G, n, i, j, wave_of(kappa));
+}
+
+// Pair number p of the n (n/2) - n/2 pairs {i, j}, i != j: column j and row j + d mod n with
+// d = 1 + p / n, so that consecutive p share d (and nearly r). False past the last one.
+BIE_HD bool pair_of(int n, int p, int* i, int* j) {
+  const int d = 1 + p / n;
+  *j = p - (d - 1) * n;
+  if (d > n / 2 || (d == n / 2 && *j >= n / 2)) return false;
+  *i = *j + d < n ? *j + d : *j + d - n;
+  return true;
 }
 
 constexpr int kCirculantMaxN = 8192;  // the shift-invariance test is O(n^2)

@@ -29,6 +29,7 @@ using namespace lucore;
 struct NodeSmem {
   LuSmem lu;
   ProblemDev P;
+  bie::Wave wave;
   int item;
 };
 
@@ -56,6 +57,7 @@ __global__ void __launch_bounds__(THREADS, 2) k_factor_solve_fp64(NodeArgs a) {
     double2 z, w;
     node_weight(rg.cre, rg.cim, rg.r, rg.N, it.j, &z, &w);
     if (tid < P.K) sm.lu.fz[tid] = eval_f(P.term[tid], z);
+    if (BIE && tid == 0) sm.wave = bie::wave_of(z);
     __syncthreads();
 
     // assemble [T(z_j) | V]
@@ -65,7 +67,7 @@ __global__ void __launch_bounds__(THREADS, 2) k_factor_solve_fp64(NodeArgs a) {
     double2* circ = M + nn;
     const bool use_circ = BIE && P.bie_circ;
     if (use_circ) {
-      for (int m = tid; m < n; m += THREADS) circ[m] = bie::dlp_entry(P.bie, n, m, 0, z);
+      for (int m = tid; m < n; m += THREADS) circ[m] = bie::dlp_entry(P.bie, n, m, 0, sm.wave);
       __syncthreads();
     }
     for (int col = 0; col < n; ++col) {
@@ -79,12 +81,17 @@ __global__ void __launch_bounds__(THREADS, 2) k_factor_solve_fp64(NodeArgs a) {
           } else if (use_circ && t.kind == PMCIM_F_HELMHOLTZ_DLP) {
             const int m = row >= col ? row - col : row - col + n;
             cfma(v, t.id, circ[m]);
-          } else {
-            cfma_term<BIE>(v, P, t, sm.lu.fz[k], row, col);
+          } else if (row == col && t.kind != PMCIM_F_HELMHOLTZ_DLP) {
+            cfma(v, sm.lu.fz[k], t.id);
           }
         }
         M[e] = v;
       }
+    }
+    if (BIE && P.bie && !use_circ) {
+      __syncthreads();
+      add_layer(P.bie, n, layer_coefficient(P), sm.wave, tid, THREADS,
+                [&](int i, int j, double2 v) { M[(size_t)j * n + i] = cadd(M[(size_t)j * n + i], v); });
     }
     if (use_circ) __syncthreads();  // circ is read above and overwritten by V below
     for (size_t e = tid; e < (size_t)n * l; e += THREADS) M[nn + e] = P.V[e];
@@ -107,6 +114,7 @@ __global__ void __launch_bounds__(THREADS, 2) k_factor_solve_fp64(NodeArgs a) {
 struct VerifySmem {
   LuSmem lu;
   ProblemDev P;
+  bie::Wave wave;
   double2 red2[THREADS / 32];
   double red[THREADS / 32];
   double2 bc;
@@ -190,16 +198,24 @@ __global__ void __launch_bounds__(THREADS, 2) k_verify_fp64(ValueArgs a) {
     double2* yv = x + 2 * n;
     const double2 lam = a.lam[it];
     if (tid < P.K) sm.lu.fz[tid] = eval_f(P.term[tid], lam);
+    if (BIE && tid == 0) sm.wave = bie::wave_of(lam);
     __syncthreads();
+    if (BIE && P.bie) {
+      for (size_t e = tid; e < nn; e += THREADS) M[e] = make_double2(0.0, 0.0);
+      __syncthreads();
+      add_layer(P.bie, n, layer_coefficient(P), sm.wave, tid, THREADS,
+                [&](int i, int j, double2 v) { M[(size_t)j * n + i] = v; });
+      __syncthreads();
+    }
     double fro = 0.0;
     for (int col = 0; col < n; ++col) {
       for (int row = tid; row < n; row += THREADS) {
         const size_t e = (size_t)col * n + row;
-        double2 v = make_double2(0.0, 0.0);
+        double2 v = BIE && P.bie ? M[e] : make_double2(0.0, 0.0);
         for (int k = 0; k < P.K; ++k) {
           const TermDesc& t = P.term[k];
           if (t.dense) cfma(v, sm.lu.fz[k], P.A[(size_t)t.mat_index * nn + e]);
-          else cfma_term<BIE>(v, P, t, sm.lu.fz[k], row, col);
+          else if (row == col && t.kind != PMCIM_F_HELMHOLTZ_DLP) cfma(v, sm.lu.fz[k], t.id);
         }
         M[e] = v;
         fro += cabs2(v);

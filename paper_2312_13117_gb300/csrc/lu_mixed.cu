@@ -331,21 +331,13 @@ __device__ void residual_fp64_col(const double2* __restrict__ X, double2* __rest
 // T(z_j) in FP64 into T (n x n, column-major), the matrix of the refinement
 // residuals, and rounded to complex64 into M32 (leading dimension n), the FP32
 // LU's matrix: the dense terms in one pass over the elements, four elements per
-// thread at a time so that their coefficient loads overlap, then a boundary-
-// integral term (bie.cuh; a circulant one from its first column, formed in
-// scratch, n values), then the identity terms on the diagonal. herm: T(z_j)^H
-// instead (the coefficients read transposed, the sum conjugated; used by the
-// certificates' bordered steps, which problems with a boundary-integral term do
-// not take).
-template <bool BIE>
-__device__ void assemble_fp64(const NodeCtx& cx, double2* __restrict__ T, float2* __restrict__ M32, bool herm,
-                              double2* __restrict__ scratch) {
+// thread at a time so that their coefficient loads overlap, then the identity
+// terms on the diagonal. herm: T(z_j)^H instead (the coefficients read transposed,
+// the sum conjugated; used by the certificates' bordered steps).
+__device__ void assemble_fp64(const NodeCtx& cx, double2* __restrict__ T, float2* __restrict__ M32, bool herm) {
   const ProblemDev& P = cx.P;
   const int n = P.n;
   const size_t nn = (size_t)n * n;
-  double2 id = make_double2(0.0, 0.0);
-  for (int k = 0; k < P.K; ++k)
-    if (!P.term[k].dense && P.term[k].kind != PMCIM_F_HELMHOLTZ_DLP) id = cadd(id, cmul(cx.fz[k], P.term[k].id));
   for (size_t e0 = gtid(); e0 < nn; e0 += 4 * (size_t)THREADS) {
     double2 v[4];
 #pragma unroll
@@ -375,26 +367,7 @@ __device__ void assemble_fp64(const NodeCtx& cx, double2* __restrict__ T, float2
     }
   }
   gsync();
-  if (BIE && P.bie && !herm) {
-    int kb = 0;
-    while (kb + 1 < P.K && P.term[kb].kind != PMCIM_F_HELMHOLTZ_DLP) ++kb;
-    const double2 cb = P.term[kb].id, zb = cx.fz[kb];
-    if (P.bie_circ) {
-      for (int m = gtid(); m < n; m += THREADS) scratch[m] = bie::dlp_entry(P.bie, n, m, 0, zb);
-      gsync();
-    }
-    for (int col = 0; col < n; ++col)
-      for (int row = gtid(); row < n; row += THREADS) {
-        const size_t e = (size_t)col * n + row;
-        const double2 kv = P.bie_circ ? scratch[row >= col ? row - col : row - col + n]
-                                      : bie::dlp_entry(P.bie, n, row, col, zb);
-        double2 t = T[e];
-        cfma(t, cb, kv);
-        T[e] = t;
-        M32[e] = make_float2((float)t.x, (float)t.y);
-      }
-    gsync();
-  }
+  double2 id = cx.fid;
   if (herm) id.y = -id.y;
   for (int i = gtid(); i < n; i += THREADS) {
     const size_t e = (size_t)i * n + i;
@@ -403,6 +376,29 @@ __device__ void assemble_fp64(const NodeCtx& cx, double2* __restrict__ T, float2
     M32[e] = make_float2((float)t.x, (float)t.y);
   }
   gsync();
+}
+
+// The FP32 LU's matrix of a boundary-integral node from the FP64 T(z_j) that
+// k_bie_assemble left: the matrix, or the first column of a circulant one, rounded once in
+// stage (n values of shared memory) where it fits.
+__device__ void round_bie(const double2* __restrict__ T, float2* __restrict__ M32, int n, bool column_only,
+                          float2* __restrict__ stage, int stage_elems) {
+  const size_t nn = (size_t)n * n;
+  if (!column_only) {
+#pragma unroll 4
+    for (size_t e = gtid(); e < nn; e += THREADS) M32[e] = make_float2((float)T[e].x, (float)T[e].y);
+    return;
+  }
+  const bool fits = n <= stage_elems;
+  if (fits)
+    for (int m = gtid(); m < n; m += THREADS) stage[m] = make_float2((float)T[m].x, (float)T[m].y);
+  gsync();
+  const int warp = gtid() >> 5, lane = gtid() & 31;
+  for (int col = warp; col < n; col += THREADS / 32)
+    for (int row = lane; row < n; row += 32) {
+      const int m = row >= col ? row - col : row - col + n;
+      M32[(size_t)col * n + row] = fits ? stage[m] : make_float2((float)T[m].x, (float)T[m].y);
+    }
 }
 
 // T(z_j) for the FP32 LU: FP32 arithmetic on the complex64 copy of the A_k
@@ -454,8 +450,8 @@ __device__ void assemble32(const NodeCtx& cx, float2* __restrict__ M32) {
   }
 }
 
-// T(z_j) into the FP32 matrix (rounded) or, for the fallback, the FP64 matrix.
-__device__ void assemble(const NodeCtx& cx, float2* M32, double2* M64) {
+// T(z_j) in FP64 for the fallback.
+__device__ void assemble(const NodeCtx& cx, double2* M64) {
   const ProblemDev& P = cx.P;
   const int n = P.n;
   const size_t nn = (size_t)n * n;
@@ -468,8 +464,7 @@ __device__ void assemble(const NodeCtx& cx, float2* M32, double2* M64) {
         if (t.dense) cfma(v, cx.fz[k], P.A[(size_t)t.mat_index * nn + e]);
         else if (row == col) cfma(v, cx.fz[k], t.id);
       }
-      if (M32) M32[e] = make_float2((float)v.x, (float)v.y);
-      else M64[e] = v;
+      M64[e] = v;
     }
   }
 }
@@ -517,11 +512,6 @@ __device__ __forceinline__ int next_index(const MixedArgs& a, int counter, int t
   return c.item;
 }
 
-// Whether the node's residuals are formed on the tensor cores.
-__device__ __forceinline__ bool node_oz(const MixedArgs& a, const ProblemDev& P, const RegionDev& rg) {
-  return a.oz && P.Adig != nullptr && !rg.herm && P.bie == nullptr;
-}
-
 constexpr uint32_t TMEM_FACTOR = 256;  // columns per CTA, two CTAs per SM
 static_assert(tcu::TMEM_COLS <= TMEM_FACTOR && 2 * tcb::ACC_COLS <= TMEM_FACTOR, "TMEM columns");
 
@@ -559,11 +549,12 @@ __global__ void __launch_bounds__(THREADS, TC ? 2 : 3) k_mixed_factor(MixedArgs 
     const int n = P.n, l = P.l, ncols = n + l;
     const size_t nn = (size_t)n * n, nl = (size_t)n * l;
     pc.mark(PH_SETUP);
-    // T(z_j) in FP64 for the residuals on the FP64 pipe, and rounded; T(z_j)^H likewise;
-    // always with a boundary-integral term (no stored coefficients to take residuals from)
-    if (rg.herm || (P.n_dense >= 2 && !a.oz) || (BIE && P.bie))
-      assemble_fp64<BIE>(c, a.t64 + (size_t)q * a.t64_stride, M32, rg.herm != 0,
-                         reinterpret_cast<double2*>(slot + mixed_residual_offset(n, l)));
+    // T(z_j) in FP64 for the residuals on the FP64 pipe, and rounded; T(z_j)^H likewise
+    if (BIE && P.bie && !rg.herm)
+      round_bie(a.t64 + (size_t)q * a.t64_stride, M32, n, mixed_column_only(a, P),
+                reinterpret_cast<float2*>(cx.stage), scratch_bytes / (int)sizeof(float2));
+    else if (rg.herm || (P.n_dense >= 2 && !a.oz))
+      assemble_fp64(c, a.t64 + (size_t)q * a.t64_stride, M32, rg.herm != 0);
     else
       assemble32(c, M32);
     for (size_t e = tid; e < nl; e += THREADS) M32[nn + e] = make_float2((float)P.V[e].x, (float)P.V[e].y);
@@ -583,7 +574,8 @@ __global__ void __launch_bounds__(THREADS, TC ? 2 : 3) k_mixed_factor(MixedArgs 
       MixedState st{};
       st.info = info;
       st.lost = sm.tc_bad != bad_before ? MIXED_LOST_LU : 0;
-      st.id = c.fid;
+      // a boundary-integral node's residual takes the whole of T(z_j) as its one dense term
+      st.id = BIE && P.bie ? make_double2(0.0, 0.0) : c.fid;
       a.state[q] = st;
     }
   }
@@ -638,7 +630,7 @@ __global__ void __launch_bounds__(THREADS, 3) k_mixed_solve(MixedArgs a, int sw)
     const int* lists = reinterpret_cast<const int*>(slot + mixed_lists_offset(n, l));
     double2* X = a.X + rg.x_off + (size_t)it.j * nl;
     MixedState st = a.state[q];
-    const bool oz = node_oz(a, P, rg);
+    const bool oz = mixed_node_oz(a, P, rg);
     bool ok = st.info == 0, done = false;
     if (sw == 0) {
       if (ok) {
@@ -772,11 +764,17 @@ __global__ void __launch_bounds__(THREADS, 2) k_mixed_fallback(MixedArgs a, size
     double2* M64 = reinterpret_cast<double2*>(a.work + (size_t)blockIdx.x * bytes_per_cta);
     int* piv = reinterpret_cast<int*>(M64 + nn + nl);
     double2* X = a.X + rg.x_off + (size_t)it.j * nl;
-    if (P.bie) {  // T(z_j) as k_mixed_factor assembled it in FP64
+    if (P.bie) {  // T(z_j) as k_bie_assemble left it
       const double2* T64 = a.t64 + (size_t)q * a.t64_stride;
-      for (size_t e = gtid(); e < nn; e += THREADS) M64[e] = T64[e];
+      if (mixed_column_only(a, P)) {
+        for (int col = 0; col < n; ++col)
+          for (int row = gtid(); row < n; row += THREADS)
+            M64[(size_t)col * n + row] = T64[row >= col ? row - col : row - col + n];
+      } else {
+        for (size_t e = gtid(); e < nn; e += THREADS) M64[e] = T64[e];
+      }
     } else {
-      assemble(c, nullptr, M64);
+      assemble(c, M64);
     }
     for (size_t e = gtid(); e < nl; e += THREADS) M64[nn + e] = P.V[e];
     gsync();
@@ -852,6 +850,10 @@ cudaError_t launch_factor_solve_mixed(const MixedArgs& a, int sms, cudaStream_t 
   cudaError_t e = cudaMemsetAsync(a.ctl, 0, mixed_ctl_zero_ints(a.n_probs, a.max_sweeps) * sizeof(int), s);
   if (e != cudaSuccess) return e;
   auto grid = [&](int per_sm) { return per_sm * sms < a.count ? per_sm * sms : a.count; };
+  if (a.bie && a.t64) {
+    e = launch_bie_assemble(a, sms, s, launched);
+    if (e != cudaSuccess) return e;
+  }
   {
     const int scratch = (int)factor_scratch_bytes(a.max_n, a.tc != 0);
     const size_t smem = kFactorHead + scratch;

@@ -18,6 +18,7 @@ struct Head {
   int item;
   ProblemDev P;
   double2 fz[PMCIM_MAX_TERMS];
+  bie::Wave wave;
 };
 constexpr size_t kHeadBytes = (sizeof(Head) + 15) & ~size_t(15);
 
@@ -45,8 +46,12 @@ __global__ void __launch_bounds__(512) k_factor_solve_resident(NodeArgs a) {
     if (tid < P.K) sm.fz[tid] = eval_f(P.term[tid], z);
     // a circulant boundary-integral term's n distinct entries, in the reciprocals' place
     const bool use_circ = BIE && P.bie_circ;
-    if (use_circ)
-      for (int m = tid; m < n; m += blockDim.x) rinv[m] = bie::dlp_entry(P.bie, n, m, 0, z);
+    if (BIE) {
+      if (tid == 0) sm.wave = bie::wave_of(z);
+      __syncthreads();
+      if (use_circ)
+        for (int m = tid; m < n; m += blockDim.x) rinv[m] = bie::dlp_entry(P.bie, n, m, 0, sm.wave);
+    }
     __syncthreads();
     const size_t nn = (size_t)n * n;
     for (int col = warp; col < n; col += nwarp)
@@ -57,10 +62,15 @@ __global__ void __launch_bounds__(512) k_factor_solve_resident(NodeArgs a) {
           if (t.dense) cfma(v, sm.fz[k], P.A[(size_t)t.mat_index * nn + (size_t)col * n + row]);
           else if (use_circ && t.kind == PMCIM_F_HELMHOLTZ_DLP)
             cfma(v, t.id, rinv[row >= col ? row - col : row - col + n]);
-          else cfma_term<BIE>(v, P, t, sm.fz[k], row, col);
+          else if (row == col && t.kind != PMCIM_F_HELMHOLTZ_DLP) cfma(v, sm.fz[k], t.id);
         }
         M[(size_t)col * ld + row] = v;
       }
+    if (BIE && P.bie && !use_circ) {
+      __syncthreads();
+      add_layer(P.bie, n, layer_coefficient(P), sm.wave, tid, blockDim.x,
+                [&](int i, int j, double2 v) { M[(size_t)j * ld + i] = cadd(M[(size_t)j * ld + i], v); });
+    }
     for (int c = warp; c < l; c += nwarp)
       for (int row = lane; row < n; row += 32) M[(size_t)(n + c) * ld + row] = P.V[(size_t)c * n + row];
     __syncthreads();

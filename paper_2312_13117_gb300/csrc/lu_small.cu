@@ -56,9 +56,7 @@ __global__ void __launch_bounds__(WARPS * 32) k_factor_solve_small(NodeArgs a) {
         for (int k = 0; k < P.K; ++k) {
           const TermDesc& t = P.term[k];
           if (t.dense) cfma(v, sm.fz[w][k], P.A[(size_t)t.mat_index * nn + e]);
-          else if (BIE && t.kind == PMCIM_F_HELMHOLTZ_DLP)  // T^H: entry (c, lane), conjugated below
-            cfma(v, t.id, bie::dlp_entry(P.bie, n, rg.herm ? c : lane, rg.herm ? lane : c, sm.fz[w][k]));
-          else if (c == lane) cfma(v, sm.fz[w][k], t.id);
+          else if (c == lane && t.kind != PMCIM_F_HELMHOLTZ_DLP) cfma(v, sm.fz[w][k], t.id);
         }
         if (rg.herm) v.y = -v.y;
         row[c] = v;
@@ -66,6 +64,14 @@ __global__ void __launch_bounds__(WARPS * 32) k_factor_solve_small(NodeArgs a) {
       for (int c = 0; c < l; ++c) row[n + c] = P.V[(size_t)c * n + lane];
     }
     __syncwarp();
+    if (BIE && P.bie) {
+      const bie::Wave W = bie::wave_of(z);
+      add_layer(P.bie, n, layer_coefficient(P), W, lane, 32, [&](int i, int j, double2 v) {
+        double2& m = rg.herm ? M[j * LDC + i] : M[i * LDC + j];  // T^H: entry (j, i) is conj(T_ij)
+        m = cadd(m, rg.herm ? cconj(v) : v);
+      });
+      __syncwarp();
+    }
     int info = 0;
     for (int j = 0; j < n; ++j) {
       double bv = -1.0;

@@ -19,6 +19,8 @@
 //                 exact as int64 sums of the orders' upper and lower half over all
 //                 inner indices; FP64 arithmetic (2 operations per SM and clock) is left
 //                 for one update of R per term.
+// A boundary-integral node has a matrix of its own: its tiles hold its own groups only,
+// and the digits are those of T(z_j) (bie_nodes.cu).
 // A wait for operands is bounded by tc_wait_cycles: when one runs out the CTA's nodes
 // are marked, and solved again in FP64. A wait between the warps is bounded by
 // handoff_wait_cycles: when one runs out the launch fails (MixedArgs::err).
@@ -50,6 +52,9 @@ __device__ __forceinline__ double pow2(int e) {
   return (e >= -1022 && e <= 1023) ? __hiloint2double((e + 1023) << 20, 0) : scalbn(1.0, e);
 }
 
+// Matrices a problem's residual multiplies: its dense terms, or T(z_j).
+__device__ __forceinline__ int terms_of(const ProblemDev& P) { return P.bie ? 1 : P.n_dense; }
+
 // Digits of f_d X of the active nodes, one CTA per node and dense term; CTA 0 also
 // counts the residual tiles before each problem.
 __global__ void __launch_bounds__(DIGIT_THREADS) k_oz_digits(MixedArgs a, int sw, int max_dense) {
@@ -64,7 +69,13 @@ __global__ void __launch_bounds__(DIGIT_THREADS) k_oz_digits(MixedArgs a, int sw
     int base = 0;
     for (int p0 = 0; p0 < a.n_probs; p0 += 32) {
       const int p = p0 + tid;
-      int v = p < a.n_probs ? (uc[p] + MAXG - 1) / MAXG * row_blocks(a.probs[p].n) : 0;
+      int v = 0;
+      if (p < a.n_probs) {
+        // problems share their tiles among nodes; a boundary-integral node has its own
+        const int ncg = (a.probs[p].l + CG - 1) / CG;
+        v = (a.probs[p].bie ? uc[p] / ncg * ((ncg + MAXG - 1) / MAXG) : (uc[p] + MAXG - 1) / MAXG) *
+            row_blocks(a.probs[p].n);
+      }
       const int own = v;
       for (int o = 1; o < 32; o <<= 1) {
         const int x = __shfl_up_sync(0xffffffffu, v, o);
@@ -80,16 +91,20 @@ __global__ void __launch_bounds__(DIGIT_THREADS) k_oz_digits(MixedArgs a, int sw
     const NodeItem it = a.items[q];
     const RegionDev rg = a.regions[it.region];
     const ProblemDev& P = a.probs[rg.prob];
-    if (dd >= P.n_dense || P.Adig == nullptr || rg.herm || P.bie) continue;  // the same in every thread
+    if (dd >= terms_of(P) || !mixed_node_oz(a, P, rg)) continue;  // the same in every thread
     const int n = P.n, l = P.l, kcn = k_chunks(n), ncg = (l + CG - 1) / CG;
     __syncthreads();  // f_sh and g of the previous node
     if (tid == 0) {
-      int k = 0;
-      for (int d = -1; k < P.K; ++k)
-        if (P.term[k].dense && ++d == dd) break;
-      double2 z, wt;
-      node_weight(rg.cre, rg.cim, rg.r, rg.N, it.j, &z, &wt);
-      f_sh = eval_f(P.term[k], z);
+      if (P.bie) {
+        f_sh = make_double2(1.0, 0.0);
+      } else {
+        int k = 0;
+        for (int d = -1; k < P.K; ++k)
+          if (P.term[k].dense && ++d == dd) break;
+        double2 z, wt;
+        node_weight(rg.cre, rg.cim, rg.r, rg.N, it.j, &z, &wt);
+        f_sh = eval_f(P.term[k], z);
+      }
     }
     __syncthreads();
     const double2 f = f_sh;
@@ -176,10 +191,16 @@ struct TileWalk {
   __device__ bool next(Tile& out) {
     if (t >= tiles[a.n_probs]) return false;
     while (tiles[p + 1] <= t) ++p;
-    const int rbn = row_blocks(a.probs[p].n), loc = t - tiles[p], u0 = loc / rbn * MAXG;
+    const int rbn = row_blocks(a.probs[p].n), loc = t - tiles[p];
+    int u0 = loc / rbn * MAXG, end = uc[p];
+    if (a.probs[p].bie) {  // a node's groups are consecutive
+      const int ncg = (a.probs[p].l + CG - 1) / CG, per = (ncg + MAXG - 1) / MAXG, node = loc / rbn / per;
+      u0 = node * ncg + loc / rbn % per * MAXG;
+      end = (node + 1) * ncg;
+    }
     out.p = p;
     out.rb = loc % rbn;
-    out.ng = min(MAXG, uc[p] - u0);
+    out.ng = min(MAXG, end - u0);
     out.units = a.units + (size_t)(sw & 1) * a.unit_cap + a.ubase[p] + u0;
     t += gridDim.x;
     return true;
@@ -247,8 +268,9 @@ __device__ void copy_role(const MixedArgs& a, int sw, GemmSmem& sm) {
     const unsigned char* src[MAXG];
     for (int g = 0; g < t.ng; ++g)
       src[g] = a.ysl + (size_t)(t.units[g] >> 3) * a.ysl_stride + (size_t)(t.units[g] & 7) * kcn * GROUP_STAGE;
-    for (int dd = 0; dd < P.n_dense && ok; ++dd) {
-      const unsigned char* asrc = P.Adig + ((size_t)dd * rbn + t.rb) * kcn * S * A_STAGE;
+    const unsigned char* digits = P.bie ? a.tdig + (size_t)(t.units[0] >> 3) * a.tdig_stride : P.Adig;
+    for (int dd = 0; dd < terms_of(P) && ok; ++dd) {
+      const unsigned char* asrc = digits + ((size_t)dd * rbn + t.rb) * kcn * S * A_STAGE;
       for (int kc = 0; kc < kcn && ok; ++kc) {
         const uint32_t bi = nb % RB2, bk = nb / RB2;
         ok = bk == 0 || wait_or_bad(&sm.b_empty[bi], (bk - 1) & 1u, a.tc_wait_cycles, &sm.bad);
@@ -284,7 +306,7 @@ __device__ void mma_role(const MixedArgs& a, int sw, GemmSmem& sm) {
     const int kcn = k_chunks(P.n);
     // kind::f16, F32 accumulator, BF16 A and B, K-major, M = 128, N = 16 per group
     const uint32_t id = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(t.ng * 2) << 17) | ((uint32_t)(TM >> 4) << 24);
-    for (int dd = 0; dd < P.n_dense && ok; ++dd)
+    for (int dd = 0; dd < terms_of(P) && ok; ++dd)
       for (int kc0 = 0; kc0 < kcn && ok; kc0 += KD / KC) {
         ok = blk == 0 || wait_or_bad(&sm.acc_empty, (blk - 1) & 1u, a.handoff_wait_cycles, &sm.bad, LOST_HANDOFF);
         if (!ok) break;
@@ -348,7 +370,7 @@ __device__ void drain_role(const MixedArgs& a, int sw, GemmSmem& sm) {
     double2* R = reinterpret_cast<double2*>(a.work + (size_t)q * a.slot_bytes + mixed_residual_offset(n, l)) +
                  (size_t)cg * CG * n + row;
     const int cols = min(CG, l - cg * CG);
-    for (int dd = 0; dd < P.n_dense; ++dd) {
+    for (int dd = 0; dd < terms_of(P); ++dd) {
       long long hi[2 * CG], lo[2 * CG];  // orders 2-5 and 6-9: hi 2^28 + lo
 #pragma unroll
       for (int c = 0; c < 2 * CG; ++c) hi[c] = lo[c] = 0;
@@ -380,7 +402,8 @@ __device__ void drain_role(const MixedArgs& a, int sw, GemmSmem& sm) {
         if (lane == 0) arrive(&sm.acc_empty);
       }
       if (mine && row < n) {
-        const int er = P.Aexp[((size_t)dd * rbn + t.rb) * TM + 32 * quad + lane];
+        const int32_t* ex = P.bie ? a.texp + (size_t)q * a.texp_stride : P.Aexp;
+        const int er = ex[((size_t)dd * rbn + t.rb) * TM + 32 * quad + lane];
         const int* ge = a.gexp + (size_t)q * a.gexp_stride + (dd * ncg + cg) * CG;
         const double2 id = a.state[q].id;
         const bool has_id = id.x != 0.0 || id.y != 0.0;

@@ -170,16 +170,29 @@ struct ProblemDev {
   TermDesc term[PMCIM_MAX_TERMS];
 };
 
-// Entry (row, col) of one non-dense term: the identity term's diagonal, or the
-// boundary-integral term's c K_n(z) entry (fz = z for it). Dense terms are read by
-// the callers from the coefficients. The kernels that assemble T are instantiated
-// twice: BIE = false (no problem of the launch has a boundary-integral term) leaves
-// out the entry's code and its registers.
-template <bool BIE>
-__device__ __forceinline__ void cfma_term(double2& v, const ProblemDev& P, const TermDesc& t, double2 fz, int row,
-                                          int col) {
-  if (BIE && t.kind == PMCIM_F_HELMHOLTZ_DLP) cfma(v, t.id, bie::dlp_entry(P.bie, P.n, row, col, fz));
-  else if (row == col) cfma(v, fz, t.id);
+// Adds a boundary-integral term c K_n(z) to a matrix, by threads tid = 0 .. nthr-1:
+// add(i, j, v) adds v to entry (i, j), once per entry. The two entries of a pair share
+// their Bessel values (bie.cuh). The kernels that assemble T are instantiated twice:
+// BIE = false (no problem of the launch has such a term) leaves out this code and its
+// registers.
+template <typename Add>
+__device__ __forceinline__ void add_layer(const double* G, int n, double2 c, const bie::Wave& W, int tid, int nthr,
+                                          Add add) {
+  for (int p = tid; p < n * (n / 2); p += nthr) {
+    int i, j;
+    if (!bie::pair_of(n, p, &i, &j)) continue;
+    double2 a, b;
+    bie::dlp_pair(G, n, i, j, W, &a, &b);
+    add(i, j, cmul(c, a));
+    add(j, i, cmul(c, b));
+  }
+  for (int j = tid; j < n; j += nthr) add(j, j, cmul(c, bie::dlp_diagonal(G, n, j)));
+}
+// The coefficient c of a problem's boundary-integral term.
+__device__ __forceinline__ double2 layer_coefficient(const ProblemDev& P) {
+  for (int k = 0; k < P.K; ++k)
+    if (P.term[k].kind == PMCIM_F_HELMHOLTZ_DLP) return P.term[k].id;
+  return make_double2(0.0, 0.0);
 }
 
 struct RegionDev {
@@ -270,7 +283,13 @@ struct MixedArgs {
   int bie;             // a problem has a boundary-integral term
   int oz;              // refinement residuals on the tensor cores
   int res64;           // a node forms its residuals on the FP64 pipe
-  double2* t64;        // per slot, T(z_j) in FP64 for those
+  // boundary-integral nodes (bie_nodes.cu): per slot, the exact digits of T(z_j) and their row
+  // exponents (NULL: residuals on the FP64 pipe)
+  unsigned char* tdig;
+  size_t tdig_stride;
+  int32_t* texp;
+  int texp_stride;
+  double2* t64;        // per slot, T(z_j) in FP64 for those and for boundary-integral nodes
   size_t t64_stride;
   unsigned char* ysl;  // per slot, the digits of f_k X (oz_refine.cu)
   size_t ysl_stride;
@@ -294,6 +313,14 @@ __host__ __device__ inline size_t mixed_ctl_zero_ints(int n_probs, int max_sweep
 }
 __host__ __device__ inline size_t mixed_ctl_ints(int n_probs, int max_sweeps) {
   return mixed_ctl_zero_ints(n_probs, max_sweeps) + n_probs + 1;
+}
+// Whether the node's residuals are formed on the tensor cores.
+__device__ __forceinline__ bool mixed_node_oz(const MixedArgs& a, const ProblemDev& P, const RegionDev& rg) {
+  return a.oz && !rg.herm && (P.bie ? a.tdig != nullptr : P.Adig != nullptr);
+}
+// Whether a node's t64 holds only the first column of T(z_j), which is circulant.
+__device__ __forceinline__ bool mixed_column_only(const MixedArgs& a, const ProblemDev& P) {
+  return a.tdig != nullptr && P.bie_circ && P.n_dense == 0;
 }
 __device__ __forceinline__ int* mixed_ucount(const MixedArgs& a, int sw) {
   return a.ctl + MIXED_CTL_UNITS + (size_t)sw * a.n_probs;
@@ -320,6 +347,8 @@ cudaError_t prepare_factor_fp64();   // shared-memory limits; call outside graph
 cudaError_t prepare_factor_mixed();
 cudaError_t launch_factor_solve_fp64(const NodeArgs& a, cudaStream_t s);
 cudaError_t launch_factor_solve_mixed(const MixedArgs& a, int sms, cudaStream_t s, int* launched);
+// T(z_j) of the boundary-integral nodes in FP64 (t64) and its digits (bie_nodes.cu)
+cudaError_t launch_bie_assemble(const MixedArgs& a, int sms, cudaStream_t s, int* launched);
 // the residuals of sweep sw's active nodes (oz_refine.cu)
 cudaError_t prepare_oz_refine();
 cudaError_t launch_oz_residual(const MixedArgs& a, int sw, int sms, cudaStream_t s);

@@ -240,6 +240,7 @@ __global__ void __launch_bounds__(RT) k_certify(ValueArgs a) {
   __shared__ double2 fz[PMCIM_MAX_TERMS];
   __shared__ double red[2][RT / 32];
   __shared__ double2 ccol[BIE ? kCircMax : 1];
+  __shared__ bie::Wave wave;
   const int m = blockIdx.x;
   load_problem(&P, a.probs + a.prob_of[m]);
   __syncthreads();
@@ -249,8 +250,12 @@ __global__ void __launch_bounds__(RT) k_certify(ValueArgs a) {
   const double2* v = a.vecs + a.vec_off[m];
   if (threadIdx.x < P.K) fz[threadIdx.x] = eval_f(P.term[threadIdx.x], lam);
   const bool circ = BIE && P.bie_circ && n <= kCircMax;
+  if (BIE) {
+    if (threadIdx.x == 0) wave = bie::wave_of(lam);
+    __syncthreads();
+  }
   if (circ)
-    for (int q = threadIdx.x; q < n; q += RT) ccol[q] = bie::dlp_entry(P.bie, n, q, 0, lam);
+    for (int q = threadIdx.x; q < n; q += RT) ccol[q] = bie::dlp_entry(P.bie, n, q, 0, wave);
   __syncthreads();
   double r2 = 0.0, f2 = 0.0;
   for (int row = threadIdx.x; row < n; row += RT) {
@@ -264,7 +269,7 @@ __global__ void __launch_bounds__(RT) k_certify(ValueArgs a) {
         if (tk.dense) cfma(t, fz[k], P.A[(size_t)tk.mat_index * nn + e]);
         else if (BIE && tk.kind == PMCIM_F_HELMHOLTZ_DLP) {  // T^H: entry (col, row), conjugated below
           const int i = a.herm ? col : row, j = a.herm ? row : col;
-          cfma(t, tk.id, circ ? ccol[i >= j ? i - j : i - j + n] : bie::dlp_entry(P.bie, n, i, j, fz[k]));
+          cfma(t, tk.id, circ ? ccol[i >= j ? i - j : i - j + n] : bie::dlp_entry(P.bie, n, i, j, wave));
         }
         else if (row == col) cfma(t, fz[k], tk.id);
       }
