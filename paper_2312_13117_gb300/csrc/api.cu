@@ -1929,7 +1929,7 @@ int pmcim_problem_create(int32_t n, int32_t K, const double* const* A, const pmc
       return fail(PMCIM_ENOMEM, "coefficient upload: %s", cudaGetErrorString(e));
     }
     for (int k = 0; k < K; ++k) {
-      if (!A[k]) continue;
+      if (p->term[k].mat_index < 0) continue;  // an identity term, or a curve
       e = cudaMemcpy(p->dA + (size_t)p->term[k].mat_index * nn, A[k], nn * sizeof(double2), cudaMemcpyDefault);
       if (e != cudaSuccess) {
         cudaFree(p->dA);
