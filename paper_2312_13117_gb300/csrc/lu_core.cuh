@@ -197,175 +197,6 @@ __device__ void cta_lu_panel(T2* __restrict__ M, int n, int ncols, int k0, int k
   }
 }
 
-// The same panel factorisation (same pivots, same arithmetic up to the order of
-// the updates of each element) in sub-panels of SB <= 8 columns held in shared
-// memory: each sub-panel is loaded once, factored column by column in shared
-// memory, written back, and then applied to the rest of the panel (its row
-// swaps as one gather, the unit lower triangular solve for its U rows, and one
-// rank-SB update). The row swaps of the columns outside the panel (and of the
-// panel's earlier sub-panels) are applied after the panel (cta_panel_swaps_lp,
-// with the sub-panel width this returns).
-// scratch: shared memory of scratch_elems elements, at least (n - k0) + 8 NB + 40
-// (then SB = 1).
-template <typename T2>
-__device__ __noinline__ int cta_lu_panel_sub(T2* __restrict__ M, int n, int ncols, int k0, int kb, int* __restrict__ piv,
-                                 LuSmemT<T2>& sm, T2* __restrict__ scratch, int scratch_elems) {
-  const int tid = gtid();
-  const size_t ld = (size_t)n;
-  const int kend = k0 + kb;
-  using R = decltype(l1abs(T2{}));
-  constexpr int SBMAX = 8, CHUNK = 8;
-  const int m0 = n - k0;
-  int SB = SBMAX;
-  while (SB > 1 && (size_t)m0 * SB + (size_t)NB * SBMAX + 40 > (size_t)scratch_elems) SB >>= 1;
-  T2* sp = scratch;                                  // sub-panel, rows p0..n-1, leading dimension m
-  T2* us = scratch + (size_t)m0 * SB;                // its U rows for the rest of the panel, [col][t]
-  int* mp = reinterpret_cast<int*>(us + NB * SBMAX);  // composed swaps: count, dst[2 SBMAX], src[2 SBMAX]
-  for (int p0 = k0; p0 < kend; p0 += SB) {
-    const int sb = min(SB, kend - p0);
-    const int m = n - p0;
-    // 1. load (many loads in flight per thread: one round trip per 16 elements)
-#pragma unroll 16
-    for (int e = tid; e < m * sb; e += THREADS) {
-      const int r = e % m, c = e / m;
-      sp[(size_t)c * m + r] = M[(size_t)(p0 + c) * ld + p0 + r];
-    }
-    gsync();
-    // 2. factor in shared memory
-    for (int j = 0; j < sb; ++j) {
-      R bv = R(-1);
-      int bi = m;
-      for (int r = j + tid; r < m; r += THREADS) {
-        const R v = l1abs(sp[(size_t)j * m + r]);
-        if (v > bv) { bv = v; bi = r; }
-      }
-      warp_argmax(bv, bi);
-      if ((tid & 31) == 0) { sm.red_v[tid >> 5] = (double)bv; sm.red_i[tid >> 5] = bi; }
-      gsync();
-      if (tid == 0) {
-        double v = sm.red_v[0];
-        int ii = sm.red_i[0];
-        for (int w = 1; w < THREADS / 32; ++w)
-          if (sm.red_v[w] > v || (sm.red_v[w] == v && sm.red_i[w] < ii)) { v = sm.red_v[w]; ii = sm.red_i[w]; }
-        if (ii >= m) ii = j;
-        sm.piv_sh = ii;
-        piv[p0 + j] = p0 + ii;
-      }
-      gsync();
-      const int pr = sm.piv_sh;
-      if (pr != j && tid < sb) {
-        const T2 t = sp[(size_t)tid * m + j];
-        sp[(size_t)tid * m + j] = sp[(size_t)tid * m + pr];
-        sp[(size_t)tid * m + pr] = t;
-      }
-      gsync();
-      const T2 pv = sp[(size_t)j * m + j];
-      const bool zero = cis_zero(pv);
-      if (zero && tid == 0 && sm.info_sh == 0) sm.info_sh = p0 + j + 1;
-      if (!zero) {
-        const T2 rp = crecip(pv);
-        for (int r = j + 1 + tid; r < m; r += THREADS) {
-          const T2 lv = cmul(sp[(size_t)j * m + r], rp);
-          sp[(size_t)j * m + r] = lv;
-          for (int c = j + 1; c < sb; ++c) cfms(sp[(size_t)c * m + r], lv, sp[(size_t)c * m + j]);
-        }
-      }
-      gsync();
-    }
-    // 3. write back
-#pragma unroll 4
-    for (int e = tid; e < m * sb; e += THREADS) {
-      const int r = e % m, c = e / m;
-      M[(size_t)(p0 + c) * ld + p0 + r] = sp[(size_t)c * m + r];
-    }
-    const int c1 = p0 + sb, nr = kend - c1;  // the rest of the panel
-    if (nr > 0) {
-      // the sub-panel's swaps composed: row dst[i] receives the old row src[i]
-      if (tid == 0) {
-        int cnt = 0;
-        int* dst = mp + 1;
-        int* src = mp + 1 + 2 * SBMAX;
-        for (int j = 0; j < sb; ++j) {
-          const int a = p0 + j, b = piv[p0 + j];
-          if (a == b) continue;
-          int ia = -1, ib = -1;
-          for (int i = 0; i < cnt; ++i) {
-            if (dst[i] == a) ia = i;
-            if (dst[i] == b) ib = i;
-          }
-          if (ia < 0) { ia = cnt; dst[cnt] = a; src[cnt] = a; ++cnt; }
-          if (ib < 0) { ib = cnt; dst[cnt] = b; src[cnt] = b; ++cnt; }
-          const int t = src[ia];
-          src[ia] = src[ib];
-          src[ib] = t;
-        }
-        mp[0] = cnt;
-      }
-      gsync();
-      {
-        const int cnt = mp[0];
-        const int* dst = mp + 1;
-        const int* src = mp + 1 + 2 * SBMAX;
-        constexpr int GU = (2 * SBMAX * NB + THREADS - 1) / THREADS;  // gather elements per thread
-        T2 tmp[GU];
-#pragma unroll
-        for (int u = 0; u < GU; ++u) {
-          const int e = tid + u * THREADS;
-          if (e < cnt * nr) tmp[u] = M[(size_t)(c1 + e / cnt) * ld + src[e % cnt]];
-        }
-        gsync();
-#pragma unroll
-        for (int u = 0; u < GU; ++u) {
-          const int e = tid + u * THREADS;
-          if (e < cnt * nr) M[(size_t)(c1 + e / cnt) * ld + dst[e % cnt]] = tmp[u];
-        }
-      }
-      gsync();
-      // U rows p0..p0+sb-1 of the rest: unit lower triangular solve with L11 (one thread per column)
-      for (int c = tid; c < nr; c += THREADS) {
-        T2 u[SBMAX];
-#pragma unroll
-        for (int t = 0; t < SBMAX; ++t)
-          if (t < sb) u[t] = M[(size_t)(c1 + c) * ld + p0 + t];
-#pragma unroll
-        for (int t = 1; t < SBMAX; ++t)
-#pragma unroll
-          for (int q = 0; q < SBMAX; ++q)
-            if (t < sb && q < t) cfms(u[t], sp[(size_t)q * m + t], u[q]);
-#pragma unroll
-        for (int t = 0; t < SBMAX; ++t)
-          if (t < sb) {
-            M[(size_t)(c1 + c) * ld + p0 + t] = u[t];
-            us[c * SBMAX + t] = u[t];
-          }
-      }
-      gsync();
-      // rank-sb update of rows p0+sb..n-1 of the rest, CHUNK columns in flight per row
-      for (int r = sb + tid; r < m; r += THREADS) {
-        T2 lr[SBMAX];
-#pragma unroll
-        for (int t = 0; t < SBMAX; ++t) lr[t] = t < sb ? sp[(size_t)t * m + r] : czero<T2>();
-        for (int cc = 0; cc < nr; cc += CHUNK) {
-          T2 v[CHUNK];
-#pragma unroll
-          for (int q = 0; q < CHUNK; ++q)
-            if (cc + q < nr) v[q] = M[(size_t)(c1 + cc + q) * ld + p0 + r];
-#pragma unroll
-          for (int q = 0; q < CHUNK; ++q)
-            if (cc + q < nr) {
-#pragma unroll
-              for (int t = 0; t < SBMAX; ++t)
-                if (t < sb) cfms(v[q], lr[t], us[(cc + q) * SBMAX + t]);
-              M[(size_t)(c1 + cc + q) * ld + p0 + r] = v[q];
-            }
-        }
-      }
-    }
-    gsync();
-  }
-  return SB;
-}
-
 // ---------------------------------------------------------------------------
 // Row interchanges in LINPACK's order (the precision form's FP32 LU): a panel's
 // swaps reach the panel's own columns and the columns right of it, never the L
@@ -396,58 +227,6 @@ __device__ inline void compose_swaps(const int* __restrict__ piv, int a, int b, 
     src[ib] = t;
   }
   list[0] = cnt;
-}
-
-// The permutation in list (shared memory, complete before the call) on columns
-// c_lo..c_hi-1 of M, staged through stage (stage_elems elements of shared memory):
-// all of a chunk's rows are read before any is written. All threads; returns with
-// the group synchronised.
-template <typename T2>
-__device__ void apply_row_perm(T2* __restrict__ M, size_t ld, int c_lo, int c_hi, const int* __restrict__ list,
-                               T2* __restrict__ stage, int stage_elems) {
-  const int cnt = list[0];
-  if (cnt > 0 && c_hi > c_lo) {
-    const int* dst = list + 1;
-    const int* src = list + 1 + 2 * NB;
-    const int per = max(1, stage_elems / cnt);
-    for (int c0 = c_lo; c0 < c_hi; c0 += per) {
-      const int tot = min(per, c_hi - c0) * cnt;
-#pragma unroll 8
-      for (int e = gtid(); e < tot; e += THREADS) stage[e] = M[(size_t)(c0 + e / cnt) * ld + src[e % cnt]];
-      gsync();
-#pragma unroll 8
-      for (int e = gtid(); e < tot; e += THREADS) M[(size_t)(c0 + e / cnt) * ld + dst[e % cnt]] = stage[e];
-      gsync();
-    }
-  }
-  gsync();
-}
-
-// After cta_lu_panel_sub (sub-panels of SB columns), in LINPACK's order: the
-// panel's swaps on the columns right of it, and on each sub-panel's columns the
-// swaps of the later sub-panels (a sub-panel's own swaps and those before it are
-// already in its columns). The panel's whole permutation is also written to
-// list_out (global memory) for the forward solves. scratch: shared memory of
-// scratch_bytes bytes, of which the last SWAP_LIST_INTS ints hold a list.
-template <typename T2>
-__device__ void cta_panel_swaps_lp(T2* __restrict__ M, int n, int ncols, int k0, int kb, const int* __restrict__ piv,
-                                   int SB, int* __restrict__ list_out, unsigned char* scratch, int scratch_bytes) {
-  const int tid = gtid();
-  const size_t ld = (size_t)n;
-  const int kend = k0 + kb;
-  int* ls = reinterpret_cast<int*>(scratch + scratch_bytes) - SWAP_LIST_INTS;
-  T2* stage = reinterpret_cast<T2*>(scratch);
-  const int elems = (int)((reinterpret_cast<unsigned char*>(ls) - scratch) / sizeof(T2));
-  gsync();
-  if (tid == 0) compose_swaps(piv, k0, kend, ls);
-  gsync();
-  for (int i = tid; i < SWAP_LIST_INTS; i += THREADS) list_out[i] = ls[i];
-  apply_row_perm(M, ld, kend, ncols, ls, stage, elems);
-  for (int q0 = k0; q0 + SB < kend; q0 += SB) {
-    if (tid == 0) compose_swaps(piv, q0 + SB, kend, ls);
-    gsync();
-    apply_row_perm(M, ld, q0, q0 + SB, ls, stage, elems);
-  }
 }
 
 // U12 = L11^{-1} A12 for rows k0..k0+kb-1, columns k0+kb..ncols-1.
@@ -684,64 +463,5 @@ __device__ void cta_back_blocked(T2* __restrict__ M, int n, int l, LuSmemT<T2>& 
     gsync();
   }
 }
-
-// L y = b for the l columns after the n x n block of M, with L from an LU whose
-// row interchanges are in LINPACK's order: before panel p's columns of L, its
-// permutation (lists + p SWAP_LIST_INTS, global memory) is applied to y.
-template <typename T2>
-__device__ void cta_fwd_blocked_lp(T2* __restrict__ M, int n, int l, LuSmemT<T2>& sm, const int* __restrict__ lists) {
-  const int tid = gtid(), lane = tid & 31, wid = tid >> 5;
-  const size_t ld = (size_t)n;
-  T2* Y = M + (size_t)n * ld;
-  constexpr int GU = 4;  // permuted elements per thread and round
-  for (int k0 = 0; k0 < n; k0 += NB) {
-    const int kb = min(NB, n - k0);
-    {
-      const int* L = lists + (size_t)(k0 / NB) * SWAP_LIST_INTS;
-      const int cnt = L[0];
-      const int* dst = L + 1;
-      const int* src = L + 1 + 2 * NB;
-      // whole columns per round, so that a column's rows are all read before any is written
-      const int per = cnt > 0 ? max(1, GU * THREADS / cnt) : l;
-      for (int c0 = 0; c0 < l && cnt > 0; c0 += per) {
-        const int tot = min(per, l - c0) * cnt;
-        T2 v[GU];
-#pragma unroll
-        for (int u = 0; u < GU; ++u) {
-          const int e = tid + u * THREADS;
-          if (e < tot) v[u] = Y[(size_t)(c0 + e / cnt) * ld + src[e % cnt]];
-        }
-        gsync();
-#pragma unroll
-        for (int u = 0; u < GU; ++u) {
-          const int e = tid + u * THREADS;
-          if (e < tot) Y[(size_t)(c0 + e / cnt) * ld + dst[e % cnt]] = v[u];
-        }
-        gsync();
-      }
-    }
-    for (int e = tid; e < kb * kb; e += THREADS) {
-      const int r = e % kb, c = e / kb;
-      sm.Ls[c * NB + r] = M[(size_t)(k0 + c) * ld + k0 + r];  // Ls[t*NB + i] = L[k0+i][k0+t]
-    }
-    gsync();
-    for (int c = wid; c < l; c += THREADS / 32) {
-      T2* yc = Y + (size_t)c * ld + k0;
-      T2 y = (lane < kb) ? yc[lane] : czero<T2>();
-      for (int t = 0; t < kb - 1; ++t) {
-        T2 yt;
-        yt.x = __shfl_sync(0xffffffffu, y.x, t);
-        yt.y = __shfl_sync(0xffffffffu, y.y, t);
-        if (lane > t && lane < kb) cfms(y, sm.Ls[t * NB + lane], yt);
-      }
-      if (lane < kb) yc[lane] = y;
-      if (lane < kb) sm.Us[lane * US_LD + c] = y;  // solved block rows, [t][c]
-    }
-    gsync();
-    for (int i = k0 + kb + tid; i < n; i += THREADS) block_update_row(M, Y, ld, i, k0, kb, l, sm);
-    gsync();
-  }
-}
-
 
 }  // namespace lucore

@@ -35,8 +35,11 @@
 // tensor cores: 3xTF32 (tc_update.cuh) or BF16 3M (tc_update_bf16.cuh).
 // node_info: bits 0-23 = 0 or 1 + first zero-pivot column, bits 24-28 = sweeps
 // run, bit 29 = a tensor-core wait ran out, bit 30 = FP64 fallback.
+#include <algorithm>
+
 #include "ozaki.cuh"
 #include "tc_update_bf16.cuh"
+#include "lu32.cuh"
 
 namespace {
 
@@ -105,28 +108,31 @@ struct FactorSmem {
 constexpr size_t kFactorHead = offsetof(FactorSmem, lu32) + offsetof(LuSmemT<float2>, Ls);
 
 // Bytes of the scratch that starts at lu32.Ls: the operand stage of the tensor-core
-// updates, or else the FMA pipes' tiles and a panel's sub-panel of 8 columns.
+// updates, or else the FMA pipes' tiles and the largest panel's scratch.
 inline size_t factor_scratch_bytes(int max_n, bool tc) {
   if (tc) return tcu::STAGE_BYTES;
-  const size_t tiles = sizeof(LuSmemT<float2>) - offsetof(LuSmemT<float2>, Ls);
-  const size_t sub = ((size_t)max_n * 8 + NB * 8 + 40) * sizeof(float2) + 1024;
-  const size_t b = sub < (size_t)tcu::STAGE_BYTES ? sub : (size_t)tcu::STAGE_BYTES;
-  return ((b > tiles ? b : tiles) + 127) & ~size_t(127);
+  size_t b = sizeof(LuSmemT<float2>) - offsetof(LuSmemT<float2>, Ls);
+  for (int rows : {max_n, 256, 512, 1024, 2048})
+    if (rows <= max_n && rows <= lu32::ROWS_MAX) b = std::max(b, lu32::panel_scratch_bytes(rows));
+  return (b + 127) & ~size_t(127);
 }
 
 template <bool RES64>
 struct SolveSmem {
   union {
-    LuSmemT<float2> lu32;   // triangular solves
+    lu32::SolveSmem32 s;    // triangular solves
     ResSmem res;            // residual tiles on the FP64 pipe
   };
   NodeCtx c;
 };
 template <>
 struct SolveSmem<false> {
-  LuSmemT<float2> lu32;
+  lu32::SolveSmem32 s;
   NodeCtx c;
 };
+// The right-hand sides of a node stay in shared memory up to this size, behind SolveSmem
+// (three CTAs per SM).
+constexpr size_t kSolveYBytes = 46 * 1024;
 
 struct FallbackSmem {
   LuSmemT<double2> lu64;
@@ -151,35 +157,37 @@ struct PhaseClock {
   }
 };
 
-// The FP32 blocked LU of lucore::cta_lu, with the trailing updates on the
-// tensor cores (use_tc, while no wait has run out) or on the FMA pipes.
-// tc: 0 = trailing updates on the FMA pipes, 1 = 3xTF32 on the tensor cores, 2 = BF16 3M on the tensor cores
+// The FP32 blocked LU: register panels (lu32.cuh; columns of more rows than they hold in
+// global memory), the trailing updates on the tensor cores (tc: 1 = 3xTF32, 2 = BF16 3M; while
+// no wait has run out) or on the FMA pipes (0). Row interchanges in LINPACK's order (none on
+// the L columns left of a panel); each panel's permutation goes to lists for the forward
+// solves, the pivots' reciprocals to rinv.
 __device__ int cta_lu32(float2* __restrict__ M, int n, int ncols, int* __restrict__ piv, int* __restrict__ lists,
-                        LuSmemT<float2>& sm, tcu::Ctx& cx, int tc, int scratch_bytes, PhaseClock& pc) {
+                        float2* __restrict__ rinv, LuSmemT<float2>& sm, tcu::Ctx& cx, int tc, PhaseClock& pc) {
   if (gtid() == 0) sm.info_sh = 0;
   gsync();
   for (int k0 = 0; k0 < n; k0 += NB) {
     const int kb = min(NB, n - k0);
-    const int kend = k0 + kb;
-    // the panel in shared-memory sub-panels, in the tensor-core stage (idle during the
-    // panel), while one sub-panel column fits there; else in global memory
-    const int kScratch = scratch_bytes / (int)sizeof(float2);
-    // row interchanges in LINPACK's order (none on the L columns left of the panel);
-    // each panel's permutation goes to lists for the forward solves
+    const int kend = k0 + kb, rows = n - k0;
     int* list = lists + (size_t)(k0 / NB) * SWAP_LIST_INTS;
-    if (n - k0 + NB * 8 + 40 <= kScratch) {
-      const int sb = cta_lu_panel_sub(M, n, ncols, k0, kb, piv, sm, reinterpret_cast<float2*>(cx.stage), kScratch);
+    if (rows <= lu32::ROWS_MAX) {
+      const int r = lu32::panel_r(rows);
+      if (r == 1) lu32::panel<1>(M, n, k0, kb, piv, rinv, list, cx.stage, &sm.info_sh);
+      else if (r == 2) lu32::panel<2>(M, n, k0, kb, piv, rinv, list, cx.stage, &sm.info_sh);
+      else if (r == 4) lu32::panel<4>(M, n, k0, kb, piv, rinv, list, cx.stage, &sm.info_sh);
+      else lu32::panel<8>(M, n, k0, kb, piv, rinv, list, cx.stage, &sm.info_sh);
       pc.mark(PH_PANEL);
-      cta_panel_swaps_lp(M, n, ncols, k0, kb, piv, sb, list, cx.stage, scratch_bytes);
-      pc.mark(PH_SWAPS);
+      if (kend >= ncols) continue;
+      lu32::swap_trsm(M, n, ncols, k0, kb, lu32::panel_smem(cx.stage, rows), reinterpret_cast<float2*>(cx.stage));
     } else {
       cta_lu_panel(M, n, ncols, k0, kb, piv, sm, k0);
       if (gtid() == 0) compose_swaps(piv, k0, kend, list);
+      if (gtid() < kb) rinv[k0 + gtid()] = lu32::recip32(M[(size_t)(k0 + gtid()) * n + k0 + gtid()]);
       gsync();
       pc.mark(PH_PANEL);
+      if (kend >= ncols) continue;
+      cta_lu_trsm(M, n, ncols, k0, kb, sm);
     }
-    if (kend >= ncols) continue;
-    cta_lu_trsm(M, n, ncols, k0, kb, sm);
     pc.mark(PH_TRSM);
     if (kend >= n) continue;
     if (tc == 2 && !*cx.bad) tcb::update(M, n, ncols, k0, kb, cx);
@@ -519,7 +527,7 @@ static_assert(tcu::TMEM_COLS <= TMEM_FACTOR && 2 * tcb::ACC_COLS <= TMEM_FACTOR,
 // BIE: the instantiation for launches with a boundary-integral term (bie.cuh); the
 // other leaves its code out. TC: a region of the launch updates on the tensor cores.
 template <bool BIE, bool TC>
-__global__ void __launch_bounds__(THREADS, TC ? 2 : 3) k_mixed_factor(MixedArgs a, int scratch_bytes) {
+__global__ void __launch_bounds__(THREADS, 2) k_mixed_factor(MixedArgs a, int scratch_bytes) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   FactorSmem& sm = *reinterpret_cast<FactorSmem*>(smem_raw);
   const int tid = gtid();
@@ -569,7 +577,8 @@ __global__ void __launch_bounds__(THREADS, TC ? 2 : 3) k_mixed_factor(MixedArgs 
     const int bad_before = sm.tc_bad;
     int* lists = reinterpret_cast<int*>(slot + mixed_lists_offset(n, l));
     int* piv = lists + (size_t)((n + NB - 1) / NB) * SWAP_LIST_INTS;
-    const int info = cta_lu32(M32, n, ncols, piv, lists, sm.lu32, cx, TC ? rg.lu_tc : 0, scratch_bytes, pc);
+    float2* rinv = reinterpret_cast<float2*>(slot + mixed_rinv_offset(n, l));
+    const int info = cta_lu32(M32, n, ncols, piv, lists, rinv, sm.lu32, cx, TC ? rg.lu_tc : 0, pc);
     if (tid == 0) {
       MixedState st{};
       st.info = info;
@@ -605,7 +614,7 @@ __device__ __forceinline__ void finish_node(const MixedArgs& a, const RegionDev&
 // The back substitution (sw = 0, every node) or sweep sw's correction (the active nodes).
 // RES64: a node of the launch forms its residuals on the FP64 pipe.
 template <bool RES64>
-__global__ void __launch_bounds__(THREADS, 3) k_mixed_solve(MixedArgs a, int sw) {
+__global__ void __launch_bounds__(THREADS, 3) k_mixed_solve(MixedArgs a, int sw, int y_bytes) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   SolveSmem<RES64>& sm = *reinterpret_cast<SolveSmem<RES64>*>(smem_raw);
   const int tid = gtid();
@@ -628,6 +637,9 @@ __global__ void __launch_bounds__(THREADS, 3) k_mixed_solve(MixedArgs a, int sw)
     const size_t nn = (size_t)n * n, nl = (size_t)n * l;
     double2* R = reinterpret_cast<double2*>(slot + mixed_residual_offset(n, l));
     const int* lists = reinterpret_cast<const int*>(slot + mixed_lists_offset(n, l));
+    const float2* rinv = reinterpret_cast<const float2*>(slot + mixed_rinv_offset(n, l));
+    float2* Y = nl * sizeof(float2) <= (size_t)y_bytes ? reinterpret_cast<float2*>(smem_raw + sizeof(SolveSmem<RES64>))
+                                                       : M32 + nn;
     double2* X = a.X + rg.x_off + (size_t)it.j * nl;
     MixedState st = a.state[q];
     const bool oz = mixed_node_oz(a, P, rg);
@@ -636,9 +648,13 @@ __global__ void __launch_bounds__(THREADS, 3) k_mixed_solve(MixedArgs a, int sw)
       if (ok) {
         // X_0 = U^-1 (L^-1 P V) in FP32 (the LU eliminated V)
         double xm = 0.0;
-        cta_back_blocked(M32, n, l, sm.lu32);
+        if (Y != M32 + nn) {
+          for (size_t e = tid; e < nl; e += THREADS) Y[e] = M32[nn + e];
+          gsync();
+        }
+        lu32::back(M32, Y, n, l, rinv, sm.s);
         for (size_t e = tid; e < nl; e += THREADS) {
-          const float2 y = M32[nn + e];
+          const float2 y = Y[e];
           const double2 x = make_double2((double)y.x, (double)y.y);
           X[e] = x;
           xm = fmax(xm, fmax(fabs(x.x), fabs(x.y)));
@@ -689,14 +705,14 @@ __global__ void __launch_bounds__(THREADS, 3) k_mixed_solve(MixedArgs a, int sw)
         // right-hand side R / |R|max; the forward solve applies the row interchanges
         for (size_t e = tid; e < nl; e += THREADS) {
           const double2 rv = R[e];
-          M32[nn + e] = make_float2((float)(rv.x * inv), (float)(rv.y * inv));
+          Y[e] = make_float2((float)(rv.x * inv), (float)(rv.y * inv));
         }
         gsync();
-        cta_fwd_blocked_lp(M32, n, l, sm.lu32, lists);
-        cta_back_blocked(M32, n, l, sm.lu32);
+        lu32::forward(M32, Y, n, l, sm.s, lists);
+        lu32::back(M32, Y, n, l, rinv, sm.s);
         double dm = 0.0, xmx = 0.0;
         for (size_t e = tid; e < nl; e += THREADS) {
-          const float2 d = M32[nn + e];
+          const float2 d = Y[e];
           double2 x = X[e];
           const double dx = (double)d.x * rm, dy = (double)d.y * rm;
           x.x += dx;
@@ -791,11 +807,10 @@ __global__ void __launch_bounds__(THREADS, 2) k_mixed_fallback(MixedArgs a, size
 }  // namespace
 
 // Slot layout: [FP32 matrix n x (n + l)] [FP64 residual n x l] [the panels' row
-// permutations, SWAP_LIST_INTS ints each] [pivots].
+// permutations, SWAP_LIST_INTS ints each] [pivots] [their reciprocals, complex64].
+static_assert(SWAP_LIST_INTS == MIXED_LIST_INTS && NB == MIXED_NB, "slot layout");
 size_t mixed_slot_bytes(int n, int l) {
-  const size_t b = mixed_lists_offset(n, l) +
-                   ((size_t)((n + NB - 1) / NB) * SWAP_LIST_INTS + (size_t)n) * sizeof(int);
-  return (b + 255) & ~(size_t)255;
+  return (mixed_rinv_offset(n, l) + (size_t)n * sizeof(float2) + 255) & ~(size_t)255;
 }
 // Bytes a slot area needs at the least: one FP64 fallback.
 size_t mixed_fallback_bytes(int n, int l) {
@@ -810,6 +825,10 @@ const void* factor_kernel(bool bie, bool tc) {
 }  // namespace
 
 static_assert(2 * (kFactorHead + tcu::STAGE_BYTES + 1024) <= 228 * 1024, "two CTAs per SM");
+static_assert(lu32::panel_scratch_bytes(lu32::ROWS_MAX) <= tcu::STAGE_BYTES && lu32::panel_scratch_bytes(1024) <= tcu::STAGE_BYTES &&
+                  lu32::panel_scratch_bytes(256) <= tcu::STAGE_BYTES && lu32::panel_scratch_bytes(512) <= tcu::STAGE_BYTES,
+              "a panel fits the operand stage");
+static_assert(3 * (sizeof(SolveSmem<false>) + kSolveYBytes + 1024) <= 228 * 1024, "three CTAs per SM");
 
 cudaError_t prepare_factor_mixed() {
   for (int i = 0; i < 4; ++i) {
@@ -821,7 +840,7 @@ cudaError_t prepare_factor_mixed() {
                                        (int)sizeof(SolveSmem<true>));
   if (e != cudaSuccess) return e;
   e = cudaFuncSetAttribute(k_mixed_solve<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)sizeof(SolveSmem<false>));
+                           (int)(sizeof(SolveSmem<false>) + kSolveYBytes));
   if (e != cudaSuccess) return e;
   e = cudaFuncSetAttribute(k_mixed_fallback, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(FallbackSmem));
   if (e != cudaSuccess) return e;
@@ -857,7 +876,7 @@ cudaError_t launch_factor_solve_mixed(const MixedArgs& a, int sms, cudaStream_t 
   {
     const int scratch = (int)factor_scratch_bytes(a.max_n, a.tc != 0);
     const size_t smem = kFactorHead + scratch;
-    const int g = grid(a.tc ? 2 : 3);
+    const int g = grid(2);
     if (a.bie && a.tc) k_mixed_factor<true, true><<<g, THREADS, smem, s>>>(a, scratch);
     else if (a.bie) k_mixed_factor<true, false><<<g, THREADS, smem, s>>>(a, scratch);
     else if (a.tc) k_mixed_factor<false, true><<<g, THREADS, smem, s>>>(a, scratch);
@@ -870,8 +889,11 @@ cudaError_t launch_factor_solve_mixed(const MixedArgs& a, int sms, cudaStream_t 
       if (e != cudaSuccess) return e;
       *launched += 2;
     }
-    if (a.res64) k_mixed_solve<true><<<grid(3), THREADS, sizeof(SolveSmem<true>), s>>>(a, sw);
-    else k_mixed_solve<false><<<grid(3), THREADS, sizeof(SolveSmem<false>), s>>>(a, sw);
+    // (the FP64-pipe residual's tiles leave no room for the right-hand sides)
+    const size_t nl = (size_t)a.max_n * a.max_l * sizeof(float2);
+    const int y = !a.res64 && nl <= kSolveYBytes ? (int)nl : 0;
+    if (a.res64) k_mixed_solve<true><<<grid(3), THREADS, sizeof(SolveSmem<true>), s>>>(a, sw, 0);
+    else k_mixed_solve<false><<<grid(3), THREADS, sizeof(SolveSmem<false>) + y, s>>>(a, sw, y);
     ++*launched;
   }
   if (a.max_sweeps > 0) {

@@ -384,6 +384,12 @@ __host__ __device__ inline size_t mixed_residual_offset(int n, int l) {
 __host__ __device__ inline size_t mixed_lists_offset(int n, int l) {
   return (mixed_residual_offset(n, l) + (size_t)n * l * 16 + 255) & ~(size_t)255;
 }
+// then the pivots and their reciprocals
+constexpr int MIXED_NB = 32, MIXED_LIST_INTS = 1 + 4 * MIXED_NB;
+__host__ __device__ inline size_t mixed_rinv_offset(int n, int l) {
+  return (mixed_lists_offset(n, l) + ((size_t)((n + MIXED_NB - 1) / MIXED_NB) * MIXED_LIST_INTS + n) * sizeof(int) + 15) &
+         ~(size_t)15;
+}
 size_t mixed_slot_bytes(int n, int l);
 size_t mixed_fallback_bytes(int n, int l);
 
