@@ -9,12 +9,16 @@
 // form of Beyn's step, M_p = sum_j w_j ((z_j - c)/r)^p X_j, p < 2K; on the nodes
 // ((z_j - c)/r)^p = e^{i p theta_j}, taken from the integer phase p j mod N.
 // Nodes are summed in index order by one thread per output element, so the
-// result is deterministic. The kernel streams X once: it is HBM-bound.
+// result is deterministic. The kernel streams X once. The nodes' weights are formed once
+// per block and kept in shared memory: with a sincospi and a hypot of its own per thread
+// and node the FP64 unit bounded the kernel (disks of 64 nodes: 0.63 ms at the least, now
+// 0.13; 100 disks of n = 256, l = 8: 1.6 -> 0.39 ms).
 #include "pmcim_internal.cuh"
 
 namespace {
 
 constexpr int RT = 256;
+constexpr int NODES = 64;  // nodes whose weights are in shared memory at a time
 
 __global__ void __launch_bounds__(RT) k_reduce_moments(LevelArgs a) {
   const int g = blockIdx.y;
@@ -22,23 +26,39 @@ __global__ void __launch_bounds__(RT) k_reduce_moments(LevelArgs a) {
   const ProblemDev* P = a.probs + rg.prob;
   const int n = P->n, l = P->l;
   const int nl = n * l;
+  __shared__ double2 sw[NODES], swz[NODES];  // w_j, w_j z_j
+  __shared__ double sa[NODES];               // |w_j|
   const int e = blockIdx.x * RT + threadIdx.x;
-  if (e >= nl) return;
-  const bool first_col = e < n;
+  if (blockIdx.x * RT >= nl) return;
+  const bool first_col = e < n, in = e < nl;
   double2 c0 = make_double2(0.0, 0.0), c1 = c0, ph = c0;
   double pa = 0.0;
   const double2* Xg = a.X + rg.x_off + e;
-  for (int j = 0; j < rg.N; ++j) {
-    double2 z, w;
-    node_weight(rg.cre, rg.cim, rg.r, rg.N, j, &z, &w);
-    const double2 x = Xg[(size_t)j * nl];
-    cfma(c0, w, x);
-    cfma(c1, cmul(w, z), x);
-    if (first_col) {
-      if (j & 1) cfma(ph, cscale(w, 2.0), x);
-      pa += hypot(w.x, w.y) * hypot(x.x, x.y);
+  for (int j0 = 0; j0 < rg.N; j0 += NODES) {
+    const int jn = min(NODES, rg.N - j0);
+    __syncthreads();
+    if (threadIdx.x < jn) {
+      double2 z, w;
+      node_weight(rg.cre, rg.cim, rg.r, rg.N, j0 + threadIdx.x, &z, &w);
+      sw[threadIdx.x] = w;
+      swz[threadIdx.x] = cmul(w, z);
+      sa[threadIdx.x] = hypot(w.x, w.y);
+    }
+    __syncthreads();
+    if (in) {
+#pragma unroll 4
+      for (int j = 0; j < jn; ++j) {
+        const double2 x = Xg[(size_t)(j0 + j) * nl];
+        cfma(c0, sw[j], x);
+        cfma(c1, swz[j], x);
+        if (first_col) {
+          if ((j0 + j) & 1) cfma(ph, cscale(sw[j], 2.0), x);
+          pa += sa[j] * hypot(x.x, x.y);
+        }
+      }
     }
   }
+  if (!in) return;
   a.C0[rg.c_off + e] = c0;
   a.C1[rg.c_off + e] = c1;
   if (a.K > 1) {
