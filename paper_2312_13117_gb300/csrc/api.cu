@@ -792,6 +792,7 @@ int run_level(Call& c, const std::vector<HostRegion>& regs, bool gate_top, bool 
     size_t items64_off, n64, items32_off, n32, itemsS_off, nS;
     size_t copies_off, n_copies;  // reused solutions copied into this wave's X
     int max_copy;
+    int small_n, small_l;                 // largest among the warp-per-node items
     std::vector<ResidentClass> resident;  // FP64 nodes whose matrices stay in shared memory
   };
   std::vector<Wave> waves;
@@ -848,7 +849,7 @@ int run_level(Call& c, const std::vector<HostRegion>& regs, bool gate_top, bool 
       std::stable_sort(it64.begin(), it64.end(), by_n);
       std::stable_sort(it32.begin(), it32.end(), by_n);
       Wave wv{g0, g1, items.size(), it64.size(), 0, it32.size(), 0, itS.size(), copies_off,
-              copies.size() - copies_off, max_copy, {}};
+              copies.size() - copies_off, max_copy, 1, 1, {}};
       items.insert(items.end(), it64.begin(), it64.end());
       wv.items32_off = items.size();
       items.insert(items.end(), it32.begin(), it32.end());
@@ -857,6 +858,10 @@ int run_level(Call& c, const std::vector<HostRegion>& regs, bool gate_top, bool 
       any64 |= !it64.empty();
       any32 |= !it32.empty();
       anyS |= !itS.empty();
+      for (const NodeItem& it : itS) {
+        wv.small_n = std::max(wv.small_n, c.pd[regs[it.region].prob].n);
+        wv.small_l = std::max(wv.small_l, c.pd[regs[it.region].prob].l);
+      }
       for (std::vector<NodeItem>& f : itF) {
         if (f.empty()) continue;
         std::stable_sort(f.begin(), f.end(), by_n);
@@ -953,6 +958,9 @@ int run_level(Call& c, const std::vector<HostRegion>& regs, bool gate_top, bool 
 
   if (any64) CU(prepare_factor_fp64());
   if (anyS) CU(prepare_factor_small());
+  if (screen_features) CU(prepare_screen_features());
+  int max_N = 0;
+  for (const HostRegion& h : regs) max_N = std::max(max_N, h.N);
   if (anyF) CU(prepare_factor_resident());
 
   if (any32) {
@@ -1017,7 +1025,7 @@ int run_level(Call& c, const std::vector<HostRegion>& regs, bool gate_top, bool 
         na.n_items = (int)wv.nS;
         na.counter = ws.counters.as<int>() + kCounters * wi + 2;
         prof_begin(PMCIM_K_FACTOR, s);
-        CU(launch_factor_solve_small(na, s));
+        CU(launch_factor_solve_small(na, wv.small_n, wv.small_l, s));
         prof_end(PMCIM_K_FACTOR, s);
       }
       for (size_t k = 0; k < wv.resident.size(); ++k) {
@@ -1035,7 +1043,7 @@ int run_level(Call& c, const std::vector<HostRegion>& regs, bool gate_top, bool 
       lw.R = wv.g1 - wv.g0;
       if (screen_features) {
         prof_begin(PMCIM_K_INDICATOR, s);
-        CU(launch_screen_features(lw, ws.ind3.as<double>() + 3 * (size_t)wv.g0, s));
+        CU(launch_screen_features(lw, max_N, ws.ind3.as<double>() + 3 * (size_t)wv.g0, s));
         prof_end(PMCIM_K_INDICATOR, s);
         continue;
       }
@@ -1595,7 +1603,9 @@ int run_bordered_step(Call& c, const std::vector<double2>& lam_in, const std::ve
     na.n_items = (int)itS.size();
     na.counter = ws.icounters.as<int>() + 2;
     prof_begin(PMCIM_K_VERIFY, s);
-    CU(launch_factor_solve_small(na, s));
+    int small_n = 1;
+    for (const NodeItem& it : itS) small_n = std::max(small_n, pdv[it.region].n);
+    CU(launch_factor_solve_small(na, small_n, 1, s));
     prof_end(PMCIM_K_VERIFY, s);
   }
   // the certificate of y, against the call's own problem table

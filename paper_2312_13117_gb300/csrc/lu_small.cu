@@ -11,22 +11,26 @@
 namespace {
 
 constexpr int WARPS = 4;
-constexpr int SN = 32;            // largest n
-constexpr int SL = 16;            // largest l
-constexpr int LDC = SN + SL + 1;  // padded row length (complex entries)
+constexpr int SN = 32;  // largest n
+constexpr int SL = 16;  // largest l
 
-struct SmallSmem {
-  double2 M[WARPS][SN * LDC];
+struct SmallSmem {  // then WARPS matrices of `rows` rows of `ldc` entries
   ProblemDev P[WARPS];
   double2 fz[WARPS][PMCIM_MAX_TERMS];
+  double2 rinv[WARPS][SN];  // the pivots' reciprocals
 };
+constexpr size_t kSmallHead = (sizeof(SmallSmem) + 15) & ~size_t(15);
+// Row length for n + l columns: odd, so that eight rows lie in distinct banks.
+__host__ __device__ inline int small_ldc(int n, int l) { return (n + l) | 1; }
 
 template <bool BIE>
-__global__ void __launch_bounds__(WARPS * 32) k_factor_solve_small(NodeArgs a) {
+__global__ void __launch_bounds__(WARPS * 32) k_factor_solve_small(NodeArgs a, int matrix_elems) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   SmallSmem& sm = *reinterpret_cast<SmallSmem*>(smem_raw);
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  double2* M = sm.M[w];
+  const int lr = lane & 7, lc = lane >> 3;  // a tile of 8 rows x 4 columns
+  double2* M = reinterpret_cast<double2*>(smem_raw + kSmallHead) + (size_t)w * matrix_elems;
+  double2* rinv = sm.rinv[w];
   ProblemDev& P = sm.P[w];
   for (;;) {
     int idx = 0;
@@ -41,7 +45,7 @@ __global__ void __launch_bounds__(WARPS * 32) k_factor_solve_small(NodeArgs a) {
       for (int i = lane; i < (int)(sizeof(ProblemDev) / sizeof(int)); i += 32) d[i] = s[i];
     }
     __syncwarp();
-    const int n = P.n, l = P.l, ncols = n + l;
+    const int n = P.n, l = P.l, ncols = n + l, LDC = small_ldc(n, l);
     double2 z, wgt;
     node_weight(rg.cre, rg.cim, rg.r, rg.N, it.j, &z, &wgt);
     if (lane < P.K) sm.fz[w][lane] = eval_f(P.term[lane], z);
@@ -98,18 +102,38 @@ __global__ void __launch_bounds__(WARPS * 32) k_factor_solve_small(NodeArgs a) {
         }
       __syncwarp();
       const double2 pv = M[j * LDC + j];
+      const double2 rp = crecip(pv);  // not finite for a zero pivot, as a division by it would be
+      if (lane == 0) rinv[j] = rp;
       if (pv.x == 0.0 && pv.y == 0.0) {
         if (info == 0) info = j + 1;
-      } else if (lane > j && lane < n) {
-        const double2 lij = cmul(M[lane * LDC + j], crecip(pv));
-        M[lane * LDC + j] = lij;
-        for (int c = j + 1; c < ncols; ++c) cfms(M[lane * LDC + c], lij, M[j * LDC + c]);
+        __syncwarp();
+        continue;
+      }
+      if (lane > j && lane < n) M[lane * LDC + j] = cmul(M[lane * LDC + j], rp);
+      __syncwarp();
+      // rank-1 update in tiles of 8 rows x 4 columns: a lane without an element costs the FP64
+      // unit as much as a busy one, and a row per lane leaves most idle in the end
+      for (int r0 = j + 1; r0 < n; r0 += 8) {
+        const int r = r0 + lr;
+        const double2 lij = r < n ? M[r * LDC + j] : make_double2(0.0, 0.0);
+        for (int c0 = j + 1 + lc; c0 < ncols; c0 += 16) {
+          double2 v[4];
+#pragma unroll
+          for (int q = 0; q < 4; ++q)
+            if (r < n && c0 + 4 * q < ncols) v[q] = M[r * LDC + c0 + 4 * q];
+#pragma unroll
+          for (int q = 0; q < 4; ++q)
+            if (r < n && c0 + 4 * q < ncols) {
+              cfms(v[q], lij, M[j * LDC + c0 + 4 * q]);
+              M[r * LDC + c0 + 4 * q] = v[q];
+            }
+        }
       }
       __syncwarp();
     }
     // back substitution U X = Y on the l right-hand columns
     for (int j = n - 1; j >= 0; --j) {
-      if (lane < l) M[j * LDC + n + lane] = cdiv(M[j * LDC + n + lane], M[j * LDC + j]);
+      if (lane < l) M[j * LDC + n + lane] = cmul(M[j * LDC + n + lane], rinv[j]);
       __syncwarp();
       if (lane < j)
         for (int c = 0; c < l; ++c) cfms(M[lane * LDC + n + c], M[lane * LDC + j], M[j * LDC + n + c]);
@@ -128,24 +152,36 @@ __global__ void __launch_bounds__(WARPS * 32) k_factor_solve_small(NodeArgs a) {
 
 bool small_kernel_fits(int n, int l) { return n <= SN && l <= SL; }
 
+namespace {
+constexpr size_t kSmallMax = kSmallHead + (size_t)WARPS * SN * ((SN + SL) | 1) * sizeof(double2);
+}  // namespace
+
 cudaError_t prepare_factor_small() {
   cudaError_t e = cudaFuncSetAttribute(k_factor_solve_small<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)sizeof(SmallSmem));
+                                       (int)kSmallMax);
   if (e != cudaSuccess) return e;
   return cudaFuncSetAttribute(k_factor_solve_small<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)sizeof(SmallSmem));
+                              (int)kSmallMax);
 }
 
-// Launch only; prepare_factor_small() must have set the shared-memory limit.
-cudaError_t launch_factor_solve_small(const NodeArgs& a, cudaStream_t s) {
+// Launch only; prepare_factor_small() must have set the shared-memory limit. max_n, max_l: the
+// largest among the items, which set how many nodes an SM holds (n = 24, l = 1: 20; at the
+// largest sizes 8). The FP64 unit bounds the kernel: reciprocals kept for the back substitution
+// (a complex division is some 90 FP64 instructions of a warp) and the narrow update tiles took
+// 3072 nodes of n = 24, l = 1 from 0.75 to 0.42 ms.
+cudaError_t launch_factor_solve_small(const NodeArgs& a, int max_n, int max_l, cudaStream_t s) {
   if (a.n_items <= 0) return cudaSuccess;
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  int grid = 2 * (sms > 0 ? sms : 1);
+  const int elems = max_n * small_ldc(max_n, max_l);
+  const size_t smem = kSmallHead + (size_t)WARPS * elems * sizeof(double2);
+  int per = (int)((227 * 1024 + 1024) / (smem + 1024));
+  if (per > 5) per = 5;
+  int grid = per * (sms > 0 ? sms : 1);
   const int need = (a.n_items + WARPS - 1) / WARPS;
   if (grid > need) grid = need;
-  if (a.bie) k_factor_solve_small<true><<<grid, WARPS * 32, sizeof(SmallSmem), s>>>(a);
-  else k_factor_solve_small<false><<<grid, WARPS * 32, sizeof(SmallSmem), s>>>(a);
+  if (a.bie) k_factor_solve_small<true><<<grid, WARPS * 32, smem, s>>>(a, elems);
+  else k_factor_solve_small<false><<<grid, WARPS * 32, smem, s>>>(a, elems);
   return cudaGetLastError();
 }

@@ -371,7 +371,7 @@ cudaError_t launch_residual_points(const ProblemDev* prob, const double2* z, int
 // warp-per-node FP64 kernel for small problems (lu_small.cu)
 bool small_kernel_fits(int n, int l);
 cudaError_t prepare_factor_small();
-cudaError_t launch_factor_solve_small(const NodeArgs& a, cudaStream_t s);
+cudaError_t launch_factor_solve_small(const NodeArgs& a, int max_n, int max_l, cudaStream_t s);
 int factor_slots_fp64(int n, int l);
 // FP64 nodes whose matrix and probe columns fit shared memory (lu_resident.cu)
 int resident_ctas(int n, int l);  // CTAs per SM, 0 when a node does not fit
@@ -462,7 +462,8 @@ cudaError_t launch_certify_products(const ValueArgs& a, const double2* W, const 
 cudaError_t launch_verify_fp64(const ValueArgs& a, cudaStream_t s);
 
 // learned screen (screen.cu)
-cudaError_t launch_screen_features(const LevelArgs& a, double* ind3, cudaStream_t s);
+cudaError_t prepare_screen_features();
+cudaError_t launch_screen_features(const LevelArgs& a, int max_N, double* ind3, cudaStream_t s);
 cudaError_t launch_make_features(int R, const double* ind3, const RegionDev* regions, float* feats, cudaStream_t s);
 cudaError_t screen_forward(int M, const float* d_feats, const float* d_params, float* d_prob, void* d_scratch,
                            cudaStream_t s);  // scratch: 2 * PMCIM_SCREEN_PARAMS bytes

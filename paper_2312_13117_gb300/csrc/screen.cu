@@ -36,20 +36,25 @@ static_assert(NPARAM == PMCIM_SCREEN_PARAMS, "parameter count");
 // ---------------------------------------------------------------------------
 constexpr int FT = 256;
 
+// A node's weight on a rule, formed once per disk.
+struct Weights {
+  const double2* w;   // w_m
+  const double* abs;  // |w_m|
+};
 // P f|_M and P f|_{M/2} (component i) on the M-node rule of disk rg, whose node m is
 // node m * (N / M) of the disk's N-node rule; s_abs = sum_m |w_m| |x_m|.
 __device__ __forceinline__ void pf_component(const LevelArgs& a, const RegionDev& rg, size_t nl, int M, int i,
-                                             double2* s_full, double2* s_half, double* s_abs) {
+                                             const Weights& wt, double2* s_full, double2* s_half, double* s_abs) {
   const int step = rg.N / M;
   double2 f = make_double2(0.0, 0.0), h = f;
   double ab = 0.0;
+#pragma unroll 4
   for (int m = 0; m < M; ++m) {
-    double2 z, w;
-    node_weight(rg.cre, rg.cim, rg.r, M, m, &z, &w);
+    const double2 w = wt.w[m];
     const double2 x = a.X[rg.x_off + (size_t)(m * step) * nl + i];
     cfma(f, w, x);
     if (m & 1) cfma(h, cscale(w, 2.0), x);
-    ab += hypot(w.x, w.y) * hypot(x.x, x.y);
+    ab += wt.abs[m] * hypot(x.x, x.y);
   }
   *s_full = f;
   *s_half = h;
@@ -58,8 +63,11 @@ __device__ __forceinline__ void pf_component(const LevelArgs& a, const RegionDev
 
 // The indicator of Eq. 3.1 at three resolutions, with the reading the indicator
 // kernel takes: 0 when P f|_M is at rounding level as a whole, else the root mean
-// square of the componentwise ratios whose P f|_{M/2} is above that level.
+// square of the componentwise ratios whose P f|_{M/2} is above that level. One thread per
+// component and resolution; the weights once per disk (48 disks of n = 24, N = 64: with
+// a thread per component, both passes summing anew with weights of its own, 0.37 ms).
 __global__ void __launch_bounds__(FT) k_screen_features(LevelArgs a, double* ind3) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ double red[6][FT / 32];
   __shared__ double tot[6];
   const int g = blockIdx.x;
@@ -69,16 +77,43 @@ __global__ void __launch_bounds__(FT) k_screen_features(LevelArgs a, double* ind
   const size_t nl = (size_t)n * l;
   const int res[3] = {8, 16, N};
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  // the weights of the three rules (24 + N nodes)
+  double2* ww = reinterpret_cast<double2*>(smem_raw);
+  double* wa = reinterpret_cast<double*>(ww + 24 + N);
+  for (int t = threadIdx.x; t < 24 + N; t += FT) {
+    double2 z, w;
+    const int q = t < 8 ? 0 : t < 24 ? 1 : 2;
+    node_weight(rg.cre, rg.cim, rg.r, res[q], t - (q == 0 ? 0 : q == 1 ? 8 : 24), &z, &w);
+    ww[t] = w;
+    wa[t] = hypot(w.x, w.y);
+  }
+  __syncthreads();
+  const Weights wt[3] = {{ww, wa}, {ww + 8, wa + 8}, {ww + 24, wa + 24}};
+  // an item is a component at a resolution; a thread keeps the sums of its first ones
+  constexpr int KEEP = 4;
+  double2 kf[KEEP], kh[KEEP];
   // pass 1, per resolution: ||P f_M||^2 and ||sum |w||x| ||^2
   double acc[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-  for (int i = threadIdx.x; i < n; i += FT)
-    for (int q = 0; q < 3; ++q) {
-      double2 f, h;
-      double ab;
-      pf_component(a, rg, nl, res[q], i, &f, &h, &ab);
-      acc[2 * q] += cabs2(f);
-      acc[2 * q + 1] += ab * ab;
-    }
+#pragma unroll
+  for (int u = 0; u < KEEP; ++u) kf[u] = kh[u] = make_double2(0.0, 0.0);
+  for (int u = 0, e = threadIdx.x; e < 3 * n; ++u, e += FT) {
+    const int q = e / n, i = e - q * n;
+    double2 f, h;
+    double ab;
+    pf_component(a, rg, nl, res[q], i, wt[q], &f, &h, &ab);
+#pragma unroll
+    for (int k = 0; k < 3; ++k)
+      if (k == q) {
+        acc[2 * k] += cabs2(f);
+        acc[2 * k + 1] += ab * ab;
+      }
+#pragma unroll
+    for (int k = 0; k < KEEP; ++k)
+      if (k == u) {
+        kf[k] = f;
+        kh[k] = h;
+      }
+  }
   for (int q = 0; q < 6; ++q)
     for (int o = 16; o > 0; o >>= 1) acc[q] += __shfl_down_sync(0xffffffffu, acc[q], o);
   if (lane == 0)
@@ -92,17 +127,25 @@ __global__ void __launch_bounds__(FT) k_screen_features(LevelArgs a, double* ind
   __syncthreads();
   // pass 2, per resolution: sum of the determined |ratio|^2 and their count
   double acc2[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-  for (int i = threadIdx.x; i < n; i += FT)
-    for (int q = 0; q < 3; ++q) {
-      double2 f, h;
-      double ab;
-      pf_component(a, rg, nl, res[q], i, &f, &h, &ab);
-      const double den = cabs2(h);
-      if (den > kPfFloor * kPfFloor * tot[2 * q + 1]) {
-        acc2[2 * q] += cabs2(f) / den;
-        acc2[2 * q + 1] += 1.0;
+  for (int u = 0, e = threadIdx.x; e < 3 * n; ++u, e += FT) {
+    const int q = e / n, i = e - q * n;
+    double2 f = kf[0], h = kh[0];
+#pragma unroll
+    for (int k = 1; k < KEEP; ++k)
+      if (k == u) {
+        f = kf[k];
+        h = kh[k];
       }
-    }
+    double ab;
+    if (u >= KEEP) pf_component(a, rg, nl, res[q], i, wt[q], &f, &h, &ab);
+    const double den = cabs2(h);
+#pragma unroll
+    for (int k = 0; k < 3; ++k)
+      if (k == q && den > kPfFloor * kPfFloor * tot[2 * k + 1]) {
+        acc2[2 * k] += cabs2(f) / den;
+        acc2[2 * k + 1] += 1.0;
+      }
+  }
   for (int q = 0; q < 6; ++q)
     for (int o = 16; o > 0; o >>= 1) acc2[q] += __shfl_down_sync(0xffffffffu, acc2[q], o);
   __syncthreads();
@@ -297,9 +340,16 @@ __global__ void k_make_features(int R, const double* __restrict__ ind3, const Re
 
 }  // namespace
 
-cudaError_t launch_screen_features(const LevelArgs& a, double* ind3, cudaStream_t s) {
+// Shared memory of k_screen_features: the weights of 24 + N nodes (N <= 4096).
+cudaError_t prepare_screen_features() {
+  return cudaFuncSetAttribute(k_screen_features, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              (24 + 4096) * (int)(sizeof(double2) + sizeof(double)));
+}
+
+// max_N: the largest rule of the disks.
+cudaError_t launch_screen_features(const LevelArgs& a, int max_N, double* ind3, cudaStream_t s) {
   if (a.R <= 0) return cudaSuccess;
-  k_screen_features<<<a.R, FT, 0, s>>>(a, ind3);
+  k_screen_features<<<a.R, FT, (24 + max_N) * (sizeof(double2) + sizeof(double)), s>>>(a, ind3);
   return cudaGetLastError();
 }
 
