@@ -11,8 +11,8 @@
 // The residual V - T(z_j) X on the FP64 unit is 8 n^2 l operations a sweep, more than the
 // whole assembly of a circulant node. As digits it is tensor work like that of the other
 // problems (oz_refine.cu); making the digits is integer arithmetic on the entries' bits.
-// Measured on whole calls with FP32 LUs, n = 256, l = 8: a circle, 6400 nodes, 118 -> 56 ms;
-// an ellipse, 768 nodes, 61.4 -> 23.4 ms.
+// Measured on whole calls with FP32 LUs, n = 256, l = 8: a circle, 6400 nodes, 118 -> 40 ms;
+// an ellipse, 768 nodes, 61.4 -> 20.2 ms.
 #include "ozaki.cuh"
 
 namespace {
@@ -43,7 +43,8 @@ __global__ void __launch_bounds__(BT, 2) k_bie_assemble(MixedArgs a, int pieces)
   __shared__ double2 fz[PMCIM_MAX_TERMS];
   __shared__ bie::Wave wave;
   for (long long w = blockIdx.x; w < (long long)a.count * pieces; w += gridDim.x) {
-    const int q = (int)(w / pieces), piece = (int)(w % pieces);
+    // (pieces outermost: the CTAs share the first pieces of all nodes, the only ones of circulant nodes)
+    const int q = (int)(w % a.count), piece = (int)(w / a.count);
     const NodeItem it = a.items[q];
     const RegionDev rg = a.regions[it.region];
     const ProblemDev& G = a.probs[rg.prob];
