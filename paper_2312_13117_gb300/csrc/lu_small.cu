@@ -168,7 +168,7 @@ cudaError_t prepare_factor_small() {
 // largest among the items, which set how many nodes an SM holds (n = 24, l = 1: 20; at the
 // largest sizes 8). The FP64 unit bounds the kernel: reciprocals kept for the back substitution
 // (a complex division is some 90 FP64 instructions of a warp) and the narrow update tiles took
-// 3072 nodes of n = 24, l = 1 from 0.75 to 0.42 ms.
+// 3072 nodes of n = 24, l = 1 from 0.75 to 0.57 ms.
 cudaError_t launch_factor_solve_small(const NodeArgs& a, int max_n, int max_l, cudaStream_t s) {
   if (a.n_items <= 0) return cudaSuccess;
   int dev = 0, sms = 0;
