@@ -1320,6 +1320,15 @@ int run_beyn_levels(Call& c, const std::vector<HostRegion>& top, bool gate_top, 
   return PMCIM_OK;
 }
 
+// CTAs that share one of m values, a power of two: as many as leave every CTA an SM of its own
+// (24 values of order 512: 77 ms with one CTA each, 44 with 2, 28 with 4, and 33 with 8, two to
+// an SM; one value: 64, 37, 23, 18) and 16 rows (order 64: 1.95 ms with 1, 1.44 with 4, 1.46 with 8).
+int verify_cluster(int m, int n) {
+  int c = 1;
+  while (c < 8 && 2 * c * (long long)m <= num_sms() && 2 * c * 16 <= n) c *= 2;
+  return c;
+}
+
 // sigma_min (full) for the given values; slots sized for the largest n among them.
 int run_verify(Call& c, const std::vector<double2>& lam, const std::vector<int>& prob, std::vector<double>* sig,
                std::vector<uint8_t>* acc, std::vector<double2>* vecs = nullptr, int* vec_stride = nullptr) {
@@ -1331,14 +1340,14 @@ int run_verify(Call& c, const std::vector<double2>& lam, const std::vector<int>&
   if (m == 0) return PMCIM_OK;
   int max_n = 1;
   for (int i = 0; i < m; ++i) max_n = std::max(max_n, c.pd[prob[i]].n);
-  const size_t slot = (size_t)max_n * max_n * sizeof(double2);
+  const size_t slot = ((size_t)max_n * max_n + verify_vec_len(max_n)) * sizeof(double2);
   const int slots = (int)std::max<size_t>(1, std::min<size_t>(std::min<size_t>(2 * num_sms(), kSlotBytes / slot), m));
   CU(ws.vlam.ensure(m * sizeof(double2)));
   CU(ws.vprob.ensure(m * sizeof(int32_t)));
   CU(ws.vsig.ensure(m * sizeof(double)));
   CU(ws.vacc.ensure(m));
-  CU(ws.vwork.ensure((size_t)slots * slot));
-  CU(ws.vvec.ensure((size_t)slots * 3 * max_n * sizeof(double2)));
+  CU(ws.vwork.ensure((size_t)slots * max_n * max_n * sizeof(double2)));
+  CU(ws.vvec.ensure(slots * verify_vec_len(max_n) * sizeof(double2)));
   CU(ws.vpiv.ensure((size_t)slots * max_n * sizeof(int32_t)));
   std::vector<int32_t> pr(prob.begin(), prob.end());
   CU(cudaMemcpyAsync(ws.vlam.p, lam.data(), m * sizeof(double2), cudaMemcpyHostToDevice, s));
@@ -1358,6 +1367,7 @@ int run_verify(Call& c, const std::vector<double2>& lam, const std::vector<int>&
   va.piv = ws.vpiv.as<int32_t>();
   va.slots = slots;
   va.max_n = max_n;
+  va.cluster = verify_cluster(m, max_n);
   if (vecs) {
     CU(ws.vout.ensure((size_t)m * max_n * sizeof(double2)));
     va.vec_out = ws.vout.as<double2>();

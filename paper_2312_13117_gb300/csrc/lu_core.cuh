@@ -74,18 +74,6 @@ __device__ __forceinline__ double block_sum(double v, double* red) {
   return t;
 }
 
-// Block sum of a complex value; every thread gets the result.
-__device__ __forceinline__ double2 block_sum2(double2 v, double2* red2) {
-  const int lane = gtid() & 31, wid = gtid() >> 5;
-  v = warp_sum2(v);
-  gsync();
-  if (lane == 0) red2[wid] = v;
-  gsync();
-  double2 t = make_double2(0.0, 0.0);
-  for (int k = 0; k < THREADS / 32; ++k) t = cadd(t, red2[k]);
-  return t;
-}
-
 // ---------------------------------------------------------------------------
 // Blocked right-looking LU of the n x n leading block of M (column-major,
 // leading dimension n, ncols >= n columns; columns n..ncols-1 receive the same
@@ -287,7 +275,7 @@ __device__ void cta_lu_trsm(T2* __restrict__ M, int n, int ncols, int k0, int kb
 // chosen by the autotuner per problem size).
 template <typename T2, int RI = 4>
 __device__ void cta_lu_update_simt(T2* __restrict__ M, int n, int ncols, int k0, int kb, LuSmemT<T2>& sm,
-                                   int first = 0) {
+                                   int first = 0, int part = 0, int parts = 1) {
   constexpr int TT = 16 * RI;
   static_assert(TT <= TILE, "the shared tiles are sized for TILE");
   const int tid = gtid();
@@ -297,7 +285,10 @@ __device__ void cta_lu_update_simt(T2* __restrict__ M, int n, int ncols, int k0,
   const int m_rows = n - kend, m_cols = ncols - kend;
   const int mt = (m_rows + TT - 1) / TT, nt = (m_cols + TT - 1) / TT;
   const int tx = tid & 15, ty = tid >> 4;
-  for (int ti = 0; ti < mt; ++ti) {
+  // this CTA's tiles lo..hi-1 in row order: all of them, or one of `parts` equal shares
+  const int lo = mt * nt * part / parts, hi = mt * nt * (part + 1) / parts;
+  if (lo >= hi) return;
+  for (int ti = lo / nt; ti <= (hi - 1) / nt; ++ti) {
     const int r0 = kend + ti * TT;
     static_assert((NB * TT) % THREADS == 0, "tile staging mapping");
 #pragma unroll
@@ -308,7 +299,8 @@ __device__ void cta_lu_update_simt(T2* __restrict__ M, int n, int ncols, int k0,
       if (kk < kb && r0 + r < n) v = M[(size_t)(k0 + kk) * ld + r0 + r];
       sm.Ls[kk * TT + r] = v;
     }
-    for (int tj = 0; tj < nt; ++tj) {
+    const int tj1 = min(nt, hi - ti * nt);
+    for (int tj = max(0, lo - ti * nt); tj < tj1; ++tj) {
       const int c0 = kend + tj * TT;
 #pragma unroll
       for (int u = 0; u < NB * TT / THREADS; ++u) {

@@ -115,65 +115,239 @@ struct VerifySmem {
   LuSmem lu;
   ProblemDev P;
   bie::Wave wave;
-  double2 red2[THREADS / 32];
   double red[THREADS / 32];
-  double2 bc;
+  int row[2 * NB], src[2 * NB];  // a panel's interchanges: row[i] takes the old row src[i]
 };
 
-// Solve U^H a = x (U upper, so U^H is lower; dot-product form over columns of U).
-__device__ void solve_UH(const double2* __restrict__ M, int n, double2* __restrict__ x, VerifySmem& sm) {
-  const size_t ld = (size_t)n;
-  for (int j = 0; j < n; ++j) {
-    const double2* uj = M + (size_t)j * ld;
-    double2 s = make_double2(0.0, 0.0);
-    for (int i = threadIdx.x; i < j; i += THREADS) cfma_conj(s, uj[i], x[i]);
-    s = block_sum2(s, sm.red2);
-    if (threadIdx.x == 0) x[j] = cdiv(csub(x[j], s), cconj(uj[j]));
-    __syncthreads();
-  }
+// Few values leave most SMs idle with one CTA per value, so the CTAs of a cluster share one:
+// the LU of order 512 takes 52 ms on one SM, on the FP64 pipe, and 18.7 on 4 (7.6 of it the
+// panels, which one CTA factors). Every CTA of a cluster reaches every barrier below.
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
 }
-// Solve L^H u = a (L unit lower, so L^H is unit upper; dot-product form).
-__device__ void solve_LH(const double2* __restrict__ M, int n, double2* __restrict__ x, VerifySmem& sm) {
-  const size_t ld = (size_t)n;
-  for (int j = n - 1; j >= 0; --j) {
-    const double2* lj = M + (size_t)j * ld;
-    double2 s = make_double2(0.0, 0.0);
-    for (int i = j + 1 + threadIdx.x; i < n; i += THREADS) cfma_conj(s, lj[i], x[i]);
-    s = block_sum2(s, sm.red2);
-    if (threadIdx.x == 0) x[j] = csub(x[j], s);
-    __syncthreads();
-  }
+__device__ __forceinline__ int cluster_rank() {
+  unsigned r;
+  asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return (int)r;
 }
-// Solve L y = b (unit lower, column axpy form).
-__device__ void solve_L(const double2* __restrict__ M, int n, double2* __restrict__ x, VerifySmem& sm) {
-  const size_t ld = (size_t)n;
-  for (int j = 0; j < n; ++j) {
-    if (threadIdx.x == 0) sm.bc = x[j];
-    __syncthreads();
-    const double2 xj = sm.bc;
-    const double2* lj = M + (size_t)j * ld;
-    for (int i = j + 1 + threadIdx.x; i < n; i += THREADS) cfms(x[i], lj[i], xj);
-    __syncthreads();
-  }
+
+__device__ __forceinline__ double2 shfl2(double2 v, int src) {
+  return make_double2(__shfl_sync(0xffffffffu, v.x, src), __shfl_sync(0xffffffffu, v.y, src));
 }
-// Solve U y = b (upper, column axpy form).
-__device__ void solve_U(const double2* __restrict__ M, int n, double2* __restrict__ x, VerifySmem& sm) {
-  const size_t ld = (size_t)n;
-  for (int j = n - 1; j >= 0; --j) {
-    const double2* uj = M + (size_t)j * ld;
-    if (threadIdx.x == 0) {
-      double2 v = cdiv(x[j], uj[j]);
-      x[j] = v;
-      sm.bc = v;
+
+// A panel's interchanges on all other columns and U12 = L11^{-1} A12 on those right of it:
+// a warp takes four columns, lane t the rows k0 + t and piv[k0 + t].
+__device__ void swap_and_trsm(double2* M, int n, int k0, int kb, const int* piv, VerifySmem& sm, int rank, int size) {
+  const int tid = threadIdx.x, lane = tid & 31;
+  if (tid < 2 * NB) {  // follow one row back through the interchanges
+    const int t = tid & (NB - 1);
+    int r = t >= kb ? 0 : (tid < NB ? k0 + t : piv[k0 + t]);
+    sm.row[tid] = r;
+    for (int j = kb - 1; j >= 0; --j) {
+      const int p = piv[k0 + j];
+      r = r == k0 + j ? p : (r == p ? k0 + j : r);
     }
-    __syncthreads();
-    const double2 xj = sm.bc;
-    for (int i = threadIdx.x; i < j; i += THREADS) cfms(x[i], uj[i], xj);
-    __syncthreads();
+    sm.src[tid] = r;
+  }
+#pragma unroll
+  for (int u = 0; u < NB * NB / THREADS; ++u) {
+    const int e = tid + u * THREADS, i = e & (NB - 1), t = e / NB;
+    sm.lu.Ls[e] = i < kb && t < kb && i > t ? M[(size_t)(k0 + t) * n + k0 + i] : make_double2(0.0, 0.0);
+  }
+  __syncthreads();
+  const bool live = lane < kb;
+  const int s0 = sm.src[lane], r1 = sm.row[NB + lane], s1 = sm.src[NB + lane];
+  constexpr int CW = 4;
+  for (int g = (rank * THREADS + tid) >> 5; g * CW < n; g += size * (THREADS / 32)) {
+    double2 x[CW], y[CW];
+#pragma unroll
+    for (int q = 0; q < CW; ++q) {
+      const int c = g * CW + q;
+      const bool in = live && c < n && (c < k0 || c >= k0 + kb);
+      x[q] = in ? M[(size_t)c * n + s0] : make_double2(0.0, 0.0);
+      y[q] = in ? M[(size_t)c * n + s1] : make_double2(0.0, 0.0);
+    }
+    __syncwarp();
+    // rows below the panel's, before the panel's own (a row piv[k0 + t] may be one of those:
+    // both then hold the same value)
+#pragma unroll
+    for (int q = 0; q < CW; ++q) {
+      const int c = g * CW + q;
+      if (live && r1 >= k0 + kb && c < n && (c < k0 || c >= k0 + kb)) M[(size_t)c * n + r1] = y[q];
+    }
+    if ((g + 1) * CW > k0 + kb)
+      for (int t = 0; t < kb - 1; ++t) {
+        const double2 lt = sm.lu.Ls[t * NB + lane];
+#pragma unroll
+        for (int q = 0; q < CW; ++q) {
+          const double2 xt = shfl2(x[q], t);
+          if (g * CW + q >= k0 + kb && lane > t) cfms(x[q], lt, xt);
+        }
+      }
+#pragma unroll
+    for (int q = 0; q < CW; ++q) {
+      const int c = g * CW + q;
+      if (live && c < n && (c < k0 || c >= k0 + kb)) M[(size_t)c * n + k0 + lane] = x[q];
+    }
   }
 }
 
-__device__ double vec_norm(const double2* __restrict__ x, int n, VerifySmem& sm) {
+// LU of the n x n matrix M by a cluster of `size` CTAs: the first factors the panels, all share
+// the interchanges, the triangular solves and the trailing updates. Returns 0, or 1 + the
+// first column whose pivot was exactly zero (*flag: its way to the other CTAs).
+__device__ int cluster_lu(double2* M, int n, int* piv, int* flag, VerifySmem& sm, int rank, int size) {
+  if (threadIdx.x == 0) sm.lu.info_sh = 0;
+  __syncthreads();
+  for (int k0 = 0; k0 < n; k0 += NB) {
+    const int kb = min(NB, n - k0);
+    if (rank == 0) {
+      cta_lu_panel(M, n, k0 + kb, k0, kb, piv, sm.lu, k0);
+      if (threadIdx.x == 0) *flag = sm.lu.info_sh;
+    }
+    cluster_sync();
+    swap_and_trsm(M, n, k0, kb, piv, sm, rank, size);
+    cluster_sync();
+    if (k0 + kb >= n) break;
+    cta_lu_update_simt<double2, 2>(M, n, n, k0, kb, sm.lu, 0, rank, size);
+    cluster_sync();
+  }
+  return *flag;
+}
+
+// ---------------------------------------------------------------------------
+// The inverse iteration's triangular solves with one right-hand side, by the whole cluster in
+// 32-row blocks. The inverses of the diagonal blocks are formed once per value, so that a
+// block's unknowns are a product instead of a chain of 32 dependent steps. The first CTA takes
+// columns 0..32/size-1 of each block, and so on: each keeps its own sums
+//   acc[rank][i] = sum over its solved columns of A[i, t] y_t
+// (a row always by the same thread), and a block's right-hand side is in - sum_rank acc[rank]:
+// one cluster barrier per block. What bounds it: 2 n^2 multiply-adds an iteration on the FP64
+// pipe and then the barrier and L2 latency of 4 n / 32 blocks. One CTA with one or two barriers a
+// row took 3.7 ms an iteration at n = 512, substitution in 32-row blocks 1.2, this 0.33 with 4 CTAs.
+// ---------------------------------------------------------------------------
+// The inverses of L's (type 0) and U's (type 1) diagonal blocks, column-major and zero-padded
+// to 32 x 32: dinv + (type * blocks + block) * NB * NB. A warp takes four columns.
+__device__ void invert_diagonals(const double2* M, int n, double2* dinv, int rank, int size) {
+  constexpr int CW = 4;
+  const int lane = threadIdx.x & 31, blocks = (n + NB - 1) / NB;
+  for (int g = (rank * THREADS + (int)threadIdx.x) >> 5; g < 2 * blocks * (NB / CW); g += size * (THREADS / 32)) {
+    const int type = g / (blocks * (NB / CW)), blk = g / (NB / CW) % blocks, c0 = g % (NB / CW) * CW;
+    const int k0 = blk * NB, kb = min(NB, n - k0);
+    const double2* D = M + (size_t)k0 * n + k0;
+    double2 x[CW];
+#pragma unroll
+    for (int q = 0; q < CW; ++q) x[q] = make_double2(lane == c0 + q && c0 + q < kb ? 1.0 : 0.0, 0.0);
+    if (type == 0) {
+      for (int t = c0; t < kb - 1; ++t) {
+        const double2 d = lane > t && lane < kb ? D[(size_t)t * n + lane] : make_double2(0.0, 0.0);
+#pragma unroll
+        for (int q = 0; q < CW; ++q) cfms(x[q], d, shfl2(x[q], t));
+      }
+    } else {
+      const double2 rd = lane < kb ? crecip(D[(size_t)lane * n + lane]) : make_double2(0.0, 0.0);
+      for (int t = min(c0 + CW, kb) - 1; t >= 0; --t) {
+        const double2 d = lane < t ? D[(size_t)t * n + lane] : make_double2(0.0, 0.0);
+#pragma unroll
+        for (int q = 0; q < CW; ++q) {
+          if (lane == t) x[q] = cmul(x[q], rd);
+          cfms(x[q], d, shfl2(x[q], t));
+        }
+      }
+    }
+    double2* out = dinv + (size_t)(type * blocks + blk) * NB * NB;
+#pragma unroll
+    for (int q = 0; q < CW; ++q) out[(c0 + q) * NB + lane] = x[q];
+  }
+}
+
+// out = A^{-1} (scale * in) with A = M's triangle, or its conjugate transpose (HERM), in the
+// order of the blocks that FORWARD gives. dinv: that triangle's inverse diagonal blocks.
+// size divides 32. Every thread of the cluster; in and out are not the same.
+template <bool HERM, bool FORWARD>
+__device__ void cluster_solve(const double2* M, int n, const double2* dinv, const double2* in, double scale,
+                              double2* out, double2* acc, VerifySmem& sm, int rank, int size) {
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  const int blocks = (n + NB - 1) / NB, cw = NB / size, t0 = rank * cw;
+  double2* mine = acc + (size_t)rank * n;
+  double2* part = sm.lu.Us;  // [warp][row]
+  const double2 zero = make_double2(0.0, 0.0);
+  const auto at = [&](int i, int t) {  // A[i, t]
+    return HERM ? cconj(M[(size_t)i * n + t]) : M[(size_t)t * n + i];
+  };
+  for (int i = tid; i < n; i += THREADS) mine[i] = zero;
+  constexpr int G = 8;  // columns whose entries are in flight
+  for (int step = 0; step < blocks; ++step) {
+    const int blk = FORWARD ? step : blocks - 1 - step;
+    const int k0 = blk * NB, kb = min(NB, n - k0);
+    // what does not depend on the block's unknowns is loaded before the barrier
+    const double2* Dk = dinv + (size_t)blk * NB * NB;
+    double2 d[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int t = 4 * wid + u;
+      d[u] = HERM ? cconj(Dk[lane * NB + t]) : Dk[t * NB + lane];
+    }
+    // this thread's rows: 32-row chunks wid, wid + 8, ... among those still to be solved
+    const int first = FORWARD ? blk + 1 : 0, last = FORWARD ? blocks : blk;
+    int chunk = first + ((wid - first) & 7);
+    int i = chunk * NB + lane;
+    bool in_rows = chunk < last && i < n;
+    double2 m[G], a = in_rows ? mine[i] : zero;
+#pragma unroll
+    for (int u = 0; u < G; ++u) m[u] = in_rows && u < cw && t0 + u < kb ? at(i, k0 + t0 + u) : zero;
+    cluster_sync();
+    // this warp's four entries of the block's right-hand side: eight lanes each
+    const int tv = 4 * wid + (lane >> 3), r = lane & 7;
+    double2 v = zero;
+    if (tv < kb) {
+      if (r < size) {
+        const double2 s = acc[(size_t)r * n + k0 + tv];
+        v = make_double2(-s.x, -s.y);
+      }
+      if (r == 0) v = cadd(v, cscale(in[k0 + tv], scale));
+    }
+    for (int o = size >> 1; o > 0; o >>= 1) {
+      v.x += __shfl_down_sync(0xffffffffu, v.x, o);
+      v.y += __shfl_down_sync(0xffffffffu, v.y, o);
+    }
+    double2 y = zero;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) cfma(y, d[u], shfl2(v, 8 * u));
+    part[wid * NB + lane] = y;
+    __syncthreads();
+    // y_t of this CTA's columns, in every warp: four lanes a column, eight columns at a time
+    for (int g = 0; g < cw; g += G) {
+      const int t = t0 + g + (lane >> 2), q = lane & 3;
+      y = g + (lane >> 2) < cw ? cadd(part[q * NB + t], part[(q + 4) * NB + t]) : zero;
+#pragma unroll
+      for (int o = 1; o < 4; o <<= 1) {
+        y.x += __shfl_xor_sync(0xffffffffu, y.x, o);
+        y.y += __shfl_xor_sync(0xffffffffu, y.y, o);
+      }
+      if (wid == 0 && q == 0 && g + (lane >> 2) < cw && t < kb) out[k0 + t] = y;
+      double2 yt[G];
+#pragma unroll
+      for (int u = 0; u < G; ++u) yt[u] = shfl2(y, 4 * u);
+      for (int c = chunk; c < last; c += THREADS / 32) {
+        if (c != chunk || g != 0) {
+          i = c * NB + lane;
+          in_rows = i < n;
+          a = in_rows ? mine[i] : zero;
+#pragma unroll
+          for (int u = 0; u < G; ++u)
+            m[u] = in_rows && g + u < cw && t0 + g + u < kb ? at(i, k0 + t0 + g + u) : zero;
+        }
+#pragma unroll
+        for (int u = 0; u < G; ++u)
+          if (u < cw) cfma(a, m[u], yt[u]);
+        if (in_rows) mine[i] = a;
+      }
+    }
+  }
+  cluster_sync();
+}
+
+__device__ double vec_norm(const double2* x, int n, VerifySmem& sm) {
   double s = 0.0;
   for (int i = threadIdx.x; i < n; i += THREADS) s += cabs2(x[i]);
   return sqrt(block_sum(s, sm.red));
@@ -184,31 +358,31 @@ __global__ void __launch_bounds__(THREADS, 2) k_verify_fp64(ValueArgs a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   VerifySmem& sm = *reinterpret_cast<VerifySmem*>(smem_raw);
   const int tid = threadIdx.x;
-  double2* M = a.work + (size_t)blockIdx.x * a.max_n * a.max_n;
-  int* piv = a.piv + (size_t)blockIdx.x * a.max_n;
-  double2* x = a.vec + (size_t)blockIdx.x * 3 * a.max_n;
+  const int size = a.cluster, rank = cluster_rank(), slot = blockIdx.x / size;
+  double2* M = a.work + (size_t)slot * a.max_n * a.max_n;
+  int* piv = a.piv + (size_t)slot * a.max_n;
+  double2* y = a.vec + (size_t)slot * verify_vec_len(a.max_n);
 
-  for (int it = blockIdx.x; it < a.m; it += gridDim.x) {
+  for (int it = slot; it < a.m; it += gridDim.x / size) {
     load_problem(&sm.P, a.probs + a.prob_of[it]);
     __syncthreads();
     const ProblemDev& P = sm.P;
     const int n = P.n;
     const size_t nn = (size_t)n * n;
-    double2* wv = x + n;
-    double2* yv = x + 2 * n;
+    double2 *x = y + n, *acc = x + n, *dinv = acc + (size_t)size * n;
+    double2* dinvU = dinv + (size_t)(n + NB - 1) / NB * NB * NB;
     const double2 lam = a.lam[it];
     if (tid < P.K) sm.lu.fz[tid] = eval_f(P.term[tid], lam);
     if (BIE && tid == 0) sm.wave = bie::wave_of(lam);
     __syncthreads();
     if (BIE && P.bie) {
-      for (size_t e = tid; e < nn; e += THREADS) M[e] = make_double2(0.0, 0.0);
-      __syncthreads();
-      add_layer(P.bie, n, layer_coefficient(P), sm.wave, tid, THREADS,
+      for (size_t e = (size_t)rank * THREADS + tid; e < nn; e += size * THREADS) M[e] = make_double2(0.0, 0.0);
+      cluster_sync();
+      add_layer(P.bie, n, layer_coefficient(P), sm.wave, rank * THREADS + tid, size * THREADS,
                 [&](int i, int j, double2 v) { M[(size_t)j * n + i] = v; });
-      __syncthreads();
+      cluster_sync();
     }
-    double fro = 0.0;
-    for (int col = 0; col < n; ++col) {
+    for (int col = rank; col < n; col += size) {
       for (int row = tid; row < n; row += THREADS) {
         const size_t e = (size_t)col * n + row;
         double2 v = BIE && P.bie ? M[e] : make_double2(0.0, 0.0);
@@ -218,52 +392,43 @@ __global__ void __launch_bounds__(THREADS, 2) k_verify_fp64(ValueArgs a) {
           else if (row == col && t.kind != PMCIM_F_HELMHOLTZ_DLP) cfma(v, sm.lu.fz[k], t.id);
         }
         M[e] = v;
-        fro += cabs2(v);
       }
     }
-    fro = sqrt(block_sum(fro, sm.red));
-    const int info = cta_lu(M, n, n, piv, sm.lu);
+    cluster_sync();
+    double fro = 0.0;
+    if (rank == 0) {
+      for (size_t e = tid; e < nn; e += THREADS) fro += cabs2(M[e]);
+      fro = sqrt(block_sum(fro, sm.red));
+    }
+    const int info = cluster_lu(M, n, piv, reinterpret_cast<int*>(dinvU + (size_t)(n + NB - 1) / NB * NB * NB), sm,
+                                rank, size);
 
-    double smin = 0.0;
+    // Inverse iteration on T^H T; T = P^T L U, and as w = T^{-H} x is only needed as P w, the
+    // interchanges drop out. Every CTA forms the norms, from the same numbers in the same order.
+    double smin = 0.0, scale = 0.0;
     if (info == 0) {
+      invert_diagonals(M, n, dinv, rank, size);
       // deterministic start vector
-      for (int i = tid; i < n; i += THREADS) x[i] = make_double2(1.0 + 0.5 * sin(0.7 * i), cos(1.3 * i));
-      __syncthreads();
-      double nx = vec_norm(x, n, sm);
-      for (int i = tid; i < n; i += THREADS) x[i] = cscale(x[i], 1.0 / nx);
-      __syncthreads();
+      if (rank == 0)
+        for (int i = tid; i < n; i += THREADS) x[i] = make_double2(1.0 + 0.5 * sin(0.7 * i), cos(1.3 * i));
+      cluster_sync();
+      scale = 1.0 / vec_norm(x, n, sm);
       double rho_prev = 0.0, rho = 0.0;
       for (int iter = 0; iter < 30; ++iter) {
-        // w = T^{-H} x:  T = P^T L U  =>  T^H = U^H L^H P
-        for (int i = tid; i < n; i += THREADS) wv[i] = x[i];
-        __syncthreads();
-        solve_UH(M, n, wv, sm);
-        solve_LH(M, n, wv, sm);
-        if (tid == 0)
-          for (int k = n - 1; k >= 0; --k) {
-            int p = piv[k];
-            if (p != k) { double2 t = wv[k]; wv[k] = wv[p]; wv[p] = t; }
-          }
-        __syncthreads();
-        rho = vec_norm(wv, n, sm);
-        // y = T^{-1} w
-        for (int i = tid; i < n; i += THREADS) yv[i] = wv[i];
-        __syncthreads();
-        if (tid == 0)
-          for (int k = 0; k < n; ++k) {
-            int p = piv[k];
-            if (p != k) { double2 t = yv[k]; yv[k] = yv[p]; yv[p] = t; }
-          }
-        __syncthreads();
-        solve_L(M, n, yv, sm);
-        solve_U(M, n, yv, sm);
-        double ny = vec_norm(yv, n, sm);
-        for (int i = tid; i < n; i += THREADS) x[i] = cscale(yv[i], 1.0 / ny);
-        __syncthreads();
+        cluster_solve<true, true>(M, n, dinvU, x, scale, y, acc, sm, rank, size);   // U^H
+        cluster_solve<true, false>(M, n, dinv, y, 1.0, x, acc, sm, rank, size);     // L^H: P w
+        rho = vec_norm(x, n, sm);
+        cluster_solve<false, true>(M, n, dinv, x, 1.0, y, acc, sm, rank, size);     // L
+        cluster_solve<false, false>(M, n, dinvU, y, 1.0, x, acc, sm, rank, size);   // U: T^{-1} w
+        scale = 1.0 / vec_norm(x, n, sm);
         if (iter > 0 && fabs(rho - rho_prev) <= 1e-12 * rho) break;
         rho_prev = rho;
       }
       smin = 1.0 / rho;
+    }
+    if (rank != 0) {
+      cluster_sync();  // the first CTA has done with the slot (below)
+      continue;
     }
     if (tid == 0) {
       a.sigma[it] = smin;
@@ -272,8 +437,8 @@ __global__ void __launch_bounds__(THREADS, 2) k_verify_fp64(ValueArgs a) {
     }
     if (a.vec_out)  // the inverse iteration's last unit vector (zero when the LU met an exact zero pivot)
       for (int i = tid; i < n; i += THREADS)
-        a.vec_out[(size_t)it * a.max_n + i] = info == 0 ? x[i] : make_double2(0.0, 0.0);
-    __syncthreads();
+        a.vec_out[(size_t)it * a.max_n + i] = info == 0 ? cscale(x[i], scale) : make_double2(0.0, 0.0);
+    cluster_sync();
   }
 }
 
@@ -320,9 +485,20 @@ cudaError_t launch_verify_fp64(const ValueArgs& a, cudaStream_t s) {
   const void* fn = a.bie ? (const void*)k_verify_fp64<true> : (const void*)k_verify_fp64<false>;
   cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  int grid = a.slots < a.m ? a.slots : a.m;
-  if (a.bie) k_verify_fp64<true><<<grid, THREADS, smem, s>>>(a);
-  else k_verify_fp64<false><<<grid, THREADS, smem, s>>>(a);
+  const int clusters = a.slots < a.m ? a.slots : a.m;
+  cudaLaunchAttribute at;
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = (unsigned)a.cluster;
+  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(clusters * a.cluster));
+  cfg.blockDim = dim3(THREADS);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  e = a.bie ? cudaLaunchKernelEx(&cfg, k_verify_fp64<true>, a) : cudaLaunchKernelEx(&cfg, k_verify_fp64<false>, a);
+  if (e != cudaSuccess) return e;
   return cudaGetLastError();
 }
 

@@ -432,6 +432,11 @@ cudaError_t launch_reduce_moments(const LevelArgs& a, cudaStream_t s);
 cudaError_t launch_indicator(const LevelArgs& a, cudaStream_t s);
 cudaError_t launch_beyn(const LevelArgs& a, cudaStream_t s);
 
+// A verification slot's vectors: two of n, the CTAs' sums of n each (8 at most), the inverses
+// of L's and U's 32 x 32 diagonal blocks and a flag.
+__host__ __device__ inline size_t verify_vec_len(int n) {
+  return (size_t)10 * n + 2 * (size_t)((n + 31) / 32) * 1024 + 1;
+}
 struct ValueArgs {
   const ProblemDev* probs;
   const int32_t* prob_of;   // per value
@@ -443,7 +448,8 @@ struct ValueArgs {
   double* sigma;
   uint8_t* accept;
   double2* work;            // verify: slots * max_n * max_n
-  double2* vec;             // verify: slots * 3 * max_n
+  double2* vec;             // verify: slots * verify_vec_len(max_n)
+  int cluster;              // verify: CTAs that share one value's LU (1 to 8)
   int32_t* piv;             // verify: slots * max_n
   int slots;
   int max_n;
