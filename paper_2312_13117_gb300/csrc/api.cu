@@ -927,10 +927,9 @@ int run_level(Call& c, const std::vector<HostRegion>& regs, bool gate_top, bool 
   // ---- factorisation workspaces, one slot per resident CTA ----
   const int sms = num_sms();
   int slots64 = 0;
-  size_t slot64 = 0, digits64 = 0;
+  size_t slot64 = 0;
   if (any64) {
-    digits64 = ((size_t)max_n * (max_n + max_l) * sizeof(double2) + 127) & ~(size_t)127;
-    slot64 = digits64 + fp64_digit_bytes(max_n, max_l);
+    slot64 = (size_t)max_n * (max_n + max_l) * sizeof(double2);
     const size_t budget = slot_budget(ws.work64.cap);
     slots64 = (int)std::max<size_t>(1, std::min<size_t>(std::min<size_t>(2 * sms, budget / slot64), total_nodes));
     CU(ws.work64.ensure((size_t)slots64 * slot64));
@@ -1031,8 +1030,6 @@ int run_level(Call& c, const std::vector<HostRegion>& regs, bool gate_top, bool 
         na.counter = ws.counters.as<int>() + kCounters * wi;
         na.work = ws.work64.as<char>();
         na.slot_bytes = slot64;
-        na.digits_off = digits64;
-        na.tc_wait_cycles = wait_limit_tc();
         na.piv = ws.piv64.as<int32_t>();
         na.slots = slots64;
         prof_begin(PMCIM_K_FACTOR, s);

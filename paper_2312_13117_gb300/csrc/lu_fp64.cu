@@ -5,15 +5,10 @@
 // solver (Eq. 2.4; Appendix, linearsolver = MATLAB backslash) and suggests
 // solving all nodes in parallel (Sec. 3.2, remark on deeper parallelism).
 // Here one CTA owns one node at a time (persistent grid, one workspace slot per
-// CTA, two CTAs per SM), so no SM waits on another. GB300 issues only ~2 DFMA per
-// SM per clock: trailing updates from shared memory tiles on the FP64 pipe were
-// nearly all of a node's time, and now run as exact digit products on the tensor
-// cores in outer blocks of 64 columns (lu_fp64_tc.cuh). What is left on the FP64
-// pipe are the panels and the triangular solves, 3/32 of a node's n^3 / 3
-// multiply-adds at n = 1024. 256 nodes of n = 1024, l = 16 take 178 ms (833 before):
-// per CTA 30 in panels, 40 in triangular solves, 10 in updates of second panels, 65 in
-// the tensor-core updates; the error against extended-precision solutions at n = 130
-// to 450 is 0.5 to 0.9 times what it was.
+// CTA, two CTAs per SM): GB300 issues only ~2 DFMA per SM per clock, so a
+// node-per-CTA schedule keeps every SM's FP64 pipe busy without cross-CTA
+// synchronisation, and the trailing updates (the O(n^3) part) run from shared
+// memory tiles with a 4x4 complex register block per thread.
 //
 // The probe block V is appended to T as l extra columns, so the row swaps and
 // trailing updates of the factorisation also perform P and L^-1 on V; only the
@@ -21,120 +16,31 @@
 //
 // Pivot rule: the row maximising |Re| + |Im| in the column, lowest row index on
 // ties (the BLAS izamax convention of LAPACK zgetrf).
-#include <algorithm>
-#include <cstddef>
-
 #include "lu_core.cuh"
-#include "lu_fp64_tc.cuh"
 
 namespace {
 
 using namespace lucore;
-
-__device__ __forceinline__ double2 shfl2(double2 v, int src) {
-  return make_double2(__shfl_sync(0xffffffffu, v.x, src), __shfl_sync(0xffffffffu, v.y, src));
-}
 
 // ---------------------------------------------------------------------------
 // Persistent kernel: node g -> X_g = T(z_g)^{-1} V.
 // ---------------------------------------------------------------------------
 // Shared memory of the node kernel: the LU tiles plus the node's problem.
 struct NodeSmem {
+  LuSmem lu;
   ProblemDev P;
   bie::Wave wave;
   int item;
-  ozlu::Shared tc;
-  LuSmem lu;  // the tensor-core update stages its operands from lu.Ls on
 };
-constexpr size_t kNodeSmemBytes =
-    std::max(sizeof(NodeSmem), offsetof(NodeSmem, lu) + offsetof(LuSmem, Ls) + (size_t)ozlu::STAGE_BYTES);
-
-// U12 of an outer block's second panel (rows k0 + 32 .., columns kend..ncols-1): the first
-// panel's update of these rows and the triangular solve, a warp four columns at a time.
-__device__ void trsm_second(double2* M, int n, int ncols, int k0, LuSmem& sm) {
-  const int tid = threadIdx.x, lane = tid & 31;
-  const size_t ld = (size_t)n;
-  const int k1 = k0 + NB, kend = k1 + NB;
-  for (int e = tid; e < 2 * NB * NB; e += THREADS)  // Ls[t * 32 + i] = L[k1 + i, k0 + t], t < 64
-    sm.Ls[e] = M[(size_t)(k0 + e / NB) * ld + k1 + e % NB];
-  __syncthreads();
-  constexpr int CW = 4;
-  for (int c0 = kend + (tid >> 5) * CW; c0 < ncols; c0 += THREADS / 32 * CW) {
-    double2 y[CW], x[CW];
-#pragma unroll
-    for (int q = 0; q < CW; ++q) {
-      const bool in = c0 + q < ncols;
-      y[q] = in ? M[(size_t)(c0 + q) * ld + k0 + lane] : make_double2(0.0, 0.0);
-      x[q] = in ? M[(size_t)(c0 + q) * ld + k1 + lane] : make_double2(0.0, 0.0);
-    }
-    for (int t = 0; t < NB; ++t) {
-      const double2 l = sm.Ls[t * NB + lane];
-#pragma unroll
-      for (int q = 0; q < CW; ++q) cfms(x[q], l, shfl2(y[q], t));
-    }
-    for (int t = 0; t < NB - 1; ++t) {
-      const double2 l = sm.Ls[(NB + t) * NB + lane];
-#pragma unroll
-      for (int q = 0; q < CW; ++q) {
-        const double2 xt = shfl2(x[q], t);
-        if (lane > t) cfms(x[q], l, xt);
-      }
-    }
-#pragma unroll
-    for (int q = 0; q < CW; ++q)
-      if (c0 + q < ncols) M[(size_t)(c0 + q) * ld + k1 + lane] = x[q];
-  }
-  __syncthreads();
-}
-
-// cta_lu with the trailing updates on the tensor cores (lu_fp64_tc.cuh) while at least
-// kTcRows rows are left below an outer block of two panels: a tile takes some 21 us however
-// few of its 128 rows are there, and the FP64 pipe 1 us a row of it. With one panel an outer
-// block the drains (a quarter of a tile) would double, with four the work left on the FP64 pipe.
-constexpr int kTcRows = 32;
-template <int RI>
-__device__ int cta_lu_tc(double2* M, int n, int ncols, int* piv, unsigned char* scratch, NodeSmem& s,
-                         ozlu::State& st, long long limit) {
-  LuSmem& sm = s.lu;
-  if (threadIdx.x == 0) sm.info_sh = 0;
-  __syncthreads();
-  for (int k0 = 0; k0 < n;) {
-    const int kb = min(NB, n - k0), kend = k0 + kb;
-    const bool outer = st.on && n - k0 >= ozlu::KO + kTcRows;
-    cta_lu_panel(M, n, ncols, k0, kb, piv, sm);
-    if (kend >= ncols) break;
-    cta_lu_trsm(M, n, ncols, k0, kb, sm);
-    if (kend >= n) break;
-    if (!outer) {
-      cta_lu_update_simt<double2, RI>(M, n, ncols, k0, kb, sm);
-      k0 = kend;
-      continue;
-    }
-    const int k1 = kend, k2 = k1 + NB;
-    cta_lu_update_simt<double2, 2>(M, n, k2, k0, NB, sm);  // the second panel's 32 columns
-    cta_lu_panel(M, n, ncols, k1, NB, piv, sm);
-    trsm_second(M, n, ncols, k0, sm);
-    if (!ozlu::update(M, n, ncols, k0, scratch, reinterpret_cast<unsigned char*>(sm.Ls), s.tc, st, limit)) {
-      cta_lu_update_simt<double2, RI>(M, n, ncols, k0, NB, sm, k2);
-      cta_lu_update_simt<double2, RI>(M, n, ncols, k1, NB, sm, k2);
-    }
-    k0 = k2;
-  }
-  __syncthreads();
-  return sm.info_sh;
-}
 
 // RI: the trailing update's register block (4: 64 x 64 tiles; 2: 32 x 32 tiles).
 template <int RI, bool BIE>
 __global__ void __launch_bounds__(THREADS, 2) k_factor_solve_fp64(NodeArgs a) {
-  extern __shared__ __align__(128) unsigned char smem_raw[];
+  extern __shared__ __align__(16) unsigned char smem_raw[];
   NodeSmem& sm = *reinterpret_cast<NodeSmem*>(smem_raw);
   const int tid = threadIdx.x;
   double2* M = reinterpret_cast<double2*>(a.work + (size_t)blockIdx.x * a.slot_bytes);
-  unsigned char* digits = reinterpret_cast<unsigned char*>(M) + a.digits_off;
   int* piv = a.piv + (size_t)blockIdx.x * a.max_n;
-  ozlu::State st;
-  ozlu::begin(sm.tc);
 
   for (;;) {
     // largest-first list, handed out by an atomic counter (no waiting on other CTAs)
@@ -191,7 +97,7 @@ __global__ void __launch_bounds__(THREADS, 2) k_factor_solve_fp64(NodeArgs a) {
     for (size_t e = tid; e < (size_t)n * l; e += THREADS) M[nn + e] = P.V[e];
     __syncthreads();
 
-    const int info = cta_lu_tc<RI>(M, n, ncols, piv, digits, sm, st, a.tc_wait_cycles);
+    const int info = cta_lu<double2, RI>(M, n, ncols, piv, sm.lu);
     cta_back_blocked(M, n, l, sm.lu);
 
     double2* Xo = a.X + rg.x_off + (size_t)it.j * n * l;
@@ -199,7 +105,6 @@ __global__ void __launch_bounds__(THREADS, 2) k_factor_solve_fp64(NodeArgs a) {
     if (tid == 0) a.node_info[rg.node_off + it.j] = info;
     __syncthreads();
   }
-  ozlu::end(sm.tc);
 }
 
 // ---------------------------------------------------------------------------
@@ -224,6 +129,10 @@ __device__ __forceinline__ int cluster_rank() {
   unsigned r;
   asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
   return (int)r;
+}
+
+__device__ __forceinline__ double2 shfl2(double2 v, int src) {
+  return make_double2(__shfl_sync(0xffffffffu, v.x, src), __shfl_sync(0xffffffffu, v.y, src));
 }
 
 // A panel's interchanges on all other columns and U12 = L11^{-1} A12 on those right of it:
@@ -535,8 +444,6 @@ __global__ void __launch_bounds__(THREADS, 2) k_verify_fp64(ValueArgs a) {
 
 }  // namespace
 
-size_t fp64_digit_bytes(int n, int l) { return ozlu::scratch_bytes(n, l); }
-
 int factor_slots_fp64(int n, int l) {
   (void)n;
   (void)l;
@@ -550,7 +457,7 @@ cudaError_t prepare_factor_fp64() {
   const void* fns[4] = {(const void*)k_factor_solve_fp64<4, false>, (const void*)k_factor_solve_fp64<2, false>,
                         (const void*)k_factor_solve_fp64<4, true>, (const void*)k_factor_solve_fp64<2, true>};
   for (const void* f : fns) {
-    cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kNodeSmemBytes);
+    cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(NodeSmem));
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;
@@ -560,7 +467,7 @@ cudaError_t prepare_factor_fp64() {
 // is not called here so that the launch can be captured into a graph).
 cudaError_t launch_factor_solve_fp64(const NodeArgs& a, cudaStream_t s) {
   if (a.n_items <= 0) return cudaSuccess;
-  const size_t smem = kNodeSmemBytes;
+  const size_t smem = sizeof(NodeSmem);
   int grid = a.slots < a.n_items ? a.slots : a.n_items;
   if (a.bie) {
     if (a.fp64_tile == 32) k_factor_solve_fp64<2, true><<<grid, THREADS, smem, s>>>(a);

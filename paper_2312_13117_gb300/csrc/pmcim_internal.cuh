@@ -241,8 +241,6 @@ struct NodeArgs {
   int32_t* piv;             // slots * max_n
   int max_n;
   int slots;
-  size_t digits_off;              // FP64 kernel: a slot's operand digits (fp64_digit_bytes, 128-byte aligned)
-  long long tc_wait_cycles;       // FP64 kernel: limit of a tensor-core wait
   int fp64_tile;                  // FP64 kernel: trailing-update tile, 32 or 64 (0: 64)
   int bie;                        // FP64 and small kernels: a problem has a boundary-integral term
 };
@@ -376,7 +374,6 @@ bool small_kernel_fits(int n, int l);
 cudaError_t prepare_factor_small();
 cudaError_t launch_factor_solve_small(const NodeArgs& a, int max_n, int max_l, cudaStream_t s);
 int factor_slots_fp64(int n, int l);
-size_t fp64_digit_bytes(int n, int l);
 // FP64 nodes whose matrix and probe columns fit shared memory (lu_resident.cu)
 int resident_ctas(int n, int l);  // CTAs per SM, 0 when a node does not fit
 cudaError_t prepare_factor_resident();
