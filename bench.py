@@ -40,13 +40,6 @@ SM_MAX_MHZ = 2070.0
 # DRAM bytes per node of k_factor_solve_fp64, from one ncu capture of a 64-node launch at n = 1024, l = 16
 # (dram__bytes_read.sum + dram__bytes_write.sum = 15.16 + 13.45 GB); scaled to a launch by its node count.
 FACTOR_FP64_TRAFFIC_PER_NODE = 28.61e9 / 64
-# DRAM bytes per node of k_factor_solve_mixed, from one ncu capture of a 384-node launch per form
-# (dram__bytes_read.sum + dram__bytes_write.sum); scaled to a launch by its node count. None: no
-# capture of the kernel as it stands
-MIXED_TRAFFIC_PER_NODE = {"fp32ir": None, "tf32x3": (71.629e9 + 44.950e9) / 384, "bf16x3": None,
-                          "tf32x3_fp64res": None}
-# sm__pipe_tensor_cycles_active (% of active cycles) of the same capture of the tensor-core form
-MIXED_TENSOR_PIPE_PCT = {"tf32x3": 8.66}
 # FP32 pipe: 128 FFMA / SM / clock (measured 73.3 TFLOP/s at ~2.0 GHz); at the 2.07 GHz maximum:
 FP32_PEAK_TFLOPS = 128 * 2 * SM_COUNT * SM_MAX_MHZ * 1e6 / 1e12
 
@@ -1024,19 +1017,17 @@ def main():
         tm_max = max_over_ranks(tm_ms, world)
         fm = profm["factor_fp32"]
         # FP64 work: per sweep one residual product T(z)X (T(z) assembled in FP64 once per node
-        # by the factor group when the problem has two or more dense terms), plus the fallback solves
+        # by the factor step when the problem has two or more dense terms), plus the fallback solves
         w_asm = msolves * 8.0 * k_dense * n * n if (k_dense >= 2 and name == "tf32x3_fp64res") else 0.0
         w_res = aggm["ir_sweeps"] * 8.0 * n * n * l
         w64 = w_res + w_asm + aggm["ir_fallbacks"] * (8.0 * n ** 3 / 3 + 8.0 * n * n * l)
         w32 = msolves * (8.0 * n ** 3 / 3 + 8.0 * n * n * l) + aggm["ir_sweeps"] * 8.0 * n * n * l
         a64 = w64 / (fm["ms"] / 1e3) / 1e12 if fm["ms"] > 0 else None
         a32 = w32 / (fm["ms"] / 1e3) / 1e12 if fm["ms"] > 0 else None
-        roof = {"bound": "alu", "kernel": "k_factor_solve_mixed (FP64 pipe: refinement residuals)",
+        roof = {"bound": "alu", "kernel": "k_mixed_solve (FP64 pipe: refinement residuals)",
                 "achieved": a64, "peak": peak64, "unit": "TFLOP/s",
                 "frac": (a64 / peak64) if a64 else None,
-                "traffic": (MIXED_TRAFFIC_PER_NODE[name] * msolves / max(1, fm["launches"])
-                            if MIXED_TRAFFIC_PER_NODE.get(name) else None),
-                "traffic_note": "ncu DRAM bytes of a small capture, scaled by nodes per launch",
+                "traffic": None, "traffic_note": "no ncu capture of the whole form at this size",
                 "peak_source": "2 DFMA/SM/clk x 152 SMs x max SM clock",
                 "fp32_work_tflops": a32, "fp32_peak_tflops": FP32_PEAK_TFLOPS,
                 "launches": fm["launches"], "avg_launch_ms": fm["ms"] / max(1, fm["launches"]),
@@ -1057,19 +1048,16 @@ def main():
             t_s = fm["ms"] / 1e3
             ach = (res_bf16 + lu_tf32 * ratio + lu_bf16) / t_s / 1e12 if t_s > 0 else None
             roof = {"bound": "tensor",
-                    "kernel": {"tf32x3": "k_factor_solve_mixed (tensor pipe: 3xTF32 LU trailing updates + BF16 "
-                                         "digit products of the refinement residuals)",
-                               "bf16x3": "k_factor_solve_mixed (tensor pipe: BF16 3M LU trailing updates + BF16 "
-                                         "digit products of the refinement residuals)"}.get(
-                        name, "k_factor_solve_mixed (tensor pipe: BF16 digit products of the refinement "
-                              "residuals; LU on the FMA pipes)"),
+                    "kernel": "k_mixed_factor, k_oz_residual, k_mixed_solve (tensor pipe: "
+                              + {"tf32x3": "3xTF32 LU trailing updates + BF16 digit products of the refinement "
+                                           "residuals)",
+                                 "bf16x3": "BF16 3M LU trailing updates + BF16 digit products of the refinement "
+                                           "residuals)"}.get(
+                        name, "BF16 digit products of the refinement residuals; LU on the FMA pipes)"),
                     "achieved": ach, "peak": BF16_SUSTAINED_TFLOPS, "unit": "TFLOP/s (BF16-equivalent)",
                     "frac": (ach / BF16_SUSTAINED_TFLOPS) if ach else None,
                     "peak_source": "MEASURED_PEAKS.json bf16_tflops_sustained; TF32 flops x 2.25/1.1",
-                    "traffic": (MIXED_TRAFFIC_PER_NODE[name] * msolves / max(1, fm["launches"])
-                                if MIXED_TRAFFIC_PER_NODE.get(name) else None),
-                    "traffic_note": "ncu DRAM bytes of a 384-node capture, scaled by nodes per launch",
-                    "ncu_tensor_pipe_active_pct": MIXED_TENSOR_PIPE_PCT.get(name),
+                    "traffic": None, "traffic_note": "no ncu capture of the whole form at this size",
                     "residual_bf16_tflops": res_bf16 / t_s / 1e12 if t_s > 0 else None,
                     "lu_tf32_tflops": lu_tf32 / t_s / 1e12 if t_s > 0 else None,
                     "lu_bf16_tflops": lu_bf16 / t_s / 1e12 if t_s > 0 else None,
@@ -1078,7 +1066,7 @@ def main():
                     "launches": fm["launches"], "avg_launch_ms": fm["ms"] / max(1, fm["launches"]),
                     "share_of_step": fm["ms"] / tm_ms if tm_ms else None}
         if cyc.get("residual_fp64") and name == "tf32x3_fp64res":
-            # SM clock cycles of the refine group inside the residual phase, summed over CTAs
+            # SM clock cycles of the CTAs inside the residual phase, summed over CTAs
             # (one CTA per SM): the FP64 pipe's rate while the residual runs
             roof["residual_dfma_per_sm_clock"] = w_res / 2.0 / cyc["residual_fp64"]
             roof["peak_dfma_per_sm_clock"] = FP64_DFMA_PER_SM_CLK

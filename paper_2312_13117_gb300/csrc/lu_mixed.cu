@@ -265,7 +265,7 @@ __device__ double block_max(double v, double* red) {
 // R = V - sum_k f_k(z) A_k X  (FP64), R and X column-major n x l.
 // R = V - id X - f_M M X in FP64 (the refinement residual), M an n x n column-major
 // matrix (NULL: none). With two or more dense terms M is T(z_j) itself, assembled
-// in FP64 once per node by the factor group (f_M = 1, id = 0), so that a sweep
+// in FP64 once per node by the factor step (f_M = 1, id = 0), so that a sweep
 // multiplies X by one matrix instead of one per term; with a single dense term M
 // is that term's A_k.
 __device__ void residual_fp64(const double2* __restrict__ X, double2* __restrict__ R, const NodeCtx& cx,
@@ -481,7 +481,7 @@ __device__ void round_bie(const double2* __restrict__ T, float2* __restrict__ M3
 
 // T(z_j) for the FP32 LU: FP32 arithmetic on the complex64 copy of the A_k
 // (the LU only has to approximate T(z_j) to FP32 accuracy; the refinement
-// residuals use the FP64 coefficients). It keeps the factor group off the FP64
+// residuals use the FP64 coefficients). It keeps the factor step off the FP64
 // pipe. The flattened element index with eight elements per thread in flight
 // keeps the loads of each term overlapped; the identity terms are added to the
 // diagonal afterwards (a test per element would cost a 64-bit division).

@@ -150,20 +150,8 @@ __device__ __forceinline__ void tmem_ld_pair(uint32_t a_re, uint32_t a_im, float
   }
 }
 
-// Allocation, by one whole warp, before a barrier that the warps using the
-// columns also pass. The column count is a power of two >= 32.
-__device__ __forceinline__ void tmem_alloc(uint32_t* dst_smem) {
-  asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(dst_smem)),
-               "r"(TMEM_COLS)
-               : "memory");
-  asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-}
-
-__device__ __forceinline__ void tmem_dealloc(uint32_t tmem) {
-  asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TMEM_COLS) : "memory");
-}
-
-// The same for a given column count (a power of two, 32..512).
+// Allocation of a power of two of columns, 32..512, by one whole warp, before a barrier that
+// the warps using the columns also pass.
 __device__ __forceinline__ void tmem_alloc_cols(uint32_t* dst_smem, uint32_t cols) {
   asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(dst_smem)),
                "r"(cols)

@@ -15,7 +15,7 @@
 //     LU assumes; 3M adds the cancellation of P3 - P1 - P2, an absolute error of
 //     the order of 2^-24 (|Lr| + |Li|)(|Ur| + |Ui|);
 //   * per tile the three products sit in three 32-column TMEM accumulators; two
-//     tiles' accumulators (192 of the factor group's 256 columns) alternate, so the
+//     tiles' accumulators (192 of the CTA's 256 columns) alternate, so the
 //     epilogue of tile t runs while the tensor cores multiply tile t+1;
 //   * the operand stage holds the nine BF16 planes of L21 (3 operands x 3 parts,
 //     128 x 32 each, 72 KB) and the nine of one U12 tile (18 KB), in the canonical
@@ -42,7 +42,7 @@ constexpr int B_BYTES = 3 * PARTS * PLANE_B;  // [Ur, Ui, Ur + Ui] x 3 parts: 18
 constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
 constexpr uint32_t ACC_COLS = 3 * TN;         // P1, P2, P3 of one tile
 static_assert(STAGE_BYTES <= tcu::STAGE_BYTES, "the operands fit the 3xTF32 form's stage");
-static_assert(2 * ACC_COLS <= 256, "two tiles' accumulators in the factor group's TMEM columns");
+static_assert(2 * ACC_COLS <= 256, "two tiles' accumulators in the CTA's TMEM columns");
 static_assert(TK == lucore::NB, "the tensor-core tile is one panel deep");
 
 // Byte offset of element (row r, inner index k) in a K-major BF16 plane of 32 inner indices.
