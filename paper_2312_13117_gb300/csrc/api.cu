@@ -244,7 +244,7 @@ struct Workspace {
   DevBuf probs, regions, items, counters, node_info, X;
   DevBuf work64, piv64, work32, t64, phase;
   DevBuf tdig, texp;                     // boundary-integral nodes: digits of T(z_j), row exponents
-  DevBuf mstate, mctl, mlists, mubase, mmaps;  // precision forms: node states, counters, node lists, list bases
+  DevBuf mstate, mctl, mlists, mubase;  // precision forms: node states, counters, node lists, list bases
   DevBuf C0, C1, pf_half, pf_abs, ind, pf_norm, pf_scale, cand;
   DevBuf bwork, bsigma, bp, blam, bvecs, bkept, bstatus;
   DevBuf vlam, vprob, voff, vsig, vacc, vwork, vvec, vpiv;
@@ -267,7 +267,7 @@ struct Workspace {
     stream = nullptr;
     ordered = nullptr;
     DevBuf* b[] = {&probs, &regions, &items, &counters, &node_info, &X, &work64, &piv64, &work32, &t64,
-                   &phase, &tdig, &texp, &mstate, &mctl, &mlists, &mubase, &mmaps, &C0, &C1, &pf_half, &pf_abs, &ind, &pf_norm, &pf_scale, &cand, &bwork, &bsigma,
+                   &phase, &tdig, &texp, &mstate, &mctl, &mlists, &mubase, &C0, &C1, &pf_half, &pf_abs, &ind, &pf_norm, &pf_scale, &cand, &bwork, &bsigma,
                    &bp, &blam, &bvecs, &bkept, &bstatus, &vlam, &vprob, &voff, &vsig, &vacc, &vwork,
                    &vvec, &vpiv, &gitems, &gdst, &gperm, &ind3, &feats, &sprob, &sparams, &sscratch, &Xkeep,
                    &citems, &vout, &Cm, &iprobs, &iregions, &iitems, &iX, &iinfo, &icounters, &ibord, &ioffs, &ysl, &gexp, &rz,
@@ -538,7 +538,7 @@ void plan_mixed(Workspace& ws, const std::vector<ProblemDev>& pd, const std::vec
 }
 
 // Allocates what the plan needs and fills the arguments that all chunks share.
-int ensure_mixed(Call& c, const std::vector<ProblemDev>& pd, const MixedPlan& mp, int max_sweeps, MixedArgs* ma) {
+int ensure_mixed(Call& c, const MixedPlan& mp, int max_sweeps, MixedArgs* ma) {
   Workspace& ws = *c.ws;
   std::memset(ma, 0, sizeof(*ma));
   const size_t cnt = mp.max_count;
@@ -560,26 +560,6 @@ int ensure_mixed(Call& c, const std::vector<ProblemDev>& pd, const MixedPlan& mp
   CU(ws.mubase.ensure(std::max<size_t>(1, mp.ubase.size()) * sizeof(int)));
   CU(cudaMemcpyAsync(ws.mubase.p, mp.ubase.data(), mp.ubase.size() * sizeof(int), cudaMemcpyHostToDevice, c.s));
   CU(prepare_factor_mixed());
-  // the tensor maps of every chunk's problems, where a region updates on the tensor cores
-  bool maps = false;
-  for (const auto& w : mp.chunks)
-    for (const MixedChunk& ch : w) maps |= ch.tc != 0;
-  if (maps) {
-    std::vector<char> host(mp.ubase.size() * mixed_map_bytes());
-    size_t k = 0;
-    for (const auto& w : mp.chunks)
-      for (const MixedChunk& ch : w)
-        for (size_t p = 0; p < mp.n_probs; ++p, ++k)
-          if (maps && ch.tc && mixed_outer(pd[p].n) && pd[p].n <= ch.max_n)
-            maps = mixed_make_maps(ws.work32.as<char>(), mixed_slot_bytes(ch.max_n, ch.max_l), (int)ch.count, pd[p].n,
-                                   pd[p].l, host.data() + k * mixed_map_bytes());
-    if (maps) {
-      CU(ws.mmaps.ensure(host.size()));
-      CU(cudaMemcpyAsync(ws.mmaps.p, host.data(), host.size(), cudaMemcpyHostToDevice, c.s));
-      CU(cudaStreamSynchronize(c.s));  // host is pageable and ends here
-    }
-  }
-  ma->maps = maps ? ws.mmaps.as<char>() : nullptr;
   ma->n_probs = (int)mp.n_probs;
   ma->work = ws.work32.as<char>();
   ma->work_bytes = mp.work;
@@ -617,7 +597,6 @@ int launch_mixed(const MixedPlan& mp, size_t wave, size_t chunk0, const MixedArg
     a.slot_bytes = mixed_slot_bytes(ch.max_n, ch.max_l);
     a.tc = ch.tc;
     a.ubase = d_ubase + (chunk0 + k) * mp.n_probs;
-    if (a.maps) a.maps += (chunk0 + k) * mp.n_probs * mixed_map_bytes();
     int launched = 0;
     prof_begin(prof_kind, s);
     CU(launch_factor_solve_mixed(a, sms, s, &launched));
@@ -940,7 +919,7 @@ int run_level(Call& c, const std::vector<HostRegion>& regs, bool gate_top, bool 
   if (any32) {
     for (const Wave& wv : waves)
       plan_mixed(ws, c.pd, rd, items, wv.items32_off, wv.n32, tc_residual(c.opt), sms, &mp);
-    CHK(ensure_mixed(c, c.pd, mp, c.opt->max_ir_sweeps, &ma));
+    CHK(ensure_mixed(c, mp, c.opt->max_ir_sweeps, &ma));
     c.st.node_ctas = std::max(c.st.node_ctas, (int32_t)std::min<size_t>(sms, mp.max_count));
   }
   const bool timed = prof_on();
@@ -1608,7 +1587,7 @@ int run_bordered_step(Call& c, const std::vector<double2>& lam_in, const std::ve
     MixedPlan mp;
     MixedArgs ma;
     plan_mixed(ws, pdv, rdv, items, 0, it32.size(), false, sms, &mp);
-    CHK(ensure_mixed(c, pdv, mp, std::max(1, c.opt->max_ir_sweeps), &ma));
+    CHK(ensure_mixed(c, mp, std::max(1, c.opt->max_ir_sweeps), &ma));
     ma.probs = ws.iprobs.as<ProblemDev>();
     ma.regions = ws.iregions.as<RegionDev>();
     ma.X = ws.iX.as<double2>();

@@ -12,8 +12,7 @@
 //     with its key, and all threads pick the winner among the eight;
 //   * the panel's permutation then falls out of the positions, and is applied to the
 //     columns right of the panel by the triangular solve, which holds the panel's rows of
-//     a column in one warp anyway;
-//   * the pivots' reciprocals are kept for the back substitutions.
+//     a column in one warp anyway.
 // Against sub-panels factored in shared memory with separate interchanges, milliseconds of a
 // CTA per node: n = 256 panels 0.89 -> 0.37 (interchanges included), n = 1024 panels,
 // interchanges and triangular solves 9.3 -> 5.9, a sweep's solves (l = 16) 2.4 -> 2.0.
@@ -59,22 +58,12 @@ __device__ __forceinline__ unsigned pivot_key(float2 a) {
   return v >= 0.f ? __float_as_uint(v) + 1u : 0u;
 }
 
-__device__ __forceinline__ float2 recip32(float2 b) {  // Smith's scaling
-  if (fabsf(b.x) >= fabsf(b.y)) {
-    const float t = b.y / b.x, d = 1.0f / (b.x + b.y * t);
-    return make_float2(d, -t * d);
-  }
-  const float t = b.x / b.y, d = 1.0f / (b.x * t + b.y);
-  return make_float2(t * d, -d);
-}
-
 // Columns j0 .. j1-1 of a sub-panel, whose rows have at most WR columns left; v[i][c] is
 // column j + c of the thread's row i, so a step's update also shifts the row left.
 template <int R, int W, int WR>
 __device__ __forceinline__ void panel_steps(float2 (&v)[R][W], int (&pos)[R], int j0, int j1, int m, int p0,
                                             float2* __restrict__ P, int pld, PanelSmem& ps,
-                                            int* __restrict__ piv, float2* __restrict__ rinv,
-                                            int* __restrict__ info) {
+                                            int* __restrict__ piv, int* __restrict__ info) {
   const int tid = gtid(), lane = tid & 31, warp = tid >> 5;
   for (int j = j0; j < j1; ++j) {
     const int b = j & 1;
@@ -122,10 +111,9 @@ __device__ __forceinline__ void panel_steps(float2 (&v)[R][W], int (&pos)[R], in
     }
     const float2 pv = u[0];
     const bool zero = cis_zero(pv);
-    const float2 rp = recip32(pv);
+    const float2 rp = crecip(pv);
     if (tid == 0) {
       piv[p0 + j] = p0 + pp;
-      rinv[p0 + j] = rp;
       if (zero && *info == 0) *info = p0 + j + 1;
     }
     float2 l[R];
@@ -161,11 +149,11 @@ __device__ __forceinline__ void panel_steps(float2 (&v)[R][W], int (&pos)[R], in
 // sub-panel's columns get the permutation and the updates of the earlier ones as they are
 // loaded. Returns with the CTA synchronised, the panel's rows in their interchanged order
 // in M, its permutation in list (global, for the forward solves) and in ps.topsrc / bdst /
-// bsrc (for swap_trsm), the reciprocals of its pivots in rinv. scratch: panel_scratch_bytes.
+// bsrc (for swap_trsm). scratch: panel_scratch_bytes.
 template <int R>
 __device__ __noinline__ void panel(float2* __restrict__ M, int n, int k0, int kb, int* __restrict__ piv,
-                                   float2* __restrict__ rinv,
-                                   unsigned char* __restrict__ scratch, int* __restrict__ info) {
+                                   int* __restrict__ list, unsigned char* __restrict__ scratch,
+                                   int* __restrict__ info) {
   constexpr int W = NB / R;
   const int tid = gtid(), lane = tid & 31, warp = tid >> 5;
   const size_t ld = (size_t)n;
@@ -241,10 +229,10 @@ __device__ __noinline__ void panel(float2* __restrict__ M, int n, int k0, int kb
       }
     }
     constexpr int Q = W / 4;
-    panel_steps<R, W, W>(v, pos, 0, min(sb, Q), m, p0, P, m0, ps, piv, rinv, info);
-    panel_steps<R, W, W - Q>(v, pos, Q, min(sb, 2 * Q), m, p0, P, m0, ps, piv, rinv, info);
-    panel_steps<R, W, W - 2 * Q>(v, pos, 2 * Q, min(sb, 3 * Q), m, p0, P, m0, ps, piv, rinv, info);
-    panel_steps<R, W, W - 3 * Q>(v, pos, 3 * Q, sb, m, p0, P, m0, ps, piv, rinv, info);
+    panel_steps<R, W, W>(v, pos, 0, min(sb, Q), m, p0, P, m0, ps, piv, info);
+    panel_steps<R, W, W - Q>(v, pos, Q, min(sb, 2 * Q), m, p0, P, m0, ps, piv, info);
+    panel_steps<R, W, W - 2 * Q>(v, pos, 2 * Q, min(sb, 3 * Q), m, p0, P, m0, ps, piv, info);
+    panel_steps<R, W, W - 3 * Q>(v, pos, 3 * Q, sb, m, p0, P, m0, ps, piv, info);
     // the finished rows to their positions (a thread reads its own entries of P)
     int id[R];
 #pragma unroll
@@ -302,6 +290,8 @@ __device__ __noinline__ void panel(float2* __restrict__ M, int n, int k0, int kb
   gsync();
   if (tid < cnt) {
     const int d = ps.dst[tid], s = ps.src[tid];
+    list[1 + tid] = k0 + d;
+    list[1 + 2 * NB + tid] = k0 + s;
     if (d < kb) {
       ps.topsrc[d] = s;
     } else {  // such a row receives one of the panel's first rows (interchange j moves row j there)
@@ -310,193 +300,7 @@ __device__ __noinline__ void panel(float2* __restrict__ M, int n, int k0, int kb
       ps.bsrc[e] = s;
     }
   }
-  gsync();
-}
-
-// The panel's permutation for the forward solves (global memory).
-__device__ __forceinline__ void write_list(const PanelSmem& ps, int k0, int* __restrict__ list) {
-  const int tid = gtid();
-  if (tid < ps.cnt) {
-    list[1 + tid] = k0 + ps.dst[tid];
-    list[1 + 2 * NB + tid] = k0 + ps.src[tid];
-  }
-  if (tid == 0) list[0] = ps.cnt;
-}
-
-// ---------------------------------------------------------------------------
-// Outer blocks of OB columns (four panels): their panels are factored on the block's own
-// columns, whose interchanges reach all of the block (its L columns too); the columns right
-// of it then get the block's whole permutation and its 128 x 128 triangular solve in one
-// pass, and one update with K = 128 (tcu::update_wide).
-// ---------------------------------------------------------------------------
-constexpr int OB = 128;
-struct OuterSmem {
-  int top[OB];             // row (relative to k0) that the block's position i holds
-  int nb;                  // rows below the block that hold one of its first rows
-  int bdst[OB], bsrc[OB];  // (all such rows hold a row of the block)
-};
-__device__ __forceinline__ void outer_begin(OuterSmem& os) {
-  if (gtid() < OB) os.top[gtid()] = gtid();
-  if (gtid() == 0) os.nb = 0;
-  gsync();
-}
-// After the panel at row off of the block (kb columns; permutation in ps, relative to the panel).
-__device__ __forceinline__ void outer_compose(OuterSmem& os, const PanelSmem& ps, int off, int ob) {
-  const int tid = gtid(), cnt = ps.cnt, nb = os.nb;
-  int val = 0, at = -1, dst = 0;
-  if (tid < cnt) {
-    const int s = off + ps.src[tid];
-    dst = off + ps.dst[tid];
-    val = s < ob ? os.top[s] : s;
-    for (int e = 0; e < nb; ++e) {
-      if (os.bdst[e] == s) val = os.bsrc[e];
-      if (os.bdst[e] == dst) at = e;
-    }
-  }
-  gsync();
-  if (tid < cnt) {
-    if (dst < ob) {
-      os.top[dst] = val;
-    } else {
-      if (at < 0) at = atomicAdd(&os.nb, 1);
-      os.bdst[at] = dst;
-      os.bsrc[at] = val;
-    }
-  }
-  gsync();
-}
-// The block's permutation for the forward solves: count, 2 OB rows, 2 OB source rows.
-__device__ __forceinline__ void outer_list(const OuterSmem& os, int k0, int ob, int* __restrict__ list) {
-  if (gtid() >= 32) return;
-  const int lane = gtid();
-  int cnt = 0;
-  for (int i0 = 0; i0 < ob; i0 += 32) {
-    const int i = i0 + lane;
-    const bool moved = i < ob && os.top[i] != i;
-    const unsigned b = __ballot_sync(0xffffffffu, moved);
-    if (moved) {
-      const int e = cnt + __popc(b & ((1u << lane) - 1u));
-      list[1 + e] = k0 + i;
-      list[1 + 2 * OB + e] = k0 + os.top[i];
-    }
-    cnt += __popc(b);
-  }
-  for (int e = lane; e < os.nb; e += 32) {
-    list[1 + cnt + e] = k0 + os.bdst[e];
-    list[1 + 2 * OB + cnt + e] = k0 + os.bsrc[e];
-  }
-  if (lane == 0) list[0] = cnt + os.nb;
-}
-
-// The panel's permutation (ps, relative to row p0) on columns c_lo .. c_hi-1, a warp per column.
-__device__ inline void swap_columns(float2* __restrict__ M, int n, int c_lo, int c_hi, int p0, const PanelSmem& ps) {
-  const int lane = gtid() & 31, wid = gtid() >> 5, cnt = ps.cnt;
-  const bool a = lane < cnt, b = lane + 32 < cnt;
-  const int d0 = a ? ps.dst[lane] : 0, s0 = a ? ps.src[lane] : 0;
-  const int d1 = b ? ps.dst[lane + 32] : 0, s1 = b ? ps.src[lane + 32] : 0;
-  constexpr int CW = 4;
-  for (int c0 = c_lo + wid * CW; c0 < c_hi; c0 += THREADS / 32 * CW) {
-    float2 x[CW], y[CW];
-#pragma unroll
-    for (int q = 0; q < CW; ++q)
-      if (c0 + q < c_hi) {
-        const float2* col = M + (size_t)(c0 + q) * n + p0;
-        x[q] = col[s0];
-        y[q] = col[s1];
-      }
-    __syncwarp();
-#pragma unroll
-    for (int q = 0; q < CW; ++q)
-      if (c0 + q < c_hi) {
-        float2* col = M + (size_t)(c0 + q) * n + p0;
-        if (a) col[d0] = x[q];
-        if (b) col[d1] = y[q];
-      }
-  }
-  gsync();
-}
-
-// Bytes of outer_trsm's scratch: the ten 32 x 32 blocks of L11's lower triangle, and two
-// columns per warp.
-constexpr size_t OUTER_SCRATCH = 10 * NB * NB * sizeof(float2) + THREADS / 32 * 2 * OB * sizeof(float2);
-
-// The block's interchanges and U12 = L11^{-1} A12 (L11 ob x ob, ob <= 128) on columns k0 + ob ..
-// ncols-1: lane i of a warp holds rows i, i + 32, i + 64, i + 96 of CW columns.
-__device__ __noinline__ void outer_trsm(float2* __restrict__ M, int n, int ncols, int k0, int ob, const OuterSmem& os,
-                                        unsigned char* __restrict__ scratch) {
-  constexpr int CW = 4, NBLK = OB / NB;
-  const int tid = gtid(), lane = tid & 31, wid = tid >> 5;
-  const size_t ld = (size_t)n;
-  float2* L = reinterpret_cast<float2*>(scratch);  // block (bi, bj) at (bi (bi + 1) / 2 + bj), [t][i]
-  float2* buf = L + 10 * NB * NB + wid * 2 * OB;
-  for (int bi = 0; bi < NBLK; ++bi)
-    for (int bj = 0; bj <= bi; ++bj)
-#pragma unroll
-      for (int u = 0; u < NB * NB / THREADS; ++u) {
-        const int e = tid + u * THREADS, i = e & (NB - 1), t = e / NB;
-        const int r = bi * NB + i, c = bj * NB + t;
-        L[(bi * (bi + 1) / 2 + bj) * NB * NB + e] =
-            r < ob && c < r ? M[(size_t)(k0 + c) * ld + k0 + r] : make_float2(0.f, 0.f);
-      }
-  gsync();
-  int ts[NBLK];
-#pragma unroll
-  for (int b = 0; b < NBLK; ++b) ts[b] = b * NB + lane < ob ? os.top[b * NB + lane] : -1;
-  for (int c0 = k0 + ob + wid * CW; c0 < ncols; c0 += THREADS / 32 * CW) {
-    float2 x[NBLK][CW];
-#pragma unroll
-    for (int h = 0; h < CW; h += 2) {
-#pragma unroll
-      for (int b = 0; b < NBLK; ++b)
-#pragma unroll
-        for (int q = 0; q < 2; ++q) {
-          const int c = c0 + h + q;
-          if (ts[b] >= 0 && c < ncols) buf[q * OB + b * NB + lane] = M[(size_t)c * ld + k0 + b * NB + lane];
-        }
-      __syncwarp();
-#pragma unroll
-      for (int b = 0; b < NBLK; ++b)
-#pragma unroll
-        for (int q = 0; q < 2; ++q) {
-          const int c = c0 + h + q;
-          float2 v = make_float2(0.f, 0.f);
-          if (ts[b] >= 0 && c < ncols) v = ts[b] < ob ? buf[q * OB + ts[b]] : M[(size_t)c * ld + k0 + ts[b]];
-          if (h == 0) x[b][q] = v;
-          else x[b][2 + q] = v;
-        }
-      __syncwarp();  // the columns' rows are all read before any is written
-      for (int e = lane; e < os.nb; e += 32)
-#pragma unroll
-        for (int q = 0; q < 2; ++q)
-          if (c0 + h + q < ncols) M[(size_t)(c0 + h + q) * ld + k0 + os.bdst[e]] = buf[q * OB + os.bsrc[e]];
-      __syncwarp();
-    }
-#pragma unroll
-    for (int bj = 0; bj < NBLK; ++bj) {
-      if (bj * NB < ob) {
-        for (int t = 0; t < NB; ++t) {
-          float2 y[CW];
-#pragma unroll
-          for (int q = 0; q < CW; ++q) {
-            y[q].x = __shfl_sync(0xffffffffu, x[bj][q].x, t);
-            y[q].y = __shfl_sync(0xffffffffu, x[bj][q].y, t);
-          }
-#pragma unroll
-          for (int bi = bj; bi < NBLK; ++bi) {
-            // (zero on and above the diagonal, and past the block)
-            const float2 l = L[(bi * (bi + 1) / 2 + bj) * NB * NB + t * NB + lane];
-#pragma unroll
-            for (int q = 0; q < CW; ++q) cfms(x[bi][q], l, y[q]);
-          }
-        }
-      }
-    }
-#pragma unroll
-    for (int b = 0; b < NBLK; ++b)
-#pragma unroll
-      for (int q = 0; q < CW; ++q)
-        if (ts[b] >= 0 && c0 + q < ncols) M[(size_t)(c0 + q) * ld + k0 + b * NB + lane] = x[b][q];
-  }
+  if (tid == 0) list[0] = cnt;
   gsync();
 }
 
@@ -618,13 +422,33 @@ __device__ __forceinline__ void load_diagonal(const float2* __restrict__ M, int 
   }
 }
 
-// The diagonal block's solve; lower: unit lower triangle, else upper with the pivots'
-// reciprocals rinv. S rows past kb and columns past l become zero.
+// Division by one pivot (Smith, cdiv to the bit: its products are rounded before they are
+// added): the ratio of the pivot's parts and the denominator are formed once, two real
+// divisions are left per quotient.
+struct Divisor {
+  float t, d;
+  bool re;  // |Re| >= |Im|
+  __device__ explicit Divisor(float2 b) : re(fabsf(b.x) >= fabsf(b.y)) {
+    const float u = re ? b.x : b.y, v = re ? b.y : b.x;
+    t = v / u;
+    d = __fadd_rn(__fmul_rn(v, t), u);
+  }
+  __device__ __forceinline__ float2 divide(float2 a) const {
+    const float p = __fmul_rn(a.x, t), q = __fmul_rn(a.y, t);
+    const float x = re ? __fadd_rn(q, a.x) : __fadd_rn(p, a.y);
+    const float y = re ? __fadd_rn(-p, a.y) : __fadd_rn(q, -a.x);
+    return make_float2(x / d, y / d);
+  }
+};
+
+// The diagonal block's solve; lower: unit lower triangle, else upper, whose unknowns are
+// quotients by the pivots (a multiplication by a rounded reciprocal would be one rounding
+// more per unknown). S rows past kb and columns past l become zero.
 template <bool LOWER>
-__device__ __forceinline__ void solve_diagonal(float2* __restrict__ Y, int n, int l, int k0, int kb,
-                                               const float2* __restrict__ rinv, SolveSmem32& sm, int ldS) {
+__device__ __forceinline__ void solve_diagonal(float2* __restrict__ Y, int n, int l, int k0, int kb, SolveSmem32& sm,
+                                               int ldS) {
   const int lane = gtid() & 31, wid = gtid() >> 5;
-  const float2 rd = !LOWER && lane < kb ? rinv[k0 + lane] : make_float2(0.f, 0.f);
+  const Divisor pivot(!LOWER && lane < kb ? sm.Ls[lane * NB + lane] : make_float2(1.f, 0.f));
   for (int c = wid; c < ldS; c += 2 * (THREADS / 32)) {
     const int c2 = c + THREADS / 32;
     float2 a = lane < kb && c < l ? Y[(size_t)c * n + k0 + lane] : make_float2(0.f, 0.f);
@@ -633,8 +457,8 @@ __device__ __forceinline__ void solve_diagonal(float2* __restrict__ Y, int n, in
       const int t = LOWER ? s : kb - 1 - s;
       const float2 lt = sm.Ls[t * NB + lane];
       if (!LOWER && lane == t) {
-        a = cmul(a, rd);
-        b = cmul(b, rd);
+        a = pivot.divide(a);
+        b = pivot.divide(b);
       }
       float2 ta, tb;
       ta.x = __shfl_sync(0xffffffffu, a.x, t);
@@ -663,52 +487,43 @@ __device__ __forceinline__ void update_any(const float2* __restrict__ M, float2*
 __device__ __forceinline__ int solve_lds(int l) { return l > 8 ? (l + 15) / 16 * 16 : 8; }
 
 // U x = y.
-__device__ inline void back(const float2* __restrict__ M, float2* __restrict__ Y, int n, int l,
-                            const float2* __restrict__ rinv, SolveSmem32& sm) {
+__device__ inline void back(const float2* __restrict__ M, float2* __restrict__ Y, int n, int l, SolveSmem32& sm) {
   const int ldS = solve_lds(l);
   for (int k0 = (n - 1) / NB * NB; k0 >= 0; k0 -= NB) {
     const int kb = min(NB, n - k0);
     load_diagonal(M, n, k0, kb, sm);
     gsync();
-    solve_diagonal<false>(Y, n, l, k0, kb, rinv, sm, ldS);
+    solve_diagonal<false>(Y, n, l, k0, kb, sm, ldS);
     gsync();
     update_any(M, Y, n, l, k0, kb, 0, k0, sm, ldS);
     gsync();
   }
 }
 
-// L y = b, the permutation of each block of `outer` panels (lists + p SWAP_LIST_INTS for its
-// first panel p, global memory: count, 64 outer rows, their source rows) applied to y before
-// the block's columns of L.
+// L y = b, each panel's permutation (lists + p SWAP_LIST_INTS, global memory) applied to y
+// before its columns of L.
 __device__ inline void forward(const float2* __restrict__ M, float2* __restrict__ Y, int n, int l, SolveSmem32& sm,
-                               const int* __restrict__ lists, int outer) {
+                               const int* __restrict__ lists) {
   const int ldS = solve_lds(l), lane = gtid() & 31, wid = gtid() >> 5;
   for (int k0 = 0; k0 < n; k0 += NB) {
     const int kb = min(NB, n - k0);
-    if (k0 % (NB * outer) == 0) {
+    {
       // a warp per column: all its rows are read before any is written
       const int* L = lists + (size_t)(k0 / NB) * SWAP_LIST_INTS;
-      const int cnt = L[0], half = 2 * NB * outer;
+      const int cnt = L[0];
+      const int d0 = lane < cnt ? L[1 + lane] : 0, s0 = lane < cnt ? L[1 + 2 * NB + lane] : 0;
+      const int d1 = lane + 32 < cnt ? L[33 + lane] : 0, s1 = lane + 32 < cnt ? L[33 + 2 * NB + lane] : 0;
       for (int c = wid; c < l; c += THREADS / 32) {
         float2* y = Y + (size_t)c * n;
-        float2 v[8];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-          const int e = lane + 32 * u;
-          if (e < cnt) v[u] = y[L[1 + half + e]];
-        }
+        const float2 a = y[s0], b = y[s1];
         __syncwarp();
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-          const int e = lane + 32 * u;
-          if (e < cnt) y[L[1 + e]] = v[u];
-        }
+        if (lane < cnt) y[d0] = a;
+        if (lane + 32 < cnt) y[d1] = b;
       }
-      gsync();
     }
     load_diagonal(M, n, k0, kb, sm);
     gsync();
-    solve_diagonal<true>(Y, n, l, k0, kb, nullptr, sm, ldS);
+    solve_diagonal<true>(Y, n, l, k0, kb, sm, ldS);
     gsync();
     update_any(M, Y, n, l, k0, kb, k0 + kb, n, sm, ldS);
     gsync();

@@ -275,12 +275,12 @@ __device__ void cta_lu_trsm(T2* __restrict__ M, int n, int ncols, int k0, int kb
 // chosen by the autotuner per problem size).
 template <typename T2, int RI = 4>
 __device__ void cta_lu_update_simt(T2* __restrict__ M, int n, int ncols, int k0, int kb, LuSmemT<T2>& sm,
-                                   int first = 0, int part = 0, int parts = 1) {
+                                   int part = 0, int parts = 1) {
   constexpr int TT = 16 * RI;
   static_assert(TT <= TILE, "the shared tiles are sized for TILE");
   const int tid = gtid();
   const size_t ld = (size_t)n;
-  const int kend = first > k0 + kb ? first : k0 + kb;  // first updated row and column
+  const int kend = k0 + kb;
   // ---- trailing update A22 -= L21 U12 over TT x TT tiles ----
   const int m_rows = n - kend, m_cols = ncols - kend;
   const int mt = (m_rows + TT - 1) / TT, nt = (m_cols + TT - 1) / TT;

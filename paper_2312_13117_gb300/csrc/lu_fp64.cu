@@ -208,7 +208,7 @@ __device__ int cluster_lu(double2* M, int n, int* piv, int* flag, VerifySmem& sm
     swap_and_trsm(M, n, k0, kb, piv, sm, rank, size);
     cluster_sync();
     if (k0 + kb >= n) break;
-    cta_lu_update_simt<double2, 2>(M, n, n, k0, kb, sm.lu, 0, rank, size);
+    cta_lu_update_simt<double2, 2>(M, n, n, k0, kb, sm.lu, rank, size);
     cluster_sync();
   }
   return *flag;

@@ -35,10 +35,7 @@
 // tensor cores: 3xTF32 (tc_update.cuh) or BF16 3M (tc_update_bf16.cuh).
 // node_info: bits 0-23 = 0 or 1 + first zero-pivot column, bits 24-28 = sweeps
 // run, bit 29 = a tensor-core wait ran out, bit 30 = FP64 fallback.
-#include <cuda.h>
-
 #include <algorithm>
-#include <cstring>
 
 #include "ozaki.cuh"
 #include "tc_update_bf16.cuh"
@@ -104,19 +101,16 @@ struct FactorSmem {
   uint64_t mbar_tc[2];    // tensor-core completion, one per accumulator
   uint32_t tmem_base;     // TMEM_FACTOR columns
   int tc_bad;             // a tensor-core wait ran out: FMA pipes from then on
-  tcu::Wide wide;         // steps of the wide updates, staging warps -> issuing thread
-  lu32::OuterSmem os;
   // last: the operand stage of the trailing update starts at lu32.Ls and runs over the
   // end of the struct
   LuSmemT<float2> lu32;
 };
 constexpr size_t kFactorHead = offsetof(FactorSmem, lu32) + offsetof(LuSmemT<float2>, Ls);
 
-constexpr size_t kTcStage = tcu::WIDE_STAGE > tcu::STAGE_BYTES ? tcu::WIDE_STAGE : tcu::STAGE_BYTES;
 // Bytes of the scratch that starts at lu32.Ls: the operand stage of the tensor-core
 // updates, or else the FMA pipes' tiles and the largest panel's scratch.
 inline size_t factor_scratch_bytes(int max_n, bool tc) {
-  if (tc) return kTcStage;
+  if (tc) return tcu::STAGE_BYTES;
   size_t b = sizeof(LuSmemT<float2>) - offsetof(LuSmemT<float2>, Ls);
   for (int rows : {max_n, 256, 512, 1024, 2048})
     if (rows <= max_n && rows <= lu32::ROWS_MAX) b = std::max(b, lu32::panel_scratch_bytes(rows));
@@ -163,79 +157,31 @@ struct PhaseClock {
   }
 };
 
-constexpr int kOuterMinN = 160;  // orders above it factor in outer blocks (3xTF32)
-
-// One panel by the rows per thread it needs.
-__device__ __forceinline__ void panel32(float2* __restrict__ M, int n, int k0, int kb, int* __restrict__ piv,
-                                        float2* __restrict__ rinv, unsigned char* stage, int* info) {
-  const int r = lu32::panel_r(n - k0);
-  if (r == 1) lu32::panel<1>(M, n, k0, kb, piv, rinv, stage, info);
-  else if (r == 2) lu32::panel<2>(M, n, k0, kb, piv, rinv, stage, info);
-  else if (r == 4) lu32::panel<4>(M, n, k0, kb, piv, rinv, stage, info);
-  else lu32::panel<8>(M, n, k0, kb, piv, rinv, stage, info);
-}
-
 // The FP32 blocked LU: register panels (lu32.cuh; columns of more rows than they hold in
 // global memory), the trailing updates on the tensor cores (tc: 1 = 3xTF32, 2 = BF16 3M; while
-// no wait has run out) or on the FMA pipes (0). Row interchanges in LINPACK's order by blocks of
-// `outer` panels (none on the L columns left of a block); each block's permutation goes to lists
-// for the forward solves, the pivots' reciprocals to rinv.
-// outer: 4 for 3xTF32 within the register panels' rows (one update with K = 128 per block
-// instead of four that each read and write the trailing matrix), else 1.
+// no wait has run out) or on the FMA pipes (0). Row interchanges in LINPACK's order (none on
+// the L columns left of a panel); each panel's permutation goes to lists for the forward
+// solves.
 __device__ int cta_lu32(float2* __restrict__ M, int n, int ncols, int* __restrict__ piv, int* __restrict__ lists,
-                        float2* __restrict__ rinv, LuSmemT<float2>& sm, lu32::OuterSmem& os, tcu::Ctx& cx, int tc,
-                        int outer, PhaseClock& pc) {
+                        LuSmemT<float2>& sm, tcu::Ctx& cx, int tc, PhaseClock& pc) {
   if (gtid() == 0) sm.info_sh = 0;
   gsync();
-  if (outer > 1) {
-    for (int k0 = 0; k0 < n; k0 += lu32::OB) {
-      const int ob = min(lu32::OB, n - k0), kend = k0 + ob;
-      lu32::outer_begin(os);
-      for (int p0 = k0; p0 < kend; p0 += NB) {
-        const int kb = min(NB, kend - p0);
-        panel32(M, n, p0, kb, piv, rinv, cx.stage, &sm.info_sh);
-        const lu32::PanelSmem& ps = lu32::panel_smem(cx.stage, n - p0);
-        lu32::outer_compose(os, ps, p0 - k0, ob);
-        if (p0 > k0) lu32::swap_columns(M, n, k0, p0, p0, ps);
-        pc.mark(PH_PANEL);
-        if (p0 + kb < kend) {
-          lu32::swap_trsm(M, n, kend, p0, kb, ps, reinterpret_cast<float2*>(cx.stage));
-          pc.mark(PH_TRSM);
-          if (!*cx.bad) tcu::update(M, n, kend, p0, kb, cx);
-          else cta_lu_update_simt(M, n, kend, p0, kb, sm);
-          pc.mark(PH_UPDATE);
-        }
-      }
-      lu32::outer_list(os, k0, ob, lists + (size_t)(k0 / NB) * SWAP_LIST_INTS);
-      if (kend >= ncols) continue;
-      lu32::outer_trsm(M, n, ncols, k0, ob, os, cx.stage);
-      pc.mark(PH_TRSM);
-      if (kend >= n) continue;
-      if (!*cx.bad) {
-        tcu::update_wide(M, n, ncols, k0, cx);
-      } else {
-        for (int p0 = k0; p0 < kend; p0 += NB) cta_lu_update_simt(M, n, ncols, p0, min(NB, kend - p0), sm, kend);
-      }
-      pc.mark(PH_UPDATE);
-    }
-    gsync();
-    return sm.info_sh;
-  }
   for (int k0 = 0; k0 < n; k0 += NB) {
     const int kb = min(NB, n - k0);
     const int kend = k0 + kb, rows = n - k0;
     int* list = lists + (size_t)(k0 / NB) * SWAP_LIST_INTS;
     if (rows <= lu32::ROWS_MAX) {
-      panel32(M, n, k0, kb, piv, rinv, cx.stage, &sm.info_sh);
-      const lu32::PanelSmem& ps = lu32::panel_smem(cx.stage, rows);
-      lu32::write_list(ps, k0, list);
+      const int r = lu32::panel_r(rows);
+      if (r == 1) lu32::panel<1>(M, n, k0, kb, piv, list, cx.stage, &sm.info_sh);
+      else if (r == 2) lu32::panel<2>(M, n, k0, kb, piv, list, cx.stage, &sm.info_sh);
+      else if (r == 4) lu32::panel<4>(M, n, k0, kb, piv, list, cx.stage, &sm.info_sh);
+      else lu32::panel<8>(M, n, k0, kb, piv, list, cx.stage, &sm.info_sh);
       pc.mark(PH_PANEL);
       if (kend >= ncols) continue;
-      lu32::swap_trsm(M, n, ncols, k0, kb, ps, reinterpret_cast<float2*>(cx.stage));
+      lu32::swap_trsm(M, n, ncols, k0, kb, lu32::panel_smem(cx.stage, rows), reinterpret_cast<float2*>(cx.stage));
     } else {
       cta_lu_panel(M, n, ncols, k0, kb, piv, sm, k0);
       if (gtid() == 0) compose_swaps(piv, k0, kend, list);
-      if (gtid() < kb) rinv[k0 + gtid()] = lu32::recip32(M[(size_t)(k0 + gtid()) * n + k0 + gtid()]);
       gsync();
       pc.mark(PH_PANEL);
       if (kend >= ncols) continue;
@@ -389,21 +335,6 @@ __device__ void residual_fp64_col(const double2* __restrict__ X, double2* __rest
   gsync();
 }
 
-// Place in the FP32 matrix or right-hand sides of element e of an array with leading
-// dimension n (the leading dimension is mixed_order(n) there): e + e / n for an odd n, the
-// quotient by a product, e ceil(2^40 / n) >> 40, which is exact for e < n^2 up to n = 10321.
-struct At32 {
-  unsigned long long m;
-  unsigned n;
-  __device__ explicit At32(int order) : m(0), n((unsigned)order) {
-    if (n & 1) m = ((1ull << 40) + n - 1) / n;
-  }
-  __device__ __forceinline__ size_t operator()(size_t e) const {
-    if (m == 0) return e;
-    return e + (n <= 10321u ? (unsigned)((e * m) >> 40) : (unsigned)e / n);
-  }
-};
-
 // T(z_j) in FP64 into T (n x n, column-major), the matrix of the refinement
 // residuals, and rounded to complex64 into M32 (leading dimension n), the FP32
 // LU's matrix: the dense terms in one pass over the elements, four elements per
@@ -413,7 +344,6 @@ struct At32 {
 __device__ void assemble_fp64(const NodeCtx& cx, double2* __restrict__ T, float2* __restrict__ M32, bool herm) {
   const ProblemDev& P = cx.P;
   const int n = P.n;
-  const At32 at(n);
   const size_t nn = (size_t)n * n;
   for (size_t e0 = gtid(); e0 < nn; e0 += 4 * (size_t)THREADS) {
     double2 v[4];
@@ -439,7 +369,7 @@ __device__ void assemble_fp64(const NodeCtx& cx, double2* __restrict__ T, float2
       if (e < nn) {
         if (herm) v[u].y = -v[u].y;
         T[e] = v[u];
-        M32[at(e)] = make_float2((float)v[u].x, (float)v[u].y);
+        M32[e] = make_float2((float)v[u].x, (float)v[u].y);
       }
     }
   }
@@ -450,7 +380,7 @@ __device__ void assemble_fp64(const NodeCtx& cx, double2* __restrict__ T, float2
     const size_t e = (size_t)i * n + i;
     const double2 t = cadd(T[e], id);
     T[e] = t;
-    M32[at(e)] = make_float2((float)t.x, (float)t.y);
+    M32[e] = make_float2((float)t.x, (float)t.y);
   }
   gsync();
 }
@@ -461,10 +391,9 @@ __device__ void assemble_fp64(const NodeCtx& cx, double2* __restrict__ T, float2
 __device__ void round_bie(const double2* __restrict__ T, float2* __restrict__ M32, int n, bool column_only,
                           float2* __restrict__ stage, int stage_elems) {
   const size_t nn = (size_t)n * n;
-  const At32 at(n);
   if (!column_only) {
 #pragma unroll 4
-    for (size_t e = gtid(); e < nn; e += THREADS) M32[at(e)] = make_float2((float)T[e].x, (float)T[e].y);
+    for (size_t e = gtid(); e < nn; e += THREADS) M32[e] = make_float2((float)T[e].x, (float)T[e].y);
     return;
   }
   const bool fits = n <= stage_elems;
@@ -475,7 +404,7 @@ __device__ void round_bie(const double2* __restrict__ T, float2* __restrict__ M3
   for (int col = warp; col < n; col += THREADS / 32)
     for (int row = lane; row < n; row += 32) {
       const int m = row >= col ? row - col : row - col + n;
-      M32[(size_t)col * mixed_order(n) + row] = fits ? stage[m] : make_float2((float)T[m].x, (float)T[m].y);
+      M32[(size_t)col * n + row] = fits ? stage[m] : make_float2((float)T[m].x, (float)T[m].y);
     }
 }
 
@@ -488,7 +417,6 @@ __device__ void round_bie(const double2* __restrict__ T, float2* __restrict__ M3
 __device__ void assemble32(const NodeCtx& cx, float2* __restrict__ M32) {
   const ProblemDev& P = cx.P;
   const int n = P.n;
-  const At32 at(n);
   const size_t nn = (size_t)n * n;
   constexpr int U = 8;
   const float2 fid = cx.fid32;
@@ -516,13 +444,13 @@ __device__ void assemble32(const NodeCtx& cx, float2* __restrict__ M32) {
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       const size_t e = e0 + (size_t)u * THREADS;
-      if (e < nn) M32[at(e)] = v[u];
+      if (e < nn) M32[e] = v[u];
     }
   }
   if (fid.x != 0.f || fid.y != 0.f) {
     gsync();
     for (int i = gtid(); i < n; i += THREADS) {
-      float2& d = M32[(size_t)i * mixed_order(n) + i];
+      float2& d = M32[(size_t)i * n + i];
       d.x += fid.x;
       d.y += fid.y;
     }
@@ -592,7 +520,7 @@ __device__ __forceinline__ int next_index(const MixedArgs& a, int counter, int t
 }
 
 constexpr uint32_t TMEM_FACTOR = 256;  // columns per CTA, two CTAs per SM
-static_assert(tcu::TMEM_COLS <= TMEM_FACTOR && tcu::WIDE_COLS <= TMEM_FACTOR && lu32::OUTER_SCRATCH <= tcu::STAGE_BYTES && 2 * tcb::ACC_COLS <= TMEM_FACTOR, "TMEM columns");
+static_assert(tcu::TMEM_COLS <= TMEM_FACTOR && 2 * tcb::ACC_COLS <= TMEM_FACTOR, "TMEM columns");
 
 // Steps 1-2: node after node, each into its own slot.
 // BIE: the instantiation for launches with a boundary-integral term (bie.cuh); the
@@ -609,16 +537,13 @@ __global__ void __launch_bounds__(THREADS, 2) k_mixed_factor(MixedArgs a, int sc
   if (tid == 0) {
     tcu::mbar_init(&sm.mbar_tc[0]);
     tcu::mbar_init(&sm.mbar_tc[1]);
-    tcu::wide_init(sm.wide);
     sm.tc_bad = 0;
   }
   tcu::fence_async_smem();
   tcu::fence_before();
   __syncthreads();
   tcu::fence_after();
-  tcu::Ctx cx{smem_raw + kFactorHead, sm.mbar_tc,         TC ? sm.tmem_base : 0u, {0u, 0u},
-              &sm.tc_bad,             a.tc_wait_cycles, &sm.wide,               0u,
-              nullptr,                0};
+  tcu::Ctx cx{smem_raw + kFactorHead, sm.mbar_tc, TC ? sm.tmem_base : 0u, {0u, 0u}, &sm.tc_bad, a.tc_wait_cycles};
   for (;;) {
     const int q = next_index(a, MIXED_CTL_FACTOR, a.count, c);
     if (q < 0) break;
@@ -628,9 +553,8 @@ __global__ void __launch_bounds__(THREADS, 2) k_mixed_factor(MixedArgs a, int sc
     RegionDev rg;
     load_node<true>(a, q, c, rg, it);
     const ProblemDev& P = c.P;
-    const int n = P.n, l = P.l, np = mixed_order(n);
-    const At32 at(n);
-    const size_t npp = (size_t)np * np, nl = (size_t)n * l;
+    const int n = P.n, l = P.l, ncols = n + l;
+    const size_t nn = (size_t)n * n, nl = (size_t)n * l;
     pc.mark(PH_SETUP);
     // T(z_j) in FP64 for the residuals on the FP64 pipe, and rounded; T(z_j)^H likewise
     if (BIE && P.bie && !rg.herm)
@@ -640,33 +564,22 @@ __global__ void __launch_bounds__(THREADS, 2) k_mixed_factor(MixedArgs a, int sc
       assemble_fp64(c, a.t64 + (size_t)q * a.t64_stride, M32, rg.herm != 0);
     else
       assemble32(c, M32);
-    for (size_t e = tid; e < nl; e += THREADS) M32[npp + at(e)] = make_float2((float)P.V[e].x, (float)P.V[e].y);
-    if (np > n) {  // the identity's last column and row
-      for (int i = tid; i < np; i += THREADS) M32[(size_t)n * np + i] = make_float2(i == n ? 1.f : 0.f, 0.f);
-      for (int c = tid; c < np + l; c += THREADS)
-        if (c != n) M32[(size_t)c * np + n] = make_float2(0.f, 0.f);
-    }
+    for (size_t e = tid; e < nl; e += THREADS) M32[nn + e] = make_float2((float)P.V[e].x, (float)P.V[e].y);
     gsync();
     if (rg.border > 0) {  // the bordered matrix of a certificate: column s of T(z_j) replaced
       const double2* bc = a.border + rg.v_off;
-      float2* col = M32 + (size_t)(rg.border - 1) * np;
+      float2* col = M32 + (size_t)(rg.border - 1) * n;
       for (int i = tid; i < n; i += THREADS) col[i] = make_float2((float)bc[i].x, (float)bc[i].y);
       gsync();
     }
     pc.mark(PH_ASSEMBLE);
     const int bad_before = sm.tc_bad;
     int* lists = reinterpret_cast<int*>(slot + mixed_lists_offset(n, l));
-    int* piv = lists + (size_t)((n + NB - 1) / NB) * SWAP_LIST_INTS;  // (an odd n fills no panel: the same count for np)
-    float2* rinv = reinterpret_cast<float2*>(slot + mixed_rinv_offset(n, l));
-    const int tc = TC ? rg.lu_tc : 0;
-    cx.maps = a.maps ? a.maps + (size_t)rg.prob * 2 * tcu::MAP_BYTES : nullptr;
-    cx.slot = q;
-    const int outer = tc == 1 && cx.maps && np > kOuterMinN && np <= lu32::ROWS_MAX ? lu32::OB / NB : 1;
-    const int info = cta_lu32(M32, np, np + l, piv, lists, rinv, sm.lu32, sm.os, cx, tc, outer, pc);
+    int* piv = lists + (size_t)((n + NB - 1) / NB) * SWAP_LIST_INTS;
+    const int info = cta_lu32(M32, n, ncols, piv, lists, sm.lu32, cx, TC ? rg.lu_tc : 0, pc);
     if (tid == 0) {
       MixedState st{};
       st.info = info;
-      st.outer = outer;
       st.lost = sm.tc_bad != bad_before ? MIXED_LOST_LU : 0;
       // a boundary-integral node's residual takes the whole of T(z_j) as its one dense term
       st.id = BIE && P.bie ? make_double2(0.0, 0.0) : c.fid;
@@ -718,14 +631,12 @@ __global__ void __launch_bounds__(THREADS, 3) k_mixed_solve(MixedArgs a, int sw,
     RegionDev rg;
     load_node<RES64>(a, q, c, rg, it);
     const ProblemDev& P = c.P;
-    const int n = P.n, l = P.l, np = mixed_order(n);
-    const At32 at(n);
-    const size_t nn = (size_t)n * n, nl = (size_t)n * l, npp = (size_t)np * np, npl = (size_t)np * l;
+    const int n = P.n, l = P.l;
+    const size_t nn = (size_t)n * n, nl = (size_t)n * l;
     double2* R = reinterpret_cast<double2*>(slot + mixed_residual_offset(n, l));
     const int* lists = reinterpret_cast<const int*>(slot + mixed_lists_offset(n, l));
-    const float2* rinv = reinterpret_cast<const float2*>(slot + mixed_rinv_offset(n, l));
-    float2* Y = npl * sizeof(float2) <= (size_t)y_bytes ? reinterpret_cast<float2*>(smem_raw + sizeof(SolveSmem<RES64>))
-                                                        : M32 + npp;
+    float2* Y = nl * sizeof(float2) <= (size_t)y_bytes ? reinterpret_cast<float2*>(smem_raw + sizeof(SolveSmem<RES64>))
+                                                       : M32 + nn;
     double2* X = a.X + rg.x_off + (size_t)it.j * nl;
     MixedState st = a.state[q];
     const bool oz = mixed_node_oz(a, P, rg);
@@ -734,13 +645,13 @@ __global__ void __launch_bounds__(THREADS, 3) k_mixed_solve(MixedArgs a, int sw,
       if (ok) {
         // X_0 = U^-1 (L^-1 P V) in FP32 (the LU eliminated V)
         double xm = 0.0;
-        if (Y != M32 + npp) {
-          for (size_t e = tid; e < npl; e += THREADS) Y[e] = M32[npp + e];
+        if (Y != M32 + nn) {
+          for (size_t e = tid; e < nl; e += THREADS) Y[e] = M32[nn + e];
           gsync();
         }
-        lu32::back(M32, Y, np, l, rinv, sm.s);
+        lu32::back(M32, Y, n, l, sm.s);
         for (size_t e = tid; e < nl; e += THREADS) {
-          const float2 y = Y[at(e)];
+          const float2 y = Y[e];
           const double2 x = make_double2((double)y.x, (double)y.y);
           X[e] = x;
           xm = fmax(xm, fmax(fabs(x.x), fabs(x.y)));
@@ -791,16 +702,14 @@ __global__ void __launch_bounds__(THREADS, 3) k_mixed_solve(MixedArgs a, int sw,
         // right-hand side R / |R|max; the forward solve applies the row interchanges
         for (size_t e = tid; e < nl; e += THREADS) {
           const double2 rv = R[e];
-          Y[at(e)] = make_float2((float)(rv.x * inv), (float)(rv.y * inv));
+          Y[e] = make_float2((float)(rv.x * inv), (float)(rv.y * inv));
         }
-        if (np > n)
-          for (int c = tid; c < l; c += THREADS) Y[(size_t)c * np + n] = make_float2(0.f, 0.f);
         gsync();
-        lu32::forward(M32, Y, np, l, sm.s, lists, st.outer);
-        lu32::back(M32, Y, np, l, rinv, sm.s);
+        lu32::forward(M32, Y, n, l, sm.s, lists);
+        lu32::back(M32, Y, n, l, sm.s);
         double dm = 0.0, xmx = 0.0;
         for (size_t e = tid; e < nl; e += THREADS) {
-          const float2 d = Y[at(e)];
+          const float2 d = Y[e];
           double2 x = X[e];
           const double dx = (double)d.x * rm, dy = (double)d.y * rm;
           x.x += dx;
@@ -895,10 +804,10 @@ __global__ void __launch_bounds__(THREADS, 2) k_mixed_fallback(MixedArgs a, size
 }  // namespace
 
 // Slot layout: [FP32 matrix n x (n + l)] [FP64 residual n x l] [the panels' row
-// permutations, SWAP_LIST_INTS ints each] [pivots] [their reciprocals, complex64].
-static_assert(SWAP_LIST_INTS == MIXED_LIST_INTS && NB == MIXED_NB, "slot layout");
+// permutations, SWAP_LIST_INTS ints each] [pivots].
 size_t mixed_slot_bytes(int n, int l) {
-  return (mixed_rinv_offset(n, l) + (size_t)mixed_order(n) * sizeof(float2) + 255) & ~(size_t)255;
+  const size_t ints = (size_t)((n + NB - 1) / NB) * SWAP_LIST_INTS + n;
+  return (mixed_lists_offset(n, l) + ints * sizeof(int) + 255) & ~(size_t)255;
 }
 // Bytes a slot area needs at the least: one FP64 fallback.
 size_t mixed_fallback_bytes(int n, int l) {
@@ -912,7 +821,7 @@ const void* factor_kernel(bool bie, bool tc) {
 }
 }  // namespace
 
-static_assert(2 * (kFactorHead + kTcStage + 1024) <= 228 * 1024, "two CTAs per SM");
+static_assert(2 * (kFactorHead + tcu::STAGE_BYTES + 1024) <= 228 * 1024, "two CTAs per SM");
 static_assert(lu32::panel_scratch_bytes(lu32::ROWS_MAX) <= tcu::STAGE_BYTES && lu32::panel_scratch_bytes(1024) <= tcu::STAGE_BYTES &&
                   lu32::panel_scratch_bytes(256) <= tcu::STAGE_BYTES && lu32::panel_scratch_bytes(512) <= tcu::STAGE_BYTES,
               "a panel fits the operand stage");
@@ -921,7 +830,7 @@ static_assert(3 * (sizeof(SolveSmem<false>) + kSolveYBytes + 1024) <= 228 * 1024
 cudaError_t prepare_factor_mixed() {
   for (int i = 0; i < 4; ++i) {
     cudaError_t e = cudaFuncSetAttribute(factor_kernel(i & 1, i & 2), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)(kFactorHead + kTcStage));
+                                         (int)(kFactorHead + tcu::STAGE_BYTES));
     if (e != cudaSuccess) return e;
   }
   cudaError_t e = cudaFuncSetAttribute(k_mixed_solve<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -949,41 +858,6 @@ cudaError_t round_coefficients_c64(const double2* src, float2* dst, size_t count
   return cudaGetLastError();
 }
 
-static_assert(sizeof(CUtensorMap) == tcu::MAP_BYTES, "a tensor map's size");
-size_t mixed_map_bytes() { return 2 * tcu::MAP_BYTES; }
-bool mixed_outer(int n) { return mixed_order(n) > kOuterMinN && mixed_order(n) <= lu32::ROWS_MAX; }
-
-// The tensor maps of a chunk's matrices of one problem (order n, l probe columns; the slots at
-// work) for the wide updates: blocks of L21, then of U12. False when the driver has no encoder.
-bool mixed_make_maps(char* work, size_t slot_bytes, int slots, int n, int l, void* out) {
-  using Encode = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
-                              const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
-                              CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-  static const Encode encode = [] {
-    void* f = nullptr;
-    cudaDriverEntryPointQueryResult r;
-    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &f, 12000, cudaEnableDefault, &r) != cudaSuccess ||
-        r != cudaDriverEntryPointSuccess)
-      f = nullptr;
-    return reinterpret_cast<Encode>(f);
-  }();
-  if (!encode) return false;
-  const cuuint64_t np = (cuuint64_t)mixed_order(n);
-  const cuuint64_t dims[3] = {np, np + (cuuint64_t)l, (cuuint64_t)slots};
-  const cuuint64_t strides[2] = {np * sizeof(float2), slot_bytes};
-  const cuuint32_t one[3] = {1, 1, 1};
-  const cuuint32_t box[2][3] = {{tcu::TM, tcu::WK, 1}, {tcu::WK, tcu::WN, 1}};
-  for (int i = 0; i < 2; ++i) {
-    CUtensorMap m;  // the encoder wants a 64-byte boundary
-    if (encode(&m, CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 3, work, dims, strides, box[i], one, CU_TENSOR_MAP_INTERLEAVE_NONE,
-               CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-      return false;
-    memcpy(static_cast<char*>(out) + i * sizeof(m), &m, sizeof(m));
-  }
-  return true;
-}
-
 // One chunk's kernels in order (no synchronisation, so that they can be captured);
 // prepare_factor_mixed() must have set the shared-memory limits. *launched: kernels.
 cudaError_t launch_factor_solve_mixed(const MixedArgs& a, int sms, cudaStream_t s, int* launched) {
@@ -997,7 +871,7 @@ cudaError_t launch_factor_solve_mixed(const MixedArgs& a, int sms, cudaStream_t 
     if (e != cudaSuccess) return e;
   }
   {
-    const int scratch = (int)factor_scratch_bytes(mixed_order(a.max_n), a.tc != 0);
+    const int scratch = (int)factor_scratch_bytes(a.max_n, a.tc != 0);
     const size_t smem = kFactorHead + scratch;
     const int g = grid(2);
     if (a.bie && a.tc) k_mixed_factor<true, true><<<g, THREADS, smem, s>>>(a, scratch);
@@ -1013,7 +887,7 @@ cudaError_t launch_factor_solve_mixed(const MixedArgs& a, int sms, cudaStream_t 
       *launched += 2;
     }
     // (the FP64-pipe residual's tiles leave no room for the right-hand sides)
-    const size_t nl = (size_t)mixed_order(a.max_n) * a.max_l * sizeof(float2);
+    const size_t nl = (size_t)a.max_n * a.max_l * sizeof(float2);
     const int y = !a.res64 && nl <= kSolveYBytes ? (int)nl : 0;
     if (a.res64) k_mixed_solve<true><<<grid(3), THREADS, sizeof(SolveSmem<true>), s>>>(a, sw, 0);
     else k_mixed_solve<false><<<grid(3), THREADS, sizeof(SolveSmem<false>) + y, s>>>(a, sw, y);

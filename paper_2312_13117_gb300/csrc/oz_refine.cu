@@ -15,10 +15,10 @@
 //                 the digits of f_d X (14 KB per group and 32 inner indices) two deep;
 //   warp 1        MMAs into all 512 TMEM columns: 8 digit orders x 64 columns;
 //   warps 4-19    drains, after every 256 inner indices. A warp owns 32 rows and one
-//                 column group. The accumulators are integers below 2^24, and so are
-//                 exact as int64 sums of the orders' upper and lower half over all
-//                 inner indices; FP64 arithmetic (2 operations per SM and clock) is left
-//                 for one update of R per term.
+//                 column group, and forms what ozk::residual forms, in the same order and
+//                 to the same bits: Horner's rule over the orders in double-float, then
+//                 one FP64 update of R (kept in registers) per 256 inner indices, which
+//                 overlaps the next products.
 // A boundary-integral node has a matrix of its own: its tiles hold its own groups only,
 // and the digits are those of T(z_j) (bie_nodes.cu).
 // A wait for operands is bounded by tc_wait_cycles: when one runs out the CTA's nodes
@@ -115,7 +115,7 @@ __global__ void __launch_bounds__(DIGIT_THREADS) k_oz_digits(MixedArgs a, int sw
         double m = 0.0;
         if (c < l)
           for (int j = tid / CG; j < n; j += DIGIT_THREADS / CG) {
-            const double2 y = cmul(f, X[(size_t)c * n + j]);
+            const double2 y = y_product(f, X[(size_t)c * n + j]);
             m = fmax(m, fmax(fabs(y.x), fabs(y.y)));
           }
         for (int o = CG; o < 32; o <<= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
@@ -133,14 +133,16 @@ __global__ void __launch_bounds__(DIGIT_THREADS) k_oz_digits(MixedArgs a, int sw
       unsigned char* dst = a.ysl + (size_t)q * a.ysl_stride + (size_t)(dd * ncg + cg) * kcn * GROUP_STAGE;
       for (int task = tid; task < CG * kcn * (KC / 8); task += DIGIT_THREADS) {
         const int cc = task & (CG - 1), j0 = (task / CG) * 8, c = cg * CG + cc;
-        const double up = pow2(DIGIT_SHIFT - g[cc]);
+        const int shift = DIGIT_SHIFT - g[cc];
+        const bool normal = shift >= -1022 && shift <= 1023;  // 2^shift is a normal number
+        const double up = normal ? pow2(shift) : 0.0;
         long long Nr[8], Ni[8];
 #pragma unroll
         for (int u = 0; u < 8; ++u) {
           double2 y = make_double2(0.0, 0.0);
-          if (c < l && j0 + u < n) y = cmul(f, X[(size_t)c * n + j0 + u]);
-          Nr[u] = __double2ll_rn(y.x * up);
-          Ni[u] = __double2ll_rn(y.y * up);
+          if (c < l && j0 + u < n) y = y_product(f, X[(size_t)c * n + j0 + u]);
+          Nr[u] = __double2ll_rn(normal ? y.x * up : scalbn(y.x, shift));
+          Ni[u] = __double2ll_rn(normal ? y.y * up : scalbn(y.y, shift));
         }
         unsigned char* st = dst + (size_t)(j0 / KC) * GROUP_STAGE;
 #pragma unroll 1
@@ -370,61 +372,69 @@ __device__ void drain_role(const MixedArgs& a, int sw, GemmSmem& sm) {
     double2* R = reinterpret_cast<double2*>(a.work + (size_t)q * a.slot_bytes + mixed_residual_offset(n, l)) +
                  (size_t)cg * CG * n + row;
     const int cols = min(CG, l - cg * CG);
-    for (int dd = 0; dd < terms_of(P); ++dd) {
-      long long hi[2 * CG], lo[2 * CG];  // orders 2-5 and 6-9: hi 2^28 + lo
+    double r[2 * CG];  // R's columns of the group: real parts, imaginary parts
+    if (mine && row < n) {
+      const double2 id = a.state[q].id;
+      const bool has_id = id.x != 0.0 || id.y != 0.0;
 #pragma unroll
-      for (int c = 0; c < 2 * CG; ++c) hi[c] = lo[c] = 0;
+      for (int c = 0; c < CG; ++c) {
+        double2 v = make_double2(0.0, 0.0);
+        if (c < cols) {
+          v = P.V[(size_t)(cg * CG + c) * n + row];
+          if (has_id) cfms(v, id, X[(size_t)c * n]);
+        }
+        r[c] = v.x;
+        r[CG + c] = v.y;
+      }
+    }
+    for (int dd = 0; dd < terms_of(P); ++dd) {
+      // the product's scale in each column, 2^(row exponent + column exponent - 61)
+      int ge[CG];
+      int er = 0;
+      if (mine && row < n) {
+        const int32_t* ex = P.bie ? a.texp + (size_t)q * a.texp_stride : P.Aexp;
+        er = ex[((size_t)dd * rbn + t.rb) * TM + 32 * quad + lane];
+#pragma unroll
+        for (int c = 0; c < CG; ++c)
+          ge[c] = a.gexp[(size_t)q * a.gexp_stride + (dd * ncg + cg) * CG + c] + er - DRAIN_SCALE;
+      }
       for (int kc0 = 0; kc0 < kcn; kc0 += KD / KC) {
         const bool ok = wait_or_bad(&sm.acc_full, blk & 1u, a.handoff_wait_cycles, &sm.bad, LOST_HANDOFF);
         if (!__all_sync(0xffffffffu, ok)) return;  // sm.bad is set
         ++blk;
         tcu::fence_after();
+        DF H[2 * CG];
         if (mine) {
+          // Horner's rule over the orders in double-float, as ozk::residual's
 #pragma unroll
-          for (int h = 0; h < 4; ++h) {
+          for (int c = 0; c < 2 * CG; ++c) H[c] = DF{0.f, 0.f};
+#pragma unroll 1
+          for (int h = 0; h < NQ; ++h) {
             uint32_t v[16];
             tmem_ld16(base + (uint32_t)(h * 16 * MAXG), v);
 #pragma unroll
             for (int c = 0; c < 2 * CG; ++c)
-              hi[c] += (long long)__float2int_rn(__uint_as_float(v[c])) * (1 << (21 - 7 * h));
-          }
-#pragma unroll
-          for (int h = 0; h < 4; ++h) {
-            uint32_t v[16];
-            tmem_ld16(base + (uint32_t)((4 + h) * 16 * MAXG), v);
-#pragma unroll
-            for (int c = 0; c < 2 * CG; ++c)
-              lo[c] += (long long)__float2int_rn(__uint_as_float(v[c])) * (1 << (21 - 7 * h));
+              H[c] = df_add_f(DF{H[c].hi * 128.f, H[c].lo * 128.f}, __uint_as_float(v[c]));
           }
         }
         tcu::fence_before();
         __syncwarp();
         if (lane == 0) arrive(&sm.acc_empty);
-      }
-      if (mine && row < n) {
-        const int32_t* ex = P.bie ? a.texp + (size_t)q * a.texp_stride : P.Aexp;
-        const int er = ex[((size_t)dd * rbn + t.rb) * TM + 32 * quad + lane];
-        const int* ge = a.gexp + (size_t)q * a.gexp_stride + (dd * ncg + cg) * CG;
-        const double2 id = a.state[q].id;
-        const bool has_id = id.x != 0.0 || id.y != 0.0;
+        // (the FP64 part while the next block's products run)
+        if (mine && row < n) {
 #pragma unroll
-        for (int c = 0; c < CG; ++c) {
-          if (c < cols) {
-            double2 r;
-            if (dd == 0) {
-              r = P.V[(size_t)(cg * CG + c) * n + row];
-              if (has_id) cfms(r, id, X[(size_t)c * n]);
-            } else {
-              r = R[(size_t)c * n];
-            }
-            const int e = er + ge[c] - DRAIN_SCALE;
-            const double s1 = -pow2(e), s2 = -pow2(e + 28);
-            r.x = fma(s2, (double)hi[c], fma(s1, (double)lo[c], r.x));
-            r.y = fma(s2, (double)hi[CG + c], fma(s1, (double)lo[CG + c], r.y));
-            R[(size_t)c * n] = r;
+          for (int c = 0; c < CG; ++c) {
+            const double sc = pow2(ge[c]);
+            r[c] = fma(-sc, (double)H[c].hi, fma(-sc, (double)H[c].lo, r[c]));
+            r[CG + c] = fma(-sc, (double)H[CG + c].hi, fma(-sc, (double)H[CG + c].lo, r[CG + c]));
           }
         }
       }
+    }
+    if (mine && row < n) {
+#pragma unroll
+      for (int c = 0; c < CG; ++c)
+        if (c < cols) R[(size_t)c * n] = make_double2(r[c], r[CG + c]);
     }
   }
 }

@@ -149,6 +149,12 @@ __device__ __forceinline__ int exponent_of(double m) {
   return e;
 }
 
+// An entry of f X. Which products are fused is fixed, so that every kernel that makes digits of
+// f X takes the same numbers.
+__device__ __forceinline__ double2 y_product(double2 f, double2 x) {
+  return make_double2(fma(f.x, x.x, -__dmul_rn(f.y, x.y)), fma(f.y, x.x, __dmul_rn(f.x, x.y)));
+}
+
 // Digit t (0 = most significant) when the digits are taken from the least
 // significant end: for t > 0 the balanced remainder of N modulo 128 (N becomes
 // the quotient), for t = 0 what is left of N.
@@ -214,7 +220,7 @@ __device__ inline void y_digits(const double2* __restrict__ X, int n, int l, int
     if (c0 + c < l) {
       const double2* xc = X + (size_t)(c0 + c) * n;
       for (int j = r0; j < n; j += THREADS_PER_GROUP / LC) {
-        const double2 y = cmul(f, xc[j]);
+        const double2 y = y_product(f, xc[j]);
         m = fmax(m, fmax(fabs(y.x), fabs(y.y)));
       }
     }
@@ -239,7 +245,7 @@ __device__ inline void y_digits(const double2* __restrict__ X, int n, int l, int
     for (int u = 0; u < 8; ++u) {
       const int j = j0 + u;
       double2 y = make_double2(0.0, 0.0);
-      if (col_ok && j < n) y = cmul(f, X[(size_t)(c0 + c) * n + j]);
+      if (col_ok && j < n) y = y_product(f, X[(size_t)(c0 + c) * n + j]);
       Nr[u] = __double2ll_rn(scalbn(y.x, DIGIT_SHIFT - e));
       Ni[u] = __double2ll_rn(scalbn(y.y, DIGIT_SHIFT - e));
     }

@@ -253,7 +253,7 @@ struct MixedState {
   int32_t info;    // 0, or 1 + first zero-pivot column of the FP32 LU
   int32_t sweeps;  // refinement sweeps run
   int32_t lost;    // MIXED_LOST_*: a tensor-core wait ran out
-  int32_t outer;   // panels per block of the LU's row interchanges
+  int32_t pad;
 };
 constexpr int MIXED_LOST_LU = 1, MIXED_LOST_RESIDUAL = 2;
 // ctl: work counters, active nodes per sweep, then the column groups per sweep and problem
@@ -302,7 +302,6 @@ struct MixedArgs {
   int* units;          // [sweep & 1][unit_cap]: their groups of 8 solution columns, 8 slot + group,
   int unit_cap;        // those of problem p from ubase[p] on
   const int* ubase;
-  const char* maps;            // per problem, tensor maps of its slots (mixed_make_maps); NULL: none
   const double2* border;       // the replacement columns of bordered nodes
   unsigned long long* phase;   // NULL, or PMCIM_PHASES clock64 counters per CTA
   int32_t* err;                // set to 1 when a wait between a kernel's warp groups ran out
@@ -378,28 +377,15 @@ int factor_slots_fp64(int n, int l);
 int resident_ctas(int n, int l);  // CTAs per SM, 0 when a node does not fit
 cudaError_t prepare_factor_resident();
 cudaError_t launch_factor_solve_resident(const NodeArgs& a, int max_l, cudaStream_t s);
-// The precision forms factor a matrix of even order, so that its columns lie on 16-byte
-// boundaries (bulk copies): an odd n gets one more row and column, those of the identity.
-__host__ __device__ inline int mixed_order(int n) { return (n + 1) & ~1; }
 __host__ __device__ inline size_t mixed_residual_offset(int n, int l) {
-  return (((size_t)mixed_order(n) * (mixed_order(n) + l) * 8) + 255) & ~(size_t)255;
+  return (((size_t)n * (n + l) * 8) + 255) & ~(size_t)255;
 }
-// the LU panels' row permutations (ints), after the FP64 residual
+// the LU panels' row permutations (ints), after the FP64 residual; then the pivots
 __host__ __device__ inline size_t mixed_lists_offset(int n, int l) {
   return (mixed_residual_offset(n, l) + (size_t)n * l * 16 + 255) & ~(size_t)255;
 }
-// then the pivots and their reciprocals
-constexpr int MIXED_NB = 32, MIXED_LIST_INTS = 1 + 4 * MIXED_NB;
-__host__ __device__ inline size_t mixed_rinv_offset(int n, int l) {
-  return (mixed_lists_offset(n, l) +
-          ((size_t)((n + MIXED_NB - 1) / MIXED_NB) * MIXED_LIST_INTS + mixed_order(n)) * sizeof(int) + 15) &
-         ~(size_t)15;
-}
 size_t mixed_slot_bytes(int n, int l);
 size_t mixed_fallback_bytes(int n, int l);
-size_t mixed_map_bytes();  // tensor maps of one problem
-bool mixed_outer(int n);   // an order that needs them: factored in outer blocks (3xTF32)
-bool mixed_make_maps(char* work, size_t slot_bytes, int slots, int n, int l, void* out);
 
 struct LevelArgs {
   const ProblemDev* probs;
