@@ -5,8 +5,8 @@
 // columns fit an SM's shared memory (lu_resident.cuh): one CTA per node, as many
 // CTAs per SM as fit. The FP64 unit (2 multiply-adds per SM and clock) bounds
 // these nodes: n = 100, l = 10 needs 0.42 ms of one SM. Measured on whole calls:
-// 3600 nodes of n = 100, l = 10 (indicator) 19.0 ms against 47.8 ms through the
-// blocked kernel, 512 nodes of n = 64, l = 8 (moments) 1.26 against 3.47 ms.
+// 3600 nodes of n = 100, l = 10 (indicator) 20.8 ms against 47.8 ms through the
+// blocked kernel, 512 nodes of n = 64, l = 8 (moments) 1.23 against 3.47 ms.
 #include "lu_resident.cuh"
 
 namespace {
@@ -39,18 +39,18 @@ __global__ void __launch_bounds__(512) k_factor_solve_resident(NodeArgs a) {
     __syncthreads();
     const ProblemDev& P = sm.P;
     const int n = P.n, l = P.l, ncols = n + l, ld = lead(n);
-    double2* rinv = M + (size_t)ld * ncols;
-    int* piv = reinterpret_cast<int*>(rinv + n);
+    double2* divisor = M + (size_t)ld * ncols;
+    int* piv = reinterpret_cast<int*>(divisor + n);
     double2 z, w;
     node_weight(rg.cre, rg.cim, rg.r, rg.N, it.j, &z, &w);
     if (tid < P.K) sm.fz[tid] = eval_f(P.term[tid], z);
-    // a circulant boundary-integral term's n distinct entries, in the reciprocals' place
+    // a circulant boundary-integral term's n distinct entries, in the divisors' place
     const bool use_circ = BIE && P.bie_circ;
     if (BIE) {
       if (tid == 0) sm.wave = bie::wave_of(z);
       __syncthreads();
       if (use_circ)
-        for (int m = tid; m < n; m += blockDim.x) rinv[m] = bie::dlp_entry(P.bie, n, m, 0, sm.wave);
+        for (int m = tid; m < n; m += blockDim.x) divisor[m] = bie::dlp_entry(P.bie, n, m, 0, sm.wave);
     }
     __syncthreads();
     const size_t nn = (size_t)n * n;
@@ -61,7 +61,7 @@ __global__ void __launch_bounds__(512) k_factor_solve_resident(NodeArgs a) {
           const TermDesc& t = P.term[k];
           if (t.dense) cfma(v, sm.fz[k], P.A[(size_t)t.mat_index * nn + (size_t)col * n + row]);
           else if (use_circ && t.kind == PMCIM_F_HELMHOLTZ_DLP)
-            cfma(v, t.id, rinv[row >= col ? row - col : row - col + n]);
+            cfma(v, t.id, divisor[row >= col ? row - col : row - col + n]);
           else if (row == col && t.kind != PMCIM_F_HELMHOLTZ_DLP) cfma(v, sm.fz[k], t.id);
         }
         M[(size_t)col * ld + row] = v;
@@ -74,8 +74,8 @@ __global__ void __launch_bounds__(512) k_factor_solve_resident(NodeArgs a) {
     for (int c = warp; c < l; c += nwarp)
       for (int row = lane; row < n; row += 32) M[(size_t)(n + c) * ld + row] = P.V[(size_t)c * n + row];
     __syncthreads();
-    factor(M, n, ncols, ld, piv, rinv, sm.ctl);
-    back(M, n, l, ld, rinv);
+    factor(M, n, ncols, ld, piv, divisor, sm.ctl);
+    back(M, n, l, ld, divisor);
     __syncthreads();
     double2* Xo = a.X + rg.x_off + (size_t)it.j * n * l;
     for (int c = warp; c < l; c += nwarp)
@@ -92,7 +92,7 @@ constexpr size_t kSmBytes = 227 * 1024;  // shared memory of an SM that CTAs can
 // CTAs per SM for an FP64 node of this size, 0 when it does not fit. An SM gives
 // each CTA 1 KB more than it asks for.
 int resident_ctas(int n, int l) {
-  const size_t b = kHeadBytes + node_bytes(n, l, sizeof(double2));
+  const size_t b = kHeadBytes + node_bytes(n, l);
   if (b > kSmBytes) return 0;
   const size_t k = (kSmBytes + 1024) / (b + 1024);
   return (int)(k < 8 ? k : 8);
@@ -111,7 +111,7 @@ cudaError_t launch_factor_solve_resident(const NodeArgs& a, int max_l, cudaStrea
   if (a.n_items <= 0) return cudaSuccess;
   const int ctas = resident_ctas(a.max_n, max_l);
   if (ctas < 1) return cudaErrorInvalidValue;
-  const size_t smem = kHeadBytes + node_bytes(a.max_n, max_l, sizeof(double2));
+  const size_t smem = kHeadBytes + node_bytes(a.max_n, max_l);
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);

@@ -17,7 +17,7 @@ constexpr int SL = 16;  // largest l
 struct SmallSmem {  // then WARPS matrices of `rows` rows of `ldc` entries
   ProblemDev P[WARPS];
   double2 fz[WARPS][PMCIM_MAX_TERMS];
-  double2 rinv[WARPS][SN];  // the pivots' reciprocals
+  double2 divisor[WARPS][SN];  // Smith's ratio and denominator of the pivots
 };
 constexpr size_t kSmallHead = (sizeof(SmallSmem) + 15) & ~size_t(15);
 // Row length for n + l columns: odd, so that eight rows lie in distinct banks.
@@ -30,7 +30,7 @@ __global__ void __launch_bounds__(WARPS * 32) k_factor_solve_small(NodeArgs a, i
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int lr = lane & 7, lc = lane >> 3;  // a tile of 8 rows x 4 columns
   double2* M = reinterpret_cast<double2*>(smem_raw + kSmallHead) + (size_t)w * matrix_elems;
-  double2* rinv = sm.rinv[w];
+  double2* divisor = sm.divisor[w];
   ProblemDev& P = sm.P[w];
   for (;;) {
     int idx = 0;
@@ -102,14 +102,15 @@ __global__ void __launch_bounds__(WARPS * 32) k_factor_solve_small(NodeArgs a, i
         }
       __syncwarp();
       const double2 pv = M[j * LDC + j];
-      const double2 rp = crecip(pv);  // not finite for a zero pivot, as a division by it would be
-      if (lane == 0) rinv[j] = rp;
+      const Smith sd(pv);
+      const double2 rp = sd.reciprocal();  // not finite for a zero pivot, as a division by it would be
+      if (lane == 0) divisor[j] = make_double2(sd.t, sd.d);
       if (pv.x == 0.0 && pv.y == 0.0) {
         if (info == 0) info = j + 1;
         __syncwarp();
         continue;
       }
-      if (lane > j && lane < n) M[lane * LDC + j] = cmul(M[lane * LDC + j], rp);
+      if (lane > j && lane < n) M[lane * LDC + j] = Smith::multiplier(M[lane * LDC + j], rp);
       __syncwarp();
       // rank-1 update in tiles of 8 rows x 4 columns: a lane without an element costs the FP64
       // unit as much as a busy one, and a row per lane leaves most idle in the end
@@ -133,7 +134,15 @@ __global__ void __launch_bounds__(WARPS * 32) k_factor_solve_small(NodeArgs a, i
     }
     // back substitution U X = Y on the l right-hand columns
     for (int j = n - 1; j >= 0; --j) {
-      if (lane < l) M[j * LDC + n + lane] = cmul(M[j * LDC + n + lane], rinv[j]);
+      // lanes c and c + 16: the real and the imaginary part of column c's quotient (l <= 16)
+      const int c = lane & (SL - 1), im = lane / SL;
+      double q = 0.0;
+      if (c < l) {
+        const double2 td = divisor[j];
+        q = Smith(M[j * LDC + j], td.x, td.y).part(M[j * LDC + n + c], im);
+      }
+      __syncwarp();
+      if (c < l) (im ? M[j * LDC + n + c].y : M[j * LDC + n + c].x) = q;
       __syncwarp();
       if (lane < j)
         for (int c = 0; c < l; ++c) cfms(M[lane * LDC + n + c], M[lane * LDC + j], M[j * LDC + n + c]);
@@ -166,9 +175,10 @@ cudaError_t prepare_factor_small() {
 
 // Launch only; prepare_factor_small() must have set the shared-memory limit. max_n, max_l: the
 // largest among the items, which set how many nodes an SM holds (n = 24, l = 1: 20; at the
-// largest sizes 8). The FP64 unit bounds the kernel: reciprocals kept for the back substitution
-// (a complex division is some 90 FP64 instructions of a warp) and the narrow update tiles took
-// 3072 nodes of n = 24, l = 1 from 0.75 to 0.57 ms.
+// largest sizes 8). The FP64 unit bounds the kernel: quotients that share the pivot's part of the
+// division (a complex division is some 90 FP64 instructions of a warp) and the narrow update tiles
+// took a call of 3072 nodes of n = 24, l = 1 from 1.26 to 0.83 ms, 0.80 with products by rounded
+// reciprocals, which are another rounding.
 cudaError_t launch_factor_solve_small(const NodeArgs& a, int max_n, int max_l, cudaStream_t s) {
   if (a.n_items <= 0) return cudaSuccess;
   int dev = 0, sms = 0;

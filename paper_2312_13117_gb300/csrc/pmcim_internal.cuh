@@ -69,6 +69,33 @@ __host__ __device__ __forceinline__ double2 cdiv(double2 a, double2 b) {
     return make_double2((a.x * t + a.y) / d, (a.y * t - a.x) / d);
   }
 }
+// Smith's division by one b in parts: what depends on b alone (the ratio t of its parts and the
+// denominator d) is formed once. The quotients are cdiv's and the multipliers those by crecip, to
+// the bit: there the denominator's and the quotients' products are rounded before they are added.
+struct Smith {
+  double t, d;
+  bool re;  // |Re b| >= |Im b|
+  __device__ __forceinline__ explicit Smith(double2 b) : re(fabs(b.x) >= fabs(b.y)) {
+    const double u = re ? b.x : b.y, v = re ? b.y : b.x;
+    t = v / u;
+    d = __dadd_rn(__dmul_rn(v, t), u);
+  }
+  __device__ __forceinline__ Smith(double2 b, double t_, double d_) : t(t_), d(d_), re(fabs(b.x) >= fabs(b.y)) {}
+  __device__ __forceinline__ double2 reciprocal() const {
+    const double u = 1.0 / d, v = t / d;
+    return re ? make_double2(u, -v) : make_double2(v, -u);
+  }
+  // a times that reciprocal
+  static __device__ __forceinline__ double2 multiplier(double2 a, double2 r) {
+    return make_double2(fma(a.x, r.x, -__dmul_rn(a.y, r.y)), fma(a.x, r.y, __dmul_rn(a.y, r.x)));
+  }
+  // the real (0) or the imaginary part (1) of a / b
+  __device__ __forceinline__ double part(double2 a, int im) const {
+    const double u = im ? (re ? a.y : -a.x) : (re ? a.x : a.y);
+    const double v = im ? (re ? -a.x : a.y) : (re ? a.y : a.x);
+    return __dadd_rn(__dmul_rn(v, t), u) / d;
+  }
+};
 __device__ __forceinline__ double l1abs(double2 a) { return fabs(a.x) + fabs(a.y); }
 
 // float2 counterparts used by the FP32 factorisation
