@@ -782,7 +782,7 @@ int run_level(Call& c, const std::vector<HostRegion>& regs, bool gate_top, bool 
   // ---- waves of whole disks whose solutions fit the wave buffer ----
   struct ResidentClass {
     size_t off, count;
-    int max_n, max_l;
+    size_t bytes;  // shared memory of the largest node (the largest n and l may lie in different ones)
   };
   // work counters of a wave: FP64, mixed, small, then one per class of resident nodes
   // (by CTAs per SM)
@@ -824,7 +824,7 @@ int run_level(Call& c, const std::vector<HostRegion>& regs, bool gate_top, bool 
       for (int g = g0; g < g1; ++g) {
         const ProblemDev& P = c.pd[regs[g].prob];
         const bool f64 = form_of(regs[g].prob) == PMCIM_PREC_FP64;
-        const int fit = f64 ? resident_ctas(P.n, P.l) : 0;
+        const int fit = f64 ? resident_ctas(resident_bytes(P.n, P.l)) : 0;
         std::vector<NodeItem>& dst = small_kernel_fits(P.n, P.l) ? itS
                                      : fit > 0 ? itF[fit - 1] : f64 ? it64 : it32;
         const bool re = reuse && reuse->src[g] >= 0;
@@ -865,10 +865,10 @@ int run_level(Call& c, const std::vector<HostRegion>& regs, bool gate_top, bool 
       for (std::vector<NodeItem>& f : itF) {
         if (f.empty()) continue;
         std::stable_sort(f.begin(), f.end(), by_n);
-        ResidentClass rc{items.size(), f.size(), 0, 0};
+        ResidentClass rc{items.size(), f.size(), 0};
         for (const NodeItem& it : f) {
-          rc.max_n = std::max(rc.max_n, c.pd[regs[it.region].prob].n);
-          rc.max_l = std::max(rc.max_l, c.pd[regs[it.region].prob].l);
+          const ProblemDev& P = c.pd[regs[it.region].prob];
+          rc.bytes = std::max(rc.bytes, resident_bytes(P.n, P.l));
         }
         items.insert(items.end(), f.begin(), f.end());
         wv.resident.push_back(rc);
@@ -1032,10 +1032,9 @@ int run_level(Call& c, const std::vector<HostRegion>& regs, bool gate_top, bool 
         const ResidentClass& rc = wv.resident[k];
         na.items = ws.items.as<NodeItem>() + rc.off;
         na.n_items = (int)rc.count;
-        na.max_n = rc.max_n;
         na.counter = ws.counters.as<int>() + kCounters * wi + 3 + k;
         prof_begin(PMCIM_K_FACTOR, s);
-        CU(launch_factor_solve_resident(na, rc.max_l, s));
+        CU(launch_factor_solve_resident(na, rc.bytes, s));
         prof_end(PMCIM_K_FACTOR, s);
       }
       LevelArgs lw = la;

@@ -89,12 +89,13 @@ constexpr size_t kSmBytes = 227 * 1024;  // shared memory of an SM that CTAs can
 
 }  // namespace
 
-// CTAs per SM for an FP64 node of this size, 0 when it does not fit. An SM gives
+size_t resident_bytes(int n, int l) { return kHeadBytes + node_bytes(n, l); }
+
+// CTAs per SM that ask for this much shared memory, 0 when one does not fit. An SM gives
 // each CTA 1 KB more than it asks for.
-int resident_ctas(int n, int l) {
-  const size_t b = kHeadBytes + node_bytes(n, l);
-  if (b > kSmBytes) return 0;
-  const size_t k = (kSmBytes + 1024) / (b + 1024);
+int resident_ctas(size_t bytes) {
+  if (bytes > kSmBytes) return 0;
+  const size_t k = (kSmBytes + 1024) / (bytes + 1024);
   return (int)(k < 8 ? k : 8);
 }
 
@@ -106,12 +107,11 @@ cudaError_t prepare_factor_resident() {
                               (int)kSmBytes);
 }
 
-// max_l: the largest l among the items (a.max_n: the largest n).
-cudaError_t launch_factor_solve_resident(const NodeArgs& a, int max_l, cudaStream_t s) {
+// bytes: the largest resident_bytes among the items.
+cudaError_t launch_factor_solve_resident(const NodeArgs& a, size_t bytes, cudaStream_t s) {
   if (a.n_items <= 0) return cudaSuccess;
-  const int ctas = resident_ctas(a.max_n, max_l);
+  const int ctas = resident_ctas(bytes);
   if (ctas < 1) return cudaErrorInvalidValue;
-  const size_t smem = kHeadBytes + node_bytes(a.max_n, max_l);
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -119,7 +119,7 @@ cudaError_t launch_factor_solve_resident(const NodeArgs& a, int max_l, cudaStrea
   if (grid > a.n_items) grid = a.n_items;
   // a CTA alone on its SM needs 16 warps to keep the FP64 units busy
   const int threads = ctas == 1 ? 512 : 256;
-  if (a.bie) k_factor_solve_resident<true><<<grid, threads, smem, s>>>(a);
-  else k_factor_solve_resident<false><<<grid, threads, smem, s>>>(a);
+  if (a.bie) k_factor_solve_resident<true><<<grid, threads, bytes, s>>>(a);
+  else k_factor_solve_resident<false><<<grid, threads, bytes, s>>>(a);
   return cudaGetLastError();
 }

@@ -401,9 +401,10 @@ cudaError_t prepare_factor_small();
 cudaError_t launch_factor_solve_small(const NodeArgs& a, int max_n, int max_l, cudaStream_t s);
 int factor_slots_fp64(int n, int l);
 // FP64 nodes whose matrix and probe columns fit shared memory (lu_resident.cu)
-int resident_ctas(int n, int l);  // CTAs per SM, 0 when a node does not fit
+size_t resident_bytes(int n, int l);  // shared memory of such a node's CTA
+int resident_ctas(size_t bytes);      // CTAs per SM, 0 when it does not fit
 cudaError_t prepare_factor_resident();
-cudaError_t launch_factor_solve_resident(const NodeArgs& a, int max_l, cudaStream_t s);
+cudaError_t launch_factor_solve_resident(const NodeArgs& a, size_t bytes, cudaStream_t s);
 __host__ __device__ inline size_t mixed_residual_offset(int n, int l) {
   return (((size_t)n * (n + l) * 8) + 255) & ~(size_t)255;
 }
