@@ -538,7 +538,7 @@ void plan_mixed(Workspace& ws, const std::vector<ProblemDev>& pd, const std::vec
 }
 
 // Allocates what the plan needs and fills the arguments that all chunks share.
-int ensure_mixed(Call& c, const MixedPlan& mp, int max_sweeps, MixedArgs* ma) {
+int ensure_mixed(Call& c, const MixedPlan& mp, int max_sweeps, const double2* border, MixedArgs* ma) {
   Workspace& ws = *c.ws;
   std::memset(ma, 0, sizeof(*ma));
   const size_t cnt = mp.max_count;
@@ -555,7 +555,7 @@ int ensure_mixed(Call& c, const MixedPlan& mp, int max_sweeps, MixedArgs* ma) {
     ma->texp_stride = mp.texp_stride;
   }
   CU(ws.mstate.ensure(cnt * sizeof(MixedState)));
-  CU(ws.mctl.ensure(mixed_ctl_ints((int)mp.n_probs, max_sweeps) * sizeof(int)));
+  CU(ws.mctl.ensure(mixed_ctl_ints((int)mp.n_probs, mixed_rounds(max_sweeps, border != nullptr)) * sizeof(int)));
   CU(ws.mlists.ensure((3 * cnt + 2 * (size_t)mp.unit_cap) * sizeof(int)));
   CU(ws.mubase.ensure(std::max<size_t>(1, mp.ubase.size()) * sizeof(int)));
   CU(cudaMemcpyAsync(ws.mubase.p, mp.ubase.data(), mp.ubase.size() * sizeof(int), cudaMemcpyHostToDevice, c.s));
@@ -578,6 +578,7 @@ int ensure_mixed(Call& c, const MixedPlan& mp, int max_sweeps, MixedArgs* ma) {
   ma->unit_cap = mp.unit_cap;
   ma->slots = (int)cnt;
   ma->max_sweeps = max_sweeps;
+  ma->border = border;
   ma->bie = any_bie(c.groups) ? 1 : 0;
   ma->tc_wait_cycles = wait_limit_tc();
   ma->handoff_wait_cycles = wait_limit_handoff();
@@ -919,7 +920,7 @@ int run_level(Call& c, const std::vector<HostRegion>& regs, bool gate_top, bool 
   if (any32) {
     for (const Wave& wv : waves)
       plan_mixed(ws, c.pd, rd, items, wv.items32_off, wv.n32, tc_residual(c.opt), sms, &mp);
-    CHK(ensure_mixed(c, mp, c.opt->max_ir_sweeps, &ma));
+    CHK(ensure_mixed(c, mp, c.opt->max_ir_sweeps, nullptr, &ma));
     c.st.node_ctas = std::max(c.st.node_ctas, (int32_t)std::min<size_t>(sms, mp.max_count));
   }
   const bool timed = prof_on();
@@ -1586,7 +1587,7 @@ int run_bordered_step(Call& c, const std::vector<double2>& lam_in, const std::ve
     MixedPlan mp;
     MixedArgs ma;
     plan_mixed(ws, pdv, rdv, items, 0, it32.size(), false, sms, &mp);
-    CHK(ensure_mixed(c, mp, std::max(1, c.opt->max_ir_sweeps), &ma));
+    CHK(ensure_mixed(c, mp, std::max(1, c.opt->max_ir_sweeps), bord, &ma));
     ma.probs = ws.iprobs.as<ProblemDev>();
     ma.regions = ws.iregions.as<RegionDev>();
     ma.X = ws.iX.as<double2>();
@@ -1594,7 +1595,6 @@ int run_bordered_step(Call& c, const std::vector<double2>& lam_in, const std::ve
     ma.tol_ir = kIrTol;
     ma.err = ws.icounters.as<int32_t>() + 3;
     ma.res64 = 1;
-    ma.border = bord;
     // verification work, timed apart from the disks' nodes
     CHK(launch_mixed(mp, 0, 0, ma, ws.iitems.as<NodeItem>(), sms, PMCIM_K_VERIFY, s, ws.mubase.as<int>()));
   }

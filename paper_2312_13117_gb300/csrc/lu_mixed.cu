@@ -606,10 +606,12 @@ __global__ void __launch_bounds__(THREADS, 2) k_mixed_factor(MixedArgs a, int sc
 __device__ __forceinline__ void finish_node(const MixedArgs& a, const RegionDev& rg, const NodeItem& it,
                                             const MixedState& st, bool ok) {
   a.node_info[rg.node_off + it.j] =
-      st.info | (st.sweeps << 24) | (st.lost ? (1 << 29) : 0) | (ok ? 0 : (1 << 30));
+      st.info | (min(st.sweeps, 31) << 24) | (st.lost ? (1 << 29) : 0) | (ok ? 0 : (1 << 30));
 }
 
-// The back substitution (sw = 0, every node) or sweep sw's correction (the active nodes).
+// The back substitution (sw = 0, every node) or sweep sw's correction (the active nodes). A
+// bordered node's sweeps all run in the launch of the first: they are not bounded by
+// MIXED_MAX_SWEEPS, and their residuals need no other kernel.
 // RES64: a node of the launch forms its residuals on the FP64 pipe.
 template <bool RES64>
 __global__ void __launch_bounds__(THREADS, 3) k_mixed_solve(MixedArgs a, int sw, int y_bytes) {
@@ -663,70 +665,73 @@ __global__ void __launch_bounds__(THREADS, 3) k_mixed_solve(MixedArgs a, int sw,
       done = a.max_sweeps == 0;
       pc.mark(PH_FIRST_SOLVE);
     } else {
-      if (oz) {
-        ok = (st.lost & MIXED_LOST_RESIDUAL) == 0;  // R is not valid where a wait ran out
-      } else if (RES64) {
-        // the matrix the residual multiplies: T(z_j) assembled once, or the one dense term
-        const double2* M = nullptr;
-        double2 fM = make_double2(1.0, 0.0), id = make_double2(0.0, 0.0);
-        if (P.n_dense >= 2 || rg.herm || P.bie) {
-          M = a.t64 + (size_t)q * a.t64_stride;
-        } else {
-          id = c.fid;
-          for (int t = 0; t < P.K; ++t)
-            if (P.term[t].dense) {
-              M = P.A + (size_t)P.term[t].mat_index * nn;
-              fM = c.fz[t];
-            }
+      for (int s = sw;; ++s) {
+        if (oz) {
+          ok = (st.lost & MIXED_LOST_RESIDUAL) == 0;  // R is not valid where a wait ran out
+        } else if (RES64) {
+          // the matrix the residual multiplies: T(z_j) assembled once, or the one dense term
+          const double2* M = nullptr;
+          double2 fM = make_double2(1.0, 0.0), id = make_double2(0.0, 0.0);
+          if (P.n_dense >= 2 || rg.herm || P.bie) {
+            M = a.t64 + (size_t)q * a.t64_stride;
+          } else {
+            id = c.fid;
+            for (int t = 0; t < P.K; ++t)
+              if (P.term[t].dense) {
+                M = P.A + (size_t)P.term[t].mat_index * nn;
+                fM = c.fz[t];
+              }
+          }
+          ResSmem& res = *reinterpret_cast<ResSmem*>(smem_raw);
+          if (l == 1) residual_fp64_col(X, R, c, res, M, fM, id);
+          else residual_fp64(X, R, c, res, M, fM, id);
         }
-        ResSmem& res = *reinterpret_cast<ResSmem*>(smem_raw);
-        if (l == 1) residual_fp64_col(X, R, c, res, M, fM, id);
-        else residual_fp64(X, R, c, res, M, fM, id);
-      }
-      if (ok && rg.border > 0) {
-        // bordered system M u = b, M = T(z_j) + (c - T(z_j) e_s) e_s^T with b = -T(z_j) e_s:
-        // R = b - T X - (c + b) X_s (l = 1)
-        const double2 xs = X[rg.border - 1];
-        const double2* bc = a.border + rg.v_off;
-        for (size_t e = tid; e < nl; e += THREADS) cfms(R[e], cadd(bc[e], P.V[e]), xs);
-      }
-      pc.mark(PH_RESIDUAL);
-      double rm = 0.0;
-      if (ok) {
-        for (size_t e = tid; e < nl; e += THREADS) rm = fmax(rm, fmax(fabs(R[e].x), fabs(R[e].y)));
-        rm = block_max(rm, c.red);
-        done = rm == 0.0;
-      }
-      if (ok && !done) {
-        const double inv = 1.0 / rm;
-        // right-hand side R / |R|max; the forward solve applies the row interchanges
-        for (size_t e = tid; e < nl; e += THREADS) {
-          const double2 rv = R[e];
-          Y[e] = make_float2((float)(rv.x * inv), (float)(rv.y * inv));
+        if (ok && rg.border > 0) {
+          // bordered system M u = b, M = T(z_j) + (c - T(z_j) e_s) e_s^T with b = -T(z_j) e_s:
+          // R = b - T X - (c + b) X_s (l = 1)
+          const double2 xs = X[rg.border - 1];
+          const double2* bc = a.border + rg.v_off;
+          for (size_t e = tid; e < nl; e += THREADS) cfms(R[e], cadd(bc[e], P.V[e]), xs);
         }
-        gsync();
-        lu32::forward(M32, Y, n, l, sm.s, lists);
-        lu32::back(M32, Y, n, l, sm.s);
-        double dm = 0.0, xmx = 0.0;
-        for (size_t e = tid; e < nl; e += THREADS) {
-          const float2 d = Y[e];
-          double2 x = X[e];
-          const double dx = (double)d.x * rm, dy = (double)d.y * rm;
-          x.x += dx;
-          x.y += dy;
-          X[e] = x;
-          dm = fmax(dm, fmax(fabs(dx), fabs(dy)));
-          xmx = fmax(xmx, fmax(fabs(x.x), fabs(x.y)));
+        pc.mark(PH_RESIDUAL);
+        double rm = 0.0;
+        if (ok) {
+          for (size_t e = tid; e < nl; e += THREADS) rm = fmax(rm, fmax(fabs(R[e].x), fabs(R[e].y)));
+          rm = block_max(rm, c.red);
+          done = rm == 0.0;
         }
-        dm = block_max(dm, c.red);
-        xmx = block_max(xmx, c.red);
-        st.sweeps = sw;
-        if (!(dm < st.dprev) && sw > 1) ok = false;  // no contraction
-        else if (dm * dm <= a.tol_ir * xmx * st.dprev) done = true;
-        else if (sw >= a.max_sweeps) ok = false;
-        st.dprev = dm;
+        if (ok && !done) {
+          const double inv = 1.0 / rm;
+          // right-hand side R / |R|max; the forward solve applies the row interchanges
+          for (size_t e = tid; e < nl; e += THREADS) {
+            const double2 rv = R[e];
+            Y[e] = make_float2((float)(rv.x * inv), (float)(rv.y * inv));
+          }
+          gsync();
+          lu32::forward(M32, Y, n, l, sm.s, lists);
+          lu32::back(M32, Y, n, l, sm.s);
+          double dm = 0.0, xmx = 0.0;
+          for (size_t e = tid; e < nl; e += THREADS) {
+            const float2 d = Y[e];
+            double2 x = X[e];
+            const double dx = (double)d.x * rm, dy = (double)d.y * rm;
+            x.x += dx;
+            x.y += dy;
+            X[e] = x;
+            dm = fmax(dm, fmax(fabs(dx), fabs(dy)));
+            xmx = fmax(xmx, fmax(fabs(x.x), fabs(x.y)));
+          }
+          dm = block_max(dm, c.red);
+          xmx = block_max(xmx, c.red);
+          st.sweeps = s;
+          if (!(dm < st.dprev) && s > 1) ok = false;  // no contraction
+          else if (dm * dm <= a.tol_ir * xmx * st.dprev) done = true;
+          else if (s >= a.max_sweeps) ok = false;
+          st.dprev = dm;
+        }
+        pc.mark(PH_CORRECTION);
+        if (done || !ok || rg.border == 0) break;
       }
-      pc.mark(PH_CORRECTION);
     }
     const bool refine = a.max_sweeps > 0;
     if ((done || !ok) && rg.border > 0) {
@@ -863,7 +868,9 @@ cudaError_t round_coefficients_c64(const double2* src, float2* dst, size_t count
 cudaError_t launch_factor_solve_mixed(const MixedArgs& a, int sms, cudaStream_t s, int* launched) {
   *launched = 0;
   if (a.count <= 0) return cudaSuccess;
-  cudaError_t e = cudaMemsetAsync(a.ctl, 0, mixed_ctl_zero_ints(a.n_probs, a.max_sweeps) * sizeof(int), s);
+  const int rounds = mixed_rounds(a.max_sweeps, a.border != nullptr);
+  if (rounds > MIXED_MAX_SWEEPS) return cudaErrorInvalidValue;  // (ctl has no counters for more)
+  cudaError_t e = cudaMemsetAsync(a.ctl, 0, mixed_ctl_zero_ints(a.n_probs, rounds) * sizeof(int), s);
   if (e != cudaSuccess) return e;
   auto grid = [&](int per_sm) { return per_sm * sms < a.count ? per_sm * sms : a.count; };
   if (a.bie && a.t64) {
@@ -880,7 +887,7 @@ cudaError_t launch_factor_solve_mixed(const MixedArgs& a, int sms, cudaStream_t 
     else k_mixed_factor<false, false><<<g, THREADS, smem, s>>>(a, scratch);
     ++*launched;
   }
-  for (int sw = 0; sw <= a.max_sweeps; ++sw) {
+  for (int sw = 0; sw <= rounds; ++sw) {
     if (sw > 0 && a.oz) {
       e = launch_oz_residual(a, sw, sms, s);
       if (e != cudaSuccess) return e;

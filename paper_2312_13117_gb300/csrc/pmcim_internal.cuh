@@ -335,11 +335,16 @@ struct MixedArgs {
   long long tc_wait_cycles;       // limit of a wait for a tensor-core commit or its operands
   long long handoff_wait_cycles;  // limit of a wait between warp groups
 };
-__host__ __device__ inline size_t mixed_ctl_zero_ints(int n_probs, int max_sweeps) {
-  return MIXED_CTL_UNITS + (size_t)(max_sweeps + 1) * n_probs;
+// Sweeps that are launches of their own, at most MIXED_MAX_SWEEPS: bordered nodes, whose number
+// of sweeps has no limit, run theirs in one.
+__host__ __device__ inline int mixed_rounds(int max_sweeps, bool border) {
+  return border && max_sweeps > 1 ? 1 : max_sweeps;
 }
-__host__ __device__ inline size_t mixed_ctl_ints(int n_probs, int max_sweeps) {
-  return mixed_ctl_zero_ints(n_probs, max_sweeps) + n_probs + 1;
+__host__ __device__ inline size_t mixed_ctl_zero_ints(int n_probs, int rounds) {
+  return MIXED_CTL_UNITS + (size_t)(rounds + 1) * n_probs;
+}
+__host__ __device__ inline size_t mixed_ctl_ints(int n_probs, int rounds) {
+  return mixed_ctl_zero_ints(n_probs, rounds) + n_probs + 1;
 }
 // Whether the node's residuals are formed on the tensor cores.
 __device__ __forceinline__ bool mixed_node_oz(const MixedArgs& a, const ProblemDev& P, const RegionDev& rg) {
@@ -353,7 +358,7 @@ __device__ __forceinline__ int* mixed_ucount(const MixedArgs& a, int sw) {
   return a.ctl + MIXED_CTL_UNITS + (size_t)sw * a.n_probs;
 }
 __device__ __forceinline__ int* mixed_tiles(const MixedArgs& a) {
-  return a.ctl + mixed_ctl_zero_ints(a.n_probs, a.max_sweeps);
+  return a.ctl + mixed_ctl_zero_ints(a.n_probs, mixed_rounds(a.max_sweeps, a.border != nullptr));
 }
 // Phase-clock slots (PMCIM_PHASES): SM cycles summed over CTAs, by step.
 enum { PH_ASSEMBLE = 0, PH_PANEL = 1, PH_FIRST_SOLVE = 2, PH_RESIDUAL = 3, PH_CORRECTION = 4, PH_FALLBACK = 5,
