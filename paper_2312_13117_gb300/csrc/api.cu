@@ -242,8 +242,8 @@ long long wait_limit_handoff() {
 // Device workspaces, reused across calls on one handle.
 struct Workspace {
   DevBuf probs, regions, items, counters, node_info, X;
-  DevBuf work64, piv64, work32, t64, phase;
-  DevBuf tdig, texp;                     // boundary-integral nodes: digits of T(z_j), row exponents
+  DevBuf work64, piv64, work32, phase;
+  DevBuf texp;                          // boundary-integral nodes: row exponents of T(z_j)'s digits
   DevBuf mstate, mctl, mlists, mubase;  // precision forms: node states, counters, node lists, list bases
   DevBuf C0, C1, pf_half, pf_abs, ind, pf_norm, pf_scale, cand;
   DevBuf bwork, bsigma, bp, blam, bvecs, bkept, bstatus;
@@ -255,7 +255,7 @@ struct Workspace {
   DevBuf ind3, feats, sprob, sparams, sscratch;
   // verification's inverse-iteration step: per-value problem table, pseudo-disks, items, solutions
   DevBuf iprobs, iregions, iitems, iX, iinfo, icounters, ibord, ioffs;
-  DevBuf ysl, gexp;                  // per slot: digits of f_k X for the tensor-core residual, exponents
+  DevBuf gexp;                       // per slot: column exponents of the digits of f_k X
   DevBuf rz, rX, rR, rstat, rysl;    // pmcim_residual: points, solutions, residuals, status, scratch
   DevBuf cW, cidx, cgram, gpart;     // certificates from coefficient products: W, index arrays, Gram data
   // the library's own stream: graphs cannot be captured on the legacy default stream
@@ -266,11 +266,11 @@ struct Workspace {
     if (ordered) cudaEventDestroy(ordered);
     stream = nullptr;
     ordered = nullptr;
-    DevBuf* b[] = {&probs, &regions, &items, &counters, &node_info, &X, &work64, &piv64, &work32, &t64,
-                   &phase, &tdig, &texp, &mstate, &mctl, &mlists, &mubase, &C0, &C1, &pf_half, &pf_abs, &ind, &pf_norm, &pf_scale, &cand, &bwork, &bsigma,
+    DevBuf* b[] = {&probs, &regions, &items, &counters, &node_info, &X, &work64, &piv64, &work32,
+                   &phase, &texp, &mstate, &mctl, &mlists, &mubase, &C0, &C1, &pf_half, &pf_abs, &ind, &pf_norm, &pf_scale, &cand, &bwork, &bsigma,
                    &bp, &blam, &bvecs, &bkept, &bstatus, &vlam, &vprob, &voff, &vsig, &vacc, &vwork,
                    &vvec, &vpiv, &gitems, &gdst, &gperm, &ind3, &feats, &sprob, &sparams, &sscratch, &Xkeep,
-                   &citems, &vout, &Cm, &iprobs, &iregions, &iitems, &iX, &iinfo, &icounters, &ibord, &ioffs, &ysl, &gexp, &rz,
+                   &citems, &vout, &Cm, &iprobs, &iregions, &iitems, &iX, &iinfo, &icounters, &ibord, &ioffs, &gexp, &rz,
                    &rX, &rR, &rstat, &rysl, &cW, &cidx, &cgram, &gpart};
     for (DevBuf* x : b) x->release();
   }
@@ -469,17 +469,19 @@ int n_bucket(int n) {
 struct MixedChunk {
   size_t off, count;  // in the item list
   int max_n, max_l;
-  int tc;
+  int tc, res64;
+  // bytes of the chunk's slots, and where the arrays of its nodes follow them (0: none)
+  size_t work, t64_off, ysl_off, tdig_off, total;
+  size_t t64_stride, ysl_stride, tdig_stride;
+  int gexp_stride, texp_stride;
 };
 
-// The chunks of a call's precision-form nodes, their workspaces and the arguments they share.
+// The chunks of a call's precision-form nodes and what their workspaces need.
 struct MixedPlan {
   std::vector<std::vector<MixedChunk>> chunks;  // per wave
   std::vector<int> ubase;                       // per chunk and problem: first unit of its list
   size_t n_probs = 0, max_count = 0;
-  size_t work = 0, t64 = 0, ysl = 0;
-  size_t t64_stride = 0, ysl_stride = 0, tdig_stride = 0;
-  int gexp_stride = 0, texp_stride = 0;
+  size_t arena = 0, gexp = 0, texp = 0;  // the most that a chunk takes (bytes, then numbers)
   int unit_cap = 0;
 };
 
@@ -489,32 +491,36 @@ void plan_mixed(Workspace& ws, const std::vector<ProblemDev>& pd, const std::vec
   mp->n_probs = pd.size();
   mp->chunks.emplace_back();
   if (count == 0) return;
-  int max_l = 1, nd = 0;
-  size_t ysl = 0, t64 = 0;
+  MixedChunk w{};  // what the wave's chunks share
+  w.max_l = 1;
+  size_t t64 = 0;
+  int nd = 0;
   for (size_t i = 0; i < count; ++i) {
     const RegionDev& r = rd[items[off + i].region];
     const ProblemDev& P = pd[r.prob];
-    max_l = std::max(max_l, P.l);
+    w.max_l = std::max(w.max_l, P.l);
     const bool column = oz && P.bie && P.bie_circ && P.n_dense == 0;  // mixed_column_only
     if (r.herm || P.bie || (P.n_dense >= 2 && !oz)) t64 = std::max(t64, (size_t)P.n * (column ? 1 : P.n));
     if (oz && !r.herm) {
       const int terms = P.bie ? 1 : P.n_dense;
-      ysl = std::max(ysl, oz_slot_bytes(P.n, P.l, terms));
+      w.ysl_stride = std::max(w.ysl_stride, oz_slot_bytes(P.n, P.l, terms));
       nd = std::max(nd, terms);
       if (P.bie) {
-        mp->tdig_stride = std::max(mp->tdig_stride, coefficient_digit_bytes(P.n, 1));
-        mp->texp_stride = std::max(mp->texp_stride, (P.n + 127) / 128 * 128);
+        w.tdig_stride = std::max(w.tdig_stride, coefficient_digit_bytes(P.n, 1));
+        w.texp_stride = std::max(w.texp_stride, (P.n + 127) / 128 * 128);
       }
     }
   }
-  mp->t64_stride = std::max(mp->t64_stride, t64);
-  mp->ysl_stride = std::max(mp->ysl_stride, ysl);
-  mp->gexp_stride = std::max(mp->gexp_stride, nd * PMCIM_MAX_L);
-  const size_t budget = slot_budget(ws.work32.cap + ws.t64.cap + ws.ysl.cap + ws.tdig.cap);
+  w.t64_stride = t64;
+  w.gexp_stride = nd * PMCIM_MAX_L;
+  const auto align = [](size_t b) { return (b + 1023) & ~(size_t)1023; };
+  const size_t budget = slot_budget(ws.work32.cap);
   for (size_t i = 0; i < count;) {
-    MixedChunk ch{off + i, 0, pd[rd[items[off + i].region].prob].n, max_l, 0};
+    MixedChunk ch = w;
+    ch.off = off + i;
+    ch.max_n = pd[rd[items[off + i].region].prob].n;
     const size_t slot = mixed_slot_bytes(ch.max_n, ch.max_l);
-    const size_t per = slot + mp->t64_stride * sizeof(double2) + mp->ysl_stride + mp->tdig_stride;
+    const size_t per = slot + ch.t64_stride * sizeof(double2) + ch.ysl_stride + ch.tdig_stride;
     const size_t cap = std::max<size_t>(
         1, std::min(budget / per, std::max<size_t>(kChunkBytes / per, (size_t)kChunkNodesPerSm * sms)));
     ch.count = std::min(cap, count - i);
@@ -523,15 +529,23 @@ void plan_mixed(Workspace& ws, const std::vector<ProblemDev>& pd, const std::vec
       const RegionDev& r = rd[items[off + i + k].region];
       units[r.prob] += (pd[r.prob].l + 7) / 8;
       ch.tc |= r.lu_tc != 0;
+      ch.res64 |= !oz || r.herm || !(pd[r.prob].bie || pd[r.prob].n_dense > 0);  // no digits to multiply
     }
     int base = 0;
     for (int u : units) {
       mp->ubase.push_back(base);
       base += u;
     }
+    ch.work = std::max(ch.count * slot, mixed_fallback_bytes(ch.max_n, ch.max_l));
+    ch.t64_off = align(ch.work);
+    ch.ysl_off = align(ch.t64_off + ch.count * ch.t64_stride * sizeof(double2));
+    ch.tdig_off = align(ch.ysl_off + ch.count * ch.ysl_stride);
+    ch.total = ch.tdig_off + ch.count * ch.tdig_stride;
     mp->unit_cap = std::max(mp->unit_cap, base);
     mp->max_count = std::max(mp->max_count, ch.count);
-    mp->work = std::max(mp->work, std::max(ch.count * slot, mixed_fallback_bytes(ch.max_n, ch.max_l)));
+    mp->arena = std::max(mp->arena, ch.total);
+    mp->gexp = std::max(mp->gexp, ch.count * ch.gexp_stride);
+    mp->texp = std::max(mp->texp, ch.count * ch.texp_stride);
     mp->chunks.back().push_back(ch);
     i += ch.count;
   }
@@ -542,18 +556,9 @@ int ensure_mixed(Call& c, const MixedPlan& mp, int max_sweeps, const double2* bo
   Workspace& ws = *c.ws;
   std::memset(ma, 0, sizeof(*ma));
   const size_t cnt = mp.max_count;
-  CU(ws.work32.ensure(mp.work));
-  if (mp.t64_stride) CU(ws.t64.ensure(cnt * mp.t64_stride * sizeof(double2)));
-  if (mp.ysl_stride) CU(ws.ysl.ensure(cnt * mp.ysl_stride));
-  if (mp.gexp_stride) CU(ws.gexp.ensure(cnt * mp.gexp_stride * sizeof(int32_t)));
-  if (mp.tdig_stride) {
-    CU(ws.tdig.ensure(cnt * mp.tdig_stride));
-    CU(ws.texp.ensure(cnt * mp.texp_stride * sizeof(int32_t)));
-    ma->tdig = ws.tdig.as<unsigned char>();
-    ma->tdig_stride = mp.tdig_stride;
-    ma->texp = ws.texp.as<int32_t>();
-    ma->texp_stride = mp.texp_stride;
-  }
+  CU(ws.work32.ensure(mp.arena));
+  if (mp.gexp) CU(ws.gexp.ensure(mp.gexp * sizeof(int32_t)));
+  if (mp.texp) CU(ws.texp.ensure(mp.texp * sizeof(int32_t)));
   CU(ws.mstate.ensure(cnt * sizeof(MixedState)));
   CU(ws.mctl.ensure(mixed_ctl_ints((int)mp.n_probs, mixed_rounds(max_sweeps, border != nullptr)) * sizeof(int)));
   CU(ws.mlists.ensure((3 * cnt + 2 * (size_t)mp.unit_cap) * sizeof(int)));
@@ -562,14 +567,8 @@ int ensure_mixed(Call& c, const MixedPlan& mp, int max_sweeps, const double2* bo
   CU(prepare_factor_mixed());
   ma->n_probs = (int)mp.n_probs;
   ma->work = ws.work32.as<char>();
-  ma->work_bytes = mp.work;
-  ma->t64 = mp.t64_stride ? ws.t64.as<double2>() : nullptr;
-  ma->t64_stride = mp.t64_stride;
-  ma->ysl = mp.ysl_stride ? ws.ysl.as<unsigned char>() : nullptr;
-  ma->ysl_stride = mp.ysl_stride;
-  ma->oz = mp.ysl_stride ? 1 : 0;
   ma->gexp = ws.gexp.as<int32_t>();
-  ma->gexp_stride = mp.gexp_stride;
+  ma->texp = ws.texp.as<int32_t>();
   ma->state = ws.mstate.as<MixedState>();
   ma->ctl = ws.mctl.as<int>();
   ma->act = ws.mlists.as<int>();
@@ -596,7 +595,18 @@ int launch_mixed(const MixedPlan& mp, size_t wave, size_t chunk0, const MixedArg
     a.max_n = ch.max_n;
     a.max_l = ch.max_l;
     a.slot_bytes = mixed_slot_bytes(ch.max_n, ch.max_l);
+    a.work_bytes = ch.work;
     a.tc = ch.tc;
+    a.res64 = ch.res64;
+    a.t64 = ch.t64_stride ? reinterpret_cast<double2*>(a.work + ch.t64_off) : nullptr;
+    a.t64_stride = ch.t64_stride;
+    a.ysl = ch.ysl_stride ? reinterpret_cast<unsigned char*>(a.work + ch.ysl_off) : nullptr;
+    a.ysl_stride = ch.ysl_stride;
+    a.oz = ch.ysl_stride ? 1 : 0;
+    a.tdig = ch.tdig_stride ? reinterpret_cast<unsigned char*>(a.work + ch.tdig_off) : nullptr;
+    a.tdig_stride = ch.tdig_stride;
+    a.texp_stride = ch.texp_stride;
+    a.gexp_stride = ch.gexp_stride;
     a.ubase = d_ubase + (chunk0 + k) * mp.n_probs;
     int launched = 0;
     prof_begin(prof_kind, s);
@@ -972,12 +982,6 @@ int run_level(Call& c, const std::vector<HostRegion>& regs, bool gate_top, bool 
     ma.tol_ir = c.opt->tol_ir > 0.0 ? c.opt->tol_ir : kIrTol;
     ma.err = ws.counters.as<int32_t>() + kCounters * waves.size();
     ma.phase = timed ? ws.phase.as<unsigned long long>() : nullptr;
-    // nodes whose residuals have no coefficient digits
-    for (const NodeItem& it : items) {
-      const ProblemDev& P = c.pd[rd[it.region].prob];
-      if (P.bie ? !ma.tdig : P.n_dense == 0) ma.res64 = 1;
-    }
-    if (!tc_residual(c.opt)) ma.res64 = 1;
   }
   // ---- the level as one CUDA graph (profiler events become graph nodes) ----
   cudaGraph_t graph = nullptr;
@@ -1594,7 +1598,6 @@ int run_bordered_step(Call& c, const std::vector<double2>& lam_in, const std::ve
     ma.node_info = ws.iinfo.as<int32_t>();
     ma.tol_ir = kIrTol;
     ma.err = ws.icounters.as<int32_t>() + 3;
-    ma.res64 = 1;
     // verification work, timed apart from the disks' nodes
     CHK(launch_mixed(mp, 0, 0, ma, ws.iitems.as<NodeItem>(), sms, PMCIM_K_VERIFY, s, ws.mubase.as<int>()));
   }
