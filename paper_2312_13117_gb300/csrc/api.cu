@@ -469,7 +469,7 @@ int n_bucket(int n) {
 struct MixedChunk {
   size_t off, count;  // in the item list
   int max_n, max_l;
-  int tc, res64;
+  int tc, res64, oz_dense;
   // bytes of the chunk's slots, and where the arrays of its nodes follow them (0: none)
   size_t work, t64_off, ysl_off, tdig_off, total;
   size_t t64_stride, ysl_stride, tdig_stride;
@@ -502,11 +502,11 @@ void plan_mixed(Workspace& ws, const std::vector<ProblemDev>& pd, const std::vec
     const bool column = oz && P.bie && P.bie_circ && P.n_dense == 0;  // mixed_column_only
     if (r.herm || P.bie || (P.n_dense >= 2 && !oz)) t64 = std::max(t64, (size_t)P.n * (column ? 1 : P.n));
     if (oz && !r.herm) {
-      const int terms = P.bie ? 1 : P.n_dense;
-      w.ysl_stride = std::max(w.ysl_stride, oz_slot_bytes(P.n, P.l, terms));
-      nd = std::max(nd, terms);
+      if (P.bie || P.n_dense > 0)
+        w.ysl_stride = std::max(w.ysl_stride, oz_slot_bytes(P.n, P.l, P.bie ? 0 : P.n_dense));
+      nd = std::max(nd, P.bie ? 1 : P.n_dense);
       if (P.bie) {
-        w.tdig_stride = std::max(w.tdig_stride, coefficient_digit_bytes(P.n, 1));
+        w.tdig_stride = std::max(w.tdig_stride, bie_digit_bytes(P.n));
         w.texp_stride = std::max(w.texp_stride, (P.n + 127) / 128 * 128);
       }
     }
@@ -529,6 +529,7 @@ void plan_mixed(Workspace& ws, const std::vector<ProblemDev>& pd, const std::vec
       const RegionDev& r = rd[items[off + i + k].region];
       units[r.prob] += (pd[r.prob].l + 7) / 8;
       ch.tc |= r.lu_tc != 0;
+      ch.oz_dense |= oz && !r.herm && !pd[r.prob].bie && pd[r.prob].n_dense > 0;
       ch.res64 |= !oz || r.herm || !(pd[r.prob].bie || pd[r.prob].n_dense > 0);  // no digits to multiply
     }
     int base = 0;
@@ -603,6 +604,7 @@ int launch_mixed(const MixedPlan& mp, size_t wave, size_t chunk0, const MixedArg
     a.ysl = ch.ysl_stride ? reinterpret_cast<unsigned char*>(a.work + ch.ysl_off) : nullptr;
     a.ysl_stride = ch.ysl_stride;
     a.oz = ch.ysl_stride ? 1 : 0;
+    a.oz_dense = ch.oz_dense;
     a.tdig = ch.tdig_stride ? reinterpret_cast<unsigned char*>(a.work + ch.tdig_off) : nullptr;
     a.tdig_stride = ch.tdig_stride;
     a.texp_stride = ch.texp_stride;

@@ -21,8 +21,9 @@ using namespace ozk;
 
 constexpr int BT = 256;
 constexpr int PIECE = 4096;  // pairs of an assembly item
+constexpr int CIRC = 1024;   // largest circulant matrix that is written from its first column
 
-// rint(x 2^shift) as an integer (ties away from zero), |result| <= 2^48, by the bits of x.
+// rint(x 2^shift) as an integer (ties away from zero), |result| <= 2^55, by the bits of x.
 __device__ __forceinline__ long long scaled_integer(double x, int shift) {
   const long long b = __double_as_longlong(x);
   const int ex = (int)((b >> 52) & 0x7ff);
@@ -42,6 +43,7 @@ __global__ void __launch_bounds__(BT, 2) k_bie_assemble(MixedArgs a, int pieces)
   __shared__ ProblemDev P;
   __shared__ double2 fz[PMCIM_MAX_TERMS];
   __shared__ bie::Wave wave;
+  __shared__ double2 first[CIRC];
   for (long long w = blockIdx.x; w < (long long)a.count * pieces; w += gridDim.x) {
     // (pieces outermost: the CTAs share the first pieces of all nodes, the only ones of circulant nodes)
     const int q = (int)(w % a.count), piece = (int)(w / a.count);
@@ -76,6 +78,16 @@ __global__ void __launch_bounds__(BT, 2) k_bie_assemble(MixedArgs a, int pieces)
       for (int m = threadIdx.x; m < n; m += BT) {
         double2 v = cmul(cb, bie::dlp_entry(P.bie, n, m, 0, wave));
         T[m] = m == 0 ? cadd(v, id) : v;
+      }
+      continue;
+    }
+    if (P.bie_circ && n <= CIRC) {  // n distinct entries: every piece forms them and writes its share
+      for (int m = threadIdx.x; m < n; m += BT) first[m] = cmul(cb, bie::dlp_entry(P.bie, n, m, 0, wave));
+      __syncthreads();
+      for (int e = 2 * piece * PIECE + threadIdx.x; e < min(n * n, 2 * (piece + 1) * PIECE); e += BT) {
+        const int j = e / n, i = e - j * n;
+        const double2 v = first[i >= j ? i - j : i - j + n];
+        store(i, j, i == j ? cadd(v, id) : v);
       }
       continue;
     }
@@ -130,10 +142,10 @@ __global__ void __launch_bounds__(BT) k_bie_digits(MixedArgs a, int max_rb) {
       a.texp[(size_t)q * a.texp_stride + rb * TM + tid] = emax[tid];
     }
     __syncthreads();
-    unsigned char* base = a.tdig + (size_t)q * a.tdig_stride + (size_t)rb * kcn * S * A_STAGE;
+    unsigned char* base = a.tdig + (size_t)q * a.tdig_stride + (size_t)rb * kcn * BIE_DIGITS * A_STAGE;
     for (int task = tid; task < TM * kcn * (KC / 8); task += BT) {
       const int r = task & (TM - 1), j0 = task / TM * 8, i = rb * TM + r;
-      const int shift = DIGIT_SHIFT - emax[r];
+      const int shift = 7 * BIE_DIGITS - 1 - emax[r];
       long long Nr[8], Ni[8];
 #pragma unroll
       for (int u = 0; u < 8; ++u) {
@@ -143,9 +155,9 @@ __global__ void __launch_bounds__(BT) k_bie_digits(MixedArgs a, int max_rb) {
         Nr[u] = scaled_integer(v.x, shift);
         Ni[u] = scaled_integer(v.y, shift);
       }
-      unsigned char* st = base + (size_t)(j0 / KC) * S * A_STAGE + tile_off(r, j0 % KC);
+      unsigned char* st = base + (size_t)(j0 / KC) * BIE_DIGITS * A_STAGE + tile_off(r, j0 % KC);
 #pragma unroll 1
-      for (int t = S - 1; t >= 0; --t) {
+      for (int t = BIE_DIGITS - 1; t >= 0; --t) {
         uint32_t pr[4], pi[4];
 #pragma unroll
         for (int u = 0; u < 8; u += 2) {
@@ -162,6 +174,8 @@ __global__ void __launch_bounds__(BT) k_bie_digits(MixedArgs a, int max_rb) {
 }
 
 }  // namespace
+
+size_t bie_digit_bytes(int n) { return (size_t)row_blocks(n) * k_chunks(n) * BIE_DIGITS * A_STAGE; }
 
 cudaError_t launch_bie_assemble(const MixedArgs& a, int sms, cudaStream_t s, int* launched) {
   const int pieces = (a.max_n * (a.max_n / 2) + PIECE - 1) / PIECE, rb = row_blocks(a.max_n);

@@ -889,9 +889,8 @@ cudaError_t launch_factor_solve_mixed(const MixedArgs& a, int sms, cudaStream_t 
   }
   for (int sw = 0; sw <= rounds; ++sw) {
     if (sw > 0 && a.oz) {
-      e = launch_oz_residual(a, sw, sms, s);
+      e = launch_oz_residual(a, sw, sms, s, launched);
       if (e != cudaSuccess) return e;
-      *launched += 2;
     }
     // (the FP64-pipe residual's tiles leave no room for the right-hand sides)
     const size_t nl = (size_t)a.max_n * a.max_l * sizeof(float2);

@@ -20,7 +20,12 @@
 //                 one FP64 update of R (kept in registers) per 256 inner indices, which
 //                 overlaps the next products.
 // A boundary-integral node has a matrix of its own: its tiles hold its own groups only,
-// and the digits are those of T(z_j) (bie_nodes.cu).
+// and the digits are those of T(z_j) (bie_nodes.cu). Its rows hold numbers of very
+// different sizes (H_1 grows like e^{-Im w}), and its residuals take the place of FP64
+// ones, so it gets 8 digits (55 bits of a row's largest number) and the pairs of total
+// order <= 10, in 9 accumulators and at most three groups a tile. Errors of such a residual
+// relative to |X|, n = 34, z = 2 - 2.8 i: 5.1e-16 (plain FP64 1.1e-15, 7 digits 7.9e-14);
+// 100 disks of 64 nodes at n = 256, l = 8 take 46.6 ms in all (45.3 with 7 digits).
 // A wait for operands is bounded by tc_wait_cycles: when one runs out the CTA's nodes
 // are marked, and solved again in FP64. A wait between the warps is bounded by
 // handoff_wait_cycles: when one runs out the launch fails (MixedArgs::err).
@@ -31,20 +36,32 @@ namespace {
 using namespace ozk;
 
 constexpr int CG = 8;                     // solution columns of a group
-constexpr int MAXG = 4;                   // groups of a tile
-constexpr int GROUP_STAGE = 2 * CG * KC * 2 * 2 * S;  // a group's digits of 32 inner indices: 14 KB
-constexpr int PART = GROUP_STAGE / 2;     // [real rows][imaginary rows]: 7 KB each
+// The digits of a form of products: dense terms (ozaki.cuh), or a boundary-integral node's T(z_j).
+template <bool BIE>
+struct Form {
+  static constexpr int S = BIE ? 8 : ozk::S, QMAX = BIE ? 10 : ozk::QMAX, NQ = QMAX - 1;
+  static constexpr int SHIFT = 7 * S - 1;   // a number's integer is rint(x 2^(SHIFT - exponent))
+  static constexpr int SCALE = 2 * SHIFT - 7 * (2 * S - QMAX);  // weight of the last order, 2^(e + g - SCALE)
+  static constexpr int MAXG = BIE ? 3 : 4;  // groups of a tile
+  static constexpr int STAGE = 2 * CG * KC * 2 * 2 * S;  // a group's digits of 32 inner indices: 14 or 16 KB
+  static constexpr int PART = STAGE / 2;                 // [real rows][imaginary rows]
+};
+static_assert(Form<false>::SHIFT == DIGIT_SHIFT && Form<false>::SCALE == DRAIN_SCALE, "the coefficients' digits");
+static_assert(Form<true>::S == BIE_DIGITS, "T(z_j)'s digits");
+static_assert(Form<true>::NQ * 16 * Form<true>::MAXG <= 512 && Form<false>::NQ * 16 * Form<false>::MAXG <= 512,
+              "TMEM columns");
+static_assert(8 * 2 * KD * 64 * 64 <= (1 << 24), "tensor-core partial sums must stay exact in FP32");
 constexpr int RA = 6;                     // A stages
 constexpr int RB2 = 2;                    // B stages
 constexpr int DRAIN_WARP0 = 4, DRAIN_WARPS = 16;
 constexpr int GEMM_THREADS = 32 * (DRAIN_WARP0 + DRAIN_WARPS);
 constexpr int DIGIT_THREADS = 256;
 
-// Byte offset of digit t, form f (0: [Yr | Yi], 1: [-Yi | Yr]), part p (0: the real
+// Byte offset of digit t, form f (0: [Yr | Yi], 1: [-Yi | Yr]), part p (of `part` bytes) (0: the real
 // accumulator rows, 1: the imaginary ones), column c, inner index k of a group's stage.
-// Consecutive 8-row blocks of a tile's operand are PART bytes apart in every (t, f).
-__device__ __forceinline__ int stage_off(int t, int f, int p, int c, int k) {
-  return p * PART + (t * 2 + f) * 512 + (k >> 3) * 128 + c * 16 + (k & 7) * 2;
+// Consecutive 8-row blocks of a tile's operand are `part` bytes apart in every (t, f).
+__device__ __forceinline__ int stage_off(int part, int t, int f, int p, int c, int k) {
+  return p * part + (t * 2 + f) * 512 + (k >> 3) * 128 + c * 16 + (k & 7) * 2;
 }
 
 // 2^e, exact for every e that a double holds.
@@ -56,7 +73,7 @@ __device__ __forceinline__ double pow2(int e) {
 __device__ __forceinline__ int terms_of(const ProblemDev& P) { return P.bie ? 1 : P.n_dense; }
 
 // Digits of f_d X of the active nodes, one CTA per node and dense term; CTA 0 also
-// counts the residual tiles before each problem.
+// counts the residual tiles before each problem, by form.
 __global__ void __launch_bounds__(DIGIT_THREADS) k_oz_digits(MixedArgs a, int sw, int max_dense) {
   __shared__ double red[DIGIT_THREADS];
   __shared__ int g[CG];
@@ -65,26 +82,28 @@ __global__ void __launch_bounds__(DIGIT_THREADS) k_oz_digits(MixedArgs a, int sw
   const int active = a.ctl[MIXED_CTL_ACTIVE + sw];
   if (blockIdx.x == 0 && tid < 32) {
     const int* uc = mixed_ucount(a, sw);
-    int* tiles = mixed_tiles(a);
-    int base = 0;
-    for (int p0 = 0; p0 < a.n_probs; p0 += 32) {
-      const int p = p0 + tid;
-      int v = 0;
-      if (p < a.n_probs) {
-        // problems share their tiles among nodes; a boundary-integral node has its own
-        const int ncg = (a.probs[p].l + CG - 1) / CG;
-        v = (a.probs[p].bie ? uc[p] / ncg * ((ncg + MAXG - 1) / MAXG) : (uc[p] + MAXG - 1) / MAXG) *
-            row_blocks(a.probs[p].n);
+    for (int f = 0; f < 2; ++f) {
+      int* tiles = mixed_tiles(a, f != 0);
+      int base = 0;
+      for (int p0 = 0; p0 < a.n_probs; p0 += 32) {
+        const int p = p0 + tid;
+        int v = 0;
+        if (p < a.n_probs && (a.probs[p].bie != nullptr) == (f != 0)) {
+          // problems share their tiles among nodes; a boundary-integral node has its own
+          const int ncg = (a.probs[p].l + CG - 1) / CG;
+          constexpr int GB = Form<true>::MAXG, GD = Form<false>::MAXG;
+          v = (f ? uc[p] / ncg * ((ncg + GB - 1) / GB) : (uc[p] + GD - 1) / GD) * row_blocks(a.probs[p].n);
+        }
+        const int own = v;
+        for (int o = 1; o < 32; o <<= 1) {
+          const int x = __shfl_up_sync(0xffffffffu, v, o);
+          if (tid >= o) v += x;
+        }
+        if (p < a.n_probs) tiles[p] = base + v - own;
+        base += __shfl_sync(0xffffffffu, v, 31);
       }
-      const int own = v;
-      for (int o = 1; o < 32; o <<= 1) {
-        const int x = __shfl_up_sync(0xffffffffu, v, o);
-        if (tid >= o) v += x;
-      }
-      if (p < a.n_probs) tiles[p] = base + v - own;
-      base += __shfl_sync(0xffffffffu, v, 31);
+      if (tid == 0) tiles[a.n_probs] = base;
     }
-    if (tid == 0) tiles[a.n_probs] = base;
   }
   for (int w = blockIdx.x; w < active * max_dense; w += gridDim.x) {
     const int q = a.act[(size_t)(sw & 1) * a.slots + w / max_dense], dd = w % max_dense;
@@ -93,6 +112,7 @@ __global__ void __launch_bounds__(DIGIT_THREADS) k_oz_digits(MixedArgs a, int sw
     const ProblemDev& P = a.probs[rg.prob];
     if (dd >= terms_of(P) || !mixed_node_oz(a, P, rg)) continue;  // the same in every thread
     const int n = P.n, l = P.l, kcn = k_chunks(n), ncg = (l + CG - 1) / CG;
+    const int digits = P.bie ? Form<true>::S : Form<false>::S, stage = P.bie ? Form<true>::STAGE : Form<false>::STAGE;
     __syncthreads();  // f_sh and g of the previous node
     if (tid == 0) {
       if (P.bie) {
@@ -130,10 +150,10 @@ __global__ void __launch_bounds__(DIGIT_THREADS) k_oz_digits(MixedArgs a, int sw
         }
         __syncthreads();
       }
-      unsigned char* dst = a.ysl + (size_t)q * a.ysl_stride + (size_t)(dd * ncg + cg) * kcn * GROUP_STAGE;
+      unsigned char* dst = a.ysl + (size_t)q * a.ysl_stride + (size_t)(dd * ncg + cg) * kcn * stage;
       for (int task = tid; task < CG * kcn * (KC / 8); task += DIGIT_THREADS) {
         const int cc = task & (CG - 1), j0 = (task / CG) * 8, c = cg * CG + cc;
-        const int shift = DIGIT_SHIFT - g[cc];
+        const int shift = 7 * digits - 1 - g[cc];
         const bool normal = shift >= -1022 && shift <= 1023;  // 2^shift is a normal number
         const double up = normal ? pow2(shift) : 0.0;
         long long Nr[8], Ni[8];
@@ -144,9 +164,9 @@ __global__ void __launch_bounds__(DIGIT_THREADS) k_oz_digits(MixedArgs a, int sw
           Nr[u] = __double2ll_rn(normal ? y.x * up : scalbn(y.x, shift));
           Ni[u] = __double2ll_rn(normal ? y.y * up : scalbn(y.y, shift));
         }
-        unsigned char* st = dst + (size_t)(j0 / KC) * GROUP_STAGE;
+        unsigned char* st = dst + (size_t)(j0 / KC) * stage;
 #pragma unroll 1
-        for (int t = S - 1; t >= 0; --t) {
+        for (int t = digits - 1; t >= 0; --t) {
           uint32_t pr[4], pi[4], nr[4];
 #pragma unroll
           for (int u = 0; u < 8; u += 2) {
@@ -157,19 +177,20 @@ __global__ void __launch_bounds__(DIGIT_THREADS) k_oz_digits(MixedArgs a, int sw
             nr[u / 2] = (uint32_t)bf16_of_int(-i0) | ((uint32_t)bf16_of_int(-i1) << 16);
           }
           const int k = j0 % KC;
-          *reinterpret_cast<uint4*>(st + stage_off(t, 0, 0, cc, k)) = make_uint4(pr[0], pr[1], pr[2], pr[3]);
-          *reinterpret_cast<uint4*>(st + stage_off(t, 0, 1, cc, k)) = make_uint4(pi[0], pi[1], pi[2], pi[3]);
-          *reinterpret_cast<uint4*>(st + stage_off(t, 1, 0, cc, k)) = make_uint4(nr[0], nr[1], nr[2], nr[3]);
-          *reinterpret_cast<uint4*>(st + stage_off(t, 1, 1, cc, k)) = make_uint4(pr[0], pr[1], pr[2], pr[3]);
+          *reinterpret_cast<uint4*>(st + stage_off(stage / 2, t, 0, 0, cc, k)) = make_uint4(pr[0], pr[1], pr[2], pr[3]);
+          *reinterpret_cast<uint4*>(st + stage_off(stage / 2, t, 0, 1, cc, k)) = make_uint4(pi[0], pi[1], pi[2], pi[3]);
+          *reinterpret_cast<uint4*>(st + stage_off(stage / 2, t, 1, 0, cc, k)) = make_uint4(nr[0], nr[1], nr[2], nr[3]);
+          *reinterpret_cast<uint4*>(st + stage_off(stage / 2, t, 1, 1, cc, k)) = make_uint4(pr[0], pr[1], pr[2], pr[3]);
         }
       }
     }
   }
 }
 
+template <bool BIE>
 struct GemmSmem {
   alignas(1024) unsigned char a[RA][A_STAGE];
-  alignas(1024) unsigned char b[RB2][MAXG * GROUP_STAGE];
+  alignas(1024) unsigned char b[RB2][Form<BIE>::MAXG * Form<BIE>::STAGE];
   uint64_t a_full[RA], a_empty[RA], b_full[RB2], b_empty[RB2], acc_full, acc_empty, last;
   uint32_t a_issued, b_issued;  // copies issued, for the settling wait
   uint32_t tmem;
@@ -183,19 +204,21 @@ struct Tile {
 };
 
 // Walks this CTA's tiles (blockIdx.x, + gridDim.x, ...) in order.
+template <bool BIE>
 struct TileWalk {
   const MixedArgs& a;
   const int* tiles;
   const int* uc;
   int sw, t, p;
   __device__ TileWalk(const MixedArgs& a_, int sw_)
-      : a(a_), tiles(mixed_tiles(a_)), uc(mixed_ucount(a_, sw_)), sw(sw_), t((int)blockIdx.x), p(0) {}
+      : a(a_), tiles(mixed_tiles(a_, BIE)), uc(mixed_ucount(a_, sw_)), sw(sw_), t((int)blockIdx.x), p(0) {}
   __device__ bool next(Tile& out) {
     if (t >= tiles[a.n_probs]) return false;
     while (tiles[p + 1] <= t) ++p;
     const int rbn = row_blocks(a.probs[p].n), loc = t - tiles[p];
+    constexpr int MAXG = Form<BIE>::MAXG;
     int u0 = loc / rbn * MAXG, end = uc[p];
-    if (a.probs[p].bie) {  // a node's groups are consecutive
+    if (BIE) {  // a node's groups are consecutive
       const int ncg = (a.probs[p].l + CG - 1) / CG, per = (ncg + MAXG - 1) / MAXG, node = loc / rbn / per;
       u0 = node * ncg + loc / rbn % per * MAXG;
       end = (node + 1) * ncg;
@@ -259,8 +282,10 @@ __device__ __forceinline__ void tmem_ld16(uint32_t addr, uint32_t (&r)[16]) {
 }
 
 // warp 0, one lane
-__device__ void copy_role(const MixedArgs& a, int sw, GemmSmem& sm) {
-  TileWalk walk(a, sw);
+template <bool BIE>
+__device__ void copy_role(const MixedArgs& a, int sw, GemmSmem<BIE>& sm) {
+  constexpr int S = Form<BIE>::S, MAXG = Form<BIE>::MAXG, STAGE = Form<BIE>::STAGE;
+  TileWalk<BIE> walk(a, sw);
   Tile t;
   uint32_t na = 0, nb = 0;
   bool ok = true;
@@ -269,18 +294,17 @@ __device__ void copy_role(const MixedArgs& a, int sw, GemmSmem& sm) {
     const int rbn = row_blocks(P.n), kcn = k_chunks(P.n), ncg = (P.l + CG - 1) / CG;
     const unsigned char* src[MAXG];
     for (int g = 0; g < t.ng; ++g)
-      src[g] = a.ysl + (size_t)(t.units[g] >> 3) * a.ysl_stride + (size_t)(t.units[g] & 7) * kcn * GROUP_STAGE;
-    const unsigned char* digits = P.bie ? a.tdig + (size_t)(t.units[0] >> 3) * a.tdig_stride : P.Adig;
+      src[g] = a.ysl + (size_t)(t.units[g] >> 3) * a.ysl_stride + (size_t)(t.units[g] & 7) * kcn * STAGE;
+    const unsigned char* digits = BIE ? a.tdig + (size_t)(t.units[0] >> 3) * a.tdig_stride : P.Adig;
     for (int dd = 0; dd < terms_of(P) && ok; ++dd) {
       const unsigned char* asrc = digits + ((size_t)dd * rbn + t.rb) * kcn * S * A_STAGE;
       for (int kc = 0; kc < kcn && ok; ++kc) {
         const uint32_t bi = nb % RB2, bk = nb / RB2;
         ok = bk == 0 || wait_or_bad(&sm.b_empty[bi], (bk - 1) & 1u, a.tc_wait_cycles, &sm.bad);
         if (!ok) break;
-        expect_tx(&sm.b_full[bi], (uint32_t)t.ng * GROUP_STAGE);
+        expect_tx(&sm.b_full[bi], (uint32_t)t.ng * STAGE);
         for (int g = 0; g < t.ng; ++g)
-          bulk_g2s(sm.b[bi] + g * GROUP_STAGE, src[g] + ((size_t)dd * ncg * kcn + kc) * GROUP_STAGE, GROUP_STAGE,
-                   &sm.b_full[bi]);
+          bulk_g2s(sm.b[bi] + g * STAGE, src[g] + ((size_t)dd * ncg * kcn + kc) * STAGE, STAGE, &sm.b_full[bi]);
         ++nb;
         for (int s = 0; s < S; ++s) {
           const uint32_t ai = na % RA, ak = na / RA;
@@ -298,8 +322,10 @@ __device__ void copy_role(const MixedArgs& a, int sw, GemmSmem& sm) {
 }
 
 // warp 1, one lane
-__device__ void mma_role(const MixedArgs& a, int sw, GemmSmem& sm) {
-  TileWalk walk(a, sw);
+template <bool BIE>
+__device__ void mma_role(const MixedArgs& a, int sw, GemmSmem<BIE>& sm) {
+  constexpr int S = Form<BIE>::S, QMAX = Form<BIE>::QMAX, MAXG = Form<BIE>::MAXG, PART = Form<BIE>::PART;
+  TileWalk<BIE> walk(a, sw);
   Tile t;
   uint32_t na = 0, nb = 0, blk = 0;
   bool ok = true;
@@ -353,11 +379,13 @@ __device__ void mma_role(const MixedArgs& a, int sw, GemmSmem& sm) {
 }
 
 // warps 4-19
-__device__ void drain_role(const MixedArgs& a, int sw, GemmSmem& sm) {
+template <bool BIE>
+__device__ void drain_role(const MixedArgs& a, int sw, GemmSmem<BIE>& sm) {
+  constexpr int NQ = Form<BIE>::NQ, MAXG = Form<BIE>::MAXG;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int quad = warp & 3, gi = (warp - DRAIN_WARP0) >> 2;
   const uint32_t base = sm.tmem + ((uint32_t)(32 * quad) << 16) + (uint32_t)(16 * gi);
-  TileWalk walk(a, sw);
+  TileWalk<BIE> walk(a, sw);
   Tile t;
   uint32_t blk = 0;
   while (walk.next(t)) {
@@ -372,6 +400,51 @@ __device__ void drain_role(const MixedArgs& a, int sw, GemmSmem& sm) {
     double2* R = reinterpret_cast<double2*>(a.work + (size_t)q * a.slot_bytes + mixed_residual_offset(n, l)) +
                  (size_t)cg * CG * n + row;
     const int cols = min(CG, l - cg * CG);
+    if constexpr (BIE) {
+      // exact sums of the orders' upper and lower part over all inner indices
+      constexpr int NHI = NQ - 4;
+      long long hi[2 * CG], lo[2 * CG];  // hi 2^28 + lo, in units of the last order
+#pragma unroll
+      for (int c = 0; c < 2 * CG; ++c) hi[c] = lo[c] = 0;
+      for (int kc0 = 0; kc0 < kcn; kc0 += KD / KC) {
+        const bool ok = wait_or_bad(&sm.acc_full, blk & 1u, a.handoff_wait_cycles, &sm.bad, LOST_HANDOFF);
+        if (!__all_sync(0xffffffffu, ok)) return;  // sm.bad is set
+        ++blk;
+        tcu::fence_after();
+        if (mine) {
+#pragma unroll
+          for (int h = 0; h < NQ; ++h) {
+            uint32_t v[16];
+            tmem_ld16(base + (uint32_t)(h * 16 * MAXG), v);
+#pragma unroll
+            for (int c = 0; c < 2 * CG; ++c) {
+              const long long d = (long long)__float2int_rn(__uint_as_float(v[c]));
+              if (h < NHI) hi[c] += d * (1 << (7 * (NHI - 1 - h)));
+              else lo[c] += d * (1 << (7 * (NQ - 1 - h)));
+            }
+          }
+        }
+        tcu::fence_before();
+        __syncwarp();
+        if (lane == 0) arrive(&sm.acc_empty);
+      }
+      if (mine && row < n) {
+        const int er = a.texp[(size_t)q * a.texp_stride + t.rb * TM + 32 * quad + lane];
+        const int* ge = a.gexp + (size_t)q * a.gexp_stride + cg * CG;
+#pragma unroll
+        for (int c = 0; c < CG; ++c) {
+          if (c < cols) {
+            double2 v = P.V[(size_t)(cg * CG + c) * n + row];
+            const int e = er + ge[c] - Form<true>::SCALE;
+            const double s1 = -pow2(e), s2 = -pow2(e + 28);
+            v.x = fma(s2, (double)hi[c], fma(s1, (double)lo[c], v.x));
+            v.y = fma(s2, (double)hi[CG + c], fma(s1, (double)lo[CG + c], v.y));
+            R[(size_t)c * n] = v;
+          }
+        }
+      }
+      continue;
+    }
     double r[2 * CG];  // R's columns of the group: real parts, imaginary parts
     if (mine && row < n) {
       const double2 id = a.state[q].id;
@@ -392,8 +465,7 @@ __device__ void drain_role(const MixedArgs& a, int sw, GemmSmem& sm) {
       int ge[CG];
       int er = 0;
       if (mine && row < n) {
-        const int32_t* ex = P.bie ? a.texp + (size_t)q * a.texp_stride : P.Aexp;
-        er = ex[((size_t)dd * rbn + t.rb) * TM + 32 * quad + lane];
+        er = P.Aexp[((size_t)dd * rbn + t.rb) * TM + 32 * quad + lane];
 #pragma unroll
         for (int c = 0; c < CG; ++c)
           ge[c] = a.gexp[(size_t)q * a.gexp_stride + (dd * ncg + cg) * CG + c] + er - DRAIN_SCALE;
@@ -439,11 +511,12 @@ __device__ void drain_role(const MixedArgs& a, int sw, GemmSmem& sm) {
   }
 }
 
+template <bool BIE>
 __global__ void __launch_bounds__(GEMM_THREADS, 1) k_oz_residual(MixedArgs a, int sw) {
   extern __shared__ __align__(1024) unsigned char smem_raw[];
-  GemmSmem& sm = *reinterpret_cast<GemmSmem*>(smem_raw);
+  GemmSmem<BIE>& sm = *reinterpret_cast<GemmSmem<BIE>*>(smem_raw);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  if ((int)blockIdx.x >= mixed_tiles(a)[a.n_probs] || *reinterpret_cast<volatile int32_t*>(a.err)) return;
+  if ((int)blockIdx.x >= mixed_tiles(a, BIE)[a.n_probs] || *reinterpret_cast<volatile int32_t*>(a.err)) return;
   const long long t0 = clock64();
   const unsigned long long w0 = global_ns();
   if (warp == 2) tcu::tmem_alloc_cols(&sm.tmem, 512);
@@ -488,7 +561,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1) k_oz_residual(MixedArgs a, in
       if (sm.bad == LOST_HANDOFF) atomicExch(a.err, 1);
     }
     // the nodes of this CTA's tiles have no valid residual
-    TileWalk walk(a, sw);
+    TileWalk<BIE> walk(a, sw);
     Tile t;
     while (walk.next(t))
       if (tid < t.ng) atomicOr(&a.state[t.units[tid] >> 3].lost, MIXED_LOST_RESIDUAL);
@@ -504,19 +577,33 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1) k_oz_residual(MixedArgs a, in
 
 }  // namespace
 
-size_t oz_slot_bytes(int n, int l, int n_dense) {
-  return (size_t)n_dense * ((l + CG - 1) / CG) * k_chunks(n) * GROUP_STAGE;
+// terms: dense terms, 0 for a boundary-integral node
+size_t oz_slot_bytes(int n, int l, int terms) {
+  const size_t groups = (size_t)((l + CG - 1) / CG) * k_chunks(n);
+  return terms > 0 ? terms * groups * Form<false>::STAGE : groups * Form<true>::STAGE;
 }
 
 cudaError_t prepare_oz_refine() {
-  return cudaFuncSetAttribute(k_oz_residual, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(GemmSmem));
+  cudaError_t e = cudaFuncSetAttribute(k_oz_residual<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)sizeof(GemmSmem<false>));
+  if (e != cudaSuccess) return e;
+  return cudaFuncSetAttribute(k_oz_residual<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              (int)sizeof(GemmSmem<true>));
 }
 
-cudaError_t launch_oz_residual(const MixedArgs& a, int sw, int sms, cudaStream_t s) {
-  static_assert(sizeof(GemmSmem) <= 227 * 1024, "one CTA per SM");
+cudaError_t launch_oz_residual(const MixedArgs& a, int sw, int sms, cudaStream_t s, int* launched) {
+  static_assert(sizeof(GemmSmem<false>) <= 227 * 1024 && sizeof(GemmSmem<true>) <= 227 * 1024, "one CTA per SM");
   const int nd = a.gexp_stride / PMCIM_MAX_L;
   const long long w = (long long)a.count * nd;
   k_oz_digits<<<(unsigned)(w < 4 * sms ? w : 4 * sms), DIGIT_THREADS, 0, s>>>(a, sw, nd);
-  k_oz_residual<<<sms, GEMM_THREADS, sizeof(GemmSmem), s>>>(a, sw);
+  ++*launched;
+  if (a.oz_dense) {
+    k_oz_residual<false><<<sms, GEMM_THREADS, sizeof(GemmSmem<false>), s>>>(a, sw);
+    ++*launched;
+  }
+  if (a.tdig) {
+    k_oz_residual<true><<<sms, GEMM_THREADS, sizeof(GemmSmem<true>), s>>>(a, sw);
+    ++*launched;
+  }
   return cudaGetLastError();
 }

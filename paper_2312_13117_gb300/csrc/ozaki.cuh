@@ -60,6 +60,7 @@ constexpr int B_STAGE = 2 * S * B_TILE;  // both operands of every digit t: 28 K
 constexpr int NA = 3;                 // A stages in the ring
 constexpr int NBUF = 2;               // B stages in the ring
 constexpr uint32_t TMEM_COLS = NQ * TN;  // 256
+constexpr int BIE_DIGITS = 8;         // of a boundary-integral node's T(z_j) (oz_refine.cu)
 constexpr int DIGIT_SHIFT = 48;       // N = rint(x 2^(48 - exponent)), |N| <= 2^48
 constexpr int DRAIN_SCALE = 61;       // H 2^(e + g - 61) is the block's product (96 - 35)
 

@@ -284,7 +284,8 @@ struct MixedState {
 };
 constexpr int MIXED_LOST_LU = 1, MIXED_LOST_RESIDUAL = 2;
 // ctl: work counters, active nodes per sweep, then the column groups per sweep and problem
-// (all zero at a chunk's start), then the residual tiles before each problem
+// (all zero at a chunk's start), then the residual tiles before each problem, those of dense
+// terms and those of boundary-integral nodes
 constexpr int MIXED_CTL_FACTOR = 0, MIXED_CTL_FIRST = 1, MIXED_CTL_FALLBACK = 2, MIXED_CTL_FALLBACK_COUNT = 3,
               MIXED_CTL_ACTIVE = 16, MIXED_CTL_SWEEP = 32, MIXED_CTL_UNITS = 48;
 constexpr int MIXED_MAX_SWEEPS = 10;
@@ -309,6 +310,7 @@ struct MixedArgs {
   int tc;              // a region updates on the tensor cores (RegionDev::lu_tc)
   int bie;             // a problem has a boundary-integral term
   int oz;              // refinement residuals on the tensor cores
+  int oz_dense;        // some of them from the digits of dense terms
   int res64;           // a node forms its residuals on the FP64 pipe
   // boundary-integral nodes (bie_nodes.cu): per slot, the exact digits of T(z_j) and their row
   // exponents (NULL: residuals on the FP64 pipe)
@@ -344,7 +346,7 @@ __host__ __device__ inline size_t mixed_ctl_zero_ints(int n_probs, int rounds) {
   return MIXED_CTL_UNITS + (size_t)(rounds + 1) * n_probs;
 }
 __host__ __device__ inline size_t mixed_ctl_ints(int n_probs, int rounds) {
-  return mixed_ctl_zero_ints(n_probs, rounds) + n_probs + 1;
+  return mixed_ctl_zero_ints(n_probs, rounds) + 2 * (n_probs + 1);
 }
 // Whether the node's residuals are formed on the tensor cores.
 __device__ __forceinline__ bool mixed_node_oz(const MixedArgs& a, const ProblemDev& P, const RegionDev& rg) {
@@ -357,8 +359,9 @@ __device__ __forceinline__ bool mixed_column_only(const MixedArgs& a, const Prob
 __device__ __forceinline__ int* mixed_ucount(const MixedArgs& a, int sw) {
   return a.ctl + MIXED_CTL_UNITS + (size_t)sw * a.n_probs;
 }
-__device__ __forceinline__ int* mixed_tiles(const MixedArgs& a) {
-  return a.ctl + mixed_ctl_zero_ints(a.n_probs, mixed_rounds(a.max_sweeps, a.border != nullptr));
+__device__ __forceinline__ int* mixed_tiles(const MixedArgs& a, bool bie) {
+  return a.ctl + mixed_ctl_zero_ints(a.n_probs, mixed_rounds(a.max_sweeps, a.border != nullptr)) +
+         (bie ? a.n_probs + 1 : 0);
 }
 // Phase-clock slots (PMCIM_PHASES): SM cycles summed over CTAs, by step.
 enum { PH_ASSEMBLE = 0, PH_PANEL = 1, PH_FIRST_SOLVE = 2, PH_RESIDUAL = 3, PH_CORRECTION = 4, PH_FALLBACK = 5,
@@ -383,8 +386,9 @@ cudaError_t launch_factor_solve_mixed(const MixedArgs& a, int sms, cudaStream_t 
 cudaError_t launch_bie_assemble(const MixedArgs& a, int sms, cudaStream_t s, int* launched);
 // the residuals of sweep sw's active nodes (oz_refine.cu)
 cudaError_t prepare_oz_refine();
-cudaError_t launch_oz_residual(const MixedArgs& a, int sw, int sms, cudaStream_t s);
-size_t oz_slot_bytes(int n, int l, int n_dense);  // digits of f_k X of one slot
+cudaError_t launch_oz_residual(const MixedArgs& a, int sw, int sms, cudaStream_t s, int* launched);
+size_t oz_slot_bytes(int n, int l, int terms);  // digits of f_k X of one slot
+size_t bie_digit_bytes(int n);                  // digits of a boundary-integral node's T(z_j)
 // dst[i] = complex64(src[i]), i < count (the FP32 copy of the coefficients)
 cudaError_t round_coefficients_c64(const double2* src, float2* dst, size_t count, cudaStream_t s);
 // Exact BF16 digits of the n_dense dense coefficients (ozaki.cu): row exponents
