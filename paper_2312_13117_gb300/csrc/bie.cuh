@@ -123,8 +123,8 @@ BIE_HD Wave wave_of(double2 kappa) {
 //    coefficients, by Horner's rule, 8 FP64 operations per term (a term with a running
 //    product and a stopping test took about 20, and FP64 bounds the assembly). The number
 //    of terms, ceil(5.9 + 3 |w| - 0.095 |w|^2), leaves out less than 1e-17 of the largest
-//    term; a warp takes its largest, so that its lanes read the same coefficients. Near the
-//    real axis the sums cancel to e^{-|w|} of their largest term, which sets the range.
+//    term; each entry takes its own, so that its value does not depend on the entries that
+//    share its warp. Near the real axis the sums cancel to e^{-|w|} of their largest term, which sets the range.
 //  6 < |w| <= 13: J_k by the backward recurrence J_{k-1} = (2k / w) J_k - J_{k+1} (DLMF
 //    3.6(iii)) from k = 46, scaled by e^{+-iw} = J_0 + 2 sum_k (+-i)^k J_k (DLMF 10.12.1; the
 //    sign that makes the left side large), and Y_1 by Neumann's series (Abramowitz & Stegun
@@ -144,9 +144,6 @@ BIE_HD void j1_h1(const Wave& W, double r, double ri, double lr, double2* J, dou
     const double2 u = make_double2(h.y * h.y - h.x * h.x, -2.0 * h.x * h.y);  // -(w/2)^2
     const float fw = (float)aw;
     int k = (int)ceilf(5.9f + fw * (3.0f - 0.095f * fw)) - 1;
-#if defined(__CUDA_ARCH__)
-    k = __reduce_max_sync(__activemask(), k);
-#endif
     double2 p = make_double2(TB.cj[k], 0.0), q = make_double2(TB.cs[k], 0.0);
     for (--k; k >= 0; --k) {
       const double px = fma(p.x, u.x, fma(-p.y, u.y, TB.cj[k])), qx = fma(q.x, u.x, fma(-q.y, u.y, TB.cs[k]));
@@ -249,10 +246,11 @@ BIE_ENTRY void dlp_pair(const double* G, int n, int i, int j, const Wave& W, dou
   const double rr = ex * ex + ey * ey;
 #if defined(__CUDA_ARCH__)
   const double ri = rsqrt(rr);
+  double r = rr * ri;
+  r = fma(0.5 * ri, fma(-r, r, rr), r);  // one Newton step: the rounding of ri stays out of r
 #else
-  const double ri = 1.0 / sqrt(rr);
+  const double r = sqrt(rr), ri = 1.0 / r;
 #endif
-  const double r = rr * ri;
   double2 J1, H1;
   j1_h1(W, r, ri, log(r), &J1, &H1);
   const int m = i > j ? i - j : i - j + n;
