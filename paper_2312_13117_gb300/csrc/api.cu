@@ -537,7 +537,9 @@ void plan_mixed(Workspace& ws, const std::vector<ProblemDev>& pd, const std::vec
       mp->ubase.push_back(base);
       base += u;
     }
-    ch.work = std::max(ch.count * slot, mixed_fallback_bytes(ch.max_n, ch.max_l));
+    // the slots, and in their place the FP64 matrices of as many nodes as are solved again at a time
+    const size_t fb = mixed_fallback_bytes(ch.max_n, ch.max_l);
+    ch.work = std::max(ch.count * slot, fb * std::max<size_t>(1, std::min({ch.count, 2 * (size_t)sms, budget / fb})));
     ch.t64_off = align(ch.work);
     ch.ysl_off = align(ch.t64_off + ch.count * ch.t64_stride * sizeof(double2));
     ch.tdig_off = align(ch.ysl_off + ch.count * ch.ysl_stride);

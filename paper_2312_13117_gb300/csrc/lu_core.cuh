@@ -423,12 +423,12 @@ __device__ __forceinline__ void block_update_row(const T2* __restrict__ M, T2* _
 }
 
 
-// U x = y, U upper with its diagonal.
+// U x = y, U upper with its diagonal, for the l columns from n + c0 on.
 template <typename T2>
-__device__ void cta_back_blocked(T2* __restrict__ M, int n, int l, LuSmemT<T2>& sm) {
+__device__ void cta_back_blocked(T2* __restrict__ M, int n, int l, LuSmemT<T2>& sm, int c0 = 0) {
   const int tid = gtid(), lane = tid & 31, wid = tid >> 5;
   const size_t ld = (size_t)n;
-  T2* Y = M + (size_t)n * ld;
+  T2* Y = M + (size_t)(n + c0) * ld;
   const int nblk = (n + NB - 1) / NB;
   for (int b = nblk - 1; b >= 0; --b) {
     const int k0 = b * NB;

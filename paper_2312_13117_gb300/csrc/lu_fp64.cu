@@ -16,7 +16,7 @@
 //
 // Pivot rule: the row maximising |Re| + |Im| in the column, lowest row index on
 // ties (the BLAS izamax convention of LAPACK zgetrf).
-#include "lu_core.cuh"
+#include "cluster_lu.cuh"
 
 namespace {
 
@@ -116,103 +116,8 @@ struct VerifySmem {
   ProblemDev P;
   bie::Wave wave;
   double red[THREADS / 32];
-  int row[2 * NB], src[2 * NB];  // a panel's interchanges: row[i] takes the old row src[i]
+  Interchanges swaps;
 };
-
-// Few values leave most SMs idle with one CTA per value, so the CTAs of a cluster share one:
-// the LU of order 512 takes 52 ms on one SM, on the FP64 pipe, and 18.7 on 4 (7.6 of it the
-// panels, which one CTA factors). Every CTA of a cluster reaches every barrier below.
-__device__ __forceinline__ void cluster_sync() {
-  asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
-}
-__device__ __forceinline__ int cluster_rank() {
-  unsigned r;
-  asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-  return (int)r;
-}
-
-__device__ __forceinline__ double2 shfl2(double2 v, int src) {
-  return make_double2(__shfl_sync(0xffffffffu, v.x, src), __shfl_sync(0xffffffffu, v.y, src));
-}
-
-// A panel's interchanges on all other columns and U12 = L11^{-1} A12 on those right of it:
-// a warp takes four columns, lane t the rows k0 + t and piv[k0 + t].
-__device__ void swap_and_trsm(double2* M, int n, int k0, int kb, const int* piv, VerifySmem& sm, int rank, int size) {
-  const int tid = threadIdx.x, lane = tid & 31;
-  if (tid < 2 * NB) {  // follow one row back through the interchanges
-    const int t = tid & (NB - 1);
-    int r = t >= kb ? 0 : (tid < NB ? k0 + t : piv[k0 + t]);
-    sm.row[tid] = r;
-    for (int j = kb - 1; j >= 0; --j) {
-      const int p = piv[k0 + j];
-      r = r == k0 + j ? p : (r == p ? k0 + j : r);
-    }
-    sm.src[tid] = r;
-  }
-#pragma unroll
-  for (int u = 0; u < NB * NB / THREADS; ++u) {
-    const int e = tid + u * THREADS, i = e & (NB - 1), t = e / NB;
-    sm.lu.Ls[e] = i < kb && t < kb && i > t ? M[(size_t)(k0 + t) * n + k0 + i] : make_double2(0.0, 0.0);
-  }
-  __syncthreads();
-  const bool live = lane < kb;
-  const int s0 = sm.src[lane], r1 = sm.row[NB + lane], s1 = sm.src[NB + lane];
-  constexpr int CW = 4;
-  for (int g = (rank * THREADS + tid) >> 5; g * CW < n; g += size * (THREADS / 32)) {
-    double2 x[CW], y[CW];
-#pragma unroll
-    for (int q = 0; q < CW; ++q) {
-      const int c = g * CW + q;
-      const bool in = live && c < n && (c < k0 || c >= k0 + kb);
-      x[q] = in ? M[(size_t)c * n + s0] : make_double2(0.0, 0.0);
-      y[q] = in ? M[(size_t)c * n + s1] : make_double2(0.0, 0.0);
-    }
-    __syncwarp();
-    // rows below the panel's, before the panel's own (a row piv[k0 + t] may be one of those:
-    // both then hold the same value)
-#pragma unroll
-    for (int q = 0; q < CW; ++q) {
-      const int c = g * CW + q;
-      if (live && r1 >= k0 + kb && c < n && (c < k0 || c >= k0 + kb)) M[(size_t)c * n + r1] = y[q];
-    }
-    if ((g + 1) * CW > k0 + kb)
-      for (int t = 0; t < kb - 1; ++t) {
-        const double2 lt = sm.lu.Ls[t * NB + lane];
-#pragma unroll
-        for (int q = 0; q < CW; ++q) {
-          const double2 xt = shfl2(x[q], t);
-          if (g * CW + q >= k0 + kb && lane > t) cfms(x[q], lt, xt);
-        }
-      }
-#pragma unroll
-    for (int q = 0; q < CW; ++q) {
-      const int c = g * CW + q;
-      if (live && c < n && (c < k0 || c >= k0 + kb)) M[(size_t)c * n + k0 + lane] = x[q];
-    }
-  }
-}
-
-// LU of the n x n matrix M by a cluster of `size` CTAs: the first factors the panels, all share
-// the interchanges, the triangular solves and the trailing updates. Returns 0, or 1 + the
-// first column whose pivot was exactly zero (*flag: its way to the other CTAs).
-__device__ int cluster_lu(double2* M, int n, int* piv, int* flag, VerifySmem& sm, int rank, int size) {
-  if (threadIdx.x == 0) sm.lu.info_sh = 0;
-  __syncthreads();
-  for (int k0 = 0; k0 < n; k0 += NB) {
-    const int kb = min(NB, n - k0);
-    if (rank == 0) {
-      cta_lu_panel(M, n, k0 + kb, k0, kb, piv, sm.lu, k0);
-      if (threadIdx.x == 0) *flag = sm.lu.info_sh;
-    }
-    cluster_sync();
-    swap_and_trsm(M, n, k0, kb, piv, sm, rank, size);
-    cluster_sync();
-    if (k0 + kb >= n) break;
-    cta_lu_update_simt<double2, 2>(M, n, n, k0, kb, sm.lu, rank, size);
-    cluster_sync();
-  }
-  return *flag;
-}
 
 // ---------------------------------------------------------------------------
 // The inverse iteration's triangular solves with one right-hand side, by the whole cluster in
@@ -400,8 +305,8 @@ __global__ void __launch_bounds__(THREADS, 2) k_verify_fp64(ValueArgs a) {
       for (size_t e = tid; e < nn; e += THREADS) fro += cabs2(M[e]);
       fro = sqrt(block_sum(fro, sm.red));
     }
-    const int info = cluster_lu(M, n, piv, reinterpret_cast<int*>(dinvU + (size_t)(n + NB - 1) / NB * NB * NB), sm,
-                                rank, size);
+    const int info = cluster_lu(M, n, n, piv, reinterpret_cast<int*>(dinvU + (size_t)(n + NB - 1) / NB * NB * NB),
+                                sm.lu, sm.swaps, rank, size);
 
     // Inverse iteration on T^H T; T = P^T L U, and as w = T^{-H} x is only needed as P w, the
     // interchanges drop out. Every CTA forms the norms, from the same numbers in the same order.

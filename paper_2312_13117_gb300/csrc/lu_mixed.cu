@@ -40,6 +40,7 @@
 #include "ozaki.cuh"
 #include "tc_update_bf16.cuh"
 #include "lu32.cuh"
+#include "cluster_lu.cuh"
 
 namespace {
 
@@ -136,6 +137,7 @@ constexpr size_t kSolveYBytes = 46 * 1024;
 
 struct FallbackSmem {
   LuSmemT<double2> lu64;
+  Interchanges swaps;
   NodeCtx c;
 };
 
@@ -457,12 +459,12 @@ __device__ void assemble32(const NodeCtx& cx, float2* __restrict__ M32) {
   }
 }
 
-// T(z_j) in FP64 for the fallback.
-__device__ void assemble(const NodeCtx& cx, double2* M64) {
+// T(z_j) in FP64 for the fallback: columns rank, rank + size, ...
+__device__ void assemble(const NodeCtx& cx, double2* M64, int rank, int size) {
   const ProblemDev& P = cx.P;
   const int n = P.n;
   const size_t nn = (size_t)n * n;
-  for (int col = 0; col < n; ++col) {
+  for (int col = rank; col < n; col += size) {
     for (int row = gtid(); row < n; row += THREADS) {
       const size_t e = (size_t)col * n + row;
       double2 v = make_double2(0.0, 0.0);
@@ -760,18 +762,25 @@ __global__ void __launch_bounds__(THREADS, 3) k_mixed_solve(MixedArgs a, int sw,
 }
 
 // Step 4: the nodes that did not converge, by the FP64 LU. The chunk's other nodes are
-// done, so the FP64 matrices take the slots' place.
-__global__ void __launch_bounds__(THREADS, 2) k_mixed_fallback(MixedArgs a, size_t bytes_per_cta) {
+// done, so the FP64 matrices take the slots' place. One such node of order 1024 is 0.36 s of an
+// SM, and nothing else runs meanwhile; so as long as there are few of them (at most `few`, which
+// leaves two CTAs per SM) the CTAs of a cluster share one (0.07 s), and else, where all SMs are
+// busy anyway, a CTA has one of its own, without barriers across SMs. The two kernels of a chunk
+// read the number of such nodes and one of them returns at once. Both round alike.
+template <bool CLUSTER>
+__global__ void __launch_bounds__(THREADS, 2) k_mixed_fallback(MixedArgs a, size_t bytes, int size, int few) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   FallbackSmem& sm = *reinterpret_cast<FallbackSmem*>(smem_raw);
   NodeCtx& c = sm.c;
   const int total = a.ctl[MIXED_CTL_FALLBACK_COUNT];
-  if (total == 0) return;
+  if (total == 0 || (total <= few) != CLUSTER || *reinterpret_cast<volatile int32_t*>(a.err)) return;
   PhaseClock pc(a.phase ? a.phase + (size_t)blockIdx.x * PMCIM_PHASES : nullptr);
   const unsigned long long t_start = global_ns();
-  for (;;) {
-    const int k = next_index(a, MIXED_CTL_FALLBACK, total, c);
-    if (k < 0) break;
+  const int rank = CLUSTER ? cluster_rank() : 0, slot = (int)blockIdx.x / size, slots = (int)gridDim.x / size;
+  for (int it_no = slot;; it_no += slots) {
+    int k = it_no;
+    if (!CLUSTER) k = next_index(a, MIXED_CTL_FALLBACK, total, c);
+    if (k < 0 || k >= total) break;
     const int q = a.fallback[k];
     NodeItem it;
     RegionDev rg;
@@ -779,29 +788,39 @@ __global__ void __launch_bounds__(THREADS, 2) k_mixed_fallback(MixedArgs a, size
     const ProblemDev& P = c.P;
     const int n = P.n, l = P.l;
     const size_t nn = (size_t)n * n, nl = (size_t)n * l;
-    double2* M64 = reinterpret_cast<double2*>(a.work + (size_t)blockIdx.x * bytes_per_cta);
+    double2* M64 = reinterpret_cast<double2*>(a.work + (size_t)slot * bytes);
     int* piv = reinterpret_cast<int*>(M64 + nn + nl);
     double2* X = a.X + rg.x_off + (size_t)it.j * nl;
     if (P.bie) {  // T(z_j) as k_bie_assemble left it
       const double2* T64 = a.t64 + (size_t)q * a.t64_stride;
-      if (mixed_column_only(a, P)) {
-        for (int col = 0; col < n; ++col)
-          for (int row = gtid(); row < n; row += THREADS)
-            M64[(size_t)col * n + row] = T64[row >= col ? row - col : row - col + n];
-      } else {
-        for (size_t e = gtid(); e < nn; e += THREADS) M64[e] = T64[e];
-      }
+      const bool column = mixed_column_only(a, P);
+      for (int col = rank; col < n; col += size)
+        for (int row = gtid(); row < n; row += THREADS)
+          M64[(size_t)col * n + row] =
+              T64[!column ? (size_t)col * n + row : (size_t)(row >= col ? row - col : row - col + n)];
     } else {
-      assemble(c, M64);
+      assemble(c, M64, rank, size);
     }
-    for (size_t e = gtid(); e < nl; e += THREADS) M64[nn + e] = P.V[e];
-    gsync();
-    MixedState st = a.state[q];
-    st.info = cta_lu(M64, n, n + l, piv, sm.lu64);
-    cta_back_blocked(M64, n, l, sm.lu64);
-    for (size_t e = gtid(); e < nl; e += THREADS) X[e] = M64[nn + e];
-    if (gtid() == 0) finish_node(a, rg, it, st, false);
+    for (size_t e = (size_t)rank * THREADS + gtid(); e < nl; e += (size_t)size * THREADS) M64[nn + e] = P.V[e];
+    int info;
+    if (CLUSTER) {
+      cluster_sync();
+      info = cluster_lu(M64, n, n + l, piv, piv + n, sm.lu64, sm.swaps, rank, size);
+    } else {
+      gsync();
+      info = cta_lu(M64, n, n + l, piv, sm.lu64);
+    }
+    // each CTA its share of the columns
+    const int c0 = l * rank / size, c1 = l * (rank + 1) / size;
+    if (c1 > c0) cta_back_blocked(M64, n, c1 - c0, sm.lu64, c0);
+    for (size_t e = (size_t)n * c0 + gtid(); e < (size_t)n * c1; e += THREADS) X[e] = M64[nn + e];
+    if (gtid() == 0 && rank == 0) {
+      MixedState st = a.state[q];
+      st.info = info;
+      finish_node(a, rg, it, st, false);
+    }
     pc.mark(PH_FALLBACK);
+    if (CLUSTER) cluster_sync();  // the matrix is no longer read
   }
   pc.wall(t_start);
 }
@@ -816,7 +835,7 @@ size_t mixed_slot_bytes(int n, int l) {
 }
 // Bytes a slot area needs at the least: one FP64 fallback.
 size_t mixed_fallback_bytes(int n, int l) {
-  return (((size_t)n * (n + l) * sizeof(double2) + (size_t)n * sizeof(int)) + 255) & ~(size_t)255;
+  return (((size_t)n * (n + l) * sizeof(double2) + (size_t)(n + 1) * sizeof(int)) + 255) & ~(size_t)255;
 }
 
 namespace {
@@ -844,8 +863,10 @@ cudaError_t prepare_factor_mixed() {
   e = cudaFuncSetAttribute(k_mixed_solve<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            (int)(sizeof(SolveSmem<false>) + kSolveYBytes));
   if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(k_mixed_fallback, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(FallbackSmem));
-  if (e != cudaSuccess) return e;
+  for (const void* f : {(const void*)k_mixed_fallback<false>, (const void*)k_mixed_fallback<true>}) {
+    e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(FallbackSmem));
+    if (e != cudaSuccess) return e;
+  }
   return prepare_oz_refine();
 }
 
@@ -899,13 +920,35 @@ cudaError_t launch_factor_solve_mixed(const MixedArgs& a, int sms, cudaStream_t 
     else k_mixed_solve<false><<<grid(3), THREADS, sizeof(SolveSmem<false>) + y, s>>>(a, sw, y);
     ++*launched;
   }
-  if (a.max_sweeps > 0) {
+  if (a.max_sweeps > 0 && !a.border) {
     const size_t per = mixed_fallback_bytes(a.max_n, a.max_l);
-    size_t g = a.work_bytes / per;
-    if (g < 1) return cudaErrorInvalidValue;
-    if (g > (size_t)grid(2)) g = (size_t)grid(2);
-    k_mixed_fallback<<<(unsigned)g, THREADS, sizeof(FallbackSmem), s>>>(a, per);
-    ++*launched;
+    const size_t mats = a.work_bytes / per;
+    if (mats < 1) return cudaErrorInvalidValue;
+    // CTAs of a cluster: a power of two that leaves each 16 rows
+    int size = 1;
+    while (size < 8 && 32 * size <= a.max_n) size *= 2;
+    const int few = size > 1 ? (int)std::min<size_t>(mats, (size_t)(2 * sms / size)) : 0;
+    if (few > 0) {
+      cudaLaunchAttribute at;
+      at.id = cudaLaunchAttributeClusterDimension;
+      at.val.clusterDim.x = (unsigned)size;
+      at.val.clusterDim.y = at.val.clusterDim.z = 1;
+      cudaLaunchConfig_t cfg = {};
+      cfg.gridDim = dim3((unsigned)(std::min(few, a.count) * size));
+      cfg.blockDim = dim3(THREADS);
+      cfg.dynamicSmemBytes = sizeof(FallbackSmem);
+      cfg.stream = s;
+      cfg.attrs = &at;
+      cfg.numAttrs = 1;
+      e = cudaLaunchKernelEx(&cfg, k_mixed_fallback<true>, a, per, size, few);
+      if (e != cudaSuccess) return e;
+      ++*launched;
+    }
+    if (few < a.count) {
+      const size_t g = std::min(mats, (size_t)grid(2));
+      k_mixed_fallback<false><<<(unsigned)g, THREADS, sizeof(FallbackSmem), s>>>(a, per, 1, few);
+      ++*launched;
+    }
   }
   return cudaGetLastError();
 }
