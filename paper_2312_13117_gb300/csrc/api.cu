@@ -113,9 +113,9 @@ constexpr size_t kMaxPmcimaRegions = size_t(1) << 20;
 // this fraction of |X|: 1e-11 keeps Beyn's eigenvalues within about 1e-14 of
 // the FP64 ones on the delay workload (simulated FP32 LU + FP64 refinement).
 constexpr double kIrTol = 1e-11;
-// Default limits of the precision-form kernel's bounded waits (clock64 cycles):
-// a tensor-core commit (about half a second at 2 GHz) and a hand-off between its
-// thread groups (about 16 s, longer than any node at n <= 4096).
+// Default limits of the precision-form kernels' bounded waits (clock64 cycles): a
+// tensor-core commit (about half a second at 2 GHz), and a hand-off between the
+// residual kernel's warps (about 16 s, longer than any launch of it at n <= 4096).
 constexpr long long kTcWaitCycles = 1ll << 30;
 constexpr long long kHandoffWaitCycles = 1ll << 35;
 std::mutex g_wait_mu;
@@ -537,9 +537,11 @@ void plan_mixed(Workspace& ws, const std::vector<ProblemDev>& pd, const std::vec
       mp->ubase.push_back(base);
       base += u;
     }
-    // the slots, and in their place the FP64 matrices of as many nodes as are solved again at a time
-    const size_t fb = mixed_fallback_bytes(ch.max_n, ch.max_l);
-    ch.work = std::max(ch.count * slot, fb * std::max<size_t>(1, std::min({ch.count, 2 * (size_t)sms, budget / fb})));
+    // the slots, and in their place the FP64 matrices of as many nodes as are solved again at a
+    // time (as far as the budget goes)
+    const size_t fb = mixed_fallback_bytes(ch.max_n, ch.max_l), beside = ch.count * (per - slot);
+    const size_t mats = std::min({ch.count, 2 * (size_t)sms, budget > beside ? (budget - beside) / fb : 0});
+    ch.work = std::max(ch.count * slot, fb * std::max<size_t>(1, mats));
     ch.t64_off = align(ch.work);
     ch.ysl_off = align(ch.t64_off + ch.count * ch.t64_stride * sizeof(double2));
     ch.tdig_off = align(ch.ysl_off + ch.count * ch.ysl_stride);
