@@ -40,6 +40,9 @@ SM_MAX_MHZ = 2070.0
 # DRAM bytes per node of k_factor_solve_fp64, from one ncu capture of a 64-node launch at n = 1024, l = 16
 # (dram__bytes_read.sum + dram__bytes_write.sum = 15.16 + 13.45 GB); scaled to a launch by its node count.
 FACTOR_FP64_TRAFFIC_PER_NODE = 28.61e9 / 64
+# DRAM bytes of the 3xTF32 form's kernels in one ncu capture of 320 nodes at n = 1024, l = 16 (two dense
+# terms): per node (k_mixed_factor and the first k_mixed_solve) and per sweep of a node
+TF32X3_TRAFFIC_PER_NODE, TF32X3_TRAFFIC_PER_SWEEP = 87.88e9 / 320, 6.03e9 / 320
 # FP32 pipe: 128 FFMA / SM / clock (measured 73.3 TFLOP/s at ~2.0 GHz); at the 2.07 GHz maximum:
 FP32_PEAK_TFLOPS = 128 * 2 * SM_COUNT * SM_MAX_MHZ * 1e6 / 1e12
 
@@ -1057,7 +1060,10 @@ def main():
                     "achieved": ach, "peak": BF16_SUSTAINED_TFLOPS, "unit": "TFLOP/s (BF16-equivalent)",
                     "frac": (ach / BF16_SUSTAINED_TFLOPS) if ach else None,
                     "peak_source": "MEASURED_PEAKS.json bf16_tflops_sustained; TF32 flops x 2.25/1.1",
-                    "traffic": None, "traffic_note": "no ncu capture of the whole form at this size",
+                    "traffic": ((TF32X3_TRAFFIC_PER_NODE * msolves + TF32X3_TRAFFIC_PER_SWEEP * aggm["ir_sweeps"])
+                                / max(1, fm["launches"]) if name == "tf32x3" else None),
+                    "traffic_note": ("ncu DRAM bytes of a 320-node capture at n = 1024, l = 16, scaled by nodes and "
+                                     "sweeps per launch" if name == "tf32x3" else "no ncu capture of this form"),
                     "residual_bf16_tflops": res_bf16 / t_s / 1e12 if t_s > 0 else None,
                     "lu_tf32_tflops": lu_tf32 / t_s / 1e12 if t_s > 0 else None,
                     "lu_bf16_tflops": lu_bf16 / t_s / 1e12 if t_s > 0 else None,

@@ -158,11 +158,14 @@ typedef struct {
      formed. 0 (default): on the tensor cores, from exact BF16 digits of the
      coefficients and of f_k(z_j) X (7 digits of 7 bits each per number, the
      digit products accumulated exactly in FP32 and combined in FP64; about the
-     accuracy of an FP64 product, see pmcim_residual). 1: on the FP64 pipe. */
+     accuracy of an FP64 product, see pmcim_residual; a boundary-integral term's
+     matrix and X in 8 digits, no less accurate than FP64). 1: on the FP64 pipe. */
   int32_t residual_fp64;
   /* FP64 node kernel: the trailing update's tile, 32 (32 x 32, less padding on
      small matrices) or 64 (64 x 64). 0 (default): 64, or under PMCIM_PREC_AUTO
-     the autotuner's choice per (n bucket, l, dense terms), timed up to n = 256. */
+     the autotuner's choice per (n bucket, l, dense terms), timed up to n = 256.
+     Orders that fit shared memory with their probe columns (up to about 118) are
+     factored there in tiles of their own, whatever this says. */
   int32_t fp64_tile;
 } pmcim_options;
 
@@ -421,8 +424,8 @@ typedef struct {
   /* precision form, with timing on: SM clock cycles summed over the CTAs of its
      kernels per step: assembly, LU panels, first solve, residual, correction
      solves, FP64 fallback, node set-up, LU triangular solves (U12), LU trailing
-     updates, 2 unused, the CTAs' lifetimes in ns (globaltimer, summed), the LU
-     panels' row interchanges on the columns outside the panel; 3 unused */
+     updates, 2 unused, the CTAs' lifetimes in ns (globaltimer, summed); 4 unused
+     (row interchanges are part of the panels and triangular solves) */
   double mixed_phase_cycles[PMCIM_PHASE_COUNT];
 } pmcim_profile;
 

@@ -11,8 +11,8 @@
 // The residual V - T(z_j) X on the FP64 unit is 8 n^2 l operations a sweep, more than the
 // whole assembly of a circulant node. As digits it is tensor work like that of the other
 // problems (oz_refine.cu); making the digits is integer arithmetic on the entries' bits.
-// Measured on whole calls with FP32 LUs, n = 256, l = 8: a circle, 6400 nodes, 118 -> 40 ms;
-// an ellipse, 768 nodes, 61.4 -> 20.2 ms.
+// Measured on whole calls with FP32 LUs, n = 256, l = 8: a circle, 6400 nodes, 118 -> 46.8 ms;
+// an ellipse, 768 nodes, 63.2 -> 23.2 ms.
 #include "ozaki.cuh"
 
 namespace {

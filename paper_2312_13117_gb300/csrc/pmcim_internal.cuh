@@ -280,7 +280,6 @@ struct MixedState {
   int32_t info;    // 0, or 1 + first zero-pivot column of the FP32 LU
   int32_t sweeps;  // refinement sweeps run
   int32_t lost;    // MIXED_LOST_*: a tensor-core wait ran out
-  int32_t pad;
 };
 constexpr int MIXED_LOST_LU = 1, MIXED_LOST_RESIDUAL = 2;
 // ctl: work counters, active nodes per sweep, then the column groups per sweep and problem
@@ -366,8 +365,7 @@ __device__ __forceinline__ int* mixed_tiles(const MixedArgs& a, bool bie) {
 // Phase-clock slots (PMCIM_PHASES): SM cycles summed over CTAs, by step.
 enum { PH_ASSEMBLE = 0, PH_PANEL = 1, PH_FIRST_SOLVE = 2, PH_RESIDUAL = 3, PH_CORRECTION = 4, PH_FALLBACK = 5,
        PH_SETUP = 6, PH_TRSM = 7, PH_UPDATE = 8,
-       PH_CTA_WALL_NS = 11,  // ns of CTA lifetime, not cycles
-       PH_SWAPS = 12 };      // the panel's row interchanges on the columns outside it
+       PH_CTA_WALL_NS = 11 };  // ns of CTA lifetime, not cycles
 __device__ __forceinline__ unsigned long long global_ns() {
   unsigned long long t;
   asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));

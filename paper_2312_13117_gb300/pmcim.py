@@ -188,10 +188,10 @@ def pmcim_profile_read() -> dict:
     tot = sum(cyc)
     if tot > 0:
         names = ["assemble", "lu_panel", "first_solve", "residual_fp64", "correction_solve", "fp64_fallback",
-                 "node_setup", "lu_trsm", "lu_update", "unused9", "unused10", "cta_wall", "lu_swaps",
+                 "node_setup", "lu_trsm", "lu_update", "unused9", "unused10", "cta_wall", "unused12",
                  "unused13", "unused14", "unused15"]
         share = {nm: c / tot for nm, c in zip(names, cyc) if c > 0}
-        share["lu_fp32"] = sum(share.get(k, 0.0) for k in ("lu_panel", "lu_swaps", "lu_trsm", "lu_update"))
+        share["lu_fp32"] = sum(share.get(k, 0.0) for k in ("lu_panel", "lu_trsm", "lu_update"))
         out["factor_fp32"]["phase_share"] = share
         out["factor_fp32"]["phase_cycles"] = {nm: c for nm, c in zip(names, cyc) if c > 0}
         if wall_ns > 0:
